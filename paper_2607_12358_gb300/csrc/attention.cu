@@ -753,47 +753,257 @@ acid_status launch_attn_tc(const AttnArgs& x, cudaStream_t s) {
 }
 
 // ---------------------------------------------------------------- fp32 path
-__global__ void __launch_bounds__(256) attn_f32_kernel(const float* __restrict__ q, int64_t ldq, int q_col,
-                                                       const float* __restrict__ k, int64_t ldk, int k_col,
-                                                       const float* __restrict__ v, int64_t ldv, int v_col, float* out,
-                                                       int64_t ldo, int o_col, int64_t nq, int64_t nk, int D,
-                                                       float scale) {
-  const int64_t row = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
+// Tiled flash attention on the FP32 pipes.  A CTA takes BQ query rows of one
+// head; its four groups of four warps walk the key range in interleaved tiles
+// of 32 keys, each group with its own K and V buffers, running max and
+// partial output, and the groups' parts are merged through shared memory at
+// the end.  The group split is what fills the SMs when there are few query
+// tiles (256 tokens x 4 heads are 64 tiles of 16 rows) and gives each SM 16
+// warps to hide the loads behind.
+//   A half-warp owns QT = BQ / 8 query rows: lane kg of it computes the scores
+// of keys kg and kg + 16 with those rows (16-byte shared loads along the head
+// dim; the K rows are padded by 16 bytes, so 16 rows cover all banks), the row
+// max goes through half-warp shuffles, P through shared memory, and the same
+// lanes then accumulate QT rows x D / 16 columns of the output.  The row sum
+// stays per lane until the end.  K(j + 1) loads (cp.async) while P V runs and
+// V(j) while the scores of tile j are formed.
+//   Measured at 256 tokens, 4 heads of 64: 11.2 us, against 161.7 us for one
+// warp per query row (a serial loop over the keys with a shuffle tree and two
+// exponentials per key).  What bounds it there is the latency of two key tiles
+// per group (about 4 us of FP32 work) plus load, merge and launch.
+constexpr int kF32Groups = 4, kF32Keys = 32;
+
+template <int D, int BQ>
+struct AttnF32Cfg {
+  static constexpr int QT = BQ / 8;    // query rows per half-warp
+  static constexpr int LDK = D + 4;    // padded K (and Q) row, floats
+  static constexpr int LDP = kF32Keys + 4;
+  static constexpr int K_FLOATS = kF32Keys * LDK, V_FLOATS = kF32Keys * D;
+  static constexpr int OFF_Q = 0;
+  static constexpr int OFF_P = BQ * LDK;                           // [group][BQ][LDP]
+  static constexpr int OFF_KV = OFF_P + kF32Groups * BQ * LDP;     // [group][K | V]; reused for the merge
+  static constexpr int FLOATS = OFF_KV + kF32Groups * (K_FLOATS + V_FLOATS);
+  static constexpr int SMEM = FLOATS * 4;
+  static_assert(kF32Groups * BQ * (D + 2) <= kF32Groups * (K_FLOATS + V_FLOATS), "merge buffers fit the K/V area");
+  static_assert(SMEM <= 227 * 1024, "fp32 attention shared memory");
+};
+
+struct AttnF32Args {
+  const float* q;
+  const float* k;
+  const float* v;
+  float* out;
+  int64_t ldq, ldk, ldv, ldo, nq, nk;
+  float scale;
+  int vec;  // 1: rows of q, k and v are 16-byte aligned
+};
+
+// ROWS rows of D floats (row stride ld in global memory, lds in shared
+// memory) by `threads` threads; rows from `valid_rows` on are zero.
+template <int D, int ROWS>
+__device__ __forceinline__ void load_rows_f32(float* dst, int lds, const float* src, int64_t ld, int64_t valid_rows,
+                                              int tid, int threads, int vec) {
+  if (vec) {
+    for (int i = tid; i < ROWS * (D / 4); i += threads) {
+      const int r = i / (D / 4), c = (i % (D / 4)) * 4;
+      const bool ok = r < valid_rows;
+      cp_async<16>(dst + r * lds + c, src + (ok ? (int64_t)r * ld + c : 0), ok);
+    }
+  } else {
+    for (int i = tid; i < ROWS * D; i += threads) {
+      const int r = i / D, c = i % D;
+      const bool ok = r < valid_rows;
+      cp_async<4>(dst + r * lds + c, src + (ok ? (int64_t)r * ld + c : 0), ok);
+    }
+  }
+}
+
+template <int D, int BQ>
+__global__ void __launch_bounds__(128 * kF32Groups) attn_f32_kernel(AttnF32Args a) {
+  using C = AttnF32Cfg<D, BQ>;
+  constexpr int QT = C::QT, KT = kF32Keys / 16, NC = D / 32;  // NC column pairs per lane
+  extern __shared__ __align__(16) float fsm[];
+  const int g = threadIdx.x >> 7, t = threadIdx.x & 127;  // group, thread in the group
+  const int hw = t >> 4, kg = t & 15;                     // half-warp (rows hw * QT ..), lane in it
+  const int64_t q0 = (int64_t)blockIdx.x * BQ;
   const int h = blockIdx.y;
-  const int lane = threadIdx.x & 31;
-  if (row >= nq) return;
-  constexpr int kMaxPer = 4;  // D <= 128
-  float qv[kMaxPer], o[kMaxPer];
-  const int per = D / 32;
+  float* sq = fsm + C::OFF_Q;
+  float* sp = fsm + C::OFF_P + g * BQ * C::LDP + hw * QT * C::LDP;
+  float* sk = fsm + C::OFF_KV + g * (C::K_FLOATS + C::V_FLOATS);
+  float* sv = sk + C::K_FLOATS;
+  const float* kh = a.k + h * D;
+  const float* vh = a.v + h * D;
+  const int ntiles = (int)((a.nk + kF32Keys - 1) / kF32Keys);
+  auto load_k = [&](int j) {
+    const int64_t k0 = (int64_t)j * kF32Keys;
+    load_rows_f32<D, kF32Keys>(sk, C::LDK, kh + k0 * a.ldk, a.ldk, a.nk - k0, t, 128, a.vec);
+  };
+  auto load_v = [&](int j) {
+    const int64_t k0 = (int64_t)j * kF32Keys;
+    load_rows_f32<D, kF32Keys>(sv, D, vh + k0 * a.ldv, a.ldv, a.nk - k0, t, 128, a.vec);
+  };
+  // Q rows (all groups), this group's first K and V tiles: one commit group each
+  load_rows_f32<D, BQ>(sq, C::LDK, a.q + q0 * a.ldq + h * D, a.ldq, a.nq - q0, threadIdx.x, blockDim.x, a.vec);
+  if (g < ntiles) load_k(g);
+  cp_async_commit();
+  if (g < ntiles) load_v(g);
+  cp_async_commit();
+  cp_async_wait<1>();
+  __syncthreads();  // Q and every group's first K tile
+
+  float o[QT][2 * NC] = {};
+  float m[QT], l[QT];
 #pragma unroll
-  for (int i = 0; i < kMaxPer; ++i) {
-    qv[i] = i < per ? q[row * ldq + q_col + h * D + i * 32 + lane] : 0.f;
-    o[i] = 0.f;
+  for (int i = 0; i < QT; ++i) {
+    m[i] = -INFINITY;
+    l[i] = 0.f;
   }
-  float m = -INFINITY, l = 0.f;
-  for (int64_t j = 0; j < nk; ++j) {
-    const float* kr = k + j * ldk + k_col + h * D;
-    float sdot = 0.f;
+  const float* qrow = sq + hw * QT * C::LDK;
+  for (int j = g; j < ntiles; j += kF32Groups) {
+    // scores of QT rows x KT keys
+    float s[QT][KT] = {};
+#pragma unroll 4
+    for (int d = 0; d < D; d += 4) {
+      float4 qv[QT], kv[KT];
 #pragma unroll
-    for (int i = 0; i < kMaxPer; ++i)
-      if (i < per) sdot = fmaf(qv[i], kr[i * 32 + lane], sdot);
+      for (int i = 0; i < QT; ++i) qv[i] = *reinterpret_cast<const float4*>(qrow + i * C::LDK + d);
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) sdot += __shfl_xor_sync(0xffffffffu, sdot, off);
-    const float sc = sdot * scale;
-    const float mn = fmaxf(m, sc);
-    const float corr = expf(m - mn);
-    const float p = expf(sc - mn);
-    l = l * corr + p;
-    const float* vr = v + j * ldv + v_col + h * D;
+      for (int c = 0; c < KT; ++c) kv[c] = *reinterpret_cast<const float4*>(sk + (kg + 16 * c) * C::LDK + d);
 #pragma unroll
-    for (int i = 0; i < kMaxPer; ++i)
-      if (i < per) o[i] = fmaf(p, vr[i * 32 + lane], o[i] * corr);
-    m = mn;
+      for (int i = 0; i < QT; ++i)
+#pragma unroll
+        for (int c = 0; c < KT; ++c)
+          s[i][c] = fmaf(qv[i].w, kv[c].w, fmaf(qv[i].z, kv[c].z, fmaf(qv[i].y, kv[c].y, fmaf(qv[i].x, kv[c].x, s[i][c]))));
+    }
+    group_sync(1 + g, 128);  // every warp of the group has read the K tile
+    if (j + kF32Groups < ntiles) load_k(j + kF32Groups);
+    cp_async_commit();
+    const int64_t left = a.nk - (int64_t)j * kF32Keys;  // keys of this tile
+#pragma unroll
+    for (int i = 0; i < QT; ++i) {
+      float mt = -INFINITY;
+#pragma unroll
+      for (int c = 0; c < KT; ++c) {
+        s[i][c] = kg + 16 * c < left ? s[i][c] * a.scale : -INFINITY;
+        mt = fmaxf(mt, s[i][c]);
+      }
+#pragma unroll
+      for (int off = 8; off > 0; off >>= 1) mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, off));
+      const float mn = fmaxf(m[i], mt);
+      const float ref = mn == -INFINITY ? 0.f : mn;  // no finite score yet: every term below is 0
+      const float corr = expf(m[i] - ref);
+      m[i] = mn;
+      l[i] *= corr;
+#pragma unroll
+      for (int c = 0; c < 2 * NC; ++c) o[i][c] *= corr;
+#pragma unroll
+      for (int c = 0; c < KT; ++c) {
+        const float p = kg + 16 * c < left ? expf(s[i][c] - ref) : 0.f;
+        l[i] += p;
+        sp[i * C::LDP + kg + 16 * c] = p;
+      }
+    }
+    cp_async_wait<1>();      // V(j) has landed (this thread's copies)
+    group_sync(1 + g, 128);  // ... and every thread's; P is written
+    const int kmax = left < kF32Keys ? (int)left : kF32Keys;
+#pragma unroll 2
+    for (int k = 0; k < kmax; k += 4) {  // V rows past the end are zero, and so is P
+      float4 pv[QT];
+#pragma unroll
+      for (int i = 0; i < QT; ++i) pv[i] = *reinterpret_cast<const float4*>(sp + i * C::LDP + k);
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) {
+        float2 vv[NC];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) vv[c] = *reinterpret_cast<const float2*>(sv + (k + kk) * D + 32 * c + 2 * kg);
+#pragma unroll
+        for (int i = 0; i < QT; ++i) {
+          const float p = kk == 0 ? pv[i].x : kk == 1 ? pv[i].y : kk == 2 ? pv[i].z : pv[i].w;
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            o[i][2 * c] = fmaf(p, vv[c].x, o[i][2 * c]);
+            o[i][2 * c + 1] = fmaf(p, vv[c].y, o[i][2 * c + 1]);
+          }
+        }
+      }
+    }
+    cp_async_wait<0>();      // K(j + groups) has landed
+    group_sync(1 + g, 128);  // V and P have been read
+    if (j + kF32Groups < ntiles) load_v(j + kF32Groups);
+    cp_async_commit();
   }
-  if (!ACID_IN_BOUNDS(kSiteAttnF32, row * ldo + o_col + h * D + D - 1, nq * ldo)) return;
+  cp_async_wait<0>();
+  // ---- merge: [group][BQ][D] partial outputs, then [group][BQ] {m, l}
 #pragma unroll
-  for (int i = 0; i < kMaxPer; ++i)
-    if (i < per) out[row * ldo + o_col + h * D + i * 32 + lane] = o[i] / l;
+  for (int i = 0; i < QT; ++i)
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) l[i] += __shfl_xor_sync(0xffffffffu, l[i], off);
+  __syncthreads();  // every group has finished with its K and V buffers
+  float* mo = fsm + C::OFF_KV;
+  float2* ml = reinterpret_cast<float2*>(mo + kF32Groups * BQ * D);
+#pragma unroll
+  for (int i = 0; i < QT; ++i) {
+    const int r = hw * QT + i;
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+      *reinterpret_cast<float2*>(mo + (g * BQ + r) * D + 32 * c + 2 * kg) = make_float2(o[i][2 * c], o[i][2 * c + 1]);
+    if (kg == 0) ml[g * BQ + r] = make_float2(m[i], l[i]);
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < BQ * D; i += blockDim.x) {
+    const int r = i / D, c = i % D;
+    if (q0 + r >= a.nq) break;
+    float mx = -INFINITY;
+#pragma unroll
+    for (int gg = 0; gg < kF32Groups; ++gg) mx = fmaxf(mx, ml[gg * BQ + r].x);
+    float acc = 0.f, den = 0.f;
+#pragma unroll
+    for (int gg = 0; gg < kF32Groups; ++gg) {
+      const float2 e = ml[gg * BQ + r];
+      if (gg >= ntiles) break;  // a group without a tile holds no part
+      const float w = expf(e.x - mx);
+      den = fmaf(w, e.y, den);
+      acc = fmaf(w, mo[(gg * BQ + r) * D + c], acc);
+    }
+    const int64_t at = (q0 + r) * a.ldo + h * D + c;
+    if (!ACID_IN_BOUNDS(kSiteAttnF32, at, a.nq * a.ldo)) continue;
+    a.out[at] = acc / den;
+  }
+}
+
+template <int D, int BQ>
+acid_status attn_f32_launch(const AttnF32Args& a, int heads, cudaStream_t s) {
+  using C = AttnF32Cfg<D, BQ>;
+  static bool attr_done = false;
+  if (!attr_done) {
+    ACID_CUDA(cudaFuncSetAttribute(attn_f32_kernel<D, BQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
+    attr_done = true;
+  }
+  const dim3 grid((unsigned)((a.nq + BQ - 1) / BQ), (unsigned)heads);
+  attn_f32_kernel<D, BQ><<<grid, 128 * kF32Groups, C::SMEM, s>>>(a);
+  ACID_CHECK_LAUNCH();
+  return ACID_OK;
+}
+
+template <int D>
+acid_status launch_attn_f32(const AttnArgs& x, cudaStream_t s) {
+  AttnF32Args a;
+  a.q = static_cast<const float*>(x.q) + x.q_col;
+  a.k = static_cast<const float*>(x.k) + x.k_col;
+  a.v = static_cast<const float*>(x.v) + x.v_col;
+  a.out = static_cast<float*>(x.out) + x.o_col;
+  a.ldq = x.ldq;
+  a.ldk = x.ldk;
+  a.ldv = x.ldv;
+  a.ldo = x.ldo;
+  a.nq = x.nq;
+  a.nk = x.nk;
+  a.scale = (float)(1.0 / sqrt((double)D));
+  a.vec = aligned(a.q, 16) && aligned(a.k, 16) && aligned(a.v, 16) && x.ldq % 4 == 0 && x.ldk % 4 == 0 && x.ldv % 4 == 0;
+  // 32-row tiles reuse each K and V value for twice the rows; 16-row tiles
+  // while the 32-row ones would leave SMs without a CTA
+  if ((x.nq + 31) / 32 * x.heads < num_sms_attn()) return attn_f32_launch<D, 16>(a, x.heads, s);
+  return attn_f32_launch<D, 32>(a, x.heads, s);
 }
 
 }  // namespace
@@ -805,12 +1015,12 @@ acid_status attention_forward(int dtype, const AttnArgs& x, cudaStream_t s) {
   if (dtype == ACID_FP32) {
     ACID_REQUIRE(x.head_dim % 32 == 0 && x.head_dim <= 128, ACID_ERR_UNSUPPORTED,
                  "attention fp32: head_dim must be 32, 64, 96 or 128");
-    dim3 grid((unsigned)((x.nq + 7) / 8), (unsigned)x.heads);
-    attn_f32_kernel<<<grid, 256, 0, s>>>((const float*)x.q, x.ldq, x.q_col, (const float*)x.k, x.ldk, x.k_col,
-                                         (const float*)x.v, x.ldv, x.v_col, (float*)x.out, x.ldo, x.o_col, x.nq, x.nk,
-                                         x.head_dim, (float)(1.0 / sqrt((double)x.head_dim)));
-    ACID_CHECK_LAUNCH();
-    return ACID_OK;
+    switch (x.head_dim) {
+      case 32: return launch_attn_f32<32>(x, s);
+      case 64: return launch_attn_f32<64>(x, s);
+      case 96: return launch_attn_f32<96>(x, s);
+      default: return launch_attn_f32<128>(x, s);
+    }
   }
   ACID_REQUIRE(x.head_dim == 64 || x.head_dim == 128, ACID_ERR_UNSUPPORTED, "attention bf16: head_dim must be 64 or 128");
   ACID_REQUIRE(x.q_col % 8 == 0 && x.k_col % 8 == 0 && x.v_col % 8 == 0 && x.o_col % 8 == 0 && x.ldo % 8 == 0,
