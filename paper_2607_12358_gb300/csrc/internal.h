@@ -63,9 +63,9 @@ constexpr size_t kSplitKScratchBytes = (size_t)80 * 256 * 256 * 4;
 acid_status linear_forward(int dtype, const void* A, int64_t lda, int64_t M, int K, const void* W,
                            int N, void* out, int64_t ldo, const Epilogue& epi, cudaStream_t s);
 
-// fp32 activations and output with fp32 or bf16 weights (FP32 pipes, fp32 accumulation)
-acid_status linear_forward_f32(const void* A, int64_t lda, int64_t M, int K, int w_dtype, const void* W, int N,
-                               void* out, int64_t ldo, const Epilogue& epi, cudaStream_t s);
+// fp32 operands and output (FP32 pipes, fp32 accumulation)
+acid_status linear_forward_f32(const void* A, int64_t lda, int64_t M, int K, const void* W, int N, void* out,
+                               int64_t ldo, const Epilogue& epi, cudaStream_t s);
 
 // ----------------------------------------------------------------- attention
 struct AttnArgs {

@@ -490,8 +490,9 @@ static acid_status patch_embed(const acid_model& m, const LoopWs& w, const float
     ACID_TRY(patchify_split(latent, w.tokens, m.latent_c, m.latent_f, m.latent_h, m.latent_w, m.pt, m.ph, m.pw, s));
     return linear_forward(ACID_BF16, w.tokens, 2 * sh.P, sh.N, (int)(2 * sh.P), w.patch_w2, sh.d, h_in, sh.d, e, s);
   }
+  ACID_REQUIRE(m.block.dtype == ACID_FP32, ACID_ERR_UNSUPPORTED, "patch embedding: bf16 needs P % 8 == 0");
   ACID_TRY(patchify(latent, ACID_FP32, w.tokens, m.latent_c, m.latent_f, m.latent_h, m.latent_w, m.pt, m.ph, m.pw, s));
-  return linear_forward_f32(w.tokens, sh.P, sh.N, (int)sh.P, m.block.dtype, m.patch.w, sh.d, h_in, sh.d, e, s);
+  return linear_forward_f32(w.tokens, sh.P, sh.N, (int)sh.P, m.patch.w, sh.d, h_in, sh.d, e, s);
 }
 
 // One branch's model evaluation at step st->step: Algorithm 1's decision,
