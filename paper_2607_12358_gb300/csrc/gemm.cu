@@ -1,15 +1,15 @@
 // Linear layers of the DiT block.
 //
-// bf16: persistent tcgen05 GEMMs.  A CTA (or, for N or K above 2048, a pair
-// of CTAs on two SMs with tcgen05.mma.cta_group::2) computes 128 x BN (pair:
-// 256 x 256) output tiles with the fp32 accumulator in tensor memory (TMEM),
-// double-buffered.  Warp 0 streams the A and B tiles with TMA (128-byte
-// swizzle) through a STAGES-deep mbarrier ring; warp 1 issues tcgen05.mma
-// from one thread; warps 2-9 read the accumulator back with tcgen05.ld (one
+// bf16: a persistent tcgen05 GEMM.  A pair of CTAs on two SMs
+// (tcgen05.mma.cta_group::2) computes 256 x bn output tiles with the fp32
+// accumulator in tensor memory (TMEM), double-buffered.  Warp 0 streams the A
+// and B tiles with TMA (128-byte swizzle) through an mbarrier ring; warp 1
+// issues tcgen05.mma; warps 2-9 read the accumulator back with tcgen05.ld (one
 // thread per output row) and apply the fused epilogue (bias, GELU-tanh, 3D
-// RoPE of q/k, gated or plain residual) before storing.  Long-K pair GEMMs
-// inside a block can finish their last round as split-K units (see
-// splitk_plan).
+// RoPE of q/k, gated or plain residual) before a TMA store.  A dual-stream
+// layer's text and video rows, with weights of their own, share a launch.
+// Long-K GEMMs inside a block can finish their last round as split-K units
+// (see splitk_plan).
 //
 // fp32: a register-tiled SIMT GEMM with the same epilogue (the fp32 mode's
 // 1e-4 tolerance rules out tf32 tensor cores).
@@ -29,6 +29,7 @@ namespace {
 struct EpiDev {
   int kind;
   const float* bias;
+  const float* bias_t;  // bias of the text rows' problem (dual-stream launches)
   const float* gate_v;
   const float* gate_t;
   int64_t gate_split;
@@ -45,6 +46,7 @@ EpiDev to_dev(const Epilogue& e) {
   EpiDev d;
   d.kind = e.kind;
   d.bias = e.bias;
+  d.bias_t = e.text_bias;
   d.gate_v = e.gate_video;
   d.gate_t = e.gate_text ? e.gate_text : e.gate_video;
   d.gate_split = e.gate_split;
@@ -139,29 +141,9 @@ __device__ __forceinline__ void epi_pair(const EpiDev& e, int64_t grow, int col,
 
 __host__ __device__ __forceinline__ bool epi_reads_res(int kind) { return kind == EPI_GATED_RES || kind == EPI_RES; }
 
-// ===========================================================================
-// tcgen05 GEMM (bf16 in, fp32 accumulate), persistent
-//
-// One CTA per SM walks output tiles (N fastest, so the CTAs running together
-// share A row blocks in L2 and the weight tiles stay L2-resident).  The TMEM
-// accumulator is double-buffered (2 x BN columns): the MMA warp fills buffer
-// b for tile i+1 while eight epilogue warps drain buffer b^1 of tile i.
-// ===========================================================================
-constexpr int BM = 128, BK = 64;
+constexpr int BM = 128, BK = 64;  // rows of A per CTA, depth of a k-step
 constexpr int kEpiWarps = 8;
 constexpr int kGemmThreads = 64 + 32 * kEpiWarps;
-
-template <int BN>
-struct TcCfg {
-  static constexpr int STAGES = BN == 256 ? 4 : (BN == 128 ? 6 : 8);
-  static constexpr int A_BYTES = BM * BK * 2;
-  static constexpr int B_BYTES = BN * BK * 2;
-  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int EPI_STAGE_FLOATS = 32 * 32;  // one 32x32 chunk per epilogue warp (swizzled units)
-  static constexpr int EPI_BYTES = kEpiWarps * EPI_STAGE_FLOATS * 4;
-  static constexpr int SMEM = STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 256;
-  static constexpr uint32_t TMEM_COLS = 2 * BN;
-};
 
 struct GemmDims {
   int64_t M;
@@ -169,71 +151,21 @@ struct GemmDims {
   void* out;
   int64_t ldo;
   int out_fp32;
-  // split-K launches of the pair kernel only: work unit = (tile, split);
-  // split s covers k-blocks [s kb_split, (s + 1) kb_split) and stores its
-  // raw fp32 accumulator at rows s m_pad + row of the partial buffer
+  // split-K launches only: work unit = (tile, split); split s covers k-blocks
+  // [s kb_split, (s + 1) kb_split) and stores its raw fp32 accumulator at
+  // rows s m_pad + row of the partial buffer
   int splits = 1, kb_split = 0;
   int64_t m_pad = 0;
+  // output columns per tile (a multiple of 32, at most 256) and the depth of
+  // the operand ring
+  int bn = 256, stages = 6;
+  // dual-stream launches: rows [0, l_text) are multiplied with the text
+  // weights, in mt_text row tiles of their own; 0: one problem
+  int l_text = 0, mt_text = 0;
+  // residual rows that overlap (row stride below N, as in a row repeated for
+  // every output row): not expressible as a tensor map, read with plain loads
+  int res_direct = 0;
 };
-
-// Epilogue of 32-row x 32-column accumulator chunks held by a warp (thread =
-// row after tcgen05.ld).  Each chunk is transposed through shared memory so
-// that every global access of the warp covers whole row segments: lane l
-// handles columns 4(l%8) .. 4(l%8)+3 of rows 4p + l/8, p = 0..7.  Residual
-// values of the next chunk are loaded while the current one is processed, so
-// each lane keeps up to 16 loads in flight.
-// R32: the residual is fp32 (else bf16); fixed per kernel so that a bf16
-// residual keeps two registers per row
-template <bool R32>
-struct ResChunk {
-  uint32_t w[8][R32 ? 4 : 2];  // residual of this lane's 4 columns on its 8 rows (bf16 pairs or fp32)
-  float bias[4], gv[4], gt[4];  // per-column bias and gates (video / text stream)
-};
-
-// Loads what the epilogue of the chunk at columns [col, col+4) needs from
-// global memory: the residual (for the residual kinds) and the per-column
-// bias and gates, through the read-only path for the vectors.  Called one
-// chunk ahead so that the loads overlap the previous chunk's work.
-template <int KIND, bool R32>
-__device__ __forceinline__ void load_chunk_inputs(const GemmDims& g, const EpiDev& e, int64_t row0, int col,
-                                                  ResChunk<R32>& rc) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    rc.bias[k] = e.bias ? __ldg(e.bias + col + k) : 0.f;
-    rc.gv[k] = KIND == EPI_GATED_RES ? __ldg(e.gate_v + col + k) : 0.f;
-    rc.gt[k] = KIND == EPI_GATED_RES ? __ldg(e.gate_t + col + k) : 0.f;
-  }
-  if constexpr (KIND == EPI_GATED_RES || KIND == EPI_RES) {
-#pragma unroll
-    for (int p = 0; p < 8; ++p) {
-      const int64_t row = row0 + 4 * p + (lane >> 3);
-      if (row >= g.M || !ACID_IN_BOUNDS(kSiteGemmResidual, row * e.ldr + col + 3, (g.M - 1) * e.ldr + g.N)) {
-        // computed but not stored by the epilogue
-#pragma unroll
-        for (int q = 0; q < (R32 ? 4 : 2); ++q) rc.w[p][q] = 0u;
-        continue;
-      }
-      if constexpr (R32) {
-        const uint4 t = *reinterpret_cast<const uint4*>(static_cast<const float*>(e.res) + row * e.ldr + col);
-        rc.w[p][0] = t.x; rc.w[p][1] = t.y; rc.w[p][2] = t.z; rc.w[p][3] = t.w;
-      } else {
-        const uint2 t = *reinterpret_cast<const uint2*>(static_cast<const __nv_bfloat16*>(e.res) + row * e.ldr + col);
-        rc.w[p][0] = t.x; rc.w[p][1] = t.y;
-      }
-    }
-  }
-}
-
-template <bool R32>
-__device__ __forceinline__ float res_value(const ResChunk<R32>& rc, int p, int k) {
-  if constexpr (R32) {
-    return __uint_as_float(rc.w[p][k]);
-  } else {
-    const uint32_t w = rc.w[p][k >> 1];
-    return (k & 1) ? bf16_hi(w) : bf16_lo(w);
-  }
-}
 
 // GELU (tanh form) of a packed pair, with the arithmetic of gelu_tanh<true>
 // done two lanes at a time: u = sqrt(2/pi) (x + 0.044715 x^3), out = h + h tanh(u)
@@ -249,167 +181,25 @@ __device__ __forceinline__ uint64_t gelu_x2(uint64_t x) {
   return f2_fma(h, t, h);
 }
 
-// The stage of one epilogue warp: 32 rows x 32 fp32 columns, row-major, the
-// eight 16-byte units of row r stored in the order u ^ (r & 7), so that both
-// the row-wise writes (lane = row) and the transposed reads (8 lanes per row)
-// touch every bank once per 128 bytes.
-__device__ __forceinline__ float4* stage_unit(float* stage, int row, int unit) {
-  return reinterpret_cast<float4*>(stage) + row * 8 + (unit ^ (row & 7));
-}
-
-// Output box of one chunk in the stage, as the tensor store reads it: 32 rows
-// x 32 columns, row-major.  fp32: 128-byte rows with the 128-byte swizzle
-// (16-byte unit u of row r at u ^ (r & 7)), the stage's own layout, so each
-// lane overwrites in place the 16 bytes it has just read.  bf16: 64-byte rows
-// with the 64-byte swizzle (unit u at u ^ ((r >> 1) & 3)); box row r lies in
-// stage row r / 2, which the warp has read by the time row group r / 4 is
-// written (row groups are written behind a __syncwarp).
-__device__ __forceinline__ void box_store_f32(float* stage, int rr, int lane, const float* v) {
-  *stage_unit(stage, rr, lane & 7) = make_float4(v[0], v[1], v[2], v[3]);
-}
-__device__ __forceinline__ void box_store_bf16(float* stage, int rr, int lane, const float* v) {
-  const int u = (lane & 7) >> 1;
-  uint8_t* p = reinterpret_cast<uint8_t*>(stage) + rr * 64 + ((u ^ ((rr >> 1) & 3)) << 4) + (lane & 1) * 8;
-  *reinterpret_cast<uint2*>(p) = make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
-}
-
-// Output stores of the epilogue: kinds without a residual write each chunk's
-// results back into the stage as the output box and hand it to one tensor
-// store (the TMA engine then writes the 2-4 KB box; rows past M and columns
-// past N are clipped by the tensor map).  The residual kinds keep a residual
-// prefetch of two chunks in registers and store directly from registers
-// (coalesced 8-16-byte stores per lane), which leaves them without spills at
-// the 168-register limit of ten warps.
+// Kinds whose epilogue reads no residual.
 template <int KIND>
-constexpr bool kTmaStore = !(KIND == EPI_GATED_RES || KIND == EPI_RES);
-
-// Epilogue of one 32-row x 32-column chunk held by a warp (thread = row, as
-// tcgen05.ld delivers it).  The chunk is transposed through the stage so that
-// each lane handles four columns of eight rows, then stored as above.  With
-// tensor stores the caller waits for the previous store to have read the
-// stage before calling again.
-template <int KIND, bool R32, bool O32>
-__device__ __forceinline__ void epilogue_chunk(const GemmDims& g, const EpiDev& e, const CUtensorMap* tmO,
-                                               float* stage, int64_t row0, int col0, const uint32_t* r,
-                                               const ResChunk<R32>& rc) {
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int u = 0; u < 8; ++u)
-    *stage_unit(stage, lane, u) = make_float4(__uint_as_float(r[4 * u]), __uint_as_float(r[4 * u + 1]),
-                                              __uint_as_float(r[4 * u + 2]), __uint_as_float(r[4 * u + 3]));
-  __syncwarp();
-  const int c = 4 * (lane & 7);
-  const int col = col0 + c;
-  // RoPE: the (cos, sin) of this lane's two pairs on its eight rows, all
-  // loaded through the read-only path before the row groups are processed
-  float2 rcs[KIND == EPI_ROPE_QKV ? 8 : 1][2];
-  if constexpr (KIND == EPI_ROPE_QKV) {
-    const int j0 = (col & (e.head_dim - 1)) >> 1;
-#pragma unroll
-    for (int p = 0; p < 8; ++p) {
-      const int64_t grow = row0 + 4 * p + (lane >> 3) + e.row_base;
-      rcs[p][0] = rcs[p][1] = make_float2(1.f, 0.f);
-      if (col < 2 * e.d && grow >= e.rope_first_video && row0 + 4 * p + (lane >> 3) < g.M) {
-        const RopePos pp = rope_pos(e.rope, (int)(grow - e.rope_first_video));
-#pragma unroll
-        for (int q = 0; q < 2; ++q)
-          if (rope_in_bounds(e.rope, rope_cs_ptr(e.rope, pp, j0 + q))) rcs[p][q] = __ldg(&rope_cs_ptr(e.rope, pp, j0 + q));
-      }
-    }
-  }
-  const uint64_t b01 = f2_pack(rc.bias[0], rc.bias[1]), b23 = f2_pack(rc.bias[2], rc.bias[3]);
-  // rows past M are computed like the others (from whatever the stage and
-  // residual registers hold); the tensor store clips them
-#pragma unroll
-  for (int p = 0; p < 8; ++p) {
-    const int rr = 4 * p + (lane >> 3);
-    const int64_t grow = row0 + rr + e.row_base;
-    const float4 sv = *stage_unit(stage, rr, lane & 7);
-    uint64_t v01 = f2_add(f2_pack(sv.x, sv.y), b01), v23 = f2_add(f2_pack(sv.z, sv.w), b23);
-    switch (KIND) {
-      case EPI_GELU:
-        v01 = gelu_x2(v01);
-        v23 = gelu_x2(v23);
-        break;
-      case EPI_ROPE_QKV: {
-        // (cos, sin) = (1, 0) on rows and columns that are not rotated; the
-        // four columns lie in one head (head_dim is a power of two)
-        float v[4];
-        f2_unpack(v01, v[0], v[1]);
-        f2_unpack(v23, v[2], v[3]);
-#pragma unroll
-        for (int k = 0; k < 4; k += 2) {
-          const float2 cs = rcs[p][k >> 1];
-          const float x0 = v[k], x1 = v[k + 1];
-          v[k] = x0 * cs.x - x1 * cs.y;
-          v[k + 1] = x0 * cs.y + x1 * cs.x;
-        }
-        v01 = f2_pack(v[0], v[1]);
-        v23 = f2_pack(v[2], v[3]);
-        break;
-      }
-      case EPI_GATED_RES: {
-        const bool text = grow < e.gate_split;
-        const uint64_t g01 = text ? f2_pack(rc.gt[0], rc.gt[1]) : f2_pack(rc.gv[0], rc.gv[1]);
-        const uint64_t g23 = text ? f2_pack(rc.gt[2], rc.gt[3]) : f2_pack(rc.gv[2], rc.gv[3]);
-        v01 = f2_fma(g01, v01, f2_pack(res_value(rc, p, 0), res_value(rc, p, 1)));
-        v23 = f2_fma(g23, v23, f2_pack(res_value(rc, p, 2), res_value(rc, p, 3)));
-        break;
-      }
-      case EPI_RES:
-        v01 = f2_add(v01, f2_pack(res_value(rc, p, 0), res_value(rc, p, 1)));
-        v23 = f2_add(v23, f2_pack(res_value(rc, p, 2), res_value(rc, p, 3)));
-        break;
-      default:
-        break;
-    }
-    float v[4];
-    f2_unpack(v01, v[0], v[1]);
-    f2_unpack(v23, v[2], v[3]);
-    if constexpr (kTmaStore<KIND>) {
-      if constexpr (O32) {
-        box_store_f32(stage, rr, lane, v);  // in place: this lane's own 16 bytes
-      } else {
-        __syncwarp();  // the stage row this box row overwrites has been read by every lane
-        box_store_bf16(stage, rr, lane, v);
-      }
-    } else {
-      const int64_t row = row0 + rr;
-      if (row >= g.M || !ACID_IN_BOUNDS(kSiteGemmStore, row * g.ldo + col + 3, (g.M - 1) * g.ldo + g.N)) continue;
-      if constexpr (O32)
-        *reinterpret_cast<float4*>(static_cast<float*>(g.out) + row * g.ldo + col) = make_float4(v[0], v[1], v[2], v[3]);
-      else
-        *reinterpret_cast<uint2*>(static_cast<__nv_bfloat16*>(g.out) + row * g.ldo + col) =
-            make_uint2(pack_bf16(v[0], v[1]), pack_bf16(v[2], v[3]));
-    }
-  }
-  if constexpr (kTmaStore<KIND>) {
-    fence_proxy_async_smem();
-    __syncwarp();
-    if (lane == 0) {
-      tma_store_2d(tmO, stage, col0, (int)row0);
-      bulk_commit_group();
-    }
-  } else {
-    __syncwarp();  // every lane has read the stage before the next chunk overwrites it
-  }
-}
+constexpr bool kNoResidual = !(KIND == EPI_GATED_RES || KIND == EPI_RES);
 
 // Bias of a chunk's 32 columns, the same for every lane (broadcast loads
 // through the read-only path; 16-byte loads where the vector is aligned).
-__device__ __forceinline__ void load_bias32(const EpiDev& e, int col0, float* bias) {
-  if (e.bias == nullptr) {
+__device__ __forceinline__ void load_bias32(const float* src, int col0, float* bias) {
+  if (src == nullptr) {
 #pragma unroll
     for (int k = 0; k < 32; ++k) bias[k] = 0.f;
-  } else if ((reinterpret_cast<uintptr_t>(e.bias + col0) & 15) == 0) {
+  } else if ((reinterpret_cast<uintptr_t>(src + col0) & 15) == 0) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const float4 t = __ldg(reinterpret_cast<const float4*>(e.bias + col0) + k);
+      const float4 t = __ldg(reinterpret_cast<const float4*>(src + col0) + k);
       bias[4 * k] = t.x; bias[4 * k + 1] = t.y; bias[4 * k + 2] = t.z; bias[4 * k + 3] = t.w;
     }
   } else {
 #pragma unroll
-    for (int k = 0; k < 32; ++k) bias[k] = __ldg(e.bias + col0 + k);
+    for (int k = 0; k < 32; ++k) bias[k] = __ldg(src + col0 + k);
   }
 }
 
@@ -486,13 +276,12 @@ __device__ __forceinline__ void epilogue_rows(const GemmDims& g, const EpiDev& e
 template <int KIND, bool O32>
 __device__ __forceinline__ void tma_kind_chunk(const GemmDims& g, const EpiDev& e, const CUtensorMap* tmO,
                                                uint8_t* stage, uint32_t taddr, int64_t row0, int64_t store_row0,
-                                               int col0, bool ok, int& nstore) {
+                                               int col0, const float* bias_src, bool live, int& nstore) {
   const int lane = threadIdx.x & 31;
   uint32_t r[32];
   float bias[32];
   tmem_ld32(taddr, r);
-  const bool live = ok && row0 < g.M && col0 < g.N;
-  if (live) load_bias32(e, col0, bias);
+  if (live) load_bias32(bias_src, col0, bias);
   tmem_wait_ld();
   if (!live) return;
   uint8_t* st = stage;
@@ -507,214 +296,184 @@ __device__ __forceinline__ void tma_kind_chunk(const GemmDims& g, const EpiDev& 
   ++nstore;
 }
 
-template <int BN, int KIND, bool R32, bool O32>
-__global__ void __launch_bounds__(kGemmThreads, 1)
-    gemm_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                   const __grid_constant__ CUtensorMap tmO, GemmDims g, EpiDev e) {
-  using C = TcCfg<BN>;
-  extern __shared__ uint8_t smem_raw[];
-  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sA = smem;
-  uint8_t* sB = smem + C::STAGES * C::A_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::STAGES * C::STAGE_BYTES + C::EPI_BYTES);
-  uint64_t* empty = full + C::STAGES;
-  uint64_t* acc_full = empty + C::STAGES;  // [2]
-  uint64_t* acc_empty = acc_full + 2;      // [2]
-  uint64_t* drain = acc_empty + 2;         // failure path: the MMAs issued so far have completed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int num_kb = (g.K + BK - 1) / BK;
-  const int num_n = (g.N + BN - 1) / BN;
-  const int num_tiles = (int)((g.M + BM - 1) / BM) * num_n;
-
-  if (warp == 0 && lane == 0) {
-    tma_prefetch_desc(&tmA);
-    tma_prefetch_desc(&tmB);
-    for (int s = 0; s < C::STAGES; ++s) {
-      mbar_init(&full[s], 1);
-      mbar_init(&empty[s], 1);
-    }
-    for (int b = 0; b < 2; ++b) {
-      mbar_init(&acc_full[b], 1);
-      mbar_init(&acc_empty[b], 32 * kEpiWarps);
-    }
-    mbar_init(drain, 1);
-    mbar_fence_init();
-  }
-  if (warp == 1) tmem_alloc(tmem_slot, C::TMEM_COLS);
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
-
-  if (warp == 0) {
-    if (lane == 0) {  // TMA producer: one continuous stage ring across tiles
-      int it = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
-        const int m_tile = tile / num_n, n_tile = tile % num_n;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = it % C::STAGES, round = it / C::STAGES;
-          if (round > 0 && !mbar_wait(&empty[s], (round - 1) & 1)) { ok = false; break; }
-          mbar_expect_tx(&full[s], C::STAGE_BYTES);
-          tma_load_2d(sA + s * C::A_BYTES, &tmA, &full[s], kb * BK, m_tile * BM);
-          tma_load_2d(sB + s * C::B_BYTES, &tmB, &full[s], kb * BK, n_tile * BN);
-        }
-      }
-      // After a wait ran out: the loads of the last STAGES issues may still be
-      // in flight; wait (bounded) until they have landed, so that no TMA
-      // writes into this CTA's shared memory after it exits.  Earlier issues
-      // were consumed by the MMA thread before their stage was refilled.
-      if (!ok)
-        for (int j = std::max(0, it - C::STAGES); j < it; ++j) mbar_wait(&full[j % C::STAGES], (j / C::STAGES) & 1);
-    }
-  } else if (warp == 1) {
-    if (lane == 0) {  // MMA issuer
-      constexpr uint32_t idesc = idesc_bf16_f32(BM, BN, false, false);
-      int it = 0, local = 0;
-      bool ok = true;
-      for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x, ++local) {
-        const int b = local & 1, use = local >> 1;
-        if (use > 0 && !mbar_wait(&acc_empty[b], (use - 1) & 1)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d = tmem + b * BN;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = it % C::STAGES, round = it / C::STAGES;
-          if (!mbar_wait(&full[s], round & 1)) { ok = false; break; }
-          tc_fence_after();
-          const uint32_t a0 = smem_u32(sA + s * C::A_BYTES);
-          const uint32_t b0 = smem_u32(sB + s * C::B_BYTES);
+// One chunk of a residual kind of the pair kernel, also in the accumulator's
+// layout.  The residual box (32 x 32, TMA-loaded into the warp's box `box` in
+// the swizzled layouts of epilogue_rows) is read by the lane that owns the
+// row, the result is written back over it and leaves by TMA store; two boxes
+// alternate.  Accumulator, bias and gate loads are issued before the wait for
+// the box: loaded after it, group by group, the gates alone cost 1500 of
+// 4100 SM clocks per chunk.  next(): issues the residual load of the chunk after this
+// one into the other box, once the store that last used it has read it.
+// Returns false if the wait ran out.
+template <int KIND, bool R32, bool O32, typename Next>
+__device__ __forceinline__ bool res_kind_chunk(const GemmDims& g, const EpiDev& e, const CUtensorMap* tmO, uint8_t* box, uint64_t* box_full,
+                                               uint32_t phase, uint32_t taddr, int64_t row0, int col0,
+                                               const float* bias_src, Next next) {
+  const int lane = threadIdx.x & 31;
+  uint32_t r[32];
+  float bv[32], gv[32];
+  tmem_ld32(taddr, r);
+  load_bias32(bias_src, col0, bv);
+  if constexpr (KIND == EPI_GATED_RES)
+    load_bias32(row0 + lane + e.row_base < e.gate_split ? e.gate_t : e.gate_v, col0, gv);
+  const bool ok = g.res_direct || mbar_wait_warp(box_full, phase);
+  tmem_wait_ld();
+  if (!ok) return false;
+  uint64_t v[16];
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t ad = smem_desc_sw128(a0 + k * 32, 16, 1024);
-            const uint64_t bd = smem_desc_sw128(b0 + k * 32, 16, 1024);
-            mma_bf16_ss(d, ad, bd, idesc, (kb | k) != 0);
-          }
-          mma_commit(&empty[s]);
-        }
-        if (ok) mma_commit(&acc_full[b]);
+  for (int u = 0; u < 4; ++u) {  // 8 columns of this lane's residual row
+    float rv[8] = {};
+    if (g.res_direct) {
+      const int64_t at = (row0 + lane) * e.ldr + col0 + 8 * u;
+      if (row0 + lane < g.M && ACID_IN_BOUNDS(kSiteGemmResidual, at + 7, (g.M - 1) * e.ldr + g.N)) {
+        if constexpr (R32)
+          load8(static_cast<const float*>(e.res) + at, rv);
+        else
+          load8(static_cast<const __nv_bfloat16*>(e.res) + at, rv);
       }
-      // After a wait ran out: let the MMAs already issued finish (bounded)
-      // before the accumulator's tensor memory is freed below.
-      if (!ok) {
-        mma_commit(drain);
-        mbar_wait(drain, 0);
+    } else if constexpr (R32) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const float4 t = *reinterpret_cast<const float4*>(box + lane * 128 + (((2 * u + h) ^ (lane & 7)) << 4));
+        rv[4 * h] = t.x; rv[4 * h + 1] = t.y; rv[4 * h + 2] = t.z; rv[4 * h + 3] = t.w;
       }
+    } else {
+      load8(reinterpret_cast<const __nv_bfloat16*>(box + lane * 64 + ((u ^ ((lane >> 1) & 3)) << 4)), rv);
     }
-  } else {  // epilogue: warps 2..9; lane quarter = warp % 4, column half = (warp - 2) / 4
-    const int q = warp & 3, half = (warp - 2) >> 2;
-    const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    float* stage = reinterpret_cast<float*>(smem + C::STAGES * C::STAGE_BYTES) + (warp - 2) * C::EPI_STAGE_FLOATS;
-    int local = 0;
-    for (int tile = blockIdx.x; tile < num_tiles; tile += gridDim.x, ++local) {
-      const int b = local & 1, use = local >> 1;
-      const int m_tile = tile / num_n, n_tile = tile % num_n;
-      const bool ok = mbar_wait(&acc_full[b], use & 1);
-      tc_fence_after();
-      const int64_t row0 = (int64_t)m_tile * BM + q * 32;
-      // this warp's chunks: columns [half * BN/2, (half + 1) * BN/2) of the tile, 32 at a time;
-      // the global inputs of chunk i+1 (residual, bias, gates) are loaded while chunk i is processed
-      constexpr int NC = BN / 64;
-      const int cbeg = half * (BN / 2);
-      const int lcol = 4 * (lane & 7);
-      auto process = [&](int i, const ResChunk<R32>& cur, ResChunk<R32>& nxt) {
-        const int c = cbeg + 32 * i;
-        uint32_t r[32];
-        tmem_ld32(tmem + lane_base + b * BN + c, r);
-        tmem_wait_ld();
-        const int col0 = n_tile * BN + c;
-        if (i + 1 < NC && row0 < g.M && col0 + 32 < g.N) load_chunk_inputs<KIND, R32>(g, e, row0, col0 + 32 + lcol, nxt);
-        if (ok && row0 < g.M && col0 < g.N) {
-          if constexpr (kTmaStore<KIND>) {
-            if (lane == 0) bulk_wait_group_read<0>();  // the previous box has left the stage
-            __syncwarp();
-          }
-          epilogue_chunk<KIND, R32, O32>(g, e, &tmO, stage, row0, col0, r, cur);
-        }
-      };
-      ResChunk<R32> rc0, rc1;
-      if (row0 < g.M && n_tile * BN + cbeg < g.N) load_chunk_inputs<KIND, R32>(g, e, row0, n_tile * BN + cbeg + lcol, rc0);
-#pragma unroll 1
-      for (int i = 0; i < NC; i += 2) {
-        process(i, rc0, rc1);
-        if (i + 1 < NC) process(i + 1, rc1, rc0);
-      }
-      tc_fence_before();
-      mbar_arrive(&acc_empty[b]);
-      if (!ok) break;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const int c = 8 * u + 2 * k;
+      const uint64_t acc = f2_add(f2_pack(__uint_as_float(r[c]), __uint_as_float(r[c + 1])), f2_pack(bv[c], bv[c + 1]));
+      const uint64_t rr = f2_pack(rv[2 * k], rv[2 * k + 1]);
+      if constexpr (KIND == EPI_GATED_RES)
+        v[4 * u + k] = f2_fma(f2_pack(gv[c], gv[c + 1]), acc, rr);
+      else
+        v[4 * u + k] = f2_add(acc, rr);
     }
-    if (lane == 0) bulk_wait_group<0>();  // tensor stores complete before the CTA exits
   }
-  tc_fence_before();
-  __syncthreads();
-  if (warp == 1) {
-    tc_fence_after();
-    tmem_dealloc(tmem, C::TMEM_COLS);
+  next();
+  __syncwarp();  // every lane has read its residual row
+  if constexpr (O32) {
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      float a0, a1, a2, a3;
+      f2_unpack(v[2 * u], a0, a1);
+      f2_unpack(v[2 * u + 1], a2, a3);
+      *reinterpret_cast<float4*>(box + lane * 128 + ((u ^ (lane & 7)) << 4)) = make_float4(a0, a1, a2, a3);
+    }
+  } else {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      uint32_t w[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        float a0, a1;
+        f2_unpack(v[4 * u + q], a0, a1);
+        w[q] = pack_bf16(a0, a1);
+      }
+      *reinterpret_cast<uint4*>(box + lane * 64 + ((u ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
   }
+  fence_proxy_async_smem();
+  __syncwarp();
+  if (lane == 0) {
+    tma_store_2d(tmO, box, col0, (int)row0);
+    bulk_commit_group();
+  }
+  return true;
 }
 
 // ===========================================================================
 // tcgen05 GEMM on SM pairs (cta_group::2), persistent
 //
-// A cluster of two CTAs on two SMs computes 256 x 256 output tiles: each CTA
-// stages its own 128 rows of A and its own 128 rows of B (half of the tile's
-// output columns) per 64-wide k-step, and one thread of CTA rank 0 issues
-// M256 N256 K16 MMAs that read both CTAs' shared memory and write each CTA's
-// 128 x 256 fp32 accumulator into that CTA's TMEM.  Per SM and k-step this
-// moves 32 KB into shared memory for 128 x 256 x 64 MACs, against 48 KB for
-// the single-SM 128 x 256 tile: the single-SM kernel is bound by that
-// L2-to-SM delivery.
+// A cluster of two CTAs on two SMs computes 256 x bn output tiles (bn up to
+// 256, see pick_bn): each CTA stages its own 128 rows of A and its own bn / 2
+// rows of B per 64-wide k-step, and one thread of CTA rank 0 issues M256 N(bn)
+// K16 MMAs that read both CTAs' shared memory and write each CTA's 128 x bn
+// fp32 accumulator into that CTA's TMEM.  At bn = 256 this moves 32 KB per SM
+// and k-step into shared memory for 128 x 256 x 64 MACs, against 48 KB for a
+// single-SM 128 x 256 tile.  Tiles go N fastest, so the pairs running together
+// share A row blocks in L2 and the weight tiles stay L2-resident; the TMEM
+// accumulator is double-buffered, so the epilogue of tile i overlaps the MMAs
+// of tile i + 1.
 //   warp 0   TMA producer in both CTAs; both CTAs' loads count on rank 0's
 //            full[s] barrier (rank 0 expects the bytes of both);
 //   warp 1   rank 0: MMA issuer; each k-step is committed to empty[s] of both
 //            CTAs, each tile to acc_full[b] of both CTAs;
-//   warps 2-9 epilogue of this CTA's 128 accumulator rows (as in
-//            gemm_tc_kernel); one lane per warp then arrives on rank 0's
-//            acc_empty[b], which counts the epilogue warps of both CTAs.
+//   warps 2-9 epilogue of this CTA's 128 accumulator rows; one lane per warp
+//            then arrives on rank 0's acc_empty[b], which counts the epilogue
+//            warps of both CTAs.
+//   What bounds it: long mainloops run into the power cap (FFN1 at 32760 rows,
+// 1536 -> 8960 with GELU: 521 us, 1730 TFLOP/s, at about 1.45 GHz; 571 us before
+// the issue loops below kept to uniform registers).  A k-step's floor is the
+// issue of its loads and MMAs: 240 SM clocks at bn = 32, where it was 580.
 // ===========================================================================
 struct Tc2Cfg {
-  static constexpr int BN = 256;  // output columns per pair tile
-  static constexpr int STAGES = 6;
-  static constexpr int A_BYTES = BM * BK * 2;        // this CTA's 128 rows of A
-  static constexpr int B_BYTES = (BN / 2) * BK * 2;  // this CTA's 128 rows of B
-  static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
-  static constexpr int EPI_STAGE_FLOATS = 32 * 32;
-  static constexpr int EPI_BYTES = kEpiWarps * EPI_STAGE_FLOATS * 4;
-  static constexpr int SMEM = STAGES * STAGE_BYTES + EPI_BYTES + 1024 + 256;
-  static constexpr uint32_t TMEM_COLS = 2 * BN;  // double-buffered 128 x 256 accumulator
+  static constexpr int MAX_BN = 256;           // output columns per pair tile (g.bn: a multiple of 32)
+  static constexpr int A_BYTES = BM * BK * 2;  // this CTA's 128 rows of A; its bn / 2 rows of B follow
+  static constexpr int MAX_STAGES = 12;
+  // Operand ring and epilogue boxes share shared memory: kinds without a
+  // residual have six 32 KB stages and 4 KB per epilogue warp, residual kinds
+  // five stages and two 4 KB boxes per warp.
+  static constexpr int RING = 6 * 32768, RING_RES = 5 * 32768;
+  static constexpr int WARP = 4096, WARP_RES = 8192;
+  static constexpr int SMEM = RING + kEpiWarps * WARP + 1024 + 512;
+  __host__ __device__ static constexpr int stage_bytes(int bn) { return A_BYTES + bn * BK; }
+  static int stages(int bn, bool res) { return std::min(MAX_STAGES, (res ? RING_RES : RING) / stage_bytes(bn)); }
+  static constexpr uint32_t TMEM_COLS = 2 * MAX_BN;  // double-buffered 128 x bn accumulator
 };
 static_assert(Tc2Cfg::SMEM <= 232448, "pair GEMM shared memory");
+static_assert(Tc2Cfg::RING_RES + kEpiWarps * Tc2Cfg::WARP_RES == Tc2Cfg::RING + kEpiWarps * Tc2Cfg::WARP,
+              "one shared memory size for both layouts");
+
+// Where a pair tile lies: its first row, its first column and whose rows it
+// holds (dual-stream launches: the text rows' tiles come first).
+struct TilePos {
+  int row, col;
+  bool text;
+};
+__device__ __forceinline__ TilePos tile_pos(const GemmDims& g, int tile, int num_n) {
+  const int m = tile / num_n;
+  TilePos t;
+  t.text = m < g.mt_text;
+  t.row = t.text ? m * 2 * BM : g.l_text + (m - g.mt_text) * 2 * BM;
+  t.col = (tile - m * num_n) * g.bn;
+  return t;
+}
 
 template <int KIND, bool R32, bool O32, bool SPLIT = false>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
     gemm_tc2_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
-                    const __grid_constant__ CUtensorMap tmO, GemmDims g, EpiDev e) {
+                    const __grid_constant__ CUtensorMap tmO, const __grid_constant__ CUtensorMap tmR,
+                    const __grid_constant__ CUtensorMap tmBt, const __grid_constant__ CUtensorMap tmOt, GemmDims g,
+                    EpiDev e) {
   using C = Tc2Cfg;
-  constexpr int BN = C::BN;
+  constexpr bool RES = !kNoResidual<KIND>;
+  constexpr int RING = RES ? C::RING_RES : C::RING, WARP = RES ? C::WARP_RES : C::WARP;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint8_t* sA = smem;
-  uint8_t* sB = smem + C::STAGES * C::A_BYTES;
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem + C::STAGES * C::STAGE_BYTES + C::EPI_BYTES);
-  uint64_t* empty = full + C::STAGES;
-  uint64_t* acc_full = empty + C::STAGES;  // [2]
-  uint64_t* acc_empty = acc_full + 2;      // [2] (rank 0's counts both CTAs' epilogue warps)
-  uint64_t* drain = acc_empty + 2;         // failure path: the MMAs issued so far have completed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain + 1);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + RING + kEpiWarps * WARP);
+  uint64_t* full = bars;                       // [MAX_STAGES]
+  uint64_t* empty = full + C::MAX_STAGES;      // [MAX_STAGES]
+  uint64_t* acc_full = empty + C::MAX_STAGES;  // [2]
+  uint64_t* acc_empty = acc_full + 2;          // [2] (rank 0's counts both CTAs' epilogue warps)
+  uint64_t* drain = acc_empty + 2;             // failure path: the MMAs issued so far have completed
+  uint64_t* res_full = drain + 1;              // [epilogue warp][2] residual box loaded
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(res_full + 2 * kEpiWarps);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const uint32_t rank = cluster_ctarank();
   const int pair = (int)blockIdx.x >> 1, npairs = (int)gridDim.x >> 1;
   const int num_kb = SPLIT ? g.kb_split : (g.K + BK - 1) / BK;
-  const int num_n = (g.N + BN - 1) / BN;
-  const int num_tiles = (int)((g.M + 2 * BM - 1) / (2 * BM)) * num_n;
-  const int num_units = SPLIT ? num_tiles * g.splits : num_tiles;  // (tile, split) pairs
+  const int num_n = (g.N + g.bn - 1) / g.bn;
+  const int num_m = g.mt_text + (int)((g.M - g.l_text + 2 * BM - 1) / (2 * BM));
+  const int num_units = SPLIT ? num_m * num_n * g.splits : num_m * num_n;  // (tile, split) pairs
+  const int stages = g.stages, stage_bytes = C::stage_bytes(g.bn);
 
   if (warp == 0 && lane == 0) {
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
-    for (int s = 0; s < C::STAGES; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
     }
@@ -722,6 +481,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
       mbar_init(&acc_full[b], 1);
       mbar_init(&acc_empty[b], 2 * kEpiWarps);
     }
+    if constexpr (RES)
+      for (int i = 0; i < 2 * kEpiWarps; ++i) mbar_init(&res_full[i], 1);
     mbar_init(drain, 1);
     mbar_fence_init();
   }
@@ -733,133 +494,169 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0) {
-    if (lane == 0) {  // TMA producer (both CTAs): one continuous stage ring across tiles
-      const uint32_t full0 = mapa_shared(smem_u32(full), 0);  // rank 0's full[0]
-      int it = 0;
-      bool ok = true;
-      for (int unit = pair; ok && unit < num_units; unit += npairs) {
-        const int tile = SPLIT ? unit / g.splits : unit;
-        const int kb0 = SPLIT ? (unit % g.splits) * num_kb : 0;
-        const int m_tile = tile / num_n, n_tile = tile % num_n;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = it % C::STAGES, round = it / C::STAGES;
-          if (round > 0 && !mbar_wait(&empty[s], (round - 1) & 1)) { ok = false; break; }
-          if (rank == 0) mbar_expect_tx(&full[s], 2 * C::STAGE_BYTES);
-          tma_load_2d_pair(sA + s * C::A_BYTES, &tmA, full0 + 8 * s, (kb0 + kb) * BK, m_tile * 2 * BM + (int)rank * BM);
-          tma_load_2d_pair(sB + s * C::B_BYTES, &tmB, full0 + 8 * s, (kb0 + kb) * BK,
-                           n_tile * BN + (int)rank * (BN / 2));
+    // TMA producer (both CTAs): one continuous stage ring across tiles; the
+    // whole warp walks the loop and one elected lane issues, as for the MMAs
+    const bool leader = elect_one();
+    const uint32_t full0 = mapa_shared(smem_u32(full), 0);  // rank 0's full[0]
+    int s = 0, issued = 0;
+    uint32_t ph = 1;  // parity of the previous use of the stage (a fresh barrier passes on 1)
+    bool ok = true;
+    for (int unit = pair; ok && unit < num_units; unit += npairs) {
+      const TilePos t = tile_pos(g, SPLIT ? unit / g.splits : unit, num_n);
+      const int k0 = SPLIT ? (unit % g.splits) * num_kb * BK : 0;
+      const CUtensorMap* tb = t.text ? &tmBt : &tmB;
+      const int arow = t.row + (int)rank * BM, brow = t.col + (int)rank * (g.bn / 2);
+      for (int kb = 0; kb < num_kb; ++kb) {
+        if (!mbar_wait_warp(&empty[s], ph)) { ok = false; break; }
+        if (leader) {
+          if (rank == 0) mbar_expect_tx(&full[s], 2 * stage_bytes);
+          uint8_t* st = smem + s * stage_bytes;
+          tma_load_2d_pair(st, &tmA, full0 + 8 * s, k0 + kb * BK, arow);
+          tma_load_2d_pair(st + C::A_BYTES, tb, full0 + 8 * s, k0 + kb * BK, brow);
+        }
+        __syncwarp();
+        ++issued;
+        if (++s == stages) {
+          s = 0;
+          ph ^= 1;
         }
       }
-      // After a wait ran out: rank 0 waits (bounded) for the last STAGES
-      // stages it expected to land.  Rank 1's loads count on rank 0's
-      // barriers, which rank 1 cannot poll; it idles about 2^16 clocks, far
-      // above the latency of a 32 KB load, before both CTAs meet at the exit.
-      if (!ok) {
-        if (rank == 0) {
-          for (int j = std::max(0, it - C::STAGES); j < it; ++j) mbar_wait(&full[j % C::STAGES], (j / C::STAGES) & 1);
-        } else {
-          const long long t0 = clock64();
-          while (clock64() - t0 < (1LL << 16)) {
-          }
+    }
+    // After a wait ran out: rank 0 waits (bounded) for the last `stages`
+    // stages it expected to land.  Rank 1's loads count on rank 0's
+    // barriers, which rank 1 cannot poll; it idles about 2^16 clocks, far
+    // above the latency of a 32 KB load, before both CTAs meet at the exit.
+    if (!ok && leader) {
+      if (rank == 0) {
+        for (int j = std::max(0, issued - stages); j < issued; ++j) mbar_wait(&full[j % stages], (j / stages) & 1);
+      } else {
+        const long long t0 = clock64();
+        while (clock64() - t0 < (1LL << 16)) {
         }
       }
     }
   } else if (warp == 1) {
-    if (lane == 0 && rank == 0) {  // MMA issuer (rank 0 only)
-      constexpr uint32_t idesc = idesc_bf16_f32(2 * BM, BN, false, false);
-      const uint32_t empty_l = smem_u32(empty), empty_r = mapa_shared(empty_l, 1);
-      const uint32_t accf_l = smem_u32(acc_full), accf_r = mapa_shared(accf_l, 1);
-      int it = 0, local = 0;
+    // MMA issuer (rank 0 only).  The whole warp walks the loop, so that the
+    // descriptors stay in uniform registers, and one elected lane issues:
+    // with the loop in a single-lane branch a k-step's four MMAs took 257 SM
+    // clocks to issue and a whole k-step 530, above the 512 they run for.
+    if (rank == 0) {
+      const bool leader = elect_one();
+      const uint32_t idesc = idesc_bf16_f32(2 * BM, g.bn, false, false);
+      const uint32_t empty_l = smem_u32(empty), accf_l = smem_u32(acc_full);
+      const uint64_t adesc = smem_desc_sw128(smem_u32(smem), 16, 1024);
+      const uint64_t bdesc = smem_desc_sw128(smem_u32(smem + C::A_BYTES), 16, 1024);
+      int s = 0, local = 0;
+      uint32_t ph = 0;
       bool ok = true;
       for (int unit = pair; ok && unit < num_units; unit += npairs, ++local) {
         const int b = local & 1, use = local >> 1;
-        if (use > 0 && !mbar_wait_cluster(&acc_empty[b], (use - 1) & 1)) { ok = false; break; }
+        if (use > 0 && !__all_sync(0xffffffffu, mbar_wait_cluster(&acc_empty[b], (use - 1) & 1))) { ok = false; break; }
         tc_fence_after();
-        const uint32_t d = tmem + b * BN;
-        for (int kb = 0; kb < num_kb; ++kb, ++it) {
-          const int s = it % C::STAGES, round = it / C::STAGES;
-          if (!mbar_wait(&full[s], round & 1)) { ok = false; break; }
+        const uint32_t d = tmem + b * C::MAX_BN;
+        for (int kb = 0; kb < num_kb; ++kb) {
+          if (!mbar_wait_warp(&full[s], ph)) { ok = false; break; }
           tc_fence_after();
-          const uint32_t a0 = smem_u32(sA + s * C::A_BYTES);
-          const uint32_t b0 = smem_u32(sB + s * C::B_BYTES);
+          const uint64_t off = (uint64_t)((s * stage_bytes) >> 4);
+          if (leader) {
 #pragma unroll
-          for (int k = 0; k < BK / 16; ++k) {
-            const uint64_t ad = smem_desc_sw128(a0 + k * 32, 16, 1024);
-            const uint64_t bd = smem_desc_sw128(b0 + k * 32, 16, 1024);
-            mma_bf16_ss_pair(d, ad, bd, idesc, (kb | k) != 0);
+            for (int k = 0; k < BK / 16; ++k)
+              mma_bf16_ss_pair(d, adesc + off + 2 * k, bdesc + off + 2 * k, idesc, (kb | k) != 0);
+            mma_commit_both(empty_l + 8 * s);
           }
-          mma_commit_pair(empty_l + 8 * s);
-          mma_commit_pair(empty_r + 8 * s);
+          __syncwarp();
+          if (++s == stages) {
+            s = 0;
+            ph ^= 1;
+          }
         }
-        if (ok) {
-          mma_commit_pair(accf_l + 8 * b);
-          mma_commit_pair(accf_r + 8 * b);
-        }
+        if (ok && leader) mma_commit_both(accf_l + 8 * b);
+        __syncwarp();
       }
-      if (!ok) {
+      if (!ok && leader) {
         mma_commit_pair(smem_u32(drain));
         mbar_wait(drain, 0);
       }
     }
   } else {  // epilogue: warps 2..9 of each CTA, this CTA's 128 rows of the pair tile
+    // lane quarter = warp % 4; the tile's 32-column chunks alternate between
+    // the two warps of a quarter
     const int q = warp & 3, half = (warp - 2) >> 2;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    float* stage = reinterpret_cast<float*>(smem + C::STAGES * C::STAGE_BYTES) + (warp - 2) * C::EPI_STAGE_FLOATS;
+    uint8_t* stage = smem + RING + (warp - 2) * WARP;
     const uint32_t acc_empty0 = mapa_shared(smem_u32(acc_empty), 0);
+    const int row_in = (int)rank * BM + q * 32, nch = g.bn / 32;
+    uint64_t* rfull = res_full + 2 * (warp - 2);
+    // Residual kinds: the position (unit, chunk) of the next residual load;
+    // seek() moves it on to the first chunk from there with rows and columns
+    // to store.  Loads are numbered like the chunks that consume them.
+    int lu = pair, lc = half, lrow = 0, lcol = 0, loads = 0, nchunk = 0;
+    auto seek = [&]() {
+      for (; lu < num_units; lu += npairs, lc = half) {
+        const TilePos t = tile_pos(g, lu, num_n);
+        lrow = t.row + row_in;
+        lcol = t.col + 32 * lc;
+        if (lc < nch && lcol < g.N && lrow < (t.text ? g.l_text : (int)g.M)) return true;
+      }
+      return false;
+    };
+    auto load_next = [&]() {  // lane 0
+      if (!seek()) return;
+      uint64_t* bar = &rfull[loads & 1];
+      mbar_expect_tx(bar, R32 ? 4096 : 2048);
+      tma_load_2d(stage + (loads & 1) * 4096, &tmR, bar, lcol, lrow);
+      ++loads;
+      lc += 2;
+    };
+    if constexpr (RES) {
+      if (lane == 0 && !g.res_direct) {
+        load_next();
+        load_next();
+      }
+    }
     int local = 0, nstore = 0;
     for (int unit = pair; unit < num_units; unit += npairs, ++local) {
-      const int tile = SPLIT ? unit / g.splits : unit;
       const int b = local & 1, use = local >> 1;
-      const int m_tile = tile / num_n, n_tile = tile % num_n;
-      const bool ok = mbar_wait(&acc_full[b], use & 1);
+      const TilePos t = tile_pos(g, SPLIT ? unit / g.splits : unit, num_n);
+      const int64_t row0 = t.row + row_in;
+      const bool rows_live = row0 < (t.text ? (int64_t)g.l_text : g.M);
+      const CUtensorMap* to = t.text ? &tmOt : &tmO;
+      const float* bias = t.text ? e.bias_t : e.bias;
+      bool ok = mbar_wait(&acc_full[b], use & 1);
       tc_fence_after();
-      const int64_t row0 = (int64_t)m_tile * 2 * BM + (int64_t)rank * BM + q * 32;
-      if constexpr (kTmaStore<KIND>) {
-        constexpr int NC = BN / 64;
-        const int cbeg = half * (BN / 2);
-        const int64_t store_row0 = SPLIT ? row0 + (int64_t)(unit % g.splits) * g.m_pad : row0;
 #pragma unroll 1
-        for (int i = 0; i < NC; ++i)
-          tma_kind_chunk<KIND, O32>(g, e, &tmO, reinterpret_cast<uint8_t*>(stage),
-                                    tmem + lane_base + b * BN + cbeg + 32 * i, row0, store_row0,
-                                    n_tile * BN + cbeg + 32 * i, ok, nstore);
-        tc_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * b);
-        if (!ok) break;
-        continue;
-      }
-      constexpr int NC = BN / 64;
-      const int cbeg = half * (BN / 2);
-      const int lcol = 4 * (lane & 7);
-      auto process = [&](int i, const ResChunk<R32>& cur, ResChunk<R32>& nxt) {
-        const int c = cbeg + 32 * i;
-        uint32_t r[32];
-        tmem_ld32(tmem + lane_base + b * BN + c, r);
-        tmem_wait_ld();
-        const int col0 = n_tile * BN + c;
-        if (i + 1 < NC && row0 < g.M && col0 + 32 < g.N) load_chunk_inputs<KIND, R32>(g, e, row0, col0 + 32 + lcol, nxt);
-        if (ok && row0 < g.M && col0 < g.N) {
-          if constexpr (kTmaStore<KIND>) {
-            if (lane == 0) bulk_wait_group_read<0>();  // the previous box has left the stage
-            __syncwarp();
-          }
-          epilogue_chunk<KIND, R32, O32>(g, e, &tmO, stage, row0, col0, r, cur);
+      for (int c = half; c < nch; c += 2) {
+        const uint32_t taddr = tmem + lane_base + b * C::MAX_BN + 32 * c;
+        const int col0 = t.col + 32 * c;
+        const bool live = ok && rows_live && col0 < g.N;  // warp-uniform
+        if constexpr (!RES) {
+          const int64_t store_row0 = SPLIT ? row0 + (int64_t)(unit % g.splits) * g.m_pad : row0;
+          tma_kind_chunk<KIND, O32>(g, e, to, stage, taddr, row0, store_row0, col0, bias, live, nstore);
+        } else if (live) {
+          const int x = nchunk & 1;
+          ok = res_kind_chunk<KIND, R32, O32>(g, e, to, stage + x * 4096, &rfull[x], (nchunk >> 1) & 1, taddr, row0, col0,
+                                              bias, [&]() {
+                                                // the other box: its chunk's store was issued one chunk ago
+                                                if (lane == 0 && nchunk > 0) {
+                                                  bulk_wait_group_read<0>();
+                                                  if (!g.res_direct) load_next();
+                                                }
+                                              });
+          if (!ok) break;
+          ++nchunk;
         }
-      };
-      ResChunk<R32> rc0, rc1;
-      if (row0 < g.M && n_tile * BN + cbeg < g.N) load_chunk_inputs<KIND, R32>(g, e, row0, n_tile * BN + cbeg + lcol, rc0);
-#pragma unroll 1
-      for (int i = 0; i < NC; i += 2) {
-        process(i, rc0, rc1);
-        if (i + 1 < NC) process(i + 1, rc1, rc0);
       }
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive_cluster(acc_empty0 + 8 * b);
       if (!ok) break;
     }
-    if (lane == 0) bulk_wait_group<0>();  // tensor stores complete before the CTA exits
+    if (lane == 0) {
+      // after a wait ran out: the residual loads already issued land before the CTA exits
+      if constexpr (RES)
+        for (; nchunk < loads; ++nchunk) mbar_wait(&rfull[nchunk & 1], (nchunk >> 1) & 1);
+      bulk_wait_group<0>();  // tensor stores complete before the CTA exits
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -921,7 +718,7 @@ acid_status make_tmap_bf16(CUtensorMap* map, const void* base, int64_t rows, int
 namespace {
 
 // The GEMM output as the epilogue's tensor stores see it: 32 x 32 boxes, the
-// swizzle of the box layout in epilogue_chunk (128-byte rows for fp32,
+// swizzle of the box layout in epilogue_rows (128-byte rows for fp32,
 // 64-byte rows for bf16).
 acid_status make_tmap_out(CUtensorMap* map, void* out, int64_t M, int N, int64_t ldo, bool fp32) {
   return fp32 ? make_tmap_2d(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, out, M, N, ldo, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B)
@@ -936,52 +733,6 @@ int num_sms() {
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
   }
   return n;
-}
-
-template <int BN, int KIND, bool R32, bool O32>
-acid_status launch_tc_kind1(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to, const GemmDims& g,
-                           const Epilogue& epi, int grid, cudaStream_t s) {
-  using C = TcCfg<BN>;
-  static bool attr_done = false;
-  if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<BN, KIND, R32, O32>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    attr_done = true;
-  }
-  gemm_tc_kernel<BN, KIND, R32, O32><<<grid, kGemmThreads, C::SMEM, s>>>(ta, tb, to, g, to_dev(epi));
-  ACID_CHECK_LAUNCH();
-  return ACID_OK;
-}
-
-// dispatch on the output dtype (a template parameter: it selects the box layout)
-template <int BN, int KIND, bool R32 = false>
-acid_status launch_tc_kind(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to, const GemmDims& g,
-                           const Epilogue& epi, int grid, cudaStream_t s) {
-  return g.out_fp32 ? launch_tc_kind1<BN, KIND, R32, true>(ta, tb, to, g, epi, grid, s)
-                    : launch_tc_kind1<BN, KIND, R32, false>(ta, tb, to, g, epi, grid, s);
-}
-
-template <int BN>
-acid_status launch_tc(const void* A, int64_t lda, int64_t M, int K, const void* W, int N, void* out, int64_t ldo,
-                      const Epilogue& epi, cudaStream_t s) {
-  CUtensorMap ta, tb, to;
-  ACID_TRY(make_tmap_bf16(&ta, A, M, K, lda, BM));
-  ACID_TRY(make_tmap_bf16(&tb, W, N, K, K, BN));
-  ACID_TRY(make_tmap_out(&to, out, M, N, ldo, epi.out_fp32));
-  GemmDims g{M, N, K, out, ldo, epi.out_fp32 ? 1 : 0};
-  const int64_t tiles = ((M + BM - 1) / BM) * ((N + BN - 1) / BN);
-  const int grid = (int)std::min<int64_t>(tiles, num_sms());
-  ProfScope prof(PROF_LINEAR, 2.0 * (double)M * N * K, s);
-  switch (epi.kind) {
-    case EPI_GELU: return launch_tc_kind<BN, EPI_GELU>(ta, tb, to, g, epi, grid, s);
-    case EPI_ROPE_QKV: return launch_tc_kind<BN, EPI_ROPE_QKV>(ta, tb, to, g, epi, grid, s);
-    case EPI_GATED_RES:
-      return epi.res_fp32 ? launch_tc_kind<BN, EPI_GATED_RES, true>(ta, tb, to, g, epi, grid, s)
-                          : launch_tc_kind<BN, EPI_GATED_RES, false>(ta, tb, to, g, epi, grid, s);
-    case EPI_RES:
-      return epi.res_fp32 ? launch_tc_kind<BN, EPI_RES, true>(ta, tb, to, g, epi, grid, s)
-                          : launch_tc_kind<BN, EPI_RES, false>(ta, tb, to, g, epi, grid, s);
-    default: return launch_tc_kind<BN, EPI_BIAS>(ta, tb, to, g, epi, grid, s);
-  }
 }
 
 // CTA pairs that can be resident at once for the pair kernel (clusters are
@@ -1004,49 +755,94 @@ int max_pairs() {
   return n;
 }
 
-template <int KIND, bool R32, bool O32>
-acid_status launch_tc2_kind1(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to, const GemmDims& g,
-                            const Epilogue& epi, int64_t tiles, cudaStream_t s) {
-  static bool attr_done = false;
-  if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(gemm_tc2_kernel<KIND, R32, O32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   Tc2Cfg::SMEM));
-    attr_done = true;
+int64_t pair_row_tiles(int64_t M, int64_t text_rows) {
+  return (text_rows + 2 * BM - 1) / (2 * BM) + (M - text_rows + 2 * BM - 1) / (2 * BM);
+}
+
+// Output columns per tile: the width with the lowest estimated time, in SM
+// clocks, of the pair that gets the most tiles.  A k-step runs for 2 bn clocks
+// on the tensor cores plus about 75, and not below its issue cost; each tile
+// adds about 500 and the last tile's epilogue 700 per pair of 32-column
+// chunks.  Narrower tiles win where a last round of 256-wide ones leaves pairs
+// idle.  Measured (us, CUDA events) at 256 columns and at the width chosen:
+// 7797 x 1920 x 1920 (M x K x N) gated residual 44.8, 40.4 at 160; 7800 x 1536 x
+// 4608 67.1, 63.0 at 192; 512 x 1536 x 3072 16.9, 11.4 at 96; 64 x 8960 x 1536
+// 49.6, 22.6 at 32; the wide layers of a 480p step stay at 256 (1536 -> 8960:
+// 521 us against 542 at 224).
+int pick_bn(int64_t m_tiles, int N, int K, int pairs) {
+  const int64_t num_kb = (K + BK - 1) / BK;
+  int best = Tc2Cfg::MAX_BN;
+  int64_t best_cost = INT64_MAX;
+  for (int bn = Tc2Cfg::MAX_BN; bn >= 32; bn -= 32) {
+    const int64_t tiles = m_tiles * ((N + bn - 1) / bn), rounds = (tiles + pairs - 1) / pairs;
+    const int64_t step = std::max(2 * bn + 75, 220 + bn / 2);
+    const int64_t cost = rounds * (num_kb * step + 500) + 700 * ((bn + 63) / 64);
+    if (cost < best_cost) {
+      best = bn;
+      best_cost = cost;
+    }
   }
-  const int pairs = max_pairs<KIND, R32, O32>();
+  return best;
+}
+
+// Tensor maps of one launch of the pair kernel.
+struct PairMaps {
+  CUtensorMap a, b, o, r, bt, ot;
+};
+
+template <int KIND, bool R32, bool O32>
+acid_status launch_tc2_kind1(const PairMaps& t, const GemmDims& g, const Epilogue& epi, int64_t tiles, cudaStream_t s) {
+  const int pairs = max_pairs<KIND, R32, O32>();  // also raises the shared memory limit
   ACID_REQUIRE(pairs > 0, ACID_ERR_CUDA, "linear: no resident CTA pair for the pair GEMM");
   const int grid = 2 * (int)std::min<int64_t>(tiles, pairs);
-  gemm_tc2_kernel<KIND, R32, O32><<<grid, kGemmThreads, Tc2Cfg::SMEM, s>>>(ta, tb, to, g, to_dev(epi));
+  gemm_tc2_kernel<KIND, R32, O32><<<grid, kGemmThreads, Tc2Cfg::SMEM, s>>>(t.a, t.b, t.o, t.r, t.bt, t.ot, g, to_dev(epi));
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
 template <int KIND, bool R32 = false>
-acid_status launch_tc2_kind(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& to, const GemmDims& g,
-                            const Epilogue& epi, int64_t tiles, cudaStream_t s) {
-  return g.out_fp32 ? launch_tc2_kind1<KIND, R32, true>(ta, tb, to, g, epi, tiles, s)
-                    : launch_tc2_kind1<KIND, R32, false>(ta, tb, to, g, epi, tiles, s);
+acid_status launch_tc2_kind(const PairMaps& t, const GemmDims& g, const Epilogue& epi, int64_t tiles, cudaStream_t s) {
+  return g.out_fp32 ? launch_tc2_kind1<KIND, R32, true>(t, g, epi, tiles, s)
+                    : launch_tc2_kind1<KIND, R32, false>(t, g, epi, tiles, s);
 }
 
 acid_status launch_tc2(const void* A, int64_t lda, int64_t M, int K, const void* W, int N, void* out, int64_t ldo,
                        const Epilogue& epi, cudaStream_t s) {
-  CUtensorMap ta, tb, to;
-  ACID_TRY(make_tmap_bf16(&ta, A, M, K, lda, BM));
-  ACID_TRY(make_tmap_bf16(&tb, W, N, K, K, Tc2Cfg::BN / 2));
-  ACID_TRY(make_tmap_out(&to, out, M, N, ldo, epi.out_fp32));
+  const int64_t m_tiles = pair_row_tiles(M, epi.text_rows);
+  const int bn = pick_bn(m_tiles, N, K, max_pairs<EPI_BIAS, false, false>());
+  const bool res = epi_reads_res(epi.kind);
+  PairMaps t;
+  ACID_TRY(make_tmap_bf16(&t.a, A, M, K, lda, BM));
+  ACID_TRY(make_tmap_bf16(&t.b, W, N, K, K, bn / 2));
+  ACID_TRY(make_tmap_out(&t.o, out, M, N, ldo, epi.out_fp32));
+  t.r = t.o;
+  const bool res_direct = res && epi.ldr < N;
+  if (res && !res_direct)
+    ACID_TRY(make_tmap_out(&t.r, const_cast<void*>(epi.residual), M, N, epi.ldr, epi.res_fp32));
+  t.bt = t.b;
+  t.ot = t.o;
   GemmDims g{M, N, K, out, ldo, epi.out_fp32 ? 1 : 0};
-  const int64_t tiles = ((M + 2 * BM - 1) / (2 * BM)) * ((N + Tc2Cfg::BN - 1) / Tc2Cfg::BN);
+  g.bn = bn;
+  g.stages = Tc2Cfg::stages(bn, res);
+  g.res_direct = res_direct;
+  if (epi.text_rows > 0) {  // the output map of the text rows ends with them
+    ACID_TRY(make_tmap_bf16(&t.bt, epi.text_w, N, K, K, bn / 2));
+    ACID_TRY(make_tmap_out(&t.ot, out, epi.text_rows, N, ldo, epi.out_fp32));
+    g.l_text = (int)epi.text_rows;
+    g.mt_text = (int)((epi.text_rows + 2 * BM - 1) / (2 * BM));
+  }
+  const int64_t tiles = m_tiles * ((N + bn - 1) / bn);
   ProfScope prof(PROF_LINEAR, 2.0 * (double)M * N * K, s);
   switch (epi.kind) {
-    case EPI_GELU: return launch_tc2_kind<EPI_GELU>(ta, tb, to, g, epi, tiles, s);
-    case EPI_ROPE_QKV: return launch_tc2_kind<EPI_ROPE_QKV>(ta, tb, to, g, epi, tiles, s);
+    case EPI_GELU: return launch_tc2_kind<EPI_GELU>(t, g, epi, tiles, s);
+    case EPI_ROPE_QKV: return launch_tc2_kind<EPI_ROPE_QKV>(t, g, epi, tiles, s);
     case EPI_GATED_RES:
-      return epi.res_fp32 ? launch_tc2_kind<EPI_GATED_RES, true>(ta, tb, to, g, epi, tiles, s)
-                          : launch_tc2_kind<EPI_GATED_RES, false>(ta, tb, to, g, epi, tiles, s);
+      return epi.res_fp32 ? launch_tc2_kind<EPI_GATED_RES, true>(t, g, epi, tiles, s)
+                          : launch_tc2_kind<EPI_GATED_RES, false>(t, g, epi, tiles, s);
     case EPI_RES:
-      return epi.res_fp32 ? launch_tc2_kind<EPI_RES, true>(ta, tb, to, g, epi, tiles, s)
-                          : launch_tc2_kind<EPI_RES, false>(ta, tb, to, g, epi, tiles, s);
-    default: return launch_tc2_kind<EPI_BIAS>(ta, tb, to, g, epi, tiles, s);
+      return epi.res_fp32 ? launch_tc2_kind<EPI_RES, true>(t, g, epi, tiles, s)
+                          : launch_tc2_kind<EPI_RES, false>(t, g, epi, tiles, s);
+    default: return launch_tc2_kind<EPI_BIAS>(t, g, epi, tiles, s);
   }
 }
 
@@ -1065,7 +861,7 @@ struct SplitKPlan {
 
 bool splitk_plan(int64_t M, int N, int K, size_t ws_bytes, int pairs, SplitKPlan* p) {
   constexpr int64_t bm = 2 * BM;
-  const int64_t n_tiles = (N + Tc2Cfg::BN - 1) / Tc2Cfg::BN, m_tiles = (M + bm - 1) / bm;
+  const int64_t n_tiles = (N + Tc2Cfg::MAX_BN - 1) / Tc2Cfg::MAX_BN, m_tiles = (M + bm - 1) / bm;
   const int64_t tiles = m_tiles * n_tiles, num_kb = (K + BK - 1) / BK;
   if (pairs <= 0 || num_kb < 64) return false;  // short mainloops: the last round is cheap
   const int64_t full = tiles / pairs, last = tiles - full * pairs;
@@ -1147,20 +943,21 @@ acid_status launch_tc2_splitk(const void* A, int64_t lda, int64_t M, int K, cons
   float* part = static_cast<float*>(epi.splitk_ws);
   CUtensorMap ta, tb, to;
   ACID_TRY(make_tmap_bf16(&ta, A, M, K, lda, BM));
-  ACID_TRY(make_tmap_bf16(&tb, W, N, K, K, Tc2Cfg::BN / 2));
+  ACID_TRY(make_tmap_bf16(&tb, W, N, K, K, Tc2Cfg::MAX_BN / 2));
   ACID_TRY(make_tmap_out(&to, part, (int64_t)sp.splits * sp.m_pad, N, N, true));
-  GemmDims g{M, N, K, part, N, 1};
+  GemmDims g{M, N, K, part, N, 1};  // 256 columns per tile
   g.splits = sp.splits;
   g.kb_split = sp.kb_split;
   g.m_pad = sp.m_pad;
   Epilogue raw;  // the accumulator as it is: no bias, fp32
   raw.out_fp32 = true;
-  const int64_t units = ((M + 2 * BM - 1) / (2 * BM)) * ((N + Tc2Cfg::BN - 1) / Tc2Cfg::BN) * sp.splits;
+  const int64_t units = ((M + 2 * BM - 1) / (2 * BM)) * ((N + Tc2Cfg::MAX_BN - 1) / Tc2Cfg::MAX_BN) * sp.splits;
   const int pairs = max_pairs<EPI_BIAS, false, true>();
   ACID_REQUIRE(pairs > 0, ACID_ERR_CUDA, "linear: no resident CTA pair for the pair GEMM");
   {
     ProfScope prof(PROF_LINEAR, 2.0 * (double)M * N * K, s);
-    kern<<<2 * (int)std::min<int64_t>(units, pairs), kGemmThreads, Tc2Cfg::SMEM, s>>>(ta, tb, to, g, to_dev(raw));
+    kern<<<2 * (int)std::min<int64_t>(units, pairs), kGemmThreads, Tc2Cfg::SMEM, s>>>(ta, tb, to, to, tb, to, g,
+                                                                                                  to_dev(raw));
     ACID_CHECK_LAUNCH();
   }
   switch (epi.kind) {
@@ -1359,42 +1156,39 @@ acid_status linear_forward(int dtype, const void* A, int64_t lda, int64_t M, int
                ACID_ERR_UNSUPPORTED, "linear: RoPE positions must be below 2^24");
   ACID_REQUIRE(!epi_reads_res(epi.kind) || epi.residual != nullptr, ACID_ERR_INVALID_ARG,
                "linear: residual epilogue needs a residual");
-  if (dtype == ACID_FP32) return linear_forward_f32(A, lda, M, K, W, N, out, ldo, epi, s);
+  ACID_REQUIRE(epi.text_rows >= 0 && epi.text_rows <= M && (epi.text_rows == 0 || epi.text_w != nullptr),
+               ACID_ERR_INVALID_ARG, "linear: bad text rows");
+  if (dtype == ACID_FP32) {
+    if (epi.text_rows > 0) {  // two streams: one launch each
+      const int64_t L = epi.text_rows;
+      Epilogue et = epi, ev = epi;
+      et.text_rows = ev.text_rows = 0;
+      et.bias = epi.text_bias;
+      ACID_TRY(linear_forward_f32(A, lda, L, K, epi.text_w, N, out, ldo, et, s));
+      ev.row_base += L;
+      if (ev.residual) ev.residual = static_cast<const float*>(ev.residual) + L * ev.ldr;
+      return linear_forward_f32(static_cast<const float*>(A) + L * lda, lda, M - L, K, W, N,
+                                static_cast<float*>(out) + L * ldo, ldo, ev, s);
+    }
+    return linear_forward_f32(A, lda, M, K, W, N, out, ldo, epi, s);
+  }
   ACID_REQUIRE(N % 32 == 0 && K % 8 == 0, ACID_ERR_UNSUPPORTED, "linear bf16: need N % 32 == 0 and K % 8 == 0");
   ACID_REQUIRE(ldo % 8 == 0 && aligned(out, 16) && (!epi.residual || (epi.ldr % 8 == 0 && aligned(epi.residual, 16))),
                ACID_ERR_UNSUPPORTED, "linear bf16: output/residual must be 16-byte aligned rows");
   ACID_REQUIRE(epi.kind != EPI_ROPE_QKV || (epi.head_dim & (epi.head_dim - 1)) == 0, ACID_ERR_UNSUPPORTED,
                "linear bf16: the RoPE epilogue needs a power-of-two head_dim");
-  // The widest tile that the output spans: a 128-wide tile moves a third more
-  // shared-memory bytes per FLOP than a 256-wide one, which costs more than
-  // the zero-filled columns of a partial last tile (N = 1920: 7% extra MMA
-  // work, against about 1.6x the throughput).
-  // SM pairs where the tiles' mainloop is long enough to matter: measured at
-  // M = 32760, pairs are 1-2% faster for N = 4608 / 8960 or K = 8960 and 2-3%
-  // slower for the 1536 x 1536 gated-residual output projection, whose
-  // residual traffic bounds it as much as its FLOPs do.
-  // Kinds without a residual leave through the pair kernel's accumulator-
-  // layout epilogue, which makes pairs faster from N = 1024 on (measured at
-  // M = 32760: cross-attention query 1535 -> 1565 TFLOP/s, the K = 128 patch
-  // embedding 40 -> 32 us); the residual kinds stay on single SMs up to 2048.
-  const bool no_res = epi.kind == EPI_BIAS || epi.kind == EPI_GELU || epi.kind == EPI_ROPE_QKV;
-  if (N > 128 && (N > 2048 || K > 2048 || (no_res && N >= 1024))) {
-    SplitKPlan sp;
-    if (epi.splitk_ws != nullptr && aligned(epi.splitk_ws, 128) &&
-        splitk_plan(M, N, K, epi.splitk_bytes, max_pairs<EPI_BIAS, false, true>(), &sp)) {
-      ACID_TRY(launch_tc2(A, lda, sp.rows_main, K, W, N, out, ldo, epi, s));
-      const size_t osz = epi.out_fp32 ? 4 : 2, rsz = epi.res_fp32 ? 4 : 2;
-      Epilogue et = epi;
-      et.row_base += sp.rows_main;
-      if (et.residual) et.residual = static_cast<const uint8_t*>(et.residual) + sp.rows_main * et.ldr * rsz;
-      return launch_tc2_splitk(static_cast<const uint8_t*>(A) + sp.rows_main * lda * 2, lda, M - sp.rows_main, K, W,
-                               N, static_cast<uint8_t*>(out) + sp.rows_main * ldo * osz, ldo, et, sp, s);
-    }
-    return launch_tc2(A, lda, M, K, W, N, out, ldo, epi, s);
+  SplitKPlan sp;
+  if (epi.splitk_ws != nullptr && aligned(epi.splitk_ws, 128) && epi.text_rows == 0 &&
+      splitk_plan(M, N, K, epi.splitk_bytes, max_pairs<EPI_BIAS, false, true>(), &sp)) {
+    ACID_TRY(launch_tc2(A, lda, sp.rows_main, K, W, N, out, ldo, epi, s));
+    const size_t osz = epi.out_fp32 ? 4 : 2, rsz = epi.res_fp32 ? 4 : 2;
+    Epilogue et = epi;
+    et.row_base += sp.rows_main;
+    if (et.residual) et.residual = static_cast<const uint8_t*>(et.residual) + sp.rows_main * et.ldr * rsz;
+    return launch_tc2_splitk(static_cast<const uint8_t*>(A) + sp.rows_main * lda * 2, lda, M - sp.rows_main, K, W, N,
+                             static_cast<uint8_t*>(out) + sp.rows_main * ldo * osz, ldo, et, sp, s);
   }
-  if (N > 128) return launch_tc<256>(A, lda, M, K, W, N, out, ldo, epi, s);
-  if (N > 64) return launch_tc<128>(A, lda, M, K, W, N, out, ldo, epi, s);
-  return launch_tc<64>(A, lda, M, K, W, N, out, ldo, epi, s);
+  return launch_tc2(A, lda, M, K, W, N, out, ldo, epi, s);
 }
 
 ACID_DEVICE_FLAG_READER(take_device_error_gemm)

@@ -49,6 +49,11 @@ struct Epilogue {
   int64_t rope_first_video = 0;
   int d = 0, head_dim = 0;
   bool out_fp32 = false;           // output dtype fp32 (else the GEMM dtype)
+  // dual-stream layers: rows [0, text_rows) of A, the residual and out are the
+  // text stream's and take these weights and bias (0: one stream)
+  const void* text_w = nullptr;
+  const float* text_bias = nullptr;
+  int64_t text_rows = 0;
   // optional device scratch for a split-K last round of the SM-pair GEMM
   // (long K only); without it the GEMM runs as one launch
   void* splitk_ws = nullptr;
