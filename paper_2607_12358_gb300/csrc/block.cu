@@ -27,6 +27,17 @@ acid_status lin(int dt, const void* A, int64_t lda, int64_t M, int K, const acid
   return linear_forward(dt, A, lda, M, K, L.w, N, out, ldo, e, s);
 }
 
+// A dual-stream layer over joint rows: the first text_rows rows take the text
+// stream's weights T.  One launch (bf16): the text rows' few tiles run beside
+// the video rows' instead of alone on a mostly idle GPU.
+acid_status lin_dual(int dt, const void* A, int64_t lda, int64_t M, int K, const acid_linear& L, const acid_linear& T,
+                     int64_t text_rows, int N, void* out, int64_t ldo, Epilogue e, cudaStream_t s) {
+  e.text_w = T.w;
+  e.text_bias = T.b;
+  e.text_rows = text_rows;
+  return lin(dt, A, lda, M, K, L, N, out, ldo, e, s);
+}
+
 }  // namespace
 
 int64_t block_rows(const acid_block_desc& d) {
@@ -111,7 +122,6 @@ acid_status block_forward_impl(const acid_block_desc& D, void* x, const float* t
   const int d = D.d, F = D.ffn, hd = d / D.heads;
   const int64_t L = D.kind == ACID_BLOCK_WAN ? 0 : D.n_text;  // joint text rows
   const int64_t rows = block_rows(D);
-  const int64_t Nv = rows - L;
   const float eps = D.ln_eps;
 
   // rope tables for the video grid
@@ -184,18 +194,15 @@ acid_status block_forward_impl(const acid_block_desc& D, void* x, const float* t
   // xm, and the FFN branch writes the final x = xm + g2 * (...) in the block
   // dtype, so a bf16 block rounds its residual stream once.
   float* xm = ws.xm;
-  auto gated_to_xm = [&](int64_t r0) {  // out: xm, residual: x (block dtype)
+  auto gated_to_xm = [&]() {  // out: xm, residual: x (block dtype)
     Epilogue e = gated(2);
-    e.row_base = r0;
-    e.residual = off(x, r0 * d, dt);
     e.res_fp32 = dt == ACID_FP32;
     e.out_fp32 = true;
     return e;
   };
-  auto gated_from_xm = [&](int64_t r0) {  // out: x (block dtype), residual: xm
+  auto gated_from_xm = [&]() {  // out: x (block dtype), residual: xm
     Epilogue e = gated(5);
-    e.row_base = r0;
-    e.residual = xm + r0 * d;
+    e.residual = xm;
     e.res_fp32 = true;
     e.out_fp32 = dt == ACID_FP32;
     e.splitk_ws = ws.splitk;  // FFN2 (K = ffn): a long mainloop
@@ -206,11 +213,7 @@ acid_status block_forward_impl(const acid_block_desc& D, void* x, const float* t
   // ---- attention branch: xm = x + g1 * O(Attn(RoPE(QKV(LNmod1 x))))
   ACID_TRY(ln_mod(dt, x, dt, ws.u, rows, d, mv, mv + d, mt, mt + d, L, eps, s));
   if (D.kind == ACID_BLOCK_HV_DUAL) {
-    Epilogue et = ep_qkv;
-    ACID_TRY(lin(dt, ws.u, d, L, d, W.t_qkv, 3 * d, ws.qkv, 3 * d, et, s));
-    Epilogue ev = ep_qkv;
-    ev.row_base = L;
-    ACID_TRY(lin(dt, off(ws.u, L * d, dt), d, Nv, d, W.qkv, 3 * d, off(ws.qkv, L * 3 * d, dt), 3 * d, ev, s));
+    ACID_TRY(lin_dual(dt, ws.u, d, rows, d, W.qkv, W.t_qkv, L, 3 * d, ws.qkv, 3 * d, ep_qkv, s));
   } else {
     ACID_TRY(lin(dt, ws.u, d, rows, d, W.qkv, 3 * d, ws.qkv, 3 * d, ep_qkv, s));
   }
@@ -218,10 +221,9 @@ acid_status block_forward_impl(const acid_block_desc& D, void* x, const float* t
   self.ldo = d;
   ACID_TRY(attention_forward(dt, self, s));
   if (D.kind == ACID_BLOCK_HV_DUAL) {
-    ACID_TRY(lin(dt, ws.att, d, L, d, W.t_o, d, xm, d, gated_to_xm(0), s));
-    ACID_TRY(lin(dt, off(ws.att, L * d, dt), d, Nv, d, W.o, d, xm + L * d, d, gated_to_xm(L), s));
+    ACID_TRY(lin_dual(dt, ws.att, d, rows, d, W.o, W.t_o, L, d, xm, d, gated_to_xm(), s));
   } else {
-    ACID_TRY(lin(dt, ws.att, d, rows, d, W.o, d, xm, d, gated_to_xm(0), s));
+    ACID_TRY(lin(dt, ws.att, d, rows, d, W.o, d, xm, d, gated_to_xm(), s));
   }
 
   // ---- cross-attention (WAN with text): xm += O_c(Attn(Q_c(LN xm), KV_c(ctx)))
@@ -263,13 +265,11 @@ acid_status block_forward_impl(const acid_block_desc& D, void* x, const float* t
   Epilogue eg;
   eg.kind = EPI_GELU;
   if (D.kind == ACID_BLOCK_HV_DUAL) {
-    ACID_TRY(lin(dt, ws.u, d, L, d, W.t_ff1, F, ws.hid, F, eg, s));
-    ACID_TRY(lin(dt, off(ws.u, L * d, dt), d, Nv, d, W.ff1, F, off(ws.hid, L * F, dt), F, eg, s));
-    ACID_TRY(lin(dt, ws.hid, F, L, F, W.t_ff2, d, x, d, gated_from_xm(0), s));
-    ACID_TRY(lin(dt, off(ws.hid, L * F, dt), F, Nv, F, W.ff2, d, off(x, L * d, dt), d, gated_from_xm(L), s));
+    ACID_TRY(lin_dual(dt, ws.u, d, rows, d, W.ff1, W.t_ff1, L, F, ws.hid, F, eg, s));
+    ACID_TRY(lin_dual(dt, ws.hid, F, rows, F, W.ff2, W.t_ff2, L, d, x, d, gated_from_xm(), s));
   } else {
     ACID_TRY(lin(dt, ws.u, d, rows, d, W.ff1, F, ws.hid, F, eg, s));
-    ACID_TRY(lin(dt, ws.hid, F, rows, F, W.ff2, d, x, d, gated_from_xm(0), s));
+    ACID_TRY(lin(dt, ws.hid, F, rows, F, W.ff2, d, x, d, gated_from_xm(), s));
   }
   return ACID_OK;
 }

@@ -1,5 +1,6 @@
 """GPU parity of the SM-pair GEMM at every tile width its dispatch can choose,
-with ragged rows, columns and K, and of residual rows that overlap."""
+with ragged rows, columns and K, of residual rows that overlap, and of
+dual-stream layers whose text and video rows share a launch."""
 
 import numpy as np
 import pytest
@@ -83,3 +84,26 @@ def test_residual_rows_that_overlap(acid, ldr, fp32):
     ref = r + O.linear(a, w, np.zeros(N, np.float32))
     absolute, rel = _tol(a, w, np.abs(r), K, fp32)
     assert np.all(np.abs(got.float().cpu().numpy() - ref) <= absolute + rel * np.abs(ref))
+
+
+@pytest.mark.parametrize("n_text", [0, 1, 255, 256, 300])
+def test_dual_stream_rows_share_a_launch(acid, n_text):
+    """Text rows of less than, exactly and more than one 256-row tile, and
+    none: each stream keeps its own weights, bias, modulation and rows."""
+    cfg = S.get_config("hv", d=256, heads=2, ffn=1024, n_text=n_text, latent_f=3, latent_h=16, latent_w=22)
+    w = S.block_weights(cfg, 0, seed=4, block_type="hv_dual", q_scale=4.0)
+    x = S.hidden(cfg, cfg.n_video + n_text, seed=n_text)
+    temb = S.temb_vector(cfg, seed=4)
+    blk = acid.DeviceBlock.upload(w, "hv_dual", torch.bfloat16, DEV)
+    got = acid.acid_dit_block_forward(acid.block_desc(cfg, "hv_dual"), _bf(x), _f32(temb), blk).float().cpu().numpy()
+    acid.check_device_error()
+    mt, mv = O.block_modulation(temb, w["txt.mod"]), O.block_modulation(temb, w["vid.mod"])
+    if n_text:
+        yt, yv = O.hv_dual_block(x[:n_text], x[n_text:], mt, mv, w, cfg.grid, cfg.heads)
+    else:  # the video stream alone: self-attention and FFN with its weights
+        vid = {k[4:]: v for k, v in w.items() if k.startswith("vid.")}
+        yt, yv = x[:0], O.wan_block(x, mv, vid, cfg.grid, cfg.heads)
+    # the block tolerance of the bf16 path, for each stream by itself
+    for g, r in ((got[:n_text], yt), (got[n_text:], yv)):
+        if r.size:
+            assert np.linalg.norm(g - r) <= 1e-2 * np.linalg.norm(r) and np.abs(g - r).max() <= 5e-2
