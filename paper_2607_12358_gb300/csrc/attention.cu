@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
   uint64_t* drain = bars + 15;    // failure path: the MMAs issued so far have completed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int item = a.item_base + (int)blockIdx.x / a.splits, split = (int)blockIdx.x % a.splits;
   const int qt = item % a.nqp, h = item / a.nqp;
   const int nkv_all = (int)((a.nk + C::BKV - 1) / C::BKV);
@@ -321,47 +321,59 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
       if (nv_issued < nkv) drain_loads(q_full, k_full, v_full, nk_issued, nv_issued);
     }
   } else if (warp == 1) {
-    if (lane == 0) {  // ---------------------------------------- MMA issuer
-      // Shared-memory descriptors are built once; an operand at byte offset o
-      // from a base is the base descriptor plus o >> 4 (the 14-bit address
-      // field cannot overflow: shared memory ends below 256 KB).
-      const uint64_t qdesc = smem_desc_sw128(smem_u32(sQ), 16, 1024);
-      const uint64_t kdesc = smem_desc_sw128(smem_u32(sK), 16, 1024);
-      const uint64_t vdesc = smem_desc_sw128(smem_u32(sV), C::CHUNK_KV, 1024);
-      // S_t(j) = Q_t K_j^T into the S region of tile t
-      auto issue_s = [&](int t, int j) {
-        issue_s_mma<D>(tmem + C::S_COL + t * C::BKV, qdesc + (uint64_t)((t * C::T_BYTES) >> 4),
-                       kdesc + (uint64_t)(((j & 1) * C::KV_BYTES) >> 4));
-        mma_commit(&s_full[t]);
-      };
-      bool ok = mbar_wait(q_full, 0) && mbar_wait(&k_full[0], 0);
-      if (ok) {
-        tc_fence_after();
+    // ------------------------------------------------------- MMA issuer
+    // The whole warp walks the loop (descriptors and flags stay in uniform
+    // registers) and one elected lane issues.  Descriptors are built once; an
+    // operand at byte offset o from a base is the base descriptor plus o >> 4
+    // (the 14-bit address field cannot overflow: shared memory ends below
+    // 256 KB).
+    const bool leader = elect_one();
+    const uint64_t qdesc = smem_desc_sw128(smem_u32(sQ), 16, 1024);
+    const uint64_t kdesc = smem_desc_sw128(smem_u32(sK), 16, 1024);
+    const uint64_t vdesc = smem_desc_sw128(smem_u32(sV), C::CHUNK_KV, 1024);
+    // S_t(j) = Q_t K_j^T into the S region of tile t
+    auto issue_s = [&](int t, int j) {
+      issue_s_mma<D>(tmem + C::S_COL + t * C::BKV, qdesc + (uint64_t)((t * C::T_BYTES) >> 4),
+                     kdesc + (uint64_t)(((j & 1) * C::KV_BYTES) >> 4));
+      mma_commit(&s_full[t]);
+    };
+    bool ok = mbar_wait_warp(q_full, 0) && mbar_wait_warp(&k_full[0], 0);
+    if (ok) {
+      tc_fence_after();
+      if (leader) {
         issue_s(0, 0);
         issue_s(1, 0);
         mma_commit(&k_empty[0]);
       }
-      for (int j = 0; ok && j < nkv; ++j) {
-        const int st = j & 1;
-        for (int t = 0; t < 2 && ok; ++t) {
-          if (!mbar_wait(&p_full[t], j & 1)) { ok = false; break; }
-          if (t == 0 && !mbar_wait(&v_full[st], (j >> 1) & 1)) { ok = false; break; }
-          tc_fence_after();
+      __syncwarp();
+    }
+    for (int j = 0; ok && j < nkv; ++j) {
+      const int st = j & 1;
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (!mbar_wait_warp(&p_full[t], j & 1)) { ok = false; break; }
+        if (t == 0 && !mbar_wait_warp(&v_full[st], (j >> 1) & 1)) { ok = false; break; }
+        tc_fence_after();
+        if (leader) {
           // O_t += P_t V_j
           issue_pv_mma<D>(tmem + C::o_col(t), tmem + C::S_COL + t * C::BKV,
                           vdesc + (uint64_t)((st * C::KV_BYTES) >> 4), j != 0);
           mma_commit(&pv_done[t]);
           if (t == 1) mma_commit(&v_empty[st]);
-          if (j + 1 < nkv) {
-            if (t == 0 && !mbar_wait(&k_full[st ^ 1], ((j + 1) >> 1) & 1)) { ok = false; break; }
-            tc_fence_after();
+        }
+        __syncwarp();
+        if (j + 1 < nkv) {
+          if (t == 0 && !mbar_wait_warp(&k_full[st ^ 1], ((j + 1) >> 1) & 1)) { ok = false; break; }
+          tc_fence_after();
+          if (leader) {
             issue_s(t, j + 1);
             if (t == 1) mma_commit(&k_empty[st ^ 1]);
           }
+          __syncwarp();
         }
       }
-      if (!ok) drain_mmas(drain);
     }
+    if (!ok && leader) drain_mmas(drain);
   } else {  // ---------------------------------------- softmax: warps 2-5 tile a, 6-9 tile b
     const int t = (warp - 2) >> 2;
     const int q = warp & 3;
@@ -456,7 +468,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
   uint64_t* drain = bars + 18;    // failure path: the MMAs issued so far have completed
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 19);
 
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = warp_index(), lane = threadIdx.x & 31;
   const int item0 = a.item_base + (int)blockIdx.x, item_step = (int)gridDim.x;
   const int n_items = item0 < a.item_end ? (a.item_end - 1 - item0) / item_step + 1 : 0;
   const int nkv = (int)((a.nk + C::BKV - 1) / C::BKV);
@@ -520,52 +532,62 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
       }
     }
   } else if (warp == 1) {
-    if (lane == 0) {  // ---------------------------------------- MMA issuer
-      const uint64_t qdesc = smem_desc_sw128(smem_u32(sQ), 16, 1024);
-      const uint64_t kdesc = smem_desc_sw128(smem_u32(sK), 16, 1024);
-      const uint64_t vdesc = smem_desc_sw128(smem_u32(sV), C::CHUNK_KV, 1024);
-      // S_t = Q_t K^T of step g into the S region of tile t; after an item's
-      // last key tile (last_tile) the producer may replace Q_t
-      auto issue_s = [&](int t, int g, bool last_tile) {
-        issue_s_mma<D>(tmem + C::S_COL + t * C::BKV, qdesc + (uint64_t)((t * C::T_BYTES) >> 4),
-                       kdesc + (uint64_t)(((g & 1) * C::KV_BYTES) >> 4));
-        mma_commit(&s_full[t]);
-        if (last_tile) mma_commit(&q_empty[t]);
-      };
-      bool ok = total > 0 && mbar_wait(&k_full[0], 0);
-      for (int t = 0; t < 2 && ok; ++t) {
-        if (!mbar_wait(&q_full[t], 0)) { ok = false; break; }
+    // ------------------------------------------------------- MMA issuer
+    // (whole warp walks, one elected lane issues, as in attn_tc_kernel)
+    const bool leader = elect_one();
+    const uint64_t qdesc = smem_desc_sw128(smem_u32(sQ), 16, 1024);
+    const uint64_t kdesc = smem_desc_sw128(smem_u32(sK), 16, 1024);
+    const uint64_t vdesc = smem_desc_sw128(smem_u32(sV), C::CHUNK_KV, 1024);
+    // S_t = Q_t K^T of step g into the S region of tile t; after an item's
+    // last key tile (last_tile) the producer may replace Q_t
+    auto issue_s = [&](int t, int g, bool last_tile) {
+      issue_s_mma<D>(tmem + C::S_COL + t * C::BKV, qdesc + (uint64_t)((t * C::T_BYTES) >> 4),
+                     kdesc + (uint64_t)(((g & 1) * C::KV_BYTES) >> 4));
+      mma_commit(&s_full[t]);
+      if (last_tile) mma_commit(&q_empty[t]);
+    };
+    bool ok = total > 0 && mbar_wait_warp(&k_full[0], 0);
+    for (int t = 0; t < 2 && ok; ++t) {
+      if (!mbar_wait_warp(&q_full[t], 0)) { ok = false; break; }
+      tc_fence_after();
+      if (leader) issue_s(t, 0, nkv == 1);
+      __syncwarp();
+    }
+    if (ok && leader) mma_commit(&k_empty[0]);
+    __syncwarp();
+    // step g (key tile j of item k): PV_a(g) S_a(g+1) PV_b(g) S_b(g+1); at an
+    // item boundary S(g+1) reads the next item's Q
+    for (int g = 0, j = 0, k = 0; ok && g < total; ++g) {
+      const int st = g & 1, gn = g + 1;
+      const bool boundary = j + 1 == nkv;  // step gn starts item k + 1
+      const int jn = boundary ? 0 : j + 1;
+#pragma unroll
+      for (int t = 0; t < 2; ++t) {
+        if (!mbar_wait_warp(&p_full[t], g & 1)) { ok = false; break; }
+        if (t == 0 && !mbar_wait_warp(&v_full[st], (g >> 1) & 1)) { ok = false; break; }
         tc_fence_after();
-        issue_s(t, 0, nkv == 1);
-      }
-      if (ok) mma_commit(&k_empty[0]);
-      // step g (key tile j of item k): PV_a(g) S_a(g+1) PV_b(g) S_b(g+1); at an
-      // item boundary S(g+1) reads the next item's Q
-      for (int g = 0, j = 0, k = 0; ok && g < total; ++g) {
-        const int st = g & 1, gn = g + 1;
-        const bool boundary = j + 1 == nkv;  // step gn starts item k + 1
-        const int jn = boundary ? 0 : j + 1;
-        for (int t = 0; t < 2 && ok; ++t) {
-          if (!mbar_wait(&p_full[t], g & 1)) { ok = false; break; }
-          if (t == 0 && !mbar_wait(&v_full[st], (g >> 1) & 1)) { ok = false; break; }
-          tc_fence_after();
+        if (leader) {
           issue_pv_mma<D>(tmem + C::o_col(t), tmem + C::S_COL + t * C::BKV,
                           vdesc + (uint64_t)((st * C::KV_BYTES) >> 4), j != 0);
           mma_commit(&pv_done[t]);
           if (t == 1) mma_commit(&v_empty[st]);
-          if (gn < total) {
-            if (t == 0 && !mbar_wait(&k_full[st ^ 1], (gn >> 1) & 1)) { ok = false; break; }
-            if (boundary && !mbar_wait(&q_full[t], (k + 1) & 1)) { ok = false; break; }
-            tc_fence_after();
+        }
+        __syncwarp();
+        if (gn < total) {
+          if (t == 0 && !mbar_wait_warp(&k_full[st ^ 1], (gn >> 1) & 1)) { ok = false; break; }
+          if (boundary && !mbar_wait_warp(&q_full[t], (k + 1) & 1)) { ok = false; break; }
+          tc_fence_after();
+          if (leader) {
             issue_s(t, gn, jn == nkv - 1);
             if (t == 1) mma_commit(&k_empty[st ^ 1]);
           }
+          __syncwarp();
         }
-        j = jn;
-        k += boundary;
       }
-      if (!ok) drain_mmas(drain);
+      j = jn;
+      k += boundary;
     }
+    if (!ok && leader) drain_mmas(drain);
   } else {  // ---------------------------------------- softmax: warps 2-5 tile a, 6-9 tile b
     const int t = (warp - 2) >> 2;
     const int q = warp & 3;
