@@ -135,13 +135,14 @@ acid_status block_forward_impl(const acid_block_desc& D, void* x, const float* t
 
   // modulation vectors
   const int nmod = D.kind == ACID_BLOCK_COG ? 12 * d : (D.kind == ACID_BLOCK_HV_SINGLE ? 3 * d : 6 * d);
-  ACID_TRY(gemv(dt, W.mod.w, W.mod.b, temb, ws.mod, nmod, d, true, s));
   const float* mv = ws.mod;  // video stream (or only stream)
   const float* mt = mv;      // text stream
   if (D.kind == ACID_BLOCK_COG) mt = ws.mod + 6 * d;
   if (D.kind == ACID_BLOCK_HV_DUAL) {
-    ACID_TRY(gemv(dt, W.t_mod.w, W.t_mod.b, temb, ws.mod_t, 6 * d, d, true, s));
+    ACID_TRY(gemv2(dt, W.mod.w, W.mod.b, ws.mod, nmod, W.t_mod.w, W.t_mod.b, ws.mod_t, 6 * d, temb, d, true, s));
     mt = ws.mod_t;
+  } else {
+    ACID_TRY(gemv(dt, W.mod.w, W.mod.b, temb, ws.mod, nmod, d, true, s));
   }
 
   Epilogue ep_qkv;

@@ -702,33 +702,81 @@ __global__ void __launch_bounds__(32 * kTemniMaxWarps, 1) temni_drift_kernel(con
 }
 
 // ---------------------------------------------------------------- GEMV
-template <typename TW>
-__global__ void __launch_bounds__(kThreads) gemv_kernel(const TW* __restrict__ W, const float* __restrict__ b,
-                                                        const float* __restrict__ x, float* __restrict__ y,
-                                                        int n_out, int k, int silu_in) {
-  extern __shared__ float xs[];
-  for (int i = threadIdx.x; i < k; i += blockDim.x) xs[i] = silu_in ? silu(x[i]) : x[i];
-  __syncthreads();
-  const int row = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
-  const int lane = threadIdx.x & 31;
-  if (row >= n_out) return;
-  const TW* wr = W + (int64_t)row * k;
-  float acc = 0.f;
-  for (int c = lane * 8; c < k; c += 256) {
-    if (!ACID_IN_BOUNDS(kSiteGemv, (int64_t)row * k + c + 7, (int64_t)n_out * k)) continue;
-    float w[8];
-    load8(wr + c, w);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) acc = fmaf(w[j], xs[c + j], acc);
+// A warp forms R outputs of one or two matrices that share the input (rows
+// from n_out on are the second's).  The input is staged once per CTA, as two
+// arrays of alternating 16-byte units, so that the warp's reads of its eight
+// values per lane are contiguous, and each read serves R weight rows: with one
+// row per warp and a 32-byte lane stride the shared-memory reads took four
+// times the cycles of the weight stream.
+struct GemvMat {
+  const void* W;
+  const float* b;
+  float* y;
+  int n_out;
+};
+
+template <typename TW, int R>
+__global__ void __launch_bounds__(kThreads, 3) gemv_kernel(GemvMat m0, GemvMat m1, const float* __restrict__ x, int k,
+                                                           int silu_in) {
+  extern __shared__ __align__(16) float xs[];  // [2][k / 2]: columns 8 i + {0..3}, then 8 i + {4..7}
+  for (int i = threadIdx.x; i < k; i += kThreads) {
+    const float v = x[i];
+    xs[(i & 4 ? k / 2 : 0) + (i >> 3) * 4 + (i & 3)] = silu_in ? silu(v) : v;
   }
-  acc = warp_sum_f(acc);
-  if (lane == 0) y[row] = acc + (b ? b[row] : 0.f);
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int total = m0.n_out + m1.n_out;
+  for (int first = (blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * R; first < total;
+       first += gridDim.x * (kThreads / 32) * R) {
+    const TW* wr[R];
+    float acc[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int row = min(first + r, total - 1);  // rows past the end repeat the last one and are not stored
+      wr[r] = row < m0.n_out ? static_cast<const TW*>(m0.W) + (int64_t)row * k
+                             : static_cast<const TW*>(m1.W) + (int64_t)(row - m0.n_out) * k;
+      acc[r] = 0.f;
+    }
+#pragma unroll 2
+    for (int c = lane * 8; c < k; c += 256) {
+      if (!ACID_IN_BOUNDS(kSiteGemv, c + 7, k)) continue;
+      float w[R][8];
+#pragma unroll
+      for (int r = 0; r < R; ++r) load8(wr[r] + c, w[r]);
+      const float4 lo = *reinterpret_cast<const float4*>(xs + c / 2);
+      const float4 hi = *reinterpret_cast<const float4*>(xs + k / 2 + c / 2);
+      const float xv[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+#pragma unroll
+      for (int r = 0; r < R; ++r)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[r] = fmaf(w[r][j], xv[j], acc[r]);
+    }
+#pragma unroll
+    for (int r = 0; r < R; ++r) acc[r] = warp_sum_f(acc[r]);
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int row = first + r;
+      if (lane == 0 && row < total) {
+        const GemvMat& m = row < m0.n_out ? m0 : m1;
+        const int o = row < m0.n_out ? row : row - m0.n_out;
+        m.y[o] = acc[r] + (m.b ? m.b[o] : 0.f);
+      }
+    }
+  }
 }
 
+// Small fp64 tables.  An SM has few fp64 units, so these run as many CTAs of
+// one warp, spread over the SMs, with the cosines and sines in separate warps:
+// 128 frequencies as one CTA of 128 threads took 5.6 us, a 1200-entry RoPE
+// table on 10 CTAs 8 us.
+constexpr int kTableThreads = 32;
+
 __device__ __forceinline__ void sinusoid_at(float* out, double t, int half, int j) {
-  const double f = exp(-log(10000.0) * (double)j / (double)half);
-  out[j] = (float)cos(t * f);
-  out[half + j] = (float)sin(t * f);
+  const double a = t * exp(-log(10000.0) * (double)j / (double)half);
+  if (blockIdx.y == 0)
+    out[j] = (float)cos(a);
+  else
+    out[half + j] = (float)sin(a);
 }
 
 __global__ void sinusoid_kernel(float* out, double t, int half) {
@@ -759,7 +807,10 @@ __global__ void rope_table_kernel(float2* tbl, int F, int H, int W, int pt, int 
   }
   const double dim = 2.0 * pairs;
   const double ang = (double)pos * pow(theta, -2.0 * j / dim);
-  tbl[i] = make_float2((float)cos(ang), (float)sin(ang));
+  if (blockIdx.y == 0)
+    tbl[i].x = (float)cos(ang);
+  else
+    tbl[i].y = (float)sin(ang);
 }
 
 // ---------------------------------------------------------------- patches
@@ -1077,22 +1128,40 @@ acid_status temni_drift(const float* h_cur, const float* h_prev, const float* mo
   return ACID_OK;
 }
 
-acid_status gemv(int w_dtype, const void* W, const float* b, const float* x, float* y, int n_out, int k,
-                 bool silu_input, cudaStream_t s) {
-  ACID_REQUIRE(k % 8 == 0 && k <= 16384, ACID_ERR_UNSUPPORTED, "gemv: k must be a multiple of 8, <= 16384");
-  const int blocks = (n_out + kThreads / 32 - 1) / (kThreads / 32);
+namespace {
+template <typename TW>
+acid_status launch_gemv(const GemvMat& m0, const GemvMat& m1, const float* x, int k, bool silu_input, cudaStream_t s) {
+  const int total = m0.n_out + m1.n_out;
   const size_t smem = sizeof(float) * k;
-  if (w_dtype == ACID_BF16)
-    gemv_kernel<__nv_bfloat16><<<blocks, kThreads, smem, s>>>((const __nv_bfloat16*)W, b, x, y, n_out, k, silu_input);
+  // four rows per warp, on as many CTAs as are resident, once every SM gets two
+  auto grid = [&](int rows) { return std::min((total + kThreads / 32 * rows - 1) / (kThreads / 32 * rows), 152 * 3); };
+  if (total >= 152 * 2 * (kThreads / 32) * 4)
+    gemv_kernel<TW, 4><<<grid(4), kThreads, smem, s>>>(m0, m1, x, k, silu_input);
+  else if (total >= 152 * 2 * (kThreads / 32) * 2)
+    gemv_kernel<TW, 2><<<grid(2), kThreads, smem, s>>>(m0, m1, x, k, silu_input);
   else
-    gemv_kernel<float><<<blocks, kThreads, smem, s>>>((const float*)W, b, x, y, n_out, k, silu_input);
+    gemv_kernel<TW, 1><<<grid(1), kThreads, smem, s>>>(m0, m1, x, k, silu_input);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
+}
+}  // namespace
+
+acid_status gemv2(int w_dtype, const void* W, const float* b, float* y, int n_out, const void* W2, const float* b2,
+                  float* y2, int n_out2, const float* x, int k, bool silu_input, cudaStream_t s) {
+  ACID_REQUIRE(k % 8 == 0 && k <= 16384, ACID_ERR_UNSUPPORTED, "gemv: k must be a multiple of 8, <= 16384");
+  const GemvMat m0{W, b, y, n_out}, m1{W2, b2, y2, n_out2};
+  return w_dtype == ACID_BF16 ? launch_gemv<__nv_bfloat16>(m0, m1, x, k, silu_input, s)
+                              : launch_gemv<float>(m0, m1, x, k, silu_input, s);
+}
+
+acid_status gemv(int w_dtype, const void* W, const float* b, const float* x, float* y, int n_out, int k,
+                 bool silu_input, cudaStream_t s) {
+  return gemv2(w_dtype, W, b, y, n_out, nullptr, nullptr, nullptr, 0, x, k, silu_input, s);
 }
 
 acid_status timestep_sinusoid(float* out, double t, int dim, cudaStream_t s) {
   const int half = dim / 2;
-  sinusoid_kernel<<<(half + 127) / 128, 128, 0, s>>>(out, t, half);
+  sinusoid_kernel<<<dim3((half + kTableThreads - 1) / kTableThreads, 2), kTableThreads, 0, s>>>(out, t, half);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1114,8 +1183,9 @@ acid_status rope_build(RopeTable& t, float2* storage, float theta, cudaStream_t 
   t.table = storage;
   const int64_t total = t.elems();
   if (total == 0) return ACID_OK;
-  rope_table_kernel<<<(int)((total + 127) / 128), 128, 0, s>>>(storage, t.grid_f, t.grid_h, t.grid_w, t.pairs_t,
-                                                              t.pairs_h, t.pairs_w, (double)theta);
+  const dim3 grid((unsigned)((total + kTableThreads - 1) / kTableThreads), 2);
+  rope_table_kernel<<<grid, kTableThreads, 0, s>>>(storage, t.grid_f, t.grid_h, t.grid_w, t.pairs_t, t.pairs_h, t.pairs_w,
+                                                   (double)theta);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1177,7 +1247,7 @@ acid_status euler_update_sig(float* latent, const float* v, int64_t n, const dou
 
 acid_status timestep_sinusoid_sig(float* out, const double* sig, const int* step, int dim, cudaStream_t s) {
   const int half = dim / 2;
-  sinusoid_sig_kernel<<<(half + 127) / 128, 128, 0, s>>>(out, sig, step, half);
+  sinusoid_sig_kernel<<<dim3((half + kTableThreads - 1) / kTableThreads, 2), kTableThreads, 0, s>>>(out, sig, step, half);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }

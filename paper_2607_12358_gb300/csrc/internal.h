@@ -112,6 +112,10 @@ acid_status temni_drift(const float* h_cur, const float* h_prev, const float* mo
 acid_status gemv(int w_dtype, const void* W, const float* b, const float* x, float* y, int n_out,
                  int k, bool silu_input, cudaStream_t s);
 
+// The same for two matrices of one input in one launch (y2 = W2 act(x) + b2).
+acid_status gemv2(int w_dtype, const void* W, const float* b, float* y, int n_out, const void* W2, const float* b2,
+                  float* y2, int n_out2, const float* x, int k, bool silu_input, cudaStream_t s);
+
 acid_status timestep_sinusoid(float* out, double t, int dim, cudaStream_t s);
 
 // drift partial sums (fixed-order two-pass reduction) and optional fused apply
