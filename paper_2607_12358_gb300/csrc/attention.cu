@@ -300,6 +300,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_begin();  // the set-up above overlaps the tail of the kernel before
 
   if (warp == 0) {
     if (lane == 0) {  // ---------------------------------------- TMA producer
@@ -498,6 +499,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_begin();  // the set-up above overlaps the tail of the kernel before
 
   if (warp == 0) {
     if (lane == 0) {  // ---------------------------------------- TMA producer
@@ -667,6 +669,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
 // One warp per row (256 rows per item), D / 32 columns per lane.
 template <int D>
 __global__ void __launch_bounds__(256) attn_merge_kernel(AttnDev a, int item0, int tail, int splits) {
+  pdl_begin();
   const int wrow = (int)(blockIdx.x * 8 + (threadIdx.x >> 5));  // row over all tail items
   const int lane = threadIdx.x & 31;
   if (wrow >= tail * kBQ) return;
@@ -757,9 +760,9 @@ acid_status launch_attn_tc(const AttnArgs& x, cudaStream_t s) {
     CUtensorMap to;
     ACID_TRY(make_tmap_bf16_box(&to, x.out, x.nq, x.ldo, x.ldo, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B));
     a.item_end = main_items;
-    attn_persist_kernel<D><<<std::min(main_items, slots), kAttnThreads, C::SMEM_P, s>>>(tq, tk, tv, to, a);
+    launch_pdl(attn_persist_kernel<D>, std::min(main_items, slots), kAttnThreads, C::SMEM_P, s, tq, tk, tv, to, a);
   } else {
-    attn_tc_kernel<D><<<main_items, kAttnThreads, C::SMEM, s>>>(tq, tk, tv, a);
+    launch_pdl(attn_tc_kernel<D>, main_items, kAttnThreads, C::SMEM, s, tq, tk, tv, a);
   }
   ACID_CHECK_LAUNCH();
   if (!split_tail) return ACID_OK;
@@ -767,9 +770,9 @@ acid_status launch_attn_tc(const AttnArgs& x, cudaStream_t s) {
   a.splits = splits;
   a.part_o = static_cast<float*>(x.part);
   a.part_ml = a.part_o + (size_t)tail * splits * kBQ * D;
-  attn_tc_kernel<D><<<tail * splits, kAttnThreads, C::SMEM, s>>>(tq, tk, tv, a);
+  launch_pdl(attn_tc_kernel<D>, tail * splits, kAttnThreads, C::SMEM, s, tq, tk, tv, a);
   ACID_CHECK_LAUNCH();
-  attn_merge_kernel<D><<<tail * kBQ / 8, 256, 0, s>>>(a, full, tail, splits);
+  launch_pdl(attn_merge_kernel<D>, tail * kBQ / 8, 256, 0, s, a, full, tail, splits);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -842,6 +845,7 @@ __device__ __forceinline__ void load_rows_f32(float* dst, int lds, const float* 
 
 template <int D, int BQ>
 __global__ void __launch_bounds__(128 * kF32Groups) attn_f32_kernel(AttnF32Args a) {
+  pdl_begin();
   using C = AttnF32Cfg<D, BQ>;
   constexpr int QT = C::QT, KT = kF32Keys / 16, NC = D / 32;  // NC column pairs per lane
   extern __shared__ __align__(16) float fsm[];
@@ -1002,7 +1006,7 @@ acid_status attn_f32_launch(const AttnF32Args& a, int heads, cudaStream_t s) {
     attr_done = true;
   }
   const dim3 grid((unsigned)((a.nq + BQ - 1) / BQ), (unsigned)heads);
-  attn_f32_kernel<D, BQ><<<grid, 128 * kF32Groups, C::SMEM, s>>>(a);
+  launch_pdl(attn_f32_kernel<D, BQ>, grid, 128 * kF32Groups, C::SMEM, s, a);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }

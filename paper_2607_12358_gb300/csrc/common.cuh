@@ -9,6 +9,7 @@
 #include <stdint.h>
 
 #include <string>
+#include <utility>
 
 #include "acid.h"
 
@@ -45,6 +46,26 @@ void count_launch();
     ACID_CUDA(cudaGetLastError()); \
   } while (0)
 
+// Launches a kernel that may start while the kernel before it on the stream is
+// still draining (programmatic dependent launch): its launch and set-up
+// overlap that kernel's tail.  Every kernel launched this way calls pdl_begin
+// (or pdl_trigger and pdl_wait) before its first access to global memory, and
+// pdl_wait returns once the kernel before has completed and its writes are
+// visible, so the stream's order of effects is kept, link by link.
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, std::forward<A>(args)...);
+}
 // Records CUDA events around one launch on its stream while profiling is on
 // (acid_profile_enable); `work` is the launch's algorithmic FLOPs or bytes.
 enum ProfKind { PROF_ATTENTION = 0, PROF_LINEAR = 1, PROF_DRIFT = 2, PROF_KINDS = 3 };
@@ -119,6 +140,18 @@ constexpr bool kBoundsChecked = false;
     else if (r.site) cudaMemcpyToSymbol(g_bounds, &z, sizeof(z));                    \
     return r;                                                                        \
   }
+
+// ---------------------------------------------------------------------------
+// Programmatic dependent launch (see launch_pdl)
+// ---------------------------------------------------------------------------
+// The next kernel may be launched once every CTA has come this far.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Waits until the kernel before this one has completed.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_begin() {
+  pdl_trigger();
+  pdl_wait();
+}
 
 // ---------------------------------------------------------------------------
 // Numeric helpers

@@ -72,6 +72,7 @@ __global__ void __launch_bounds__(kThreads, 4) drift_partials_kernel(const T* __
                                                                      const T* __restrict__ cur,
                                                                      const T* __restrict__ resid, T* out,
                                                                      int64_t n, double2* __restrict__ partials) {
+  pdl_begin();
   constexpr int V = Vec<T>::N;
   constexpr int U = kApply ? 2 : 4;  // 16-byte vectors in flight per thread and tensor
   const int64_t nvec = n / V;
@@ -151,6 +152,7 @@ __device__ __forceinline__ void write_drift_result(double num, double den, doubl
 // Fixed-order reduction of the CTA partials; result = {rel, num, den}.
 __global__ void __launch_bounds__(kThreads) drift_final_kernel(const double2* __restrict__ partials, int nparts,
                                                                double* __restrict__ result) {
+  pdl_begin();
   double n = 0.0, d = 0.0;
   for (int i = threadIdx.x; i < nparts; i += kThreads) {
     n += partials[i].x;
@@ -173,6 +175,7 @@ __global__ void __launch_bounds__(kThreads) drift_final_kernel(const double2* __
 template <typename T>
 __global__ void __launch_bounds__(kThreads) add_vec_kernel(const T* __restrict__ a, const T* __restrict__ b, T* out,
                                                            int64_t n) {
+  pdl_begin();
   constexpr int V = Vec<T>::N;
   const int64_t nvec = n / V;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -191,6 +194,7 @@ __global__ void __launch_bounds__(kThreads) add_vec_kernel(const T* __restrict__
 
 template <typename TA, typename TB, typename TO>
 __global__ void add_mixed_kernel(const TA* __restrict__ a, const TB* __restrict__ b, TO* out, int64_t n, float bs) {
+  pdl_begin();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
     io<TO>::st(out + i, io<TA>::ld(a + i) + bs * io<TB>::ld(b + i));
@@ -200,6 +204,7 @@ __global__ void add_mixed_kernel(const TA* __restrict__ a, const TB* __restrict_
 // READ_B false: out = a (b_scale 0, b not read).
 template <typename TA, typename TB, typename TO, bool READ_B>
 __global__ void add_mixed8_kernel(const TA* __restrict__ a, const TB* __restrict__ b, TO* out, int64_t n, float bs) {
+  pdl_begin();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (int64_t i = tid; i < n / 8; i += stride) {
@@ -352,6 +357,7 @@ constexpr int kLnThreads = 128;
 // FULL: the row fills every lane (d = 128 NV).
 template <typename Tin, typename Tout, int NV, bool FULL>
 __global__ void __launch_bounds__(kLnThreads, NV <= 12 ? 5 : 4) ln_mod_rows_kernel(LnArgs a) {
+  pdl_begin();
   const int64_t row = ((int64_t)blockIdx.x * kLnThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31, d = a.d;
   if (row >= a.rows) return;
@@ -406,6 +412,7 @@ constexpr int kLnMaxWarps = NV * RowVec<Tin>::kN <= 64 ? 16 : 12;
 
 template <typename Tin, typename Tout, int NV, bool FULL>
 __global__ void __launch_bounds__(32 * kLnMaxWarps<Tin, NV>, 1) ln_mod_bulk_kernel(LnArgs a) {
+  pdl_begin();
   constexpr int N = RowVec<Tin>::kN;
   extern __shared__ __align__(128) uint8_t lsm[];
   const int nwarps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -532,6 +539,7 @@ __global__ void __launch_bounds__(32 * kTemniMaxWarps, 1) temni_drift_kernel(con
                                                                             const float* __restrict__ scp, float eps,
                                                                             double2* __restrict__ partials,
                                                                             unsigned int* done, double* result) {
+  pdl_begin();
   extern __shared__ __align__(128) uint8_t tsm[];
   const int nwarps = blockDim.x >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -718,6 +726,7 @@ struct GemvMat {
 template <typename TW, int R>
 __global__ void __launch_bounds__(kThreads, 3) gemv_kernel(GemvMat m0, GemvMat m1, const float* __restrict__ x, int k,
                                                            int silu_in) {
+  pdl_begin();
   extern __shared__ __align__(16) float xs[];  // [2][k / 2]: columns 8 i + {0..3}, then 8 i + {4..7}
   for (int i = threadIdx.x; i < k; i += kThreads) {
     const float v = x[i];
@@ -780,17 +789,20 @@ __device__ __forceinline__ void sinusoid_at(float* out, double t, int half, int 
 }
 
 __global__ void sinusoid_kernel(float* out, double t, int half) {
+  pdl_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < half) sinusoid_at(out, t, half, j);
 }
 
 // t = 1000 sigma[step] with the step index read from device memory
 __global__ void sinusoid_sig_kernel(float* out, const double* sig, const int* step, int half) {
+  pdl_begin();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < half) sinusoid_at(out, 1000.0 * sig[*step], half, j);
 }
 
 __global__ void rope_table_kernel(float2* tbl, int F, int H, int W, int pt, int ph, int pw, double theta) {
+  pdl_begin();
   // pt / ph / pw: rotation pairs per axis (t, h, w)
   const int64_t total = (int64_t)F * pt + (int64_t)H * ph + (int64_t)W * pw;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -817,6 +829,7 @@ __global__ void rope_table_kernel(float2* tbl, int F, int H, int W, int pt, int 
 template <typename TO>
 __global__ void patchify_kernel(const float* __restrict__ lat, TO* __restrict__ tok, int C, int F, int H, int W,
                                 int pt, int ph, int pw) {
+  pdl_begin();
   const int Hp = H / ph, Wp = W / pw;
   const int P = C * pt * ph * pw;
   const int64_t total = (int64_t)(F / pt) * Hp * Wp * P;
@@ -842,6 +855,7 @@ __global__ void patchify_kernel(const float* __restrict__ lat, TO* __restrict__ 
 // tensor cores.
 __global__ void patchify_split_kernel(const float* __restrict__ lat, __nv_bfloat16* __restrict__ tok, int C, int F,
                                       int H, int W, int pt, int ph, int pw) {
+  pdl_begin();
   const int Hp = H / ph, Wp = W / pw;
   const int P = C * pt * ph * pw;
   const int64_t total = (int64_t)(F / pt) * Hp * Wp * P;
@@ -868,6 +882,7 @@ __global__ void patchify_split_kernel(const float* __restrict__ lat, __nv_bfloat
 
 __global__ void unpatchify_euler_kernel(const float* __restrict__ vtok, float* __restrict__ vout, float* lat, int C,
                                         int F, int H, int W, int pt, int ph, int pw, float dsig) {
+  pdl_begin();
   const int Hp = H / ph, Wp = W / pw;
   const int P = C * pt * ph * pw;
   const int64_t total = (int64_t)C * F * H * W;
@@ -887,6 +902,7 @@ __global__ void unpatchify_euler_kernel(const float* __restrict__ vtok, float* _
 }
 
 __global__ void euler_kernel(float* lat, const float* __restrict__ v, int64_t n, float dsig) {
+  pdl_begin();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) lat[i] = fmaf(dsig, v[i], lat[i]);
 }
@@ -894,6 +910,7 @@ __global__ void euler_kernel(float* lat, const float* __restrict__ v, int64_t n,
 // Classifier-free guidance and the Euler step: x += dsig * (v_u + g (v_c - v_u)).
 __global__ void guided_euler_kernel(float* lat, const float* __restrict__ vc, const float* __restrict__ vu, int64_t n,
                                     float g, float dsig) {
+  pdl_begin();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const float u = vu[i];
@@ -904,6 +921,7 @@ __global__ void guided_euler_kernel(float* lat, const float* __restrict__ vc, co
 // The same with dsigma read from device memory (graph-launched loops).
 __global__ void guided_euler_sig_kernel(float* lat, const float* __restrict__ vc, const float* __restrict__ vu,
                                         int64_t n, float g, const double* sig, const int* step) {
+  pdl_begin();
   const int i0 = *step;
   const float dsig = (float)(sig[i0 + 1] - sig[i0]);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -916,6 +934,7 @@ __global__ void guided_euler_sig_kernel(float* lat, const float* __restrict__ vc
 // dsigma = sigma[step + 1] - sigma[step] with the step index read from device memory
 __global__ void euler_sig_kernel(float* lat, const float* __restrict__ v, int64_t n, const double* sig,
                                  const int* step) {
+  pdl_begin();
   const int i0 = *step;
   const float dsig = (float)(sig[i0 + 1] - sig[i0]);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -951,21 +970,21 @@ acid_status drift_launch(int dtype, const void* prev, const void* cur, const voi
   if (dtype == ACID_BF16) {
     using T = __nv_bfloat16;
     if (resid)
-      drift_partials_kernel<T, true><<<grid, kThreads, 0, s>>>((const T*)prev, (const T*)cur, (const T*)resid,
+      launch_pdl(drift_partials_kernel<T, true>, grid, kThreads, 0, s, (const T*)prev, (const T*)cur, (const T*)resid,
                                                               (T*)out, n, parts);
     else
-      drift_partials_kernel<T, false><<<grid, kThreads, 0, s>>>((const T*)prev, (const T*)cur, nullptr, nullptr, n,
+      launch_pdl(drift_partials_kernel<T, false>, grid, kThreads, 0, s, (const T*)prev, (const T*)cur, nullptr, nullptr, n,
                                                                parts);
   } else {
     if (resid)
-      drift_partials_kernel<float, true><<<grid, kThreads, 0, s>>>((const float*)prev, (const float*)cur,
+      launch_pdl(drift_partials_kernel<float, true>, grid, kThreads, 0, s, (const float*)prev, (const float*)cur,
                                                                   (const float*)resid, (float*)out, n, parts);
     else
-      drift_partials_kernel<float, false><<<grid, kThreads, 0, s>>>((const float*)prev, (const float*)cur, nullptr,
+      launch_pdl(drift_partials_kernel<float, false>, grid, kThreads, 0, s, (const float*)prev, (const float*)cur, nullptr,
                                                                    nullptr, n, parts);
   }
   ACID_CHECK_LAUNCH();
-  drift_final_kernel<<<1, kThreads, 0, s>>>(parts, grid, d_result);
+  launch_pdl(drift_final_kernel, 1, kThreads, 0, s, parts, grid, d_result);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -974,10 +993,10 @@ acid_status add_same(int dtype, const void* a, const void* b, void* out, int64_t
   const int V = dtype == ACID_BF16 ? 8 : 4;
   const int grid = grid_for(n / V + 1, kThreads, 152 * 8);
   if (dtype == ACID_BF16)
-    add_vec_kernel<__nv_bfloat16><<<grid, kThreads, 0, s>>>((const __nv_bfloat16*)a, (const __nv_bfloat16*)b,
+    launch_pdl(add_vec_kernel<__nv_bfloat16>, grid, kThreads, 0, s, (const __nv_bfloat16*)a, (const __nv_bfloat16*)b,
                                                             (__nv_bfloat16*)out, n);
   else
-    add_vec_kernel<float><<<grid, kThreads, 0, s>>>((const float*)a, (const float*)b, (float*)out, n);
+    launch_pdl(add_vec_kernel<float>, grid, kThreads, 0, s, (const float*)a, (const float*)b, (float*)out, n);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -988,11 +1007,11 @@ acid_status add_mixed(int ad, const void* a, int bd, const void* b, int od, void
   const bool vec = aligned(a, 16) && aligned(b, 16) && aligned(out, 16);
   const int grid = vec ? grid_for(n / 8 + 1, kThreads, 152 * 8) : grid_for(n);
 #define ACID_ADD(TA, TB, TO)                                                                                   \
-  (!vec ? add_mixed_kernel<TA, TB, TO><<<grid, kThreads, 0, s>>>((const TA*)a, (const TB*)b, (TO*)out, n, bs)  \
+  (!vec ? launch_pdl(add_mixed_kernel<TA, TB, TO>, grid, kThreads, 0, s, (const TA*)a, (const TB*)b, (TO*)out, n, bs)  \
    : bs == 0.0f                                                                                                \
-       ? add_mixed8_kernel<TA, TB, TO, false><<<grid, kThreads, 0, s>>>((const TA*)a, (const TB*)b, (TO*)out, n, \
+       ? launch_pdl(add_mixed8_kernel<TA, TB, TO, false>, grid, kThreads, 0, s, (const TA*)a, (const TB*)b, (TO*)out, n, \
                                                                        bs)                                   \
-       : add_mixed8_kernel<TA, TB, TO, true><<<grid, kThreads, 0, s>>>((const TA*)a, (const TB*)b, (TO*)out, n, bs))
+       : launch_pdl(add_mixed8_kernel<TA, TB, TO, true>, grid, kThreads, 0, s, (const TA*)a, (const TB*)b, (TO*)out, n, bs))
   const int key = ad * 4 + bd * 2 + od;  // ACID_BF16 = 0, ACID_FP32 = 1
   switch (key) {
     case 0: ACID_ADD(H, H, H); break;
@@ -1014,9 +1033,9 @@ acid_status launch_ln_rows(const LnArgs& a, cudaStream_t s) {
   constexpr int64_t per_block = kLnThreads / 32;
   const unsigned grid = (unsigned)((a.rows + per_block - 1) / per_block);
   if (a.d == 128 * NV)
-    ln_mod_rows_kernel<Tin, Tout, NV, true><<<grid, kLnThreads, 0, s>>>(a);
+    launch_pdl(ln_mod_rows_kernel<Tin, Tout, NV, true>, grid, kLnThreads, 0, s, a);
   else
-    ln_mod_rows_kernel<Tin, Tout, NV, false><<<grid, kLnThreads, 0, s>>>(a);
+    launch_pdl(ln_mod_rows_kernel<Tin, Tout, NV, false>, grid, kLnThreads, 0, s, a);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1033,7 +1052,7 @@ acid_status launch_ln_bulk_full(const LnArgs& a, cudaStream_t s) {
   const size_t per_warp = ln_warp_bytes<Tin, Tout>(a.d), mod = (size_t)a.vecs * 8 * a.d;
   const int warps = (int)std::min<size_t>(kLnMaxWarps<Tin, NV>, (kSmemMax - mod) / per_warp);
   const int grid = (int)std::min<int64_t>(num_sms_elem(), (a.rows + warps - 1) / warps);
-  ln_mod_bulk_kernel<Tin, Tout, NV, FULL><<<grid, 32 * warps, mod + warps * per_warp, s>>>(a);
+  launch_pdl(ln_mod_bulk_kernel<Tin, Tout, NV, FULL>, grid, 32 * warps, mod + warps * per_warp, s, a);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1094,7 +1113,7 @@ acid_status launch_temni_drift(const float* h_cur, const float* h_prev, const fl
   const size_t smem = 16 * (size_t)d + warps * ring_per_warp;
   const int grid = (int)std::min<int64_t>(std::min<int64_t>(kDriftMaxBlocks, (int64_t)num_sms_elem()),
                                           std::max<int64_t>(1, (rows + warps - 1) / warps));
-  temni_drift_kernel<NV4, HOLD><<<grid, 32 * warps, smem, s>>>(h_cur, h_prev, step_dev, step_host, rows, d, mod_cur,
+  launch_pdl(temni_drift_kernel<NV4, HOLD>, grid, 32 * warps, smem, s, h_cur, h_prev, step_dev, step_host, rows, d, mod_cur,
                                                                mod_cur + d, mod_prev, mod_prev + d, eps, parts,
                                                                done, result);
   ACID_CHECK_LAUNCH();
@@ -1122,7 +1141,7 @@ acid_status temni_drift(const float* h_cur, const float* h_prev, const float* mo
     ACID_TRY((launch_temni_drift<24, false>(h_cur, h_prev, mod_cur, mod_prev, step_dev, step_host, rows, d, eps, parts,
                                            done, d_result, s, &grid)));
   if (done == nullptr) {
-    drift_final_kernel<<<1, kThreads, 0, s>>>(parts, grid, d_result);
+    launch_pdl(drift_final_kernel, 1, kThreads, 0, s, parts, grid, d_result);
     ACID_CHECK_LAUNCH();
   }
   return ACID_OK;
@@ -1136,11 +1155,11 @@ acid_status launch_gemv(const GemvMat& m0, const GemvMat& m1, const float* x, in
   // four rows per warp, on as many CTAs as are resident, once every SM gets two
   auto grid = [&](int rows) { return std::min((total + kThreads / 32 * rows - 1) / (kThreads / 32 * rows), 152 * 3); };
   if (total >= 152 * 2 * (kThreads / 32) * 4)
-    gemv_kernel<TW, 4><<<grid(4), kThreads, smem, s>>>(m0, m1, x, k, silu_input);
+    launch_pdl(gemv_kernel<TW, 4>, grid(4), kThreads, smem, s, m0, m1, x, k, silu_input);
   else if (total >= 152 * 2 * (kThreads / 32) * 2)
-    gemv_kernel<TW, 2><<<grid(2), kThreads, smem, s>>>(m0, m1, x, k, silu_input);
+    launch_pdl(gemv_kernel<TW, 2>, grid(2), kThreads, smem, s, m0, m1, x, k, silu_input);
   else
-    gemv_kernel<TW, 1><<<grid(1), kThreads, smem, s>>>(m0, m1, x, k, silu_input);
+    launch_pdl(gemv_kernel<TW, 1>, grid(1), kThreads, smem, s, m0, m1, x, k, silu_input);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1161,7 +1180,7 @@ acid_status gemv(int w_dtype, const void* W, const float* b, const float* x, flo
 
 acid_status timestep_sinusoid(float* out, double t, int dim, cudaStream_t s) {
   const int half = dim / 2;
-  sinusoid_kernel<<<dim3((half + kTableThreads - 1) / kTableThreads, 2), kTableThreads, 0, s>>>(out, t, half);
+  launch_pdl(sinusoid_kernel, dim3((half + kTableThreads - 1) / kTableThreads, 2), kTableThreads, 0, s, out, t, half);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1184,7 +1203,7 @@ acid_status rope_build(RopeTable& t, float2* storage, float theta, cudaStream_t 
   const int64_t total = t.elems();
   if (total == 0) return ACID_OK;
   const dim3 grid((unsigned)((total + kTableThreads - 1) / kTableThreads), 2);
-  rope_table_kernel<<<grid, kTableThreads, 0, s>>>(storage, t.grid_f, t.grid_h, t.grid_w, t.pairs_t, t.pairs_h, t.pairs_w,
+  launch_pdl(rope_table_kernel, grid, kTableThreads, 0, s, storage, t.grid_f, t.grid_h, t.grid_w, t.pairs_t, t.pairs_h, t.pairs_w,
                                                    (double)theta);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
@@ -1195,9 +1214,9 @@ acid_status patchify(const float* latent, int out_dtype, void* tokens, int C, in
   const int64_t total = (int64_t)C * F * H * W;
   const int grid = grid_for(total);
   if (out_dtype == ACID_BF16)
-    patchify_kernel<__nv_bfloat16><<<grid, kThreads, 0, s>>>(latent, (__nv_bfloat16*)tokens, C, F, H, W, pt, ph, pw);
+    launch_pdl(patchify_kernel<__nv_bfloat16>, grid, kThreads, 0, s, latent, (__nv_bfloat16*)tokens, C, F, H, W, pt, ph, pw);
   else
-    patchify_kernel<float><<<grid, kThreads, 0, s>>>(latent, (float*)tokens, C, F, H, W, pt, ph, pw);
+    launch_pdl(patchify_kernel<float>, grid, kThreads, 0, s, latent, (float*)tokens, C, F, H, W, pt, ph, pw);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1205,7 +1224,7 @@ acid_status patchify(const float* latent, int out_dtype, void* tokens, int C, in
 acid_status patchify_split(const float* latent, void* tokens, int C, int F, int H, int W, int pt, int ph, int pw,
                            cudaStream_t s) {
   const int64_t total = (int64_t)C * F * H * W;
-  patchify_split_kernel<<<grid_for(total), kThreads, 0, s>>>(latent, (__nv_bfloat16*)tokens, C, F, H, W, pt, ph, pw);
+  launch_pdl(patchify_split_kernel, grid_for(total), kThreads, 0, s, latent, (__nv_bfloat16*)tokens, C, F, H, W, pt, ph, pw);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1213,41 +1232,41 @@ acid_status patchify_split(const float* latent, void* tokens, int C, int F, int 
 acid_status unpatchify_euler(const float* vtok, float* v_out, float* latent, int C, int F, int H, int W, int pt,
                              int ph, int pw, float dsigma, cudaStream_t s) {
   const int64_t total = (int64_t)C * F * H * W;
-  unpatchify_euler_kernel<<<grid_for(total), kThreads, 0, s>>>(vtok, v_out, latent, C, F, H, W, pt, ph, pw, dsigma);
+  launch_pdl(unpatchify_euler_kernel, grid_for(total), kThreads, 0, s, vtok, v_out, latent, C, F, H, W, pt, ph, pw, dsigma);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
 acid_status euler_update(float* latent, const float* v, int64_t n, float dsigma, cudaStream_t s) {
-  euler_kernel<<<grid_for(n), kThreads, 0, s>>>(latent, v, n, dsigma);
+  launch_pdl(euler_kernel, grid_for(n), kThreads, 0, s, latent, v, n, dsigma);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
 acid_status guided_euler_update(float* latent, const float* v_cond, const float* v_uncond, int64_t n, float scale,
                                float dsigma, cudaStream_t s) {
-  guided_euler_kernel<<<grid_for(n), kThreads, 0, s>>>(latent, v_cond, v_uncond, n, scale, dsigma);
+  launch_pdl(guided_euler_kernel, grid_for(n), kThreads, 0, s, latent, v_cond, v_uncond, n, scale, dsigma);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
 acid_status guided_euler_update_sig(float* latent, const float* v_cond, const float* v_uncond, int64_t n, float scale,
                                    const double* sig, const int* step, cudaStream_t s) {
-  guided_euler_sig_kernel<<<grid_for(n), kThreads, 0, s>>>(latent, v_cond, v_uncond, n, scale, sig, step);
+  launch_pdl(guided_euler_sig_kernel, grid_for(n), kThreads, 0, s, latent, v_cond, v_uncond, n, scale, sig, step);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
 acid_status euler_update_sig(float* latent, const float* v, int64_t n, const double* sig, const int* step,
                              cudaStream_t s) {
-  euler_sig_kernel<<<grid_for(n), kThreads, 0, s>>>(latent, v, n, sig, step);
+  launch_pdl(euler_sig_kernel, grid_for(n), kThreads, 0, s, latent, v, n, sig, step);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
 acid_status timestep_sinusoid_sig(float* out, const double* sig, const int* step, int dim, cudaStream_t s) {
   const int half = dim / 2;
-  sinusoid_sig_kernel<<<dim3((half + kTableThreads - 1) / kTableThreads, 2), kTableThreads, 0, s>>>(out, sig, step, half);
+  launch_pdl(sinusoid_sig_kernel, dim3((half + kTableThreads - 1) / kTableThreads, 2), kTableThreads, 0, s, out, sig, step, half);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }

@@ -492,6 +492,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   cluster_sync();  // both CTAs' barriers exist before any cross-CTA arrival
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
+  pdl_begin();  // the set-up above overlaps the tail of the kernel before
 
   if (warp == 0) {
     // TMA producer (both CTAs): one continuous stage ring across tiles; the
@@ -795,7 +796,7 @@ acid_status launch_tc2_kind1(const PairMaps& t, const GemmDims& g, const Epilogu
   const int pairs = max_pairs<KIND, R32, O32>();  // also raises the shared memory limit
   ACID_REQUIRE(pairs > 0, ACID_ERR_CUDA, "linear: no resident CTA pair for the pair GEMM");
   const int grid = 2 * (int)std::min<int64_t>(tiles, pairs);
-  gemm_tc2_kernel<KIND, R32, O32><<<grid, kGemmThreads, Tc2Cfg::SMEM, s>>>(t.a, t.b, t.o, t.r, t.bt, t.ot, g, to_dev(epi));
+  launch_pdl(gemm_tc2_kernel<KIND, R32, O32>, grid, kGemmThreads, Tc2Cfg::SMEM, s, t.a, t.b, t.o, t.r, t.bt, t.ot, g, to_dev(epi));
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -881,6 +882,7 @@ bool splitk_plan(int64_t M, int N, int K, size_t ws_bytes, int pairs, SplitKPlan
 template <int KIND, bool R32, bool O32>
 __global__ void __launch_bounds__(256) splitk_fixup_kernel(const float* __restrict__ part, int splits, int64_t m_pad,
                                                            int64_t M, int N, void* out, int64_t ldo, EpiDev e) {
+  pdl_begin();
   const int64_t npair = N / 2, total = M * npair;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
@@ -918,7 +920,7 @@ acid_status launch_splitk_fixup(const SplitKPlan& sp, const float* part, int64_t
                                 const Epilogue& epi, cudaStream_t s) {
   const int64_t total = M * (N / 2);
   const int grid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)num_sms() * 8);
-  splitk_fixup_kernel<KIND, R32, O32><<<grid, 256, 0, s>>>(part, sp.splits, sp.m_pad, M, N, out, ldo, to_dev(epi));
+  launch_pdl(splitk_fixup_kernel<KIND, R32, O32>, grid, 256, 0, s, part, sp.splits, sp.m_pad, M, N, out, ldo, to_dev(epi));
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -956,7 +958,7 @@ acid_status launch_tc2_splitk(const void* A, int64_t lda, int64_t M, int K, cons
   ACID_REQUIRE(pairs > 0, ACID_ERR_CUDA, "linear: no resident CTA pair for the pair GEMM");
   {
     ProfScope prof(PROF_LINEAR, 2.0 * (double)M * N * K, s);
-    kern<<<2 * (int)std::min<int64_t>(units, pairs), kGemmThreads, Tc2Cfg::SMEM, s>>>(ta, tb, to, to, tb, to, g,
+    launch_pdl(kern, 2 * (int)std::min<int64_t>(units, pairs), kGemmThreads, Tc2Cfg::SMEM, s, ta, tb, to, to, tb, to, g,
                                                                                                   to_dev(raw));
     ACID_CHECK_LAUNCH();
   }
@@ -1027,6 +1029,7 @@ template <int TM, int TN>
 __global__ void __launch_bounds__(64 * kFGroups) gemm_f32_kernel(const float* __restrict__ A, int64_t lda, int64_t M,
                                                                  int K, const float* __restrict__ W, int N, float* out,
                                                                  int64_t ldo, EpiDev e, bool vec) {
+  pdl_begin();
   using C = F32Cfg<TM, TN>;
   constexpr int MT = TM / 8, NT = TN / 8;
   extern __shared__ __align__(16) float fsm[];
@@ -1121,7 +1124,7 @@ acid_status launch_f32(const float* A, int64_t lda, int64_t M, int K, const floa
   }
   const bool vec = aligned(A, 16) && aligned(W, 16) && lda % 4 == 0 && K % 4 == 0;
   const dim3 grid((unsigned)((N + TN - 1) / TN), (unsigned)((M + TM - 1) / TM));
-  gemm_f32_kernel<TM, TN><<<grid, 64 * kFGroups, C::SMEM, s>>>(A, lda, M, K, W, N, out, ldo, to_dev(epi), vec);
+  launch_pdl(gemm_f32_kernel<TM, TN>, grid, 64 * kFGroups, C::SMEM, s, A, lda, M, K, W, N, out, ldo, to_dev(epi), vec);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }

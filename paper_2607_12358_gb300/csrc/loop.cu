@@ -298,6 +298,7 @@ acid_status run_blocks(const acid_model& m, const LoopWs& w, cudaStream_t s, int
 template <typename T>
 __global__ void dicache_update_kernel(const T* __restrict__ h_out, const float* __restrict__ p_t, float* d1,
                                       float* d2, float* p1, float* p2, int64_t n, const int* count) {
+  pdl_begin();
   const int c = *count;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -315,13 +316,17 @@ __global__ void dicache_update_kernel(const T* __restrict__ h_out, const float* 
   }
 }
 
-__global__ void dicache_count_kernel(int* count) { *count = min(*count + 1, 2); }
+__global__ void dicache_count_kernel(int* count) {
+  pdl_begin();
+  *count = min(*count + 1, 2);
+}
 
 // Reuse: H_out = P_t + D_1 + g (D_1 - D_2), g = sum|P_t - P_1| / sum|P_1 - P_2|
 // (0 when the denominator is 0); the sums are read from device memory.
 template <typename T>
 __global__ void dicache_reuse_kernel(T* out, const float* __restrict__ p_t, const float* __restrict__ d1,
                                      const float* __restrict__ d2, int64_t n, const double* num, const double* den) {
+  pdl_begin();
   const double dn = *den;
   const float g = dn > 0.0 ? (float)(*num / dn) : 0.0f;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -335,13 +340,12 @@ int elem_grid(int64_t n) { return (int)std::min<int64_t>(152 * 16, std::max<int6
 
 acid_status dicache_update(int dt, const void* h_out, const float* p_t, const LoopWs& w, int64_t n, cudaStream_t s) {
   if (dt == ACID_BF16)
-    dicache_update_kernel<__nv_bfloat16><<<elem_grid(n), 256, 0, s>>>(
-        static_cast<const __nv_bfloat16*>(h_out), p_t, w.resid, w.dc_d2, w.dc_p1, w.dc_p2, n, w.dc_count);
+    launch_pdl(dicache_update_kernel<__nv_bfloat16>, elem_grid(n), 256, 0, s, static_cast<const __nv_bfloat16*>(h_out), p_t, w.resid, w.dc_d2, w.dc_p1, w.dc_p2, n, w.dc_count);
   else
-    dicache_update_kernel<float><<<elem_grid(n), 256, 0, s>>>(static_cast<const float*>(h_out), p_t, w.resid,
+    launch_pdl(dicache_update_kernel<float>, elem_grid(n), 256, 0, s, static_cast<const float*>(h_out), p_t, w.resid,
                                                               w.dc_d2, w.dc_p1, w.dc_p2, n, w.dc_count);
   ACID_CHECK_LAUNCH();
-  dicache_count_kernel<<<1, 1, 0, s>>>(w.dc_count);
+  launch_pdl(dicache_count_kernel, 1, 1, 0, s, w.dc_count);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -353,10 +357,10 @@ acid_status dicache_reuse(int dt, void* out, const float* p_t, const LoopWs& w, 
   ACID_TRY(drift_launch(ACID_FP32, w.dc_p2, w.dc_p1, nullptr, nullptr, n, w.dres + 3, w.drift_ws,
                         drift_workspace_bytes(0), s));
   if (dt == ACID_BF16)
-    dicache_reuse_kernel<__nv_bfloat16><<<elem_grid(n), 256, 0, s>>>(static_cast<__nv_bfloat16*>(out), p_t, w.resid,
+    launch_pdl(dicache_reuse_kernel<__nv_bfloat16>, elem_grid(n), 256, 0, s, static_cast<__nv_bfloat16*>(out), p_t, w.resid,
                                                                      w.dc_d2, n, w.dres + 1, w.dres + 4);
   else
-    dicache_reuse_kernel<float><<<elem_grid(n), 256, 0, s>>>(static_cast<float*>(out), p_t, w.resid, w.dc_d2, n,
+    launch_pdl(dicache_reuse_kernel<float>, elem_grid(n), 256, 0, s, static_cast<float*>(out), p_t, w.resid, w.dc_d2, n,
                                                             w.dres + 1, w.dres + 4);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
