@@ -74,6 +74,30 @@ bool is_device_pointer(const void* p) {
   return attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
 }
 
+DriftOutputs::DriftOutputs(double* rel_, double* sums_) : rel(rel_), sums(sums_) {
+  rel_dev = is_device_pointer(rel);
+  sums_dev = sums ? is_device_pointer(sums) : true;
+  if (rel_dev && aligned(rel, sizeof(double))) rel_direct = rel;
+  if (sums && sums_dev && aligned(sums, sizeof(double))) sums_direct = sums;
+}
+
+acid_status DriftOutputs::finish(const double* d_result, cudaStream_t s) const {
+  if (rel_dev && !rel_direct) ACID_CUDA(cudaMemcpyAsync(rel, d_result, sizeof(double), cudaMemcpyDeviceToDevice, s));
+  if (sums && sums_dev && !sums_direct)
+    ACID_CUDA(cudaMemcpyAsync(sums, d_result + 1, 2 * sizeof(double), cudaMemcpyDeviceToDevice, s));
+  if (!rel_dev || !sums_dev) {
+    double h[3];
+    ACID_CUDA(cudaMemcpyAsync(h, d_result, sizeof(h), cudaMemcpyDeviceToHost, s));
+    ACID_CUDA(cudaStreamSynchronize(s));
+    if (!rel_dev) *rel = h[0];
+    if (sums && !sums_dev) {
+      sums[0] = h[1];
+      sums[1] = h[2];
+    }
+  }
+  return ACID_OK;
+}
+
 // Runs the drift reduction (and the fused apply when resid != null) and
 // delivers the results to device or host outputs.
 static acid_status drift_entry(const void* prev, const void* cur, const void* resid, void* out, int64_t n,
@@ -94,27 +118,15 @@ static acid_status drift_entry(const void* prev, const void* cur, const void* re
   const size_t need = drift_workspace_bytes(n) + 64;
   ACID_REQUIRE(ws_bytes >= need, ACID_ERR_WORKSPACE, "drift: workspace too small (need " + std::to_string(need) + ")");
   double* result = reinterpret_cast<double*>(static_cast<uint8_t*>(ws) + drift_workspace_bytes(n));
+  DriftOutputs outs(out_rel, out_sums);
   if (n == 0) {
+    outs.rel_direct = outs.sums_direct = nullptr;
     ACID_CUDA(cudaMemsetAsync(result, 0, 3 * sizeof(double), s));
   } else {
-    ACID_TRY(drift_launch(dtype, prev, cur, resid, out, n, result, ws, drift_workspace_bytes(n), s));
+    ACID_TRY(drift_launch(dtype, prev, cur, resid, out, n, result, ws, drift_workspace_bytes(n), s, outs.rel_direct,
+                          outs.sums_direct));
   }
-  const bool rel_dev = is_device_pointer(out_rel);
-  const bool sums_dev = out_sums ? is_device_pointer(out_sums) : true;
-  if (rel_dev) ACID_CUDA(cudaMemcpyAsync(out_rel, result, sizeof(double), cudaMemcpyDeviceToDevice, s));
-  if (out_sums && sums_dev)
-    ACID_CUDA(cudaMemcpyAsync(out_sums, result + 1, 2 * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  if (!rel_dev || !sums_dev) {
-    double h[3];
-    ACID_CUDA(cudaMemcpyAsync(h, result, sizeof(h), cudaMemcpyDeviceToHost, s));
-    ACID_CUDA(cudaStreamSynchronize(s));
-    if (!rel_dev) *out_rel = h[0];
-    if (out_sums && !sums_dev) {
-      out_sums[0] = h[1];
-      out_sums[1] = h[2];
-    }
-  }
-  return ACID_OK;
+  return outs.finish(result, s);
 }
 
 }  // namespace acid
@@ -224,28 +236,15 @@ extern "C" acid_status acid_temni_drift(const float* h_prev, const float* h_cur,
   ACID_REQUIRE(ws_bytes >= need, ACID_ERR_WORKSPACE,
                "temni_drift: workspace too small (need " + std::to_string(need) + ")");
   double* result = reinterpret_cast<double*>(static_cast<uint8_t*>(ws) + drift_workspace_bytes(n));
+  DriftOutputs outs(out_rel, out_sums);
   if (rows == 0) {
+    outs.rel_direct = outs.sums_direct = nullptr;
     ACID_CUDA(cudaMemsetAsync(result, 0, 3 * sizeof(double), s));
   } else {
     ACID_TRY(temni_drift(h_cur, h_prev, mod_cur, mod_prev, nullptr, 1, rows, d, eps, result, ws,
-                         drift_workspace_bytes(n), s));
+                         drift_workspace_bytes(n), s, nullptr, outs.rel_direct, outs.sums_direct));
   }
-  const bool rel_dev = is_device_pointer(out_rel);
-  const bool sums_dev = out_sums ? is_device_pointer(out_sums) : true;
-  if (rel_dev) ACID_CUDA(cudaMemcpyAsync(out_rel, result, sizeof(double), cudaMemcpyDeviceToDevice, s));
-  if (out_sums && sums_dev)
-    ACID_CUDA(cudaMemcpyAsync(out_sums, result + 1, 2 * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  if (!rel_dev || !sums_dev) {
-    double h[3];
-    ACID_CUDA(cudaMemcpyAsync(h, result, sizeof(h), cudaMemcpyDeviceToHost, s));
-    ACID_CUDA(cudaStreamSynchronize(s));
-    if (!rel_dev) *out_rel = h[0];
-    if (out_sums && !sums_dev) {
-      out_sums[0] = h[1];
-      out_sums[1] = h[2];
-    }
-  }
-  return ACID_OK;
+  return outs.finish(result, s);
 }
 
 extern "C" acid_status acid_drift_signal(const void* prev, const void* cur, int64_t n, int32_t dtype,

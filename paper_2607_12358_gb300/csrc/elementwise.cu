@@ -149,9 +149,10 @@ __device__ __forceinline__ void write_drift_result(double num, double den, doubl
   result[2] = den;
 }
 
-// Fixed-order reduction of the CTA partials; result = {rel, num, den}.
+// Fixed-order reduction of the CTA partials; result = {rel, num, den}, and the
+// caller's own rel and {num, den} where given.
 __global__ void __launch_bounds__(kThreads) drift_final_kernel(const double2* __restrict__ partials, int nparts,
-                                                               double* __restrict__ result) {
+                                                               double* result, double* rel_out, double* sums_out) {
   pdl_begin();
   double n = 0.0, d = 0.0;
   for (int i = threadIdx.x; i < nparts; i += kThreads) {
@@ -169,7 +170,14 @@ __global__ void __launch_bounds__(kThreads) drift_final_kernel(const double2* __
     }
     __syncthreads();
   }
-  if (threadIdx.x == 0) write_drift_result(sn[0], sd[0], result);
+  if (threadIdx.x == 0) {
+    write_drift_result(sn[0], sd[0], result);
+    if (rel_out != nullptr) *rel_out = result[0];
+    if (sums_out != nullptr) {
+      sums_out[0] = sn[0];
+      sums_out[1] = sd[0];
+    }
+  }
 }
 
 template <typename T>
@@ -959,7 +967,8 @@ ACID_BOUNDS_READER(take_bounds_elementwise)
 size_t drift_workspace_bytes(int64_t) { return sizeof(double2) * kDriftMaxBlocks + 64; }
 
 acid_status drift_launch(int dtype, const void* prev, const void* cur, const void* resid, void* out, int64_t n,
-                         double* d_result, void* workspace, size_t ws_bytes, cudaStream_t s) {
+                         double* d_result, void* workspace, size_t ws_bytes, cudaStream_t s, double* rel_out,
+                         double* sums_out) {
   ACID_REQUIRE(ws_bytes >= sizeof(double2) * kDriftMaxBlocks, ACID_ERR_WORKSPACE, "drift: workspace too small");
   double2* parts = static_cast<double2*>(workspace);
   const int V = dtype == ACID_BF16 ? 8 : 4;
@@ -984,7 +993,7 @@ acid_status drift_launch(int dtype, const void* prev, const void* cur, const voi
                                                                    nullptr, n, parts);
   }
   ACID_CHECK_LAUNCH();
-  launch_pdl(drift_final_kernel, 1, kThreads, 0, s, parts, grid, d_result);
+  launch_pdl(drift_final_kernel, 1, kThreads, 0, s, parts, grid, d_result, rel_out, sums_out);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1123,7 +1132,8 @@ acid_status launch_temni_drift(const float* h_cur, const float* h_prev, const fl
 
 acid_status temni_drift(const float* h_cur, const float* h_prev, const float* mod_cur, const float* mod_prev,
                         const int* step_dev, int step_host, int64_t rows, int d, float eps, double* d_result,
-                        void* workspace, size_t ws_bytes, cudaStream_t s, unsigned int* done) {
+                        void* workspace, size_t ws_bytes, cudaStream_t s, unsigned int* done, double* rel_out,
+                        double* sums_out) {
   ACID_REQUIRE(d % 8 == 0 && d <= 3072, ACID_ERR_UNSUPPORTED, "temni_drift: d must be a multiple of 8, <= 3072");
   ACID_REQUIRE(ws_bytes >= sizeof(double2) * kDriftMaxBlocks, ACID_ERR_WORKSPACE, "temni_drift: workspace too small");
   ACID_REQUIRE(aligned(h_cur, 16) && aligned(h_prev, 16) && aligned(mod_cur, 16) && aligned(mod_prev, 16),
@@ -1141,7 +1151,7 @@ acid_status temni_drift(const float* h_cur, const float* h_prev, const float* mo
     ACID_TRY((launch_temni_drift<24, false>(h_cur, h_prev, mod_cur, mod_prev, step_dev, step_host, rows, d, eps, parts,
                                            done, d_result, s, &grid)));
   if (done == nullptr) {
-    launch_pdl(drift_final_kernel, 1, kThreads, 0, s, parts, grid, d_result);
+    launch_pdl(drift_final_kernel, 1, kThreads, 0, s, parts, grid, d_result, rel_out, sums_out);
     ACID_CHECK_LAUNCH();
   }
   return ACID_OK;

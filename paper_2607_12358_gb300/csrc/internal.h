@@ -106,7 +106,8 @@ acid_status ln_mod(int in_dtype, const void* x, int out_dtype, void* y, int64_t 
 // leaves the counter at zero again.
 acid_status temni_drift(const float* h_cur, const float* h_prev, const float* mod_cur, const float* mod_prev,
                         const int* step_dev, int step_host, int64_t rows, int d, float eps, double* d_result,
-                        void* workspace, size_t ws_bytes, cudaStream_t s, unsigned int* done = nullptr);
+                        void* workspace, size_t ws_bytes, cudaStream_t s, unsigned int* done = nullptr,
+                        double* rel_out = nullptr, double* sums_out = nullptr);
 
 // y[j] = sum_k W[j, k] act(x[k]) + b[j]; act = SiLU if silu_input.
 acid_status gemv(int w_dtype, const void* W, const float* b, const float* x, float* y, int n_out,
@@ -122,7 +123,20 @@ acid_status timestep_sinusoid(float* out, double t, int dim, cudaStream_t s);
 size_t drift_workspace_bytes(int64_t n);
 acid_status drift_launch(int dtype, const void* prev, const void* cur, const void* resid, void* out,
                          int64_t n, double* d_result /* device double[3]: rel, num, den */,
-                         void* workspace, size_t ws_bytes, cudaStream_t s);
+                         void* workspace, size_t ws_bytes, cudaStream_t s, double* rel_out = nullptr,
+                         double* sums_out = nullptr);
+
+// Delivers the results of a drift call, host side: which of the caller's
+// outputs the final kernel can write itself (device memory, aligned for a
+// double), and the copies of the others from d_result afterwards (to host
+// memory, which synchronises the stream).
+struct DriftOutputs {
+  double *rel, *sums;                              // as the caller gave them (sums may be null)
+  double *rel_direct = nullptr, *sums_direct = nullptr;  // for the kernel
+  bool rel_dev = false, sums_dev = true;
+  DriftOutputs(double* rel_, double* sums_);
+  acid_status finish(const double* d_result, cudaStream_t s) const;
+};
 
 // out = a + b elementwise, one dtype, 16-byte vectors
 acid_status add_same(int dtype, const void* a, const void* b, void* out, int64_t n, cudaStream_t s);

@@ -18,8 +18,6 @@
 
 namespace acid {
 
-bool is_device_pointer(const void* p);
-
 namespace {
 
 constexpr size_t kNoAllocScratchBytes = 16 * 1024;
@@ -112,27 +110,15 @@ extern "C" acid_status acid_drift_signal_noalloc(const void* prev, const void* c
   ACID_TRY(scratch_address(&scratch));
   cudaStream_t s = (cudaStream_t)stream;
   double* result = reinterpret_cast<double*>(static_cast<uint8_t*>(scratch) + part_bytes);
+  DriftOutputs outs(out_rel_l1, out_sums);
   // Every partial slot the final pass reads is written earlier in the same
   // call, and the results are overwritten, so nothing needs clearing here.
   if (n == 0) {
+    outs.rel_direct = outs.sums_direct = nullptr;
     ACID_CUDA(cudaMemsetAsync(result, 0, 3 * sizeof(double), s));
   } else {
-    ACID_TRY(drift_launch(dtype, prev, cur, nullptr, nullptr, n, result, scratch, part_bytes, s));
+    ACID_TRY(drift_launch(dtype, prev, cur, nullptr, nullptr, n, result, scratch, part_bytes, s, outs.rel_direct,
+                          outs.sums_direct));
   }
-  const bool rel_dev = is_device_pointer(out_rel_l1);
-  const bool sums_dev = out_sums ? is_device_pointer(out_sums) : true;
-  if (rel_dev) ACID_CUDA(cudaMemcpyAsync(out_rel_l1, result, sizeof(double), cudaMemcpyDeviceToDevice, s));
-  if (out_sums && sums_dev)
-    ACID_CUDA(cudaMemcpyAsync(out_sums, result + 1, 2 * sizeof(double), cudaMemcpyDeviceToDevice, s));
-  if (!rel_dev || !sums_dev) {
-    double h[3];
-    ACID_CUDA(cudaMemcpyAsync(h, result, sizeof(h), cudaMemcpyDeviceToHost, s));
-    ACID_CUDA(cudaStreamSynchronize(s));
-    if (!rel_dev) *out_rel_l1 = h[0];
-    if (out_sums && !sums_dev) {
-      out_sums[0] = h[1];
-      out_sums[1] = h[2];
-    }
-  }
-  return ACID_OK;
+  return outs.finish(result, s);
 }
