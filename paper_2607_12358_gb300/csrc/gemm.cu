@@ -102,6 +102,21 @@ __device__ __forceinline__ bool rope_in_bounds(const RopeTable& t, const float2&
   return ACID_IN_BOUNDS(kSiteGemmRope, &e - t.table, n);
 }
 
+// The (cos, sin) of the 16 consecutive pairs from j0 on (within the head) at a
+// position.  The table index is formed with selects, so that the 16 loads go
+// out together: behind a branch per pair each waited for the one before.
+__device__ __forceinline__ void rope_cs16(const RopeTable& t, const RopePos& p, int j0, float2* cs) {
+  const int end_t = t.pairs_t, end_h = end_t + t.pairs_h;
+  const int off_h = t.grid_f * t.pairs_t, off_w = off_h + t.grid_h * t.pairs_h;
+  const int base_t = p.f * t.pairs_t, base_h = off_h + p.h * t.pairs_h - end_t, base_w = off_w + p.w * t.pairs_w - end_h;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    const int jj = j0 + k;
+    const float2* e = t.table + (jj + (jj < end_t ? base_t : jj < end_h ? base_h : base_w));
+    cs[k] = rope_in_bounds(t, *e) ? __ldg(e) : make_float2(1.f, 0.f);
+  }
+}
+
 // Applies the epilogue to the adjacent outputs (grow, col) and (grow, col+1).
 // r0/r1: residual values (read by the caller) for the residual kinds.
 template <bool kFastGelu>
@@ -215,7 +230,7 @@ __device__ __forceinline__ void load_bias32(const float* src, int col0, float* b
 template <int KIND, bool O32>
 __device__ __forceinline__ void epilogue_rows(const GemmDims& g, const EpiDev& e, const CUtensorMap* tmO,
                                               uint8_t* stage, int64_t row0, int64_t store_row0, int col0,
-                                              const uint32_t* r, const float* bias) {
+                                              const uint32_t* r, const float* bias, const float2* cs) {
   const int lane = threadIdx.x & 31;
   uint64_t v[16];
 #pragma unroll
@@ -226,18 +241,12 @@ __device__ __forceinline__ void epilogue_rows(const GemmDims& g, const EpiDev& e
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = gelu_x2(v[k]);
   } else if constexpr (KIND == EPI_ROPE_QKV) {
-    // the chunk's 16 pairs lie in one head (head_dim is a power of two >= 32)
-    const int64_t row = row0 + lane, grow = row + e.row_base;
-    if (col0 < 2 * e.d && grow >= e.rope_first_video && row < g.M) {
-      const RopePos pp = rope_pos(e.rope, (int)(grow - e.rope_first_video));
-      const int j0 = (col0 & (e.head_dim - 1)) >> 1;
+    if (cs != nullptr) {
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
-        const float2& ce = rope_cs_ptr(e.rope, pp, j0 + k);
-        const float2 cs = rope_in_bounds(e.rope, ce) ? __ldg(&ce) : make_float2(1.f, 0.f);
         float x0, x1;
         f2_unpack(v[k], x0, x1);
-        v[k] = f2_pack(x0 * cs.x - x1 * cs.y, x0 * cs.y + x1 * cs.x);
+        v[k] = f2_pack(x0 * cs[k].x - x1 * cs[k].y, x0 * cs[k].y + x1 * cs[k].x);
       }
     }
   }
@@ -282,6 +291,22 @@ __device__ __forceinline__ void tma_kind_chunk(const GemmDims& g, const EpiDev& 
   float bias[32];
   tmem_ld32(taddr, r);
   if (live) load_bias32(bias_src, col0, bias);
+  // RoPE of q and k on video rows: the chunk's 16 pairs lie in one head
+  // (head_dim is a power of two >= 32); other rows are rotated by (1, 0)
+  float2 cs[KIND == EPI_ROPE_QKV ? 16 : 1];
+  bool rotate = false;
+  if constexpr (KIND == EPI_ROPE_QKV) {
+    rotate = live && col0 < 2 * e.d;  // warp-uniform
+    if (rotate) {
+      const int64_t row = row0 + lane, grow = row + e.row_base;
+      const bool video = grow >= e.rope_first_video && row < g.M;
+      rope_cs16(e.rope, rope_pos(e.rope, video ? (int)(grow - e.rope_first_video) : 0), (col0 & (e.head_dim - 1)) >> 1, cs);
+      if (!video) {
+#pragma unroll
+        for (int k = 0; k < 16; ++k) cs[k] = make_float2(1.f, 0.f);
+      }
+    }
+  }
   tmem_wait_ld();
   if (!live) return;
   uint8_t* st = stage;
@@ -292,7 +317,7 @@ __device__ __forceinline__ void tma_kind_chunk(const GemmDims& g, const EpiDev& 
     if (lane == 0) bulk_wait_group_read<1>();
   }
   __syncwarp();
-  epilogue_rows<KIND, O32>(g, e, tmO, st, row0, store_row0, col0, r, bias);
+  epilogue_rows<KIND, O32>(g, e, tmO, st, row0, store_row0, col0, r, bias, rotate ? cs : nullptr);
   ++nstore;
 }
 
