@@ -291,6 +291,18 @@ __device__ __forceinline__ void load_quad(const __nv_bfloat16* p, uint64_t* v) {
   v[1] = f2_pack(bf16_lo(u.y), bf16_hi(u.y));
 }
 __device__ __forceinline__ void load_quad(const float* p, uint64_t* v) { RowVec<float>::ld(p, v); }
+// a pair rounded to T
+template <typename T>
+__device__ __forceinline__ uint64_t round_to(uint64_t v) {
+  if constexpr (sizeof(T) == 2) {
+    float a, b;
+    f2_unpack(v, a, b);
+    const uint32_t w = pack_bf16(a, b);
+    return f2_pack(bf16_lo(w), bf16_hi(w));
+  } else {
+    return v;
+  }
+}
 template <int N>  // N values, N / 2 pairs
 __device__ __forceinline__ void store_pairs(__nv_bfloat16* p, const uint64_t* v) {
   uint32_t w[N / 2];
@@ -347,9 +359,18 @@ __device__ __forceinline__ float row_center(uint64_t (&v)[NV][N / 2], int lane, 
   return rsqrtf(warp_sum_f(a + b) / d + eps);
 }
 
+// What a row kernel does beside the LayerNorm of x.
+enum LnMode : int {
+  kLnPlain = 0,
+  kLnReuse = 1,  // x = h + r first, rounded to TX (the reused step's state)
+  kLnResid = 2   // also r = x - h (the computed step's residual)
+};
+
 struct LnArgs {
   const void* x;
   void* y;
+  const float* h;       // kLnReuse, kLnResid: the stack's input
+  float* r;             // kLnReuse: read, kLnResid: written
   int64_t rows, split;  // rows below split take the text vectors
   int d, vecs;          // vecs: modulation streams (0, 1 video only, 2 video and text)
   const float *shv, *scv, *sht, *sct;
@@ -362,8 +383,10 @@ struct LnArgs {
 // warp.
 constexpr int kLnThreads = 128;
 
-// FULL: the row fills every lane (d = 128 NV).
-template <typename Tin, typename Tout, int NV, bool FULL>
+// FULL: the row fills every lane (d = 128 NV).  The cached residual of a
+// TeaCache step is applied (kLnReuse) or stored (kLnResid) in the same pass:
+// apart, the state was written and read again, or read a second time.
+template <typename Tin, typename Tout, int NV, bool FULL, int MODE>
 __global__ void __launch_bounds__(kLnThreads, NV <= 12 ? 5 : 4) ln_mod_rows_kernel(LnArgs a) {
   pdl_begin();
   const int64_t row = ((int64_t)blockIdx.x * kLnThreads + threadIdx.x) >> 5;
@@ -376,7 +399,23 @@ __global__ void __launch_bounds__(kLnThreads, NV <= 12 ? 5 : 4) ln_mod_rows_kern
   for (int i = 0; i < NV; ++i) {
     const int c = (i * 32 + lane) * 4;
     if (!FULL || kBoundsChecked) v[i][0] = v[i][1] = 0;
-    if ((FULL || c < d) && ACID_IN_BOUNDS(kSiteLayerNorm, row * d + c + 3, a.rows * d)) load_quad(xr + c, v[i]);
+    if (!((FULL || c < d) && ACID_IN_BOUNDS(kSiteLayerNorm, row * d + c + 3, a.rows * d))) continue;
+    if constexpr (MODE == kLnReuse) {
+      uint64_t r[2];
+      load_quad(a.h + row * d + c, v[i]);
+      load_quad(a.r + row * d + c, r);
+      v[i][0] = round_to<Tin>(f2_add(v[i][0], r[0]));
+      v[i][1] = round_to<Tin>(f2_add(v[i][1], r[1]));
+    } else {
+      load_quad(xr + c, v[i]);
+    }
+    if constexpr (MODE == kLnResid) {
+      const float4 h = *reinterpret_cast<const float4*>(a.h + row * d + c);
+      float x0, x1, x2, x3;
+      f2_unpack(v[i][0], x0, x1);
+      f2_unpack(v[i][1], x2, x3);
+      *reinterpret_cast<float4*>(a.r + row * d + c) = make_float4(x0 - h.x, x1 - h.y, x2 - h.z, x3 - h.w);
+    }
   }
   const float rstd = row_center<NV, 4, FULL>(v, lane, d, a.eps);
   const uint64_t rs = f2_pack(rstd, rstd);
@@ -754,7 +793,7 @@ __global__ void __launch_bounds__(kThreads, 3) gemv_kernel(GemvMat m0, GemvMat m
                              : static_cast<const TW*>(m1.W) + (int64_t)(row - m0.n_out) * k;
       acc[r] = 0.f;
     }
-#pragma unroll 2
+#pragma unroll(8 / R)
     for (int c = lane * 8; c < k; c += 256) {
       if (!ACID_IN_BOUNDS(kSiteGemv, c + 7, k)) continue;
       float w[R][8];
@@ -834,8 +873,97 @@ __global__ void rope_table_kernel(float2* tbl, int F, int H, int W, int pt, int 
 }
 
 // ---------------------------------------------------------------- patches
-template <typename TO>
-__global__ void patchify_kernel(const float* __restrict__ lat, TO* __restrict__ tok, int C, int F, int H, int W,
+// One CTA moves the tokens of up to 32 patches along a latent row: rows of the
+// latent in and token vectors out (or back), both contiguous, through a
+// shared-memory tile [patch][P].  Element by element in token order the
+// latent accesses covered 8 bytes a line, behind six 64-bit divisions each.
+// Patch vectors of more than kPatchMaxP values take the element kernels below.
+constexpr int kPatchTile = 32, kPatchMaxP = 256;
+
+struct PatchGeo {
+  int C, F, H, W, pt, ph, pw;
+};
+// The tile of this CTA (blockIdx.x: tile along the row, y: patch row, z:
+// frame): its first token, its patch count, and element e of it: shared index,
+// latent index.
+struct PatchTile {
+  PatchGeo g;
+  int w0, nw, P;
+  int64_t n0;
+  __device__ __forceinline__ explicit PatchTile(const PatchGeo& geo) : g(geo) {
+    const int Wp = g.W / g.pw;
+    w0 = blockIdx.x * kPatchTile;
+    nw = min(kPatchTile, Wp - w0);
+    P = g.C * g.pt * g.ph * g.pw;
+    n0 = ((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * Wp + w0;
+  }
+  // e counts latent row by latent row: r = (c, dt, dh), then nw * pw columns
+  __device__ __forceinline__ void at(int e, int& sidx, int64_t& lidx) const {
+    const int cols = nw * g.pw, r = e / cols, x = e - r * cols;
+    const int dh = r % g.ph, q = r / g.ph, dt = q % g.pt, c = q / g.pt;
+    const int tok = x / g.pw;
+    sidx = tok * (P + 1) + r * g.pw + (x - tok * g.pw);
+    lidx = (((int64_t)c * g.F + (int)blockIdx.z * g.pt + dt) * g.H + (int)blockIdx.y * g.ph + dh) * g.W + w0 * g.pw + x;
+  }
+};
+
+// SPLIT: bf16 tokens of width 2P that carry each fp32 value as the sum of two
+// bf16 parts: hi = bf16(x) in column p, lo = bf16(x - hi) in column P + p.
+// x - hi is exact in fp32 and lo rounds it to 8 bits, so hi + lo equals x to
+// within 2^-17 |x|; a bf16 GEMM against the weights repeated along K ([W | W])
+// then forms the fp32-input patch embedding on tensor cores.  Otherwise fp32
+// tokens.
+template <bool SPLIT>
+__global__ void __launch_bounds__(kThreads) patchify_tile_kernel(const float* __restrict__ lat, void* tok, PatchGeo geo) {
+  pdl_begin();
+  extern __shared__ float tile[];
+  const PatchTile t(geo);
+  const int n = t.nw * t.P;
+  for (int e = threadIdx.x; e < n; e += kThreads) {
+    int si;
+    int64_t li;
+    t.at(e, si, li);
+    tile[si] = ACID_IN_BOUNDS(kSitePatchify, li, (int64_t)geo.C * geo.F * geo.H * geo.W) ? lat[li] : 0.f;
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < n; e += kThreads) {
+    const int k = e / t.P, p = e - k * t.P;
+    const float x = tile[k * (t.P + 1) + p];
+    if constexpr (SPLIT) {
+      __nv_bfloat16* o = static_cast<__nv_bfloat16*>(tok) + (t.n0 + k) * 2 * t.P + p;
+      const __nv_bfloat16 hi = __float2bfloat16_rn(x);
+      o[0] = hi;
+      o[t.P] = __float2bfloat16_rn(x - __bfloat162float(hi));
+    } else {
+      static_cast<float*>(tok)[(t.n0 + k) * t.P + p] = x;
+    }
+  }
+}
+
+__global__ void __launch_bounds__(kThreads) unpatchify_tile_kernel(const float* __restrict__ vtok,
+                                                                   float* __restrict__ vout, float* lat, PatchGeo geo,
+                                                                   float dsig) {
+  pdl_begin();
+  extern __shared__ float tile[];
+  const PatchTile t(geo);
+  const int n = t.nw * t.P;
+  for (int e = threadIdx.x; e < n; e += kThreads) {
+    const int k = e / t.P;
+    tile[k * (t.P + 1) + (e - k * t.P)] = vtok[t.n0 * t.P + e];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < n; e += kThreads) {
+    int si;
+    int64_t li;
+    t.at(e, si, li);
+    if (!ACID_IN_BOUNDS(kSiteUnpatchify, li, (int64_t)geo.C * geo.F * geo.H * geo.W)) continue;
+    const float v = tile[si];
+    if (vout) vout[li] = v;
+    if (lat) lat[li] = fmaf(dsig, v, lat[li]);
+  }
+}
+
+__global__ void patchify_kernel(const float* __restrict__ lat, float* __restrict__ tok, int C, int F, int H, int W,
                                 int pt, int ph, int pw) {
   pdl_begin();
   const int Hp = H / ph, Wp = W / pw;
@@ -851,16 +979,11 @@ __global__ void patchify_kernel(const float* __restrict__ lat, TO* __restrict__ 
     const int dt = p % pt; p /= pt;
     const int c = p;
     const int64_t src = (((int64_t)c * F + (f * pt + dt)) * H + (h * ph + dh)) * W + (w * pw + dw);
-    if (ACID_IN_BOUNDS(kSitePatchify, src, (int64_t)C * F * H * W)) io<TO>::st(tok + i, lat[src]);
+    if (ACID_IN_BOUNDS(kSitePatchify, src, (int64_t)C * F * H * W)) tok[i] = lat[src];
   }
 }
 
-// The same gather into bf16 tokens of width 2P that carry each fp32 value as
-// the sum of two bf16 parts: hi = bf16(x) in column p, lo = bf16(x - hi) in
-// column P + p.  x - hi is exact in fp32 and lo rounds it to 8 bits, so
-// hi + lo equals x to within 2^-17 |x|; a bf16 GEMM against the weights
-// repeated along K ([W | W]) then forms the fp32-input patch embedding on
-// tensor cores.
+// The same as hi and lo bf16 parts (see patchify_tile_kernel).
 __global__ void patchify_split_kernel(const float* __restrict__ lat, __nv_bfloat16* __restrict__ tok, int C, int F,
                                       int H, int W, int pt, int ph, int pw) {
   pdl_begin();
@@ -1037,16 +1160,24 @@ acid_status add_mixed(int ad, const void* a, int bd, const void* b, int od, void
   return ACID_OK;
 }
 
-template <typename Tin, typename Tout, int NV>
+template <typename Tin, typename Tout, int NV, int MODE>
 acid_status launch_ln_rows(const LnArgs& a, cudaStream_t s) {
   constexpr int64_t per_block = kLnThreads / 32;
   const unsigned grid = (unsigned)((a.rows + per_block - 1) / per_block);
   if (a.d == 128 * NV)
-    launch_pdl(ln_mod_rows_kernel<Tin, Tout, NV, true>, grid, kLnThreads, 0, s, a);
+    launch_pdl(ln_mod_rows_kernel<Tin, Tout, NV, true, MODE>, grid, kLnThreads, 0, s, a);
   else
-    launch_pdl(ln_mod_rows_kernel<Tin, Tout, NV, false>, grid, kLnThreads, 0, s, a);
+    launch_pdl(ln_mod_rows_kernel<Tin, Tout, NV, false, MODE>, grid, kLnThreads, 0, s, a);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
+}
+
+template <typename Tin, typename Tout, int MODE>
+acid_status ln_rows_types(const LnArgs& a, cudaStream_t s) {
+  if (a.d <= 128 * 4) return launch_ln_rows<Tin, Tout, 4, MODE>(a, s);
+  if (a.d <= 128 * 12) return launch_ln_rows<Tin, Tout, 12, MODE>(a, s);
+  if (a.d <= 128 * 16) return launch_ln_rows<Tin, Tout, 16, MODE>(a, s);
+  return launch_ln_rows<Tin, Tout, 24, MODE>(a, s);
 }
 
 template <typename Tin, typename Tout, int NV, bool FULL>
@@ -1079,10 +1210,7 @@ acid_status ln_mod_types(const LnArgs& a, cudaStream_t s) {
   // warp per row; fp32 in 37.1, 47.3; 67576 x 3072 bf16 144, 180; 4846 x 3072 fp32
   // 20.5, 16.4; 7800 x 1536 bf16 12.3, 11.5; 20000 x 256 bf16 12.3, 8.7.
   if (a.rows < kLnBulkRows || a.d <= 512) {
-    if (a.d <= 128 * 4) return launch_ln_rows<Tin, Tout, 4>(a, s);
-    if (a.d <= 128 * 12) return launch_ln_rows<Tin, Tout, 12>(a, s);
-    if (a.d <= 128 * 16) return launch_ln_rows<Tin, Tout, 16>(a, s);
-    return launch_ln_rows<Tin, Tout, 24>(a, s);
+    return ln_rows_types<Tin, Tout, kLnPlain>(a, s);
   }
   constexpr int U = RowVec<Tin>::kN == 8 ? 1 : 2;  // 16-byte vectors per 8 columns
   if (a.d <= 1536) return launch_ln_bulk<Tin, Tout, 6 * U>(a, s);
@@ -1096,11 +1224,21 @@ acid_status ln_mod(int in_dtype, const void* x, int out_dtype, void* y, int64_t 
   ACID_REQUIRE(d % 8 == 0 && d <= 3072, ACID_ERR_UNSUPPORTED, "ln_mod: d must be a multiple of 8, <= 3072");
   if (rows == 0) return ACID_OK;
   const bool two = scv != nullptr && sht != nullptr && split > 0 && (sht != shv || sct != scv);
-  const LnArgs a{x, y, rows, split, d, scv == nullptr ? 0 : two ? 2 : 1, shv, scv, sht, sct, eps};
+  const LnArgs a{x, y, nullptr, nullptr, rows, split, d, scv == nullptr ? 0 : two ? 2 : 1, shv, scv, sht, sct, eps};
   if (in_dtype == ACID_BF16 && out_dtype == ACID_BF16) return ln_mod_types<H, H>(a, s);
   if (in_dtype == ACID_BF16) return ln_mod_types<H, float>(a, s);
   if (out_dtype == ACID_BF16) return ln_mod_types<float, H>(a, s);
   return ln_mod_types<float, float>(a, s);
+}
+
+acid_status ln_mod_cached(int dtype, bool reuse, const void* x, const float* h, float* r, void* y, int64_t rows, int d,
+                          const float* sh, const float* sc, float eps, cudaStream_t s) {
+  using H = __nv_bfloat16;
+  ACID_REQUIRE(d % 8 == 0 && d <= 3072, ACID_ERR_UNSUPPORTED, "ln_mod: d must be a multiple of 8, <= 3072");
+  if (rows == 0) return ACID_OK;
+  const LnArgs a{x, y, h, r, rows, 0, d, 1, sh, sc, nullptr, nullptr, eps};
+  if (dtype == ACID_BF16) return reuse ? ln_rows_types<H, H, kLnReuse>(a, s) : ln_rows_types<H, H, kLnResid>(a, s);
+  return reuse ? ln_rows_types<float, float, kLnReuse>(a, s) : ln_rows_types<float, float, kLnResid>(a, s);
 }
 
 template <int NV4, bool HOLD>
@@ -1219,30 +1357,56 @@ acid_status rope_build(RopeTable& t, float2* storage, float theta, cudaStream_t 
   return ACID_OK;
 }
 
-acid_status patchify(const float* latent, int out_dtype, void* tokens, int C, int F, int H, int W, int pt, int ph,
-                     int pw, cudaStream_t s) {
-  const int64_t total = (int64_t)C * F * H * W;
-  const int grid = grid_for(total);
-  if (out_dtype == ACID_BF16)
-    launch_pdl(patchify_kernel<__nv_bfloat16>, grid, kThreads, 0, s, latent, (__nv_bfloat16*)tokens, C, F, H, W, pt, ph, pw);
+namespace {
+// grid and shared memory of the tile kernels; false if the patch is too long
+// (or the grid too tall) for them
+bool patch_tiles(const PatchGeo& g, dim3* grid, size_t* smem) {
+  const int P = g.C * g.pt * g.ph * g.pw;
+  const int Wp = g.W / g.pw, Hp = g.H / g.ph, Fp = g.F / g.pt;
+  if (P > kPatchMaxP || Hp > 65535 || Fp > 65535) return false;
+  *grid = dim3((unsigned)((Wp + kPatchTile - 1) / kPatchTile), (unsigned)Hp, (unsigned)Fp);
+  *smem = sizeof(float) * kPatchTile * (P + 1);
+  return true;
+}
+}  // namespace
+
+acid_status patchify(const float* latent, float* tokens, int C, int F, int H, int W, int pt, int ph, int pw,
+                     cudaStream_t s) {
+  const PatchGeo g{C, F, H, W, pt, ph, pw};
+  dim3 grid;
+  size_t smem;
+  if (patch_tiles(g, &grid, &smem))
+    launch_pdl(patchify_tile_kernel<false>, grid, kThreads, smem, s, latent, (void*)tokens, g);
   else
-    launch_pdl(patchify_kernel<float>, grid, kThreads, 0, s, latent, (float*)tokens, C, F, H, W, pt, ph, pw);
+    launch_pdl(patchify_kernel, grid_for((int64_t)C * F * H * W), kThreads, 0, s, latent, tokens, C, F, H, W, pt, ph, pw);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
 acid_status patchify_split(const float* latent, void* tokens, int C, int F, int H, int W, int pt, int ph, int pw,
                            cudaStream_t s) {
-  const int64_t total = (int64_t)C * F * H * W;
-  launch_pdl(patchify_split_kernel, grid_for(total), kThreads, 0, s, latent, (__nv_bfloat16*)tokens, C, F, H, W, pt, ph, pw);
+  const PatchGeo g{C, F, H, W, pt, ph, pw};
+  dim3 grid;
+  size_t smem;
+  if (patch_tiles(g, &grid, &smem))
+    launch_pdl(patchify_tile_kernel<true>, grid, kThreads, smem, s, latent, tokens, g);
+  else
+    launch_pdl(patchify_split_kernel, grid_for((int64_t)C * F * H * W), kThreads, 0, s, latent, (__nv_bfloat16*)tokens,
+               C, F, H, W, pt, ph, pw);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
 acid_status unpatchify_euler(const float* vtok, float* v_out, float* latent, int C, int F, int H, int W, int pt,
                              int ph, int pw, float dsigma, cudaStream_t s) {
-  const int64_t total = (int64_t)C * F * H * W;
-  launch_pdl(unpatchify_euler_kernel, grid_for(total), kThreads, 0, s, vtok, v_out, latent, C, F, H, W, pt, ph, pw, dsigma);
+  const PatchGeo g{C, F, H, W, pt, ph, pw};
+  dim3 grid;
+  size_t smem;
+  if (patch_tiles(g, &grid, &smem))
+    launch_pdl(unpatchify_tile_kernel, grid, kThreads, smem, s, vtok, v_out, latent, g, dsigma);
+  else
+    launch_pdl(unpatchify_euler_kernel, grid_for((int64_t)C * F * H * W), kThreads, 0, s, vtok, v_out, latent, C, F, H,
+               W, pt, ph, pw, dsigma);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }

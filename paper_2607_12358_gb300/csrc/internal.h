@@ -97,6 +97,12 @@ acid_status ln_mod(int in_dtype, const void* x, int out_dtype, void* y, int64_t 
                    const float* shift_v, const float* scale_v, const float* shift_t,
                    const float* scale_t, int64_t split, float eps, cudaStream_t s);
 
+// The final layer's LayerNorm (y and x of one dtype, modulated) together with
+// the TeaCache residual r [rows, d]: reuse forms x = h + r, rounded to dtype,
+// instead of reading x; otherwise r = x - h is written.
+acid_status ln_mod_cached(int dtype, bool reuse, const void* x, const float* h, float* r, void* y, int64_t rows, int d,
+                          const float* shift, const float* scale, float eps, cudaStream_t s);
+
 // TeaCache signal sums from the fp32 patch embeddings of two consecutive steps
 // and their block-0 modulations (shift then scale, d each): TEMNI of both
 // steps formed in registers, 8 bytes read per element.  Result {rel, num, den}
@@ -145,8 +151,9 @@ acid_status add_same(int dtype, const void* a, const void* b, void* out, int64_t
 acid_status add_mixed(int a_dtype, const void* a, int b_dtype, const void* b, int out_dtype,
                       void* out, int64_t n, float b_scale, cudaStream_t s);
 
-acid_status patchify(const float* latent, int out_dtype, void* tokens, int C, int F, int H, int W,
-                     int pt, int ph, int pw, cudaStream_t s);
+// fp32 tokens [N, P]
+acid_status patchify(const float* latent, float* tokens, int C, int F, int H, int W, int pt, int ph, int pw,
+                     cudaStream_t s);
 // bf16 tokens [N, 2P]: each fp32 patch value x as hi = bf16(x) in column p and
 // lo = bf16(x - hi) in column P + p (hi + lo = x to within 2^-17 |x|)
 acid_status patchify_split(const float* latent, void* tokens, int C, int F, int H, int W, int pt, int ph, int pw,

@@ -367,18 +367,34 @@ acid_status dicache_reuse(int dt, void* out, const float* p_t, const LoopWs& w, 
 }
 
 // Final layer + unpatchify: v (optional) and the Euler update of the latent.
+// A TeaCache step forms the final layer's modulation with block 0's
+// (cache != kNoCache) and applies or stores its residual in the LayerNorm pass.
+enum CacheUse { kNoCache, kReuse, kStore };
 acid_status final_layer(const acid_model& m, const LoopWs& w, const void* h_out, float* v_out, float* latent,
-                        float dsig, cudaStream_t s) {
+                        float dsig, cudaStream_t s, CacheUse cache = kNoCache, const float* h_in = nullptr) {
   const Shape sh = shape_of(m);
   const int dt = m.block.dtype;
-  ACID_TRY(gemv(dt, m.final_mod.w, m.final_mod.b, w.temb, w.fmod, 2 * sh.d, sh.d, true, s));
-  ACID_TRY(ln_mod(dt, h_out, dt, w.y, sh.N, sh.d, w.fmod, w.fmod + sh.d, nullptr, nullptr, 0, m.block.ln_eps, s));
+  if (cache == kNoCache) {
+    ACID_TRY(gemv(dt, m.final_mod.w, m.final_mod.b, w.temb, w.fmod, 2 * sh.d, sh.d, true, s));
+    ACID_TRY(ln_mod(dt, h_out, dt, w.y, sh.N, sh.d, w.fmod, w.fmod + sh.d, nullptr, nullptr, 0, m.block.ln_eps, s));
+  } else {
+    ACID_TRY(ln_mod_cached(dt, cache == kReuse, h_out, h_in, w.resid, w.y, sh.N, sh.d, w.fmod, w.fmod + sh.d,
+                           m.block.ln_eps, s));
+  }
   Epilogue e;
   e.bias = m.final_out.b;
   e.out_fp32 = true;
   ACID_TRY(linear_forward(dt, w.y, sh.d, sh.N, sh.d, m.final_out.w, (int)sh.P, w.vtok, sh.P, e, s));
   return unpatchify_euler(w.vtok, v_out, latent, m.latent_c, m.latent_f, m.latent_h, m.latent_w, m.pt, m.ph, m.pw,
                           dsig, s);
+}
+
+// The step's modulations that need only temb: block 0's (shift, scale) for the
+// TeaCache signal and the final layer's, in one launch.
+acid_status teacache_mods(const acid_model& m, const LoopWs& w, float* mod0, cudaStream_t s) {
+  const int d = m.block.d;
+  return gemv2(m.block.dtype, m.blocks[0].mod.w, m.blocks[0].mod.b, mod0, 2 * d, m.final_mod.w, m.final_mod.b, w.fmod,
+               2 * d, w.temb, d, true, s);
 }
 
 }  // namespace
@@ -495,7 +511,7 @@ static acid_status patch_embed(const acid_model& m, const LoopWs& w, const float
     return linear_forward(ACID_BF16, w.tokens, 2 * sh.P, sh.N, (int)(2 * sh.P), w.patch_w2, sh.d, h_in, sh.d, e, s);
   }
   ACID_REQUIRE(m.block.dtype == ACID_FP32, ACID_ERR_UNSUPPORTED, "patch embedding: bf16 needs P % 8 == 0");
-  ACID_TRY(patchify(latent, ACID_FP32, w.tokens, m.latent_c, m.latent_f, m.latent_h, m.latent_w, m.pt, m.ph, m.pw, s));
+  ACID_TRY(patchify(latent, reinterpret_cast<float*>(w.tokens), m.latent_c, m.latent_f, m.latent_h, m.latent_w, m.pt, m.ph, m.pw, s));
   return linear_forward_f32(w.tokens, sh.P, sh.N, (int)sh.P, m.patch.w, sh.d, h_in, sh.d, e, s);
 }
 
@@ -547,7 +563,7 @@ static acid_status branch_step(const acid_model* m, const acid_loop_cfg* cfg, ac
     // s_t: rel_l1 of block 0's modulated input (TEMNI) between consecutive
     // steps, both TEMNIs formed from this and the previous step's H_in and
     // block-0 modulation in one read-only pass
-    ACID_TRY(gemv(dt, m->blocks[0].mod.w, m->blocks[0].mod.b, w.temb, w.mod0[par], 2 * sh.d, sh.d, true, s));
+    ACID_TRY(teacache_mods(*m, w, w.mod0[par], s));
     ACID_TRY(temni_drift(h_in, w.h_in[par ^ 1], w.mod0[par], w.mod0[par ^ 1], nullptr, i, sh.N, sh.d,
                          m->block.ln_eps, w.dres, w.drift_ws, drift_workspace_bytes(0), s, w.drift_done));
     if (!warm) {
@@ -559,12 +575,10 @@ static acid_status branch_step(const acid_model* m, const acid_loop_cfg* cfg, ac
     if (compute || !st->have_cache) {
       compute = true;
       ACID_TRY(run_model());
-      ACID_TRY(add_mixed(dt, x_video, ACID_FP32, h_in, ACID_FP32, w.resid, sh.N * sh.d, -1.0f, s));
       st->have_cache = 1;
-    } else {
-      ACID_TRY(add_mixed(ACID_FP32, h_in, ACID_FP32, w.resid, dt, x_video, sh.N * sh.d, 1.0f, s));
     }
-    ACID_TRY(final_layer(*m, w, x_video, defer_euler ? w.v[0] : nullptr, defer_euler ? nullptr : latent, dsig, s));
+    ACID_TRY(final_layer(*m, w, x_video, defer_euler ? w.v[0] : nullptr, defer_euler ? nullptr : latent, dsig, s,
+                         compute ? kStore : kReuse, h_in));
     if (defer_euler) *v_out = w.v[0];
   } else if (cfg->method == ACID_METHOD_DICACHE) {
     // probe: the first probe_blocks blocks on every step; P_i (fp32) in temni[i & 1]
@@ -894,7 +908,7 @@ acid_status capture_branch(const acid_model& m, const acid_loop_cfg& cfg, LoopWs
   float* p_prev = w.temni[par ^ 1];
   const int pb = cfg.probe_blocks;
   if (cfg.method == ACID_METHOD_TEACACHE) {
-    ACID_TRY(gemv(dt, m.blocks[0].mod.w, m.blocks[0].mod.b, w.temb, w.mod0[par], 2 * sh.d, sh.d, true, s));
+    ACID_TRY(teacache_mods(m, w, w.mod0[par], s));
     ACID_TRY(temni_drift(h_in, w.h_in[par ^ 1], w.mod0[par], w.mod0[par ^ 1], step, 0, sh.N, sh.d, m.block.ln_eps,
                          w.dres, w.drift_ws, drift_workspace_bytes(0), s, w.drift_done));
   } else if (cfg.method == ACID_METHOD_DICACHE) {
@@ -927,7 +941,7 @@ acid_status capture_branch(const acid_model& m, const acid_loop_cfg& cfg, LoopWs
   }
   if (cfg.method == ACID_METHOD_DICACHE) {
   } else if (cfg.method == ACID_METHOD_TEACACHE) {
-    ACID_TRY(add_mixed(dt, x_video, ACID_FP32, h_in, ACID_FP32, w.resid, sh.N * sh.d, -1.0f, s2));
+    ACID_TRY(final_layer(m, w, x_video, v, nullptr, 0.0f, s2, kStore, h_in));
   } else {
     ACID_TRY(final_layer(m, w, x_video, v, nullptr, 0.0f, s2));
     ACID_TRY(drift_launch(ACID_FP32, v_prev, v, nullptr, nullptr, sh.latent, w.dres, w.drift_ws,
@@ -943,7 +957,7 @@ acid_status capture_branch(const acid_model& m, const acid_loop_cfg& cfg, LoopWs
   // ---- reuse body: cached residual / offset
   ACID_CUDA(cudaStreamBeginCaptureToGraph(s2, br[1], nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed));
   if (cfg.method == ACID_METHOD_TEACACHE)
-    ACID_TRY(add_mixed(ACID_FP32, h_in, ACID_FP32, w.resid, dt, x_video, sh.N * sh.d, 1.0f, s2));
+    ACID_TRY(final_layer(m, w, x_video, v, nullptr, 0.0f, s2, kReuse, h_in));
   else if (cfg.method == ACID_METHOD_DICACHE)
     ACID_TRY(dicache_reuse(dt, x_video, p_cur, w, sh.N * sh.d, s2));
   else
@@ -951,11 +965,10 @@ acid_status capture_branch(const acid_model& m, const acid_loop_cfg& cfg, LoopWs
   ACID_CUDA(cudaStreamEndCapture(s2, &tmp));
 
   // ---- output: the velocity, and the previous step's values
-  if (cfg.method == ACID_METHOD_TEACACHE) {
+  // (TeaCache: the final layer ran in the compute or reuse body)
+  if (cfg.method == ACID_METHOD_DICACHE) {
     ACID_TRY(final_layer(m, w, x_video, v, nullptr, 0.0f, s));
-  } else if (cfg.method == ACID_METHOD_DICACHE) {
-    ACID_TRY(final_layer(m, w, x_video, v, nullptr, 0.0f, s));
-  } else {
+  } else if (cfg.method == ACID_METHOD_EASYCACHE) {
     ACID_CUDA(cudaMemcpyAsync(w.x_prev, latent, sh.latent * sizeof(float), cudaMemcpyDeviceToDevice, s));
     ACID_CUDA(cudaMemcpyAsync(v_prev, v, sh.latent * sizeof(float), cudaMemcpyDeviceToDevice, s));
   }
