@@ -31,8 +31,15 @@ def _dtype(t: torch.Tensor) -> int:
     return _DT[t.dtype]
 
 
+# The current stream's handle without building a Stream object: 0.3 us against
+# 2.9 us, a third of a small call's whole host time.
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
 def _stream(stream=None) -> int:
     if stream is None:
+        if _raw_stream is not None:
+            return _raw_stream(torch.cuda.current_device())
         return torch.cuda.current_stream().cuda_stream
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
