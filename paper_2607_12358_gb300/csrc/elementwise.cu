@@ -159,18 +159,19 @@ __global__ void __launch_bounds__(kThreads) drift_final_kernel(const double2* __
     n += partials[i].x;
     d += partials[i].y;
   }
-  __shared__ double sn[kThreads], sd[kThreads];
-  sn[threadIdx.x] = n;
-  sd[threadIdx.x] = d;
-  __syncthreads();
-  for (int s = kThreads / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) {
-      sn[threadIdx.x] += sn[threadIdx.x + s];
-      sd[threadIdx.x] += sd[threadIdx.x + s];
-    }
-    __syncthreads();
+  __shared__ double sn[kThreads / 32], sd[kThreads / 32];
+  n = warp_sum_d(n);
+  d = warp_sum_d(d);
+  if ((threadIdx.x & 31) == 0) {
+    sn[threadIdx.x >> 5] = n;
+    sd[threadIdx.x >> 5] = d;
   }
+  __syncthreads();
   if (threadIdx.x == 0) {
+    for (int w = 1; w < kThreads / 32; ++w) {
+      sn[0] += sn[w];
+      sd[0] += sd[w];
+    }
     write_drift_result(sn[0], sd[0], result);
     if (rel_out != nullptr) *rel_out = result[0];
     if (sums_out != nullptr) {
