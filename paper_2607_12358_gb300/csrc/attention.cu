@@ -300,7 +300,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  pdl_begin();  // the set-up above overlaps the tail of the kernel before
+  pdl_wait();  // the set-up above overlaps the tail of the kernel before
 
   if (warp == 0) {
     if (lane == 0) {  // ---------------------------------------- TMA producer
@@ -499,7 +499,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  pdl_begin();  // the set-up above overlaps the tail of the kernel before
+  pdl_wait();  // the set-up above overlaps the tail of the kernel before
 
   if (warp == 0) {
     if (lane == 0) {  // ---------------------------------------- TMA producer
@@ -669,7 +669,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
 // One warp per row (256 rows per item), D / 32 columns per lane.
 template <int D>
 __global__ void __launch_bounds__(256) attn_merge_kernel(AttnDev a, int item0, int tail, int splits) {
-  pdl_begin();
+  pdl_wait();
   const int wrow = (int)(blockIdx.x * 8 + (threadIdx.x >> 5));  // row over all tail items
   const int lane = threadIdx.x & 31;
   if (wrow >= tail * kBQ) return;
@@ -845,7 +845,7 @@ __device__ __forceinline__ void load_rows_f32(float* dst, int lds, const float* 
 
 template <int D, int BQ>
 __global__ void __launch_bounds__(128 * kF32Groups) attn_f32_kernel(AttnF32Args a) {
-  pdl_begin();
+  pdl_wait();
   using C = AttnF32Cfg<D, BQ>;
   constexpr int QT = C::QT, KT = kF32Keys / 16, NC = D / 32;  // NC column pairs per lane
   extern __shared__ __align__(16) float fsm[];

@@ -48,10 +48,14 @@ void count_launch();
 
 // Launches a kernel that may start while the kernel before it on the stream is
 // still draining (programmatic dependent launch): its launch and set-up
-// overlap that kernel's tail.  Every kernel launched this way calls pdl_begin
-// (or pdl_trigger and pdl_wait) before its first access to global memory, and
-// pdl_wait returns once the kernel before has completed and its writes are
-// visible, so the stream's order of effects is kept, link by link.
+// overlap that kernel's tail.  Every kernel launched this way calls pdl_wait
+// before its first access to global memory, which returns once the kernel
+// before has completed and its writes are visible, so the stream's order of
+// effects is kept, link by link.
+//   Kernels leave the moment their successor may start to the default, the end
+// of their CTAs.  Allowed earlier, the successor's CTAs pile up on the few SMs
+// that the running kernel leaves free: a 128-CTA fp32 GEMM in a chain ran
+// 17.5 us instead of 9.2, the toy generation 1187 us instead of 1018.
 template <typename... P, typename... A>
 cudaError_t launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A&&... args) {
   cudaLaunchConfig_t cfg = {};
@@ -144,14 +148,8 @@ constexpr bool kBoundsChecked = false;
 // ---------------------------------------------------------------------------
 // Programmatic dependent launch (see launch_pdl)
 // ---------------------------------------------------------------------------
-// The next kernel may be launched once every CTA has come this far.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 // Waits until the kernel before this one has completed.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_begin() {
-  pdl_trigger();
-  pdl_wait();
-}
 
 // ---------------------------------------------------------------------------
 // Numeric helpers

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(kThreads, 4) drift_partials_kernel(const T* __
                                                                      const T* __restrict__ cur,
                                                                      const T* __restrict__ resid, T* out,
                                                                      int64_t n, double2* __restrict__ partials) {
-  pdl_begin();
+  pdl_wait();
   constexpr int V = Vec<T>::N;
   constexpr int U = kApply ? 2 : 4;  // 16-byte vectors in flight per thread and tensor
   const int64_t nvec = n / V;
@@ -153,7 +153,7 @@ __device__ __forceinline__ void write_drift_result(double num, double den, doubl
 // caller's own rel and {num, den} where given.
 __global__ void __launch_bounds__(kThreads) drift_final_kernel(const double2* __restrict__ partials, int nparts,
                                                                double* result, double* rel_out, double* sums_out) {
-  pdl_begin();
+  pdl_wait();
   double n = 0.0, d = 0.0;
   for (int i = threadIdx.x; i < nparts; i += kThreads) {
     n += partials[i].x;
@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(kThreads) drift_final_kernel(const double2* __
 template <typename T>
 __global__ void __launch_bounds__(kThreads) add_vec_kernel(const T* __restrict__ a, const T* __restrict__ b, T* out,
                                                            int64_t n) {
-  pdl_begin();
+  pdl_wait();
   constexpr int V = Vec<T>::N;
   const int64_t nvec = n / V;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kThreads) add_vec_kernel(const T* __restrict__
 
 template <typename TA, typename TB, typename TO>
 __global__ void add_mixed_kernel(const TA* __restrict__ a, const TB* __restrict__ b, TO* out, int64_t n, float bs) {
-  pdl_begin();
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
     io<TO>::st(out + i, io<TA>::ld(a + i) + bs * io<TB>::ld(b + i));
@@ -213,7 +213,7 @@ __global__ void add_mixed_kernel(const TA* __restrict__ a, const TB* __restrict_
 // READ_B false: out = a (b_scale 0, b not read).
 template <typename TA, typename TB, typename TO, bool READ_B>
 __global__ void add_mixed8_kernel(const TA* __restrict__ a, const TB* __restrict__ b, TO* out, int64_t n, float bs) {
-  pdl_begin();
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   for (int64_t i = tid; i < n / 8; i += stride) {
@@ -389,7 +389,7 @@ constexpr int kLnThreads = 128;
 // apart, the state was written and read again, or read a second time.
 template <typename Tin, typename Tout, int NV, bool FULL, int MODE>
 __global__ void __launch_bounds__(kLnThreads, NV <= 12 ? 5 : 4) ln_mod_rows_kernel(LnArgs a) {
-  pdl_begin();
+  pdl_wait();
   const int64_t row = ((int64_t)blockIdx.x * kLnThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31, d = a.d;
   if (row >= a.rows) return;
@@ -460,7 +460,7 @@ constexpr int kLnMaxWarps = NV * RowVec<Tin>::kN <= 64 ? 16 : 12;
 
 template <typename Tin, typename Tout, int NV, bool FULL>
 __global__ void __launch_bounds__(32 * kLnMaxWarps<Tin, NV>, 1) ln_mod_bulk_kernel(LnArgs a) {
-  pdl_begin();
+  pdl_wait();
   constexpr int N = RowVec<Tin>::kN;
   extern __shared__ __align__(128) uint8_t lsm[];
   const int nwarps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -587,7 +587,7 @@ __global__ void __launch_bounds__(32 * kTemniMaxWarps, 1) temni_drift_kernel(con
                                                                             const float* __restrict__ scp, float eps,
                                                                             double2* __restrict__ partials,
                                                                             unsigned int* done, double* result) {
-  pdl_begin();
+  pdl_wait();
   extern __shared__ __align__(128) uint8_t tsm[];
   const int nwarps = blockDim.x >> 5;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -774,7 +774,7 @@ struct GemvMat {
 template <typename TW, int R>
 __global__ void __launch_bounds__(kThreads, 3) gemv_kernel(GemvMat m0, GemvMat m1, const float* __restrict__ x, int k,
                                                            int silu_in) {
-  pdl_begin();
+  pdl_wait();
   extern __shared__ __align__(16) float xs[];  // [2][k / 2]: columns 8 i + {0..3}, then 8 i + {4..7}
   for (int i = threadIdx.x; i < k; i += kThreads) {
     const float v = x[i];
@@ -837,20 +837,20 @@ __device__ __forceinline__ void sinusoid_at(float* out, double t, int half, int 
 }
 
 __global__ void sinusoid_kernel(float* out, double t, int half) {
-  pdl_begin();
+  pdl_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < half) sinusoid_at(out, t, half, j);
 }
 
 // t = 1000 sigma[step] with the step index read from device memory
 __global__ void sinusoid_sig_kernel(float* out, const double* sig, const int* step, int half) {
-  pdl_begin();
+  pdl_wait();
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j < half) sinusoid_at(out, 1000.0 * sig[*step], half, j);
 }
 
 __global__ void rope_table_kernel(float2* tbl, int F, int H, int W, int pt, int ph, int pw, double theta) {
-  pdl_begin();
+  pdl_wait();
   // pt / ph / pw: rotation pairs per axis (t, h, w)
   const int64_t total = (int64_t)F * pt + (int64_t)H * ph + (int64_t)W * pw;
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -916,7 +916,7 @@ struct PatchTile {
 // tokens.
 template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads) patchify_tile_kernel(const float* __restrict__ lat, void* tok, PatchGeo geo) {
-  pdl_begin();
+  pdl_wait();
   extern __shared__ float tile[];
   const PatchTile t(geo);
   const int n = t.nw * t.P;
@@ -944,7 +944,7 @@ __global__ void __launch_bounds__(kThreads) patchify_tile_kernel(const float* __
 __global__ void __launch_bounds__(kThreads) unpatchify_tile_kernel(const float* __restrict__ vtok,
                                                                    float* __restrict__ vout, float* lat, PatchGeo geo,
                                                                    float dsig) {
-  pdl_begin();
+  pdl_wait();
   extern __shared__ float tile[];
   const PatchTile t(geo);
   const int n = t.nw * t.P;
@@ -966,7 +966,7 @@ __global__ void __launch_bounds__(kThreads) unpatchify_tile_kernel(const float* 
 
 __global__ void patchify_kernel(const float* __restrict__ lat, float* __restrict__ tok, int C, int F, int H, int W,
                                 int pt, int ph, int pw) {
-  pdl_begin();
+  pdl_wait();
   const int Hp = H / ph, Wp = W / pw;
   const int P = C * pt * ph * pw;
   const int64_t total = (int64_t)(F / pt) * Hp * Wp * P;
@@ -987,7 +987,7 @@ __global__ void patchify_kernel(const float* __restrict__ lat, float* __restrict
 // The same as hi and lo bf16 parts (see patchify_tile_kernel).
 __global__ void patchify_split_kernel(const float* __restrict__ lat, __nv_bfloat16* __restrict__ tok, int C, int F,
                                       int H, int W, int pt, int ph, int pw) {
-  pdl_begin();
+  pdl_wait();
   const int Hp = H / ph, Wp = W / pw;
   const int P = C * pt * ph * pw;
   const int64_t total = (int64_t)(F / pt) * Hp * Wp * P;
@@ -1014,7 +1014,7 @@ __global__ void patchify_split_kernel(const float* __restrict__ lat, __nv_bfloat
 
 __global__ void unpatchify_euler_kernel(const float* __restrict__ vtok, float* __restrict__ vout, float* lat, int C,
                                         int F, int H, int W, int pt, int ph, int pw, float dsig) {
-  pdl_begin();
+  pdl_wait();
   const int Hp = H / ph, Wp = W / pw;
   const int P = C * pt * ph * pw;
   const int64_t total = (int64_t)C * F * H * W;
@@ -1034,7 +1034,7 @@ __global__ void unpatchify_euler_kernel(const float* __restrict__ vtok, float* _
 }
 
 __global__ void euler_kernel(float* lat, const float* __restrict__ v, int64_t n, float dsig) {
-  pdl_begin();
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) lat[i] = fmaf(dsig, v[i], lat[i]);
 }
@@ -1042,7 +1042,7 @@ __global__ void euler_kernel(float* lat, const float* __restrict__ v, int64_t n,
 // Classifier-free guidance and the Euler step: x += dsig * (v_u + g (v_c - v_u)).
 __global__ void guided_euler_kernel(float* lat, const float* __restrict__ vc, const float* __restrict__ vu, int64_t n,
                                     float g, float dsig) {
-  pdl_begin();
+  pdl_wait();
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     const float u = vu[i];
@@ -1053,7 +1053,7 @@ __global__ void guided_euler_kernel(float* lat, const float* __restrict__ vc, co
 // The same with dsigma read from device memory (graph-launched loops).
 __global__ void guided_euler_sig_kernel(float* lat, const float* __restrict__ vc, const float* __restrict__ vu,
                                         int64_t n, float g, const double* sig, const int* step) {
-  pdl_begin();
+  pdl_wait();
   const int i0 = *step;
   const float dsig = (float)(sig[i0 + 1] - sig[i0]);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -1066,7 +1066,7 @@ __global__ void guided_euler_sig_kernel(float* lat, const float* __restrict__ vc
 // dsigma = sigma[step + 1] - sigma[step] with the step index read from device memory
 __global__ void euler_sig_kernel(float* lat, const float* __restrict__ v, int64_t n, const double* sig,
                                  const int* step) {
-  pdl_begin();
+  pdl_wait();
   const int i0 = *step;
   const float dsig = (float)(sig[i0 + 1] - sig[i0]);
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;

@@ -517,7 +517,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
   cluster_sync();  // both CTAs' barriers exist before any cross-CTA arrival
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
-  pdl_begin();  // the set-up above overlaps the tail of the kernel before
+  pdl_wait();  // the set-up above overlaps the tail of the kernel before
 
   if (warp == 0) {
     // TMA producer (both CTAs): one continuous stage ring across tiles; the
@@ -907,7 +907,7 @@ bool splitk_plan(int64_t M, int N, int K, size_t ws_bytes, int pairs, SplitKPlan
 template <int KIND, bool R32, bool O32>
 __global__ void __launch_bounds__(256) splitk_fixup_kernel(const float* __restrict__ part, int splits, int64_t m_pad,
                                                            int64_t M, int N, void* out, int64_t ldo, EpiDev e) {
-  pdl_begin();
+  pdl_wait();
   const int64_t npair = N / 2, total = M * npair;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
@@ -1054,7 +1054,7 @@ template <int TM, int TN>
 __global__ void __launch_bounds__(64 * kFGroups) gemm_f32_kernel(const float* __restrict__ A, int64_t lda, int64_t M,
                                                                  int K, const float* __restrict__ W, int N, float* out,
                                                                  int64_t ldo, EpiDev e, bool vec) {
-  pdl_begin();
+  pdl_wait();
   using C = F32Cfg<TM, TN>;
   constexpr int MT = TM / 8, NT = TN / 8;
   extern __shared__ __align__(16) float fsm[];

@@ -298,7 +298,7 @@ acid_status run_blocks(const acid_model& m, const LoopWs& w, cudaStream_t s, int
 template <typename T>
 __global__ void dicache_update_kernel(const T* __restrict__ h_out, const float* __restrict__ p_t, float* d1,
                                       float* d2, float* p1, float* p2, int64_t n, const int* count) {
-  pdl_begin();
+  pdl_wait();
   const int c = *count;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
@@ -317,7 +317,7 @@ __global__ void dicache_update_kernel(const T* __restrict__ h_out, const float* 
 }
 
 __global__ void dicache_count_kernel(int* count) {
-  pdl_begin();
+  pdl_wait();
   *count = min(*count + 1, 2);
 }
 
@@ -326,7 +326,7 @@ __global__ void dicache_count_kernel(int* count) {
 template <typename T>
 __global__ void dicache_reuse_kernel(T* out, const float* __restrict__ p_t, const float* __restrict__ d1,
                                      const float* __restrict__ d2, int64_t n, const double* num, const double* den) {
-  pdl_begin();
+  pdl_wait();
   const double dn = *den;
   const float g = dn > 0.0 ? (float)(*num / dn) : 0.0f;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
