@@ -3,6 +3,8 @@
 // tables, patchify / unpatchify + Euler update.
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "internal.h"
 
@@ -560,49 +562,50 @@ __global__ void __launch_bounds__(32 * kLnMaxWarps<Tin, NV>, 1) ln_mod_bulk_kern
 // embeddings H_in_t (xc) and H_in_{t-1} (xp), so the kernel reads 8 bytes per
 // element and writes nothing but one fp64 partial pair per CTA (reduced by
 // drift_final_kernel, or with a done counter by the CTA that finishes last).
-// One warp per row pair (rows counted from the end: gw, gw + total warps, ...
-// from the last row down), reductions by warp
-// shuffles only.  Lane 0 of each warp streams the warp's row pairs into its
-// own two-stage shared-memory ring with 1D bulk copies (completion counted on
-// the stage's mbarrier), so the bytes in flight come from shared memory, not
-// registers; the stage is refilled as soon as every lane has read it.  The
-// four modulation vectors (shift and 1 + scale of both steps) are staged once
-// per CTA in shared memory.  Row statistics: mean and variance from sums of
-// (x - K) and (x - K)^2 with K the row's first element, which keeps the
-// fp32 cancellation small (K lies within a few standard deviations of the
-// mean).  HOLD: rows of up to 1536 values stay in registers after one read of
-// the stage (16 per lane), else the stage is read again for the final pass.
-// Step 0 gives zero sums.
+// A group of WPR warps takes one row pair at a time (rows counted from the
+// end: g, g + total groups, ... from the last row down) and streams its row pairs
+// into its own two-stage shared-memory ring with 1D bulk copies (completion
+// counted on the stage's mbarrier), so the bytes in flight come from shared
+// memory, not registers; a lane keeps its NV4 x 4 columns of both rows in
+// registers after one read of the stage, which is refilled as soon as the
+// group has read it.  Long rows leave shared memory for few groups (three at
+// 3072 columns), so several warps share a row: with one warp each, three warps
+// per SM did all the arithmetic (16000 x 3072: 122 us).  The four modulation
+// vectors (shift and 1 + scale of both steps) are staged once per CTA in
+// shared memory.  Row statistics: mean and variance from sums of (x - K) and
+// (x - K)^2 with K the row's first element, which keeps the fp32 cancellation
+// small (K lies within a few standard deviations of the mean), by warp shuffles
+// and, across a group's warps, through shared memory.  Step 0 gives zero sums.
 constexpr int kTemniStages = 2;
-constexpr int kTemniMaxWarps = 8;
+constexpr int kTemniMaxWarps = 16, kTemniMaxGroups = 8;
 
-template <int NV4, bool HOLD>
-__global__ void __launch_bounds__(32 * kTemniMaxWarps, 1) temni_drift_kernel(const float* __restrict__ xc,
-                                                                            const float* __restrict__ xp,
-                                                                            const int* step_dev, int step_host,
-                                                                            int64_t rows, int d,
-                                                                            const float* __restrict__ shc,
-                                                                            const float* __restrict__ scc,
-                                                                            const float* __restrict__ shp,
-                                                                            const float* __restrict__ scp, float eps,
-                                                                            double2* __restrict__ partials,
-                                                                            unsigned int* done, double* result) {
+template <int NV4, int WPR>
+__global__ void __launch_bounds__(32 * (WPR == 1 ? kTemniMaxGroups : kTemniMaxWarps), 1)
+    temni_drift_kernel(const float* __restrict__ xc, const float* __restrict__ xp, const int* step_dev, int step_host,
+                       int64_t rows, int d, const float* __restrict__ shc, const float* __restrict__ scc,
+                       const float* __restrict__ shp, const float* __restrict__ scp, float eps,
+                       double2* __restrict__ partials, unsigned int* done, double* result) {
   pdl_wait();
   extern __shared__ __align__(128) uint8_t tsm[];
-  const int nwarps = blockDim.x >> 5;
+  const int nwarps = blockDim.x >> 5, ngroups = nwarps / WPR;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int grp = warp / WPR, wg = warp % WPR;  // group, warp in the group
   // four d-long vectors: shift_c, 1 + scale_c, shift_p, 1 + scale_p (separate
   // arrays, so that a warp's 16-byte reads of one vector are contiguous)
   float4* mod = reinterpret_cast<float4*>(tsm);
-  float* ring = reinterpret_cast<float*>(tsm + (size_t)16 * d);                       // [warp][stage][2][d]
-  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)nwarps * kTemniStages * 2 * d);  // [warp][stage]
+  float* ring = reinterpret_cast<float*>(tsm + (size_t)16 * d);                                   // [group][stage][2][d]
+  uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)ngroups * kTemniStages * 2 * d);    // [group][stage]
   __shared__ double rd[2][kTemniMaxWarps];
+  __shared__ float4 stats[2][kTemniMaxWarps];  // partial row sums, by row parity
+  __shared__ int gave_up[kTemniMaxWarps];      // by group
+  if (threadIdx.x < kTemniMaxWarps) gave_up[threadIdx.x] = 0;
   const int step = step_dev ? *step_dev : step_host;
-  float* wr = ring + (size_t)warp * kTemniStages * 2 * d;
-  uint64_t* wf = full + warp * kTemniStages;
-  const int64_t gw = (int64_t)blockIdx.x * nwarps + warp, nw = (int64_t)gridDim.x * nwarps;
+  float* wr = ring + (size_t)grp * kTemniStages * 2 * d;
+  uint64_t* wf = full + grp * kTemniStages;
+  const int64_t gw = (int64_t)blockIdx.x * ngroups + grp, nw = (int64_t)gridDim.x * ngroups;
   const int64_t n_my = (step > 0 && gw < rows) ? (rows - 1 - gw) / nw + 1 : 0;
   const uint32_t row_bytes = (uint32_t)d * sizeof(float);
+  const bool leader = wg == 0 && lane == 0;
   // Rows from the last one down: the patch embedding that writes h_cur just
   // before this kernel leaves its last rows in L2 (dirty), so they are read
   // first.  The previous step's rows are not read again in this step: they
@@ -617,9 +620,9 @@ __global__ void __launch_bounds__(32 * kTemniMaxWarps, 1) temni_drift_kernel(con
     bulk_load(wr + (size_t)st * 2 * d, xc + row * d, row_bytes, &wf[st]);
     bulk_load_hint(wr + (size_t)st * 2 * d + d, xp + row * d, row_bytes, &wf[st], prev_policy);
   };
-  // each warp's first copies are issued before the modulation vectors are
+  // each group's first copies are issued before the modulation vectors are
   // staged, so their latency overlaps the staging
-  if (lane == 0) {
+  if (leader) {
     for (int i = 0; i < kTemniStages; ++i) mbar_init(&wf[i], 1);
     mbar_fence_init();
     for (int64_t k = 0; k < n_my && k < kTemniStages; ++k) issue(k);
@@ -640,22 +643,20 @@ __global__ void __launch_bounds__(32 * kTemniMaxWarps, 1) temni_drift_kernel(con
   for (; k < n_my; ++k) {
     const int st = (int)(k % kTemniStages);
     const bool ok = __all_sync(0xffffffffu, mbar_wait(&wf[st], (uint32_t)((k / kTemniStages) & 1)));
-    if (!ok) break;
+    if (WPR == 1 && !ok) break;
     const float4* rc = reinterpret_cast<const float4*>(wr + (size_t)st * 2 * d);
     const float4* rp = rc + d / 4;
-    // lane's vectors: i * 32 + lane, i < NV4 (4 columns each)
-    float4 cv[HOLD ? NV4 : 1], pv[HOLD ? NV4 : 1];
+    // lane's vectors: (i * WPR + wg) * 32 + lane, i < NV4 (4 columns each)
+    float4 cv[NV4], pv[NV4];
     const float kc = wr[(size_t)st * 2 * d], kp = wr[(size_t)st * 2 * d + d];  // shifts: the rows' first elements
     float s1c = 0.f, s2c = 0.f, s1p = 0.f, s2p = 0.f;
 #pragma unroll
     for (int i = 0; i < NV4; ++i) {
-      const int v = i * 32 + lane;
+      const int v = (i * WPR + wg) * 32 + lane;
       if (v < d / 4) {
         const float4 c = rc[v], p = rp[v];
-        if constexpr (HOLD) {
-          cv[i] = c;
-          pv[i] = p;
-        }
+        cv[i] = c;
+        pv[i] = p;
         const float c0 = c.x - kc, c1 = c.y - kc, c2 = c.z - kc, c3 = c.w - kc;
         const float p0 = p.x - kp, p1 = p.y - kp, p2 = p.z - kp, p3 = p.w - kp;
         s1c += (c0 + c1) + (c2 + c3);
@@ -664,7 +665,7 @@ __global__ void __launch_bounds__(32 * kTemniMaxWarps, 1) temni_drift_kernel(con
         s2p = fmaf(p0, p0, fmaf(p1, p1, fmaf(p2, p2, fmaf(p3, p3, s2p))));
       }
     }
-    if (HOLD) {
+    if constexpr (WPR == 1) {
       __syncwarp();
       if (lane == 0 && k + kTemniStages < n_my) issue(k + kTemniStages);  // every lane holds its values
     }
@@ -675,22 +676,32 @@ __global__ void __launch_bounds__(32 * kTemniMaxWarps, 1) temni_drift_kernel(con
       s1p += __shfl_xor_sync(0xffffffffu, s1p, o);
       s2p += __shfl_xor_sync(0xffffffffu, s2p, o);
     }
+    if constexpr (WPR > 1) {
+      // the sums of row k + 2 overwrite these behind the barrier of row k + 1
+      if (lane == 0) stats[k & 1][warp] = make_float4(s1c, s2c, s1p, s2p);
+      if (!ok && lane == 0) gave_up[grp] = 1;
+      group_sync(1 + grp, 32 * WPR);
+      if (gave_up[grp]) break;  // a wait of one of its warps ran out: the group leaves together
+      if (leader && k + kTemniStages < n_my) issue(k + kTemniStages);  // the whole group holds its values
+      s1c = s2c = s1p = s2p = 0.f;
+#pragma unroll
+      for (int w = 0; w < WPR; ++w) {
+        const float4 t = stats[k & 1][grp * WPR + w];
+        s1c += t.x;
+        s2c += t.y;
+        s1p += t.z;
+        s2p += t.w;
+      }
+    }
     const float dc = s1c * inv_d, dp = s1p * inv_d;  // mean - K
     const float mc = kc + dc, mp = kp + dp;
     const float rsc = rsqrtf(fmaxf(s2c * inv_d - dc * dc, 0.f) + eps);
     const float rsp = rsqrtf(fmaxf(s2p * inv_d - dp * dp, 0.f) + eps);
 #pragma unroll
     for (int i = 0; i < NV4; ++i) {
-      const int v = i * 32 + lane;
+      const int v = (i * WPR + wg) * 32 + lane;
       if (v < d / 4) {
-        float4 c, p;
-        if constexpr (HOLD) {
-          c = cv[i];
-          p = pv[i];
-        } else {
-          c = rc[v];
-          p = rp[v];
-        }
+        const float4 c = cv[i], p = pv[i];
         const int q = d / 4;
         const float4 bcv = mod[v], acv = mod[q + v], bpv = mod[2 * q + v], apv = mod[3 * q + v];
         const float cc[4] = {c.x, c.y, c.z, c.w}, pp[4] = {p.x, p.y, p.z, p.w};
@@ -705,13 +716,9 @@ __global__ void __launch_bounds__(32 * kTemniMaxWarps, 1) temni_drift_kernel(con
         }
       }
     }
-    if (!HOLD) {
-      __syncwarp();
-      if (lane == 0 && k + kTemniStages < n_my) issue(k + kTemniStages);  // every lane is done with the stage
-    }
   }
   // after a wait ran out: the copies already issued land before the CTA exits
-  if (k < n_my && lane == 0)
+  if (k < n_my && leader)
     for (int64_t j = k; j < n_my && j < k + kTemniStages; ++j)
       mbar_wait(&wf[j % kTemniStages], (uint32_t)((j / kTemniStages) & 1));
   double dn = warp_sum_d((double)num), dd = warp_sum_d((double)den);
@@ -1242,28 +1249,28 @@ acid_status ln_mod_cached(int dtype, bool reuse, const void* x, const float* h, 
   return reuse ? ln_rows_types<float, float, kLnReuse>(a, s) : ln_rows_types<float, float, kLnResid>(a, s);
 }
 
-template <int NV4, bool HOLD>
+template <int NV4, int WPR>
 acid_status launch_temni_drift(const float* h_cur, const float* h_prev, const float* mod_cur, const float* mod_prev,
                                const int* step_dev, int step_host, int64_t rows, int d, float eps, double2* parts,
                                unsigned int* done, double* result, cudaStream_t s, int* grid_out) {
-  constexpr int kSmemMax = 226 * 1024;  // dynamic shared memory, below the 227 KB limit less the static part
+  constexpr int kSmemMax = 225 * 1024;  // dynamic shared memory, below the 227 KB limit less the static part
   static bool attr_done = false;
   if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(temni_drift_kernel<NV4, HOLD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    ACID_CUDA(cudaFuncSetAttribute(temni_drift_kernel<NV4, WPR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                    kSmemMax));
     attr_done = true;
   }
-  // warps per CTA: as many two-stage rings (8 d bytes per stage) as fit
-  // beside the staged modulation vectors (16 d bytes), at most eight
-  const size_t ring_per_warp = (size_t)kTemniStages * 8 * d + kTemniStages * sizeof(uint64_t);
-  const int warps = (int)std::max<size_t>(1, std::min<size_t>(kTemniMaxWarps, (kSmemMax - 16 * (size_t)d) /
-                                                                                   ring_per_warp));
-  const size_t smem = 16 * (size_t)d + warps * ring_per_warp;
+  // groups per CTA: as many two-stage rings (8 d bytes per stage) as fit
+  // beside the staged modulation vectors (16 d bytes), within the group and
+  // warp limits
+  const size_t ring_per_group = (size_t)kTemniStages * 8 * d + kTemniStages * sizeof(uint64_t);
+  const int groups = (int)std::max<size_t>(1, std::min<size_t>(std::min(kTemniMaxGroups, kTemniMaxWarps / WPR),
+                                                               (kSmemMax - 16 * (size_t)d) / ring_per_group));
+  const size_t smem = 16 * (size_t)d + groups * ring_per_group;
   const int grid = (int)std::min<int64_t>(std::min<int64_t>(kDriftMaxBlocks, (int64_t)num_sms_elem()),
-                                          std::max<int64_t>(1, (rows + warps - 1) / warps));
-  launch_pdl(temni_drift_kernel<NV4, HOLD>, grid, 32 * warps, smem, s, h_cur, h_prev, step_dev, step_host, rows, d, mod_cur,
-                                                               mod_cur + d, mod_prev, mod_prev + d, eps, parts,
-                                                               done, result);
+                                          std::max<int64_t>(1, (rows + groups - 1) / groups));
+  launch_pdl(temni_drift_kernel<NV4, WPR>, grid, 32 * WPR * groups, smem, s, h_cur, h_prev, step_dev, step_host, rows, d,
+             mod_cur, mod_cur + d, mod_prev, mod_prev + d, eps, parts, done, result);
   ACID_CHECK_LAUNCH();
   *grid_out = grid;
   return ACID_OK;
@@ -1280,15 +1287,20 @@ acid_status temni_drift(const float* h_cur, const float* h_prev, const float* mo
   double2* parts = static_cast<double2*>(workspace);
   ProfScope prof(PROF_DRIFT, (double)rows * d * 8.0, s);  // read both steps' H_in (fp32)
   int grid = 1;
+  auto run = [&](auto nv4, auto wpr) {
+    return launch_temni_drift<decltype(nv4)::value, decltype(wpr)::value>(h_cur, h_prev, mod_cur, mod_prev, step_dev,
+                                                                          step_host, rows, d, eps, parts, done, d_result,
+                                                                          s, &grid);
+  };
+  using std::integral_constant;
   if (d <= 512)
-    ACID_TRY((launch_temni_drift<4, true>(h_cur, h_prev, mod_cur, mod_prev, step_dev, step_host, rows, d, eps, parts, done,
-                                         d_result, s, &grid)));
+    ACID_TRY(run(integral_constant<int, 4>{}, integral_constant<int, 1>{}));
   else if (d <= 1536)
-    ACID_TRY((launch_temni_drift<12, true>(h_cur, h_prev, mod_cur, mod_prev, step_dev, step_host, rows, d, eps, parts,
-                                          done, d_result, s, &grid)));
+    ACID_TRY(run(integral_constant<int, 12>{}, integral_constant<int, 1>{}));  // 66.5 us at 32760 x 1536; two warps a row: 68.8
+  else if (d <= 2048)
+    ACID_TRY(run(integral_constant<int, 4>{}, integral_constant<int, 4>{}));
   else
-    ACID_TRY((launch_temni_drift<24, false>(h_cur, h_prev, mod_cur, mod_prev, step_dev, step_host, rows, d, eps, parts,
-                                           done, d_result, s, &grid)));
+    ACID_TRY(run(integral_constant<int, 6>{}, integral_constant<int, 4>{}));
   if (done == nullptr) {
     launch_pdl(drift_final_kernel, 1, kThreads, 0, s, parts, grid, d_result, rel_out, sums_out);
     ACID_CHECK_LAUNCH();
