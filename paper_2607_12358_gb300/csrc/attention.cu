@@ -19,11 +19,10 @@
 //               in TMEM only when the running max grows by more than 2^8 (the
 //               final division by the sum makes the result independent of
 //               when rescaling happens).
-// attn_tc_kernel runs one item per CTA (long key ranges: self and joint
-// attention).  attn_persist_kernel runs items of a few key tiles (cross
-// attention over a short text) on persistent CTAs: the next item's Q loads
-// and first S MMAs overlap the current item's last softmax, and the output
-// leaves through shared memory and TMA stores.
+// attn_tc_kernel runs one item per CTA (head dim 64 over long key ranges, and
+// the split last wave).  attn_persist_kernel runs the items on persistent
+// CTAs: the next item's Q loads and first S MMAs overlap the current item's
+// last softmax, and the output leaves through shared memory and TMA stores.
 // fp32 path: one warp per query row, exact expf, for the fp32 mode.
 #include <cudaTypedefs.h>
 #include <math.h>
@@ -437,7 +436,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
   }
 }
 
-// Persistent variant for items of a few key tiles.  Each CTA walks the items
+// Persistent variant.  Each CTA walks the items
 // item_base + blockIdx.x + k * gridDim.x; one counter g numbers its key-tile
 // steps across items, and every per-step barrier phase and ring slot follows
 // it.  Q_t of the next item is loaded once the current item's last S_t MMA
@@ -706,7 +705,7 @@ int num_sms_attn() {
   return n;
 }
 
-// Items with at most this many key tiles run on persistent CTAs.
+// Key ranges of at most this many tiles are short: no split of a last wave.
 constexpr int kPersistMaxKeyTiles = 8;
 
 template <int D>
@@ -740,19 +739,24 @@ acid_status launch_attn_tc(const AttnArgs& x, cudaStream_t s) {
   a.part_ml = nullptr;
   const int items = a.nqp * x.heads;
   const int nkv_all = (int)((x.nk + C::BKV - 1) / C::BKV);
-  // Long key ranges: items fill whole waves of CTAS_PER_SM CTAs per SM; the
-  // items of a last, partial wave are split along the key range so that they
-  // fill one wave together, and their partial results are merged.  Short key
-  // ranges: persistent CTAs take all items, and the few CTAs that take one
-  // item more cost less than a split wave's start-up and merge (measured:
-  // 109 against 121 us for 32760 x 512 keys).
+  // Head dim 128, and short key ranges at head dim 64, run on persistent CTAs
+  // (measured at head dim 128, us, persistent / one item per CTA: 4846 tokens, 24
+  // heads 179 / 188; 7800, 12 heads 248 / 254; 1100, 12 heads 18.5 / 22.2; head
+  // dim 64 at 17776 tokens, 30 heads 2326 / 2154).  Long key ranges: items fill
+  // whole waves of CTAS_PER_SM CTAs per SM; the items of a last, partial wave
+  // are split along the key range so that they fill one wave together, and
+  // their partial results are merged.  Short key ranges: the persistent CTAs
+  // take all items, and the few CTAs that take one item more cost less than a
+  // split wave's start-up and merge (measured: 109 against 121 us for
+  // 32760 x 512 keys).
   const int slots = num_sms_attn() * C::CTAS_PER_SM;
   const int full = (items / slots) * slots, tail = items - full;
   int splits = tail > 0 ? std::min(std::min(kAttnPartCtas, slots) / tail, nkv_all) : 1;
   const size_t part_need = (size_t)tail * splits * kBQ * (D + 2) * sizeof(float);
-  const bool persist = nkv_all <= kPersistMaxKeyTiles;
+  const bool short_keys = nkv_all <= kPersistMaxKeyTiles;
+  const bool persist = D == 128 || short_keys;
   const bool split_tail =
-      !persist && full > 0 && tail > 0 && splits >= 2 && x.part != nullptr && x.part_bytes >= part_need;
+      !short_keys && full > 0 && tail > 0 && splits >= 2 && x.part != nullptr && x.part_bytes >= part_need;
   ProfScope prof(PROF_ATTENTION, 4.0 * (double)x.nq * (double)x.nk * D * x.heads, s);
   const int main_items = split_tail ? full : items;
   if (persist) {
