@@ -12,6 +12,7 @@
 
 namespace acid {
 
+unsigned int take_device_error_elementwise();
 unsigned int take_device_error_gemm();
 unsigned int take_device_error_attention();
 BoundsRecord take_bounds_elementwise();
@@ -204,7 +205,8 @@ extern "C" acid_status acid_selftest_wait_timeout(int64_t budget_cycles, acid_st
 extern "C" acid_status acid_check_device_error(void) {
   clear_error();
   ACID_CUDA(cudaDeviceSynchronize());
-  const unsigned int flag = take_device_error_gemm() | take_device_error_attention() | take_device_error_capi();
+  const unsigned int flag = take_device_error_elementwise() | take_device_error_gemm() |
+                            take_device_error_attention() | take_device_error_capi();
   if (flag) {
     set_error("a bounded device-side wait timed out");
     return ACID_ERR_TIMEOUT;

@@ -1089,6 +1089,7 @@ int grid_for(int64_t work, int per_block = kThreads, int cap = 152 * 16) {
 
 }  // namespace
 
+ACID_DEVICE_FLAG_READER(take_device_error_elementwise)
 ACID_BOUNDS_READER(take_bounds_elementwise)
 
 // =========================================================================
