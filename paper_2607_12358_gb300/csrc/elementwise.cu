@@ -234,8 +234,8 @@ __global__ void add_mixed8_kernel(const TA* __restrict__ a, const TB* __restrict
     io<TO>::st(out + i, READ_B ? io<TA>::ld(a + i) + bs * io<TB>::ld(b + i) : io<TA>::ld(a + i));
 }
 
-// 1D bulk copies between global and shared memory (16-byte aligned, sizes
-// multiples of 16).
+// 1D bulk copies from global to shared memory (16-byte aligned, sizes multiples
+// of 16).
 __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                    smem_u32(dst)),
@@ -258,42 +258,20 @@ __device__ __forceinline__ uint64_t l2_policy_evict_first() {
   return p;
 }
 
-__device__ __forceinline__ void bulk_store(void* dst, const void* src, uint32_t bytes) {
-  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(reinterpret_cast<uint64_t>(dst)),
-               "r"(smem_u32(src)), "r"(bytes)
-               : "memory");
-}
-
 // ---------------------------------------------------------------- LayerNorm
-// Both kernels keep a row in one warp's registers and run the two-pass
-// statistics and the modulation on packed fp32 pairs, unpacked once and
-// centred in place.
-template <typename T> struct RowVec;  // 16 bytes of a row: kN values as packed fp32 pairs
-template <> struct RowVec<__nv_bfloat16> {
-  static constexpr int kN = 8;
-  static __device__ __forceinline__ void ld(const __nv_bfloat16* p, uint64_t* v) {
-    const uint4 u = *reinterpret_cast<const uint4*>(p);
-    v[0] = f2_pack(bf16_lo(u.x), bf16_hi(u.x));
-    v[1] = f2_pack(bf16_lo(u.y), bf16_hi(u.y));
-    v[2] = f2_pack(bf16_lo(u.z), bf16_hi(u.z));
-    v[3] = f2_pack(bf16_lo(u.w), bf16_hi(u.w));
-  }
-};
-template <> struct RowVec<float> {
-  static constexpr int kN = 4;
-  static __device__ __forceinline__ void ld(const float* p, uint64_t* v) {
-    const float4 u = *reinterpret_cast<const float4*>(p);
-    v[0] = f2_pack(u.x, u.y);
-    v[1] = f2_pack(u.z, u.w);
-  }
-};
+// Both kernels keep a row in registers and run the two-pass statistics and the
+// modulation on packed fp32 pairs, unpacked once and centred in place.
 // four values of a row
 __device__ __forceinline__ void load_quad(const __nv_bfloat16* p, uint64_t* v) {
   const uint2 u = *reinterpret_cast<const uint2*>(p);
   v[0] = f2_pack(bf16_lo(u.x), bf16_hi(u.x));
   v[1] = f2_pack(bf16_lo(u.y), bf16_hi(u.y));
 }
-__device__ __forceinline__ void load_quad(const float* p, uint64_t* v) { RowVec<float>::ld(p, v); }
+__device__ __forceinline__ void load_quad(const float* p, uint64_t* v) {
+  const float4 u = *reinterpret_cast<const float4*>(p);
+  v[0] = f2_pack(u.x, u.y);
+  v[1] = f2_pack(u.z, u.w);
+}
 // a pair rounded to T
 template <typename T>
 __device__ __forceinline__ uint64_t round_to(uint64_t v) {
@@ -306,59 +284,42 @@ __device__ __forceinline__ uint64_t round_to(uint64_t v) {
     return v;
   }
 }
-template <int N>  // N values, N / 2 pairs
-__device__ __forceinline__ void store_pairs(__nv_bfloat16* p, const uint64_t* v) {
-  uint32_t w[N / 2];
-#pragma unroll
-  for (int k = 0; k < N / 2; ++k) {
-    float a, b;
-    f2_unpack(v[k], a, b);
-    w[k] = pack_bf16(a, b);
-  }
-  if constexpr (N == 8)
-    *reinterpret_cast<uint4*>(p) = make_uint4(w[0], w[1], w[2], w[3]);
-  else
-    *reinterpret_cast<uint2*>(p) = make_uint2(w[0], w[1]);
+__device__ __forceinline__ void store_quad(__nv_bfloat16* p, const uint64_t* v) {
+  float a, b, c, d;
+  f2_unpack(v[0], a, b);
+  f2_unpack(v[1], c, d);
+  *reinterpret_cast<uint2*>(p) = make_uint2(pack_bf16(a, b), pack_bf16(c, d));
 }
-template <int N>
-__device__ __forceinline__ void store_pairs(float* p, const uint64_t* v) {
-#pragma unroll
-  for (int k = 0; k < N / 2; k += 2) {
-    float a, b, c, d;
-    f2_unpack(v[k], a, b);
-    f2_unpack(v[k + 1], c, d);
-    *reinterpret_cast<float4*>(p + 2 * k) = make_float4(a, b, c, d);
-  }
+__device__ __forceinline__ void store_quad(float* p, const uint64_t* v) {
+  float a, b, c, d;
+  f2_unpack(v[0], a, b);
+  f2_unpack(v[1], c, d);
+  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
 }
 
-// v[NV][N / 2] holds a lane's values (columns (i * 32 + lane) * N ..), zeros
+// v holds a lane's quads (columns (i * 32 + lane) * 4 ..) of a warp's row, zeros
 // past d: centres them in place and returns 1 / sqrt(var + eps).
-template <int NV, int N, bool FULL = false>
-__device__ __forceinline__ float row_center(uint64_t (&v)[NV][N / 2], int lane, int d, float eps) {
-  uint64_t s[N / 2] = {};
+template <int NV, bool FULL>
+__device__ __forceinline__ float row_center(uint64_t (&v)[NV][2], int lane, int d, float eps) {
+  uint64_t s[2] = {}, t[2] = {};
 #pragma unroll
   for (int i = 0; i < NV; ++i)
 #pragma unroll
-    for (int q = 0; q < N / 2; ++q) s[q] = f2_add(s[q], v[i][q]);
-#pragma unroll
-  for (int q = 1; q < N / 2; ++q) s[0] = f2_add(s[0], s[q]);
+    for (int q = 0; q < 2; ++q) s[q] = f2_add(s[q], v[i][q]);
   float a, b;
-  f2_unpack(s[0], a, b);
+  f2_unpack(f2_add(s[0], s[1]), a, b);
   const float mean = warp_sum_f(a + b) / d;
   const uint64_t nm = f2_pack(-mean, -mean);
-  uint64_t t[N / 2] = {};
 #pragma unroll
   for (int i = 0; i < NV; ++i)
-    if (FULL || (i * 32 + lane) * N < d) {
+    if (FULL || (i * 32 + lane) * 4 < d) {
 #pragma unroll
-      for (int q = 0; q < N / 2; ++q) {
+      for (int q = 0; q < 2; ++q) {
         v[i][q] = f2_add(v[i][q], nm);
         t[q] = f2_fma(v[i][q], v[i][q], t[q]);
       }
     }
-#pragma unroll
-  for (int q = 1; q < N / 2; ++q) t[0] = f2_add(t[0], t[q]);
-  f2_unpack(t[0], a, b);
+  f2_unpack(f2_add(t[0], t[1]), a, b);
   return rsqrtf(warp_sum_f(a + b) / d + eps);
 }
 
@@ -380,7 +341,7 @@ struct LnArgs {
   float eps;
 };
 
-// Few rows: one warp per row, straight from and to global memory.  A lane
+// Rows of up to 512 columns: one warp per row, straight from and to global memory.  A lane
 // holds four consecutive columns in every 128, so that its loads and stores
 // of bf16 (8 bytes) and fp32 (16 bytes) rows and vectors are contiguous over the
 // warp.
@@ -390,7 +351,7 @@ constexpr int kLnThreads = 128;
 // TeaCache step is applied (kLnReuse) or stored (kLnResid) in the same pass:
 // apart, the state was written and read again, or read a second time.
 template <typename Tin, typename Tout, int NV, bool FULL, int MODE>
-__global__ void __launch_bounds__(kLnThreads, NV <= 12 ? 5 : 4) ln_mod_rows_kernel(LnArgs a) {
+__global__ void __launch_bounds__(kLnThreads, 5) ln_mod_rows_kernel(LnArgs a) {
   pdl_wait();
   const int64_t row = ((int64_t)blockIdx.x * kLnThreads + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31, d = a.d;
@@ -420,7 +381,7 @@ __global__ void __launch_bounds__(kLnThreads, NV <= 12 ? 5 : 4) ln_mod_rows_kern
       *reinterpret_cast<float4*>(a.r + row * d + c) = make_float4(x0 - h.x, x1 - h.y, x2 - h.z, x3 - h.w);
     }
   }
-  const float rstd = row_center<NV, 4, FULL>(v, lane, d, a.eps);
+  const float rstd = row_center<NV, FULL>(v, lane, d, a.eps);
   const uint64_t rs = f2_pack(rstd, rstd);
   const bool text = a.vecs == 2 && row < a.split;
   const float *sc = text ? a.sct : a.scv, *sh = text ? a.sht : a.shv;
@@ -435,124 +396,155 @@ __global__ void __launch_bounds__(kLnThreads, NV <= 12 ? 5 : 4) ln_mod_rows_kern
       v[i][0] = f2_fma(v[i][0], f2_pack(1.f + p.x, 1.f + p.y), f2_pack(q.x, q.y));
       v[i][1] = f2_fma(v[i][1], f2_pack(1.f + p.z, 1.f + p.w), f2_pack(q.z, q.w));
     }
-    if (ACID_IN_BOUNDS(kSiteLayerNorm, row * d + c + 3, a.rows * d)) store_pairs<4>(yr + c, v[i]);
+    if (ACID_IN_BOUNDS(kSiteLayerNorm, row * d + c + 3, a.rows * d)) store_quad(yr + c, v[i]);
   }
 }
 
-// Many rows: persistent warps.  Lane 0 streams the warp's next rows into a
-// two-stage shared-memory ring with bulk copies; a row is read once into
-// registers (16 bytes a lane), its stage is refilled at once, and the result
-// leaves through shared memory and a bulk store.  The modulation vectors
-// (1 + scale and shift of each stream) are staged once per CTA, for bf16 rows
-// as two arrays of alternating 16-byte units so that a warp's reads are
-// contiguous.
-constexpr int kLnStages = 2;
-// From this many rows on the persistent kernel is used: five rows a warp
-// (152 CTAs of 16 warps) pay for its start.
-constexpr int64_t kLnBulkRows = 152 * 16 * 5;
+// Rows of more than 512 columns: persistent CTAs of four warps, a row at a
+// time.  One thread streams the CTA's next rows into a shared-memory ring with
+// bulk copies; a lane keeps NQ quads of the row and of its modulation (1 + scale,
+// shift) in registers, so that the vectors are read once per CTA and stream and
+// not once per row, and a row's serial chain (read, two reductions, store) is
+// a fraction of what one warp makes of it.  HBM bounds large row counts, the
+// rows' chains small ones.  Measured (us, one warp a row -> this): 4846 x 3072
+// bf16 11.0 -> 9.1, 9000 x 3072 bf16 26.6 -> 17.0, 17776 x 1920 bf16 25.4 -> 21.2,
+// 50000 x 3072 fp32 to bf16 158 -> 142.  A reused step's pass over 7800 x 1536:
+// 20.5 -> 15.4.
+constexpr int kLnMaxStages = 4;
+// CTAs per SM: 16 to 18 warps, as many as the registers of a lane's quads and
+// their modulation leave room for.
+template <int WPR>
+constexpr int kLnCtas = WPR == 3 ? 6 : 16 / WPR;
 
-// Shared memory of one warp: ring, output row, barriers.
-template <typename Tin, typename Tout>
-__host__ __device__ constexpr size_t ln_warp_bytes(int d) {
-  return (size_t)d * (kLnStages * sizeof(Tin) + sizeof(Tout)) + kLnStages * sizeof(uint64_t);
-}
-// Warps per CTA: as many as the values held per lane leave registers for.
-template <typename Tin, int NV>
-constexpr int kLnMaxWarps = NV * RowVec<Tin>::kN <= 64 ? 16 : 12;
-
-template <typename Tin, typename Tout, int NV, bool FULL>
-__global__ void __launch_bounds__(32 * kLnMaxWarps<Tin, NV>, 1) ln_mod_bulk_kernel(LnArgs a) {
-  pdl_wait();
-  constexpr int N = RowVec<Tin>::kN;
+template <typename Tin, typename Tout, int WPR, int NQ, bool FULL, int MODE>
+__global__ void __launch_bounds__(32 * WPR, kLnCtas<WPR>) ln_mod_team_kernel(LnArgs a, int stages) {
   extern __shared__ __align__(128) uint8_t lsm[];
-  const int nwarps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int d = a.d;
-  float* mod = reinterpret_cast<float*>(lsm);  // [stream][1 + scale | shift][d]
-  uint8_t* rings = lsm + (size_t)a.vecs * 8 * d;
-  Tin* ring = reinterpret_cast<Tin*>(rings) + (size_t)warp * kLnStages * d;
-  Tout* orow = reinterpret_cast<Tout*>(rings + (size_t)nwarps * kLnStages * d * sizeof(Tin)) + (size_t)warp * d;
-  uint64_t* full = reinterpret_cast<uint64_t*>(rings + (size_t)nwarps * d * (kLnStages * sizeof(Tin) + sizeof(Tout))) +
-                   warp * kLnStages;
-  const Tin* x = static_cast<const Tin*>(a.x);
-  Tout* y = static_cast<Tout*>(a.y);
-  const int64_t gw = (int64_t)blockIdx.x * nwarps + warp, nw = (int64_t)gridDim.x * nwarps;
-  const int64_t mine = gw < a.rows ? (a.rows - 1 - gw) / nw + 1 : 0;
-  const uint32_t row_bytes = (uint32_t)(d * sizeof(Tin));
-  auto issue = [&](int64_t k) {
-    const int st = (int)(k % kLnStages);
-    int64_t row = gw + k * nw;
+  constexpr int kTeam = 32 * WPR;
+  __shared__ __align__(16) float red[2][4];
+  __shared__ uint64_t full[kLnMaxStages];
+  __shared__ int gave_up;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, d = a.d;
+  using T0 = std::conditional_t<MODE == kLnReuse, float, Tin>;
+  const T0* src0 = static_cast<const T0*>(MODE == kLnReuse ? (const void*)a.h : a.x);
+  const float* src1 = MODE == kLnReuse ? a.r : a.h;
+  const uint32_t bytes0 = d * (uint32_t)sizeof(T0), bytes1 = MODE == kLnPlain ? 0 : d * 4u;
+  const int64_t mine = blockIdx.x < a.rows ? (a.rows - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+  auto issue = [&](int64_t k, int st) {
+    int64_t row = blockIdx.x + k * gridDim.x;
     if (!ACID_IN_BOUNDS(kSiteLayerNorm, row, a.rows)) row = 0;  // (debug builds) read row 0 instead
-    mbar_expect_tx(&full[st], row_bytes);
-    bulk_load(ring + (size_t)st * d, x + row * d, row_bytes, &full[st]);
+    uint8_t* dst = lsm + (size_t)st * (bytes0 + bytes1);
+    mbar_expect_tx(&full[st], bytes0 + bytes1);
+    bulk_load(dst, src0 + row * d, bytes0, &full[st]);
+    if constexpr (MODE != kLnPlain) bulk_load(dst + bytes0, src1 + row * d, bytes1, &full[st]);
   };
-  if (lane == 0) {
-    for (int i = 0; i < kLnStages; ++i) mbar_init(&full[i], 1);
+  if (tid < 8) red[tid >> 2][tid & 3] = 0.f;
+  if (tid == 0) {
+    gave_up = 0;
+    for (int i = 0; i < stages; ++i) mbar_init(&full[i], 1);
     mbar_fence_init();
-    for (int64_t k = 0; k < mine && k < kLnStages; ++k) issue(k);
   }
-  for (int i = threadIdx.x; i < a.vecs * (d / 4); i += blockDim.x) {
-    const int t = i / (d / 4), u = i % (d / 4);
-    const float4 sc = reinterpret_cast<const float4*>(t ? a.sct : a.scv)[u];
-    const float4 sh = reinterpret_cast<const float4*>(t ? a.sht : a.shv)[u];
-    const int at = N == 8 ? (u & 1) * (d / 2) + (u >> 1) * 4 : u * 4;
-    float* m = mod + (size_t)t * 2 * d;
-    *reinterpret_cast<float4*>(m + at) = make_float4(1.f + sc.x, 1.f + sc.y, 1.f + sc.z, 1.f + sc.w);
-    *reinterpret_cast<float4*>(m + d + at) = sh;
-  }
-  __syncthreads();
-  int64_t k = 0;
-  for (; k < mine; ++k) {
-    const int st = (int)(k % kLnStages);
-    if (!__all_sync(0xffffffffu, mbar_wait(&full[st], (uint32_t)((k / kLnStages) & 1)))) break;
-    const int64_t row = gw + k * nw;
-    uint64_t v[NV][N / 2];
+  pdl_wait();
+  if (tid == 0)
+    for (int k = 0; k < mine && k < stages; ++k) issue(k, k);
+  uint64_t sc[NQ][2], sh[NQ][2];
+  auto load_mod = [&](const float* scp, const float* shp) {
 #pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const int c = (i * 32 + lane) * N;
-      if constexpr (!FULL) {
-#pragma unroll
-        for (int q = 0; q < N / 2; ++q) v[i][q] = 0;
-      }
-      if (FULL || c < d) RowVec<Tin>::ld(ring + (size_t)st * d + c, v[i]);
-    }
-    __syncwarp();
-    if (lane == 0 && k + kLnStages < mine) issue(k + kLnStages);  // every lane holds its values
-    const float rstd = row_center<NV, N, FULL>(v, lane, d, a.eps);
-    const uint64_t rs = f2_pack(rstd, rstd);
-    if (lane == 0) bulk_wait_group_read<0>();  // the previous row has left the output buffer
-    __syncwarp();
-    const float* m = mod + (a.vecs == 2 && row < a.split ? 2 * d : 0);
-#pragma unroll
-    for (int i = 0; i < NV; ++i) {
-      const int c = (i * 32 + lane) * N;
+    for (int i = 0; i < NQ; ++i) {
+      const int c = (i * kTeam + tid) * 4;
       if (!FULL && c >= d) continue;
-#pragma unroll
-      for (int q = 0; q < N / 2; ++q) v[i][q] = f2_mul(v[i][q], rs);
-      if (a.vecs) {
-        const int at = N == 8 ? c / 2 : c;
-#pragma unroll
-        for (int h = 0; h < N / 4; ++h) {
-          const float4 p = *reinterpret_cast<const float4*>(m + at + h * (d / 2));
-          const float4 q = *reinterpret_cast<const float4*>(m + d + at + h * (d / 2));
-          v[i][2 * h] = f2_fma(v[i][2 * h], f2_pack(p.x, p.y), f2_pack(q.x, q.y));
-          v[i][2 * h + 1] = f2_fma(v[i][2 * h + 1], f2_pack(p.z, p.w), f2_pack(q.z, q.w));
-        }
-      }
-      store_pairs<N>(orow + c, v[i]);
+      const float4 p = *reinterpret_cast<const float4*>(scp + c), q = *reinterpret_cast<const float4*>(shp + c);
+      sc[i][0] = f2_pack(1.f + p.x, 1.f + p.y);
+      sc[i][1] = f2_pack(1.f + p.z, 1.f + p.w);
+      sh[i][0] = f2_pack(q.x, q.y);
+      sh[i][1] = f2_pack(q.z, q.w);
     }
-    fence_proxy_async_smem();
-    __syncwarp();
-    if (lane == 0) {
-      bulk_store(y + row * d, orow, (uint32_t)(d * sizeof(Tout)));
-      bulk_commit_group();
+  };
+  bool text = a.vecs == 2 && blockIdx.x < a.split;
+  if (a.vecs) load_mod(text ? a.sct : a.scv, text ? a.sht : a.shv);
+  __syncthreads();
+  // the sum over the CTA of each warp's share
+  auto team_sum = [&](uint64_t s, float* r) {
+    float x, y;
+    f2_unpack(s, x, y);
+    x = warp_sum_f(x + y);
+    if (lane == 0) r[warp] = x;
+    __syncthreads();
+    const float4 t = *reinterpret_cast<const float4*>(r);
+    return (t.x + t.y) + (t.z + t.w);
+  };
+  int st = 0;
+  uint32_t phase = 0;
+  auto next = [&] {
+    if (++st == stages) {
+      st = 0;
+      phase ^= 1;
+    }
+  };
+  int64_t k = 0, row = blockIdx.x;
+  for (; k < mine; ++k, row += gridDim.x, next()) {
+    if (!mbar_wait(&full[st], phase)) gave_up = 1;
+    const uint8_t* buf = lsm + (size_t)st * (bytes0 + bytes1);
+    const T0* r0 = reinterpret_cast<const T0*>(buf);
+    const float* r1 = reinterpret_cast<const float*>(buf + bytes0);
+    uint64_t v[NQ][2], s = 0, t = 0;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const int c = (i * kTeam + tid) * 4;
+      v[i][0] = v[i][1] = 0;
+      if (!FULL && c >= d) continue;
+      load_quad(r0 + c, v[i]);
+      if constexpr (MODE == kLnReuse) {
+        uint64_t r[2];
+        load_quad(r1 + c, r);
+        v[i][0] = round_to<Tin>(f2_add(v[i][0], r[0]));
+        v[i][1] = round_to<Tin>(f2_add(v[i][1], r[1]));
+      }
+      if constexpr (MODE == kLnResid) {
+        const float4 h = *reinterpret_cast<const float4*>(r1 + c);
+        float x0, x1, x2, x3;
+        f2_unpack(v[i][0], x0, x1);
+        f2_unpack(v[i][1], x2, x3);
+        if (ACID_IN_BOUNDS(kSiteLayerNorm, row * d + c + 3, a.rows * d))
+          *reinterpret_cast<float4*>(a.r + row * d + c) = make_float4(x0 - h.x, x1 - h.y, x2 - h.z, x3 - h.w);
+      }
+      s = f2_add(s, f2_add(v[i][0], v[i][1]));
+    }
+    const float mean = team_sum(s, red[0]) / d;
+    if (gave_up) break;  // a wait ran out: the CTA leaves together
+    if (tid == 0 && k + stages < mine) issue(k + stages, st);  // every lane holds its values
+    const uint64_t nm = f2_pack(-mean, -mean);
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      if (!FULL && (i * kTeam + tid) * 4 >= d) continue;
+      v[i][0] = f2_add(v[i][0], nm);
+      v[i][1] = f2_add(v[i][1], nm);
+      t = f2_fma(v[i][0], v[i][0], t);
+      t = f2_fma(v[i][1], v[i][1], t);
+    }
+    // a warp writes red[0] of the next row behind this barrier, red[1] behind the next row's first
+    const float rstd = rsqrtf(team_sum(t, red[1]) / d + a.eps);
+    const uint64_t rs = f2_pack(rstd, rstd);
+    if (text && row >= a.split) {
+      text = false;
+      load_mod(a.scv, a.shv);
+    }
+    Tout* yr = static_cast<Tout*>(a.y) + row * d;
+#pragma unroll
+    for (int i = 0; i < NQ; ++i) {
+      const int c = (i * kTeam + tid) * 4;
+      if (!FULL && c >= d) continue;
+      v[i][0] = f2_mul(v[i][0], rs);
+      v[i][1] = f2_mul(v[i][1], rs);
+      if (a.vecs) {
+        v[i][0] = f2_fma(v[i][0], sc[i][0], sh[i][0]);
+        v[i][1] = f2_fma(v[i][1], sc[i][1], sh[i][1]);
+      }
+      if (ACID_IN_BOUNDS(kSiteLayerNorm, row * d + c + 3, a.rows * d)) store_quad(yr + c, v[i]);
     }
   }
   // after a wait ran out: the copies already issued land before the CTA exits
-  if (lane == 0) {
-    for (int64_t j = k; j < mine && j < k + kLnStages; ++j)
-      mbar_wait(&full[j % kLnStages], (uint32_t)((j / kLnStages) & 1));
-    bulk_wait_group<0>();
-  }
+  if (tid == 0)
+    for (int64_t j = k; j < mine && j < k + stages; ++j, next()) mbar_wait(&full[st], phase);
 }
 
 // ------------------------------------------- TEMNI drift from two H_in rows
@@ -1181,50 +1173,40 @@ acid_status launch_ln_rows(const LnArgs& a, cudaStream_t s) {
   return ACID_OK;
 }
 
-template <typename Tin, typename Tout, int MODE>
-acid_status ln_rows_types(const LnArgs& a, cudaStream_t s) {
-  if (a.d <= 128 * 4) return launch_ln_rows<Tin, Tout, 4, MODE>(a, s);
-  if (a.d <= 128 * 12) return launch_ln_rows<Tin, Tout, 12, MODE>(a, s);
-  if (a.d <= 128 * 16) return launch_ln_rows<Tin, Tout, 16, MODE>(a, s);
-  return launch_ln_rows<Tin, Tout, 24, MODE>(a, s);
-}
-
-template <typename Tin, typename Tout, int NV, bool FULL>
-acid_status launch_ln_bulk_full(const LnArgs& a, cudaStream_t s) {
-  constexpr size_t kSmemMax = 226 * 1024;
+template <typename Tin, typename Tout, int WPR, int NQ, bool FULL, int MODE>
+acid_status launch_ln_team(const LnArgs& a, cudaStream_t s) {
+  constexpr size_t kSmemMax = 216 * 1024 / kLnCtas<WPR>;
   static bool attr_done = false;
   if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(ln_mod_bulk_kernel<Tin, Tout, NV, FULL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)kSmemMax));
+    ACID_CUDA(cudaFuncSetAttribute(ln_mod_team_kernel<Tin, Tout, WPR, NQ, FULL, MODE>,
+                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     attr_done = true;
   }
-  const size_t per_warp = ln_warp_bytes<Tin, Tout>(a.d), mod = (size_t)a.vecs * 8 * a.d;
-  const int warps = (int)std::min<size_t>(kLnMaxWarps<Tin, NV>, (kSmemMax - mod) / per_warp);
-  const int grid = (int)std::min<int64_t>(num_sms_elem(), (a.rows + warps - 1) / warps);
-  launch_pdl(ln_mod_bulk_kernel<Tin, Tout, NV, FULL>, grid, 32 * warps, mod + warps * per_warp, s, a);
+  const size_t row = (size_t)a.d * (MODE == kLnPlain ? sizeof(Tin) : MODE == kLnReuse ? 8 : sizeof(Tin) + 4);
+  // Two rows ahead keep HBM busy and its reads in order (bf16, 50000 x 3072: 93 us,
+  // 109 with four); rows that largely stay in L2 are latency's, which four cover
+  // (16000 x 1920: 19.5 us, 21.4 with two; the line lies between 154 and 200 MB).
+  const double bytes = (double)a.rows * a.d * (sizeof(Tin) + sizeof(Tout));
+  const int stages = row <= 6144 && bytes < 160e6 ? kLnMaxStages : 2;
+  const unsigned grid = (unsigned)std::min<int64_t>(a.rows, (int64_t)num_sms_elem() * kLnCtas<WPR>);
+  launch_pdl(ln_mod_team_kernel<Tin, Tout, WPR, NQ, FULL, MODE>, grid, 32 * WPR, stages * row, s, a, stages);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
-template <typename Tin, typename Tout, int NV>
-acid_status launch_ln_bulk(const LnArgs& a, cudaStream_t s) {
-  return a.d == 32 * RowVec<Tin>::kN * NV ? launch_ln_bulk_full<Tin, Tout, NV, true>(a, s)
-                                         : launch_ln_bulk_full<Tin, Tout, NV, false>(a, s);
+template <typename Tin, typename Tout, int WPR, int NQ, int MODE>
+acid_status launch_ln_team(const LnArgs& a, cudaStream_t s) {
+  return a.d == 128 * WPR * NQ ? launch_ln_team<Tin, Tout, WPR, NQ, true, MODE>(a, s)
+                               : launch_ln_team<Tin, Tout, WPR, NQ, false, MODE>(a, s);
 }
 
-// Vectors per lane sized to the row.
-template <typename Tin, typename Tout>
+// Warps and quads per lane sized to the row.
+template <typename Tin, typename Tout, int MODE>
 acid_status ln_mod_types(const LnArgs& a, cudaStream_t s) {
-  // Measured (us, modulated, bf16 out): 17776 x 1920 bf16 in 28.5 bulk, 41.0 one
-  // warp per row; fp32 in 37.1, 47.3; 67576 x 3072 bf16 144, 180; 4846 x 3072 fp32
-  // 20.5, 16.4; 7800 x 1536 bf16 12.3, 11.5; 20000 x 256 bf16 12.3, 8.7.
-  if (a.rows < kLnBulkRows || a.d <= 512) {
-    return ln_rows_types<Tin, Tout, kLnPlain>(a, s);
-  }
-  constexpr int U = RowVec<Tin>::kN == 8 ? 1 : 2;  // 16-byte vectors per 8 columns
-  if (a.d <= 1536) return launch_ln_bulk<Tin, Tout, 6 * U>(a, s);
-  if (a.d <= 2048) return launch_ln_bulk<Tin, Tout, 8 * U>(a, s);
-  return launch_ln_bulk<Tin, Tout, 12 * U>(a, s);
+  if (a.d <= 512) return launch_ln_rows<Tin, Tout, 4, MODE>(a, s);
+  if (a.d <= 1536) return launch_ln_team<Tin, Tout, 2, 6, MODE>(a, s);
+  if (a.d <= 1920) return launch_ln_team<Tin, Tout, 3, 5, MODE>(a, s);
+  return launch_ln_team<Tin, Tout, 4, 6, MODE>(a, s);
 }
 
 acid_status ln_mod(int in_dtype, const void* x, int out_dtype, void* y, int64_t rows, int d, const float* shv,
@@ -1234,10 +1216,10 @@ acid_status ln_mod(int in_dtype, const void* x, int out_dtype, void* y, int64_t 
   if (rows == 0) return ACID_OK;
   const bool two = scv != nullptr && sht != nullptr && split > 0 && (sht != shv || sct != scv);
   const LnArgs a{x, y, nullptr, nullptr, rows, split, d, scv == nullptr ? 0 : two ? 2 : 1, shv, scv, sht, sct, eps};
-  if (in_dtype == ACID_BF16 && out_dtype == ACID_BF16) return ln_mod_types<H, H>(a, s);
-  if (in_dtype == ACID_BF16) return ln_mod_types<H, float>(a, s);
-  if (out_dtype == ACID_BF16) return ln_mod_types<float, H>(a, s);
-  return ln_mod_types<float, float>(a, s);
+  if (in_dtype == ACID_BF16 && out_dtype == ACID_BF16) return ln_mod_types<H, H, kLnPlain>(a, s);
+  if (in_dtype == ACID_BF16) return ln_mod_types<H, float, kLnPlain>(a, s);
+  if (out_dtype == ACID_BF16) return ln_mod_types<float, H, kLnPlain>(a, s);
+  return ln_mod_types<float, float, kLnPlain>(a, s);
 }
 
 acid_status ln_mod_cached(int dtype, bool reuse, const void* x, const float* h, float* r, void* y, int64_t rows, int d,
@@ -1246,8 +1228,8 @@ acid_status ln_mod_cached(int dtype, bool reuse, const void* x, const float* h, 
   ACID_REQUIRE(d % 8 == 0 && d <= 3072, ACID_ERR_UNSUPPORTED, "ln_mod: d must be a multiple of 8, <= 3072");
   if (rows == 0) return ACID_OK;
   const LnArgs a{x, y, h, r, rows, 0, d, 1, sh, sc, nullptr, nullptr, eps};
-  if (dtype == ACID_BF16) return reuse ? ln_rows_types<H, H, kLnReuse>(a, s) : ln_rows_types<H, H, kLnResid>(a, s);
-  return reuse ? ln_rows_types<float, float, kLnReuse>(a, s) : ln_rows_types<float, float, kLnResid>(a, s);
+  if (dtype == ACID_BF16) return reuse ? ln_mod_types<H, H, kLnReuse>(a, s) : ln_mod_types<H, H, kLnResid>(a, s);
+  return reuse ? ln_mod_types<float, float, kLnReuse>(a, s) : ln_mod_types<float, float, kLnResid>(a, s);
 }
 
 template <int NV4, int WPR>

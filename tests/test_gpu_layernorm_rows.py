@@ -1,7 +1,8 @@
-"""GPU parity of the two LayerNorm kernels (one warp per row; persistent warps
-on bulk copies) on both sides of the row count between them, with rows that
-do not fill the last lanes, ragged last rounds and every pair of types, and
-of the joint blocks' split between text and video modulation."""
+"""GPU parity of the two LayerNorm kernels (one warp per row up to 512 columns;
+persistent teams of two, three or four warps on bulk copies) on both sides of
+the widths between them, with rows that do not fill the last lanes, ragged
+last rounds, rings of two and four rows and every pair of types, and of the
+joint blocks' split between text and video modulation."""
 
 import numpy as np
 import pytest
@@ -27,10 +28,12 @@ def acid():
     return a
 
 
-# 12160 rows are the first that take the persistent kernel (for rows of more
-# than 512 values); 12161 leave one warp a sixth row
+# 512, 1536 and 1920 columns are the widest of their kernel; 1216, 912 and 608
+# rows give each team of two, three and four warps one; the last two sizes lie on
+# both sides of 160 MB in bf16
 @pytest.mark.parametrize("rows,d", [(1, 8), (5, 264), (12159, 520), (12160, 520), (12161, 1536), (12300, 1544),
-                                    (12200, 2048), (12170, 3072), (12163, 512), (777, 1928), (300, 3064)])
+                                    (12200, 2048), (12170, 3072), (12163, 512), (777, 1928), (300, 3064), (1217, 1528),
+                                    (913, 1920), (4000, 1912), (609, 3072), (13020, 3072), (13024, 3072)])
 @pytest.mark.parametrize("tin,tout", [("bf16", "bf16"), ("bf16", "fp32"), ("fp32", "bf16"), ("fp32", "fp32")])
 @pytest.mark.parametrize("mod", [True, False])
 def test_layernorm_kernels(acid, rows, d, tin, tout, mod):
@@ -56,8 +59,8 @@ def test_layernorm_kernels(acid, rows, d, tin, tout, mod):
 
 @pytest.mark.parametrize("n_text,f", [(37, 3), (226, 48)])
 def test_joint_block_streams_keep_their_modulation(acid, n_text, f):
-    """A joint block of 829 rows (one warp per row) and of 12898 rows
-    (persistent warps), checked by the oracle on the rows around the split, where
+    """A joint block of 829 rows (a row a team) and of 12898 rows
+    (several), checked by the oracle on the rows around the split, where
     the text stream's modulation ends, and at both ends."""
     cfg = S.get_config("cog", d=576, heads=9, ffn=128, n_text=n_text, latent_f=f, latent_h=16, latent_w=66)
     w = S.block_weights(cfg, 0, seed=3)
