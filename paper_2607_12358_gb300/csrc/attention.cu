@@ -4,25 +4,26 @@
 // operands.
 //
 // bf16 path: a flash-attention kernel on tcgen05 tensor cores.  A work item
-// is two 128-row query tiles (a, b) of one head; its CTA streams 128-key K/V
-// tiles that both query tiles share:
-//   warp 0      TMA producer: Q_a, Q_b once, then K_j and V_j into 2-deep rings
+// is two 128-row query tiles (a, b) of one head; its CTA streams K/V tiles (128
+// keys; 64 for short ranges at head dim 64) that both query tiles share:
+//   warp 0      TMA producer: Q_a, Q_b once per item, K_j and V_j into rings
 //               (128-byte swizzle);
-//   warp 1      MMA issuer, in the order S_a(0) S_b(0) | PV_a(j) S_a(j+1)
-//               PV_b(j) S_b(j+1) | ... so that the tensor core works on one
-//               query tile while the softmax of the other runs;
-//               S_t = Q_t K_j^T lands in TMEM, P_t is written back over S_t
-//               (bf16, two per column) and O_t += P_t V_j reads P_t from TMEM
-//               and V_j from shared memory;
+//   warp 1      MMA issuer: S_t = Q_t K_j^T lands in a region of TMEM, P_t is
+//               written back over it (bf16, two per column) and O_t += P_t V_j
+//               reads P_t from TMEM and V_j from shared memory.  The tiles
+//               alternate, and each PV is followed by the S that takes its
+//               region over, so that the tensor core works on one query tile
+//               while the softmax of the other runs;
 //   warps 2-5   softmax of tile a, warps 6-9 softmax of tile b: one thread
 //               per query row keeps the running max and sum, and rescales O_t
 //               in TMEM only when the running max grows by more than 2^8 (the
 //               final division by the sum makes the result independent of
 //               when rescaling happens).
-// attn_tc_kernel runs one item per CTA (head dim 64 over long key ranges, and
-// the split last wave).  attn_persist_kernel runs the items on persistent
-// CTAs: the next item's Q loads and first S MMAs overlap the current item's
-// last softmax, and the output leaves through shared memory and TMA stores.
+// attn_persist_kernel runs whole items on persistent CTAs: the next item's Q
+// loads and first S MMAs overlap the current item's last softmax, and the
+// output leaves through shared memory and TMA stores.  attn_split_kernel runs
+// the items of a partial last wave, each split along its key range over
+// several CTAs, and attn_merge_kernel puts their parts together.
 // fp32 path: one warp per query row, exact expf, for the fp32 mode.
 #include <cudaTypedefs.h>
 #include <math.h>
@@ -43,7 +44,7 @@ namespace {
 constexpr int kTileQ = 128;  // query rows per tile (two tiles per CTA)
 constexpr int kBQ = 2 * kTileQ;
 constexpr int kAttnThreads = 320;
-constexpr float kRescaleLog2 = 8.0f;
+constexpr float kRescaleLog2 = 8.0f, kRescale = 256.0f;
 constexpr int kAttnPartCtas = kAttnSplitCtas;  // CTAs of a split tail wave (partials workspace capacity)
 
 struct AttnDev {
@@ -53,12 +54,11 @@ struct AttnDev {
   int64_t ldo;
   int o_col;
   float scale_log2;  // log2(e) / sqrt(head_dim)
-  // work item = (query-tile pair, head), numbered head-major.  attn_tc_kernel:
+  // work item = (query-tile pair, head), numbered head-major.  attn_split_kernel:
   // CTA blockIdx.x handles item item_base + blockIdx.x / splits and the
-  // split-th part of the key range; with splits > 1 it writes its
-  // unnormalised output and (max, sum) per row to part_o / part_ml instead of
-  // the final output.  attn_persist_kernel: CTA blockIdx.x handles items
-  // item_base + blockIdx.x + k * gridDim.x below item_end.
+  // split-th part of the key range, and writes its unnormalised output and
+  // (max, sum) per row to part_o / part_ml.  attn_persist_kernel: CTA blockIdx.x
+  // handles items item_base + blockIdx.x + k * gridDim.x below item_end.
   int nqp;
   int item_base, item_end;
   int splits;
@@ -66,58 +66,118 @@ struct AttnDev {
   float* part_ml;  // [CTA][256 rows][2]
 };
 
-template <int D>
+// Head dim and keys per K/V tile of a kernel.
+template <int HEAD_DIM, int KEYS>
 struct AttnCfg {
-  // Keys per K/V tile.  Head dim 128: 128-key tiles, one CTA per SM (S and O
-  // of both query tiles fill TMEM).  Head dim 64: 64-key tiles, so a CTA needs
-  // 256 TMEM columns and about 64 KB of shared memory and two CTAs share an
-  // SM, four query tiles in flight: at this head dim the exponentials, not
-  // the MMAs, set the pace and need more warps to overlap.
-  static constexpr int BKV = D <= 64 ? 64 : 128;
-  static constexpr int CTAS_PER_SM = D <= 64 ? 2 : 1;
+  static constexpr int D = HEAD_DIM, BKV = KEYS;
+  // S regions in TMEM.  Step n of a CTA (2 * key-tile step + query tile: the
+  // tiles alternate) uses region n % NB, and S(n + NB) is issued right after
+  // PV(n), which reads P(n) from it.  Head dim 128: S and O of both query tiles
+  // fill TMEM.  Head dim 64: O needs half the columns, and a third region lets
+  // the tensor cores run ahead of the softmax warps, which set the pace at this
+  // head dim: a step costs them about 630 clocks whatever its keys and 9.4 more
+  // per key (4726 tokens, 30 heads: 197.6 us in 64-key tiles on four regions,
+  // 163.1 in 96-key tiles on four, 146.6 in 128-key tiles on these three).
+  // 64-key tiles are for the shortest key ranges, where starting and ending
+  // items weighs most: 256 columns, two CTAs on an SM.
+  static constexpr int CTAS_PER_SM = BKV == 64 ? 2 : 1;
+  static constexpr int NB = D <= 64 && BKV == 128 ? 3 : 2;
+  static constexpr int KVS = NB == 3 ? 4 : 2;        // K and V ring depth
+  // Whether a tile's row max is formed before its exponentials or only where the
+  // row sum asks for it (softmax_tile).  At head dim 128 the MMAs and power set
+  // the pace and the two take the same time; two CTAs on an SM leave too few
+  // registers to keep a row until its sum is known.
+  static constexpr bool MAX_FIRST = !(D == 64 && BKV == 128);
   static constexpr int CH = D / 64;                  // 64-column chunks per row
   static constexpr int CHUNK_Q = 128 * 128;          // 128 rows x 128 bytes
   static constexpr int CHUNK_KV = BKV * 128;         // BKV rows x 128 bytes
   static constexpr int T_BYTES = CH * CHUNK_Q;       // one 128-row tile of Q
   static constexpr int KV_BYTES = CH * CHUNK_KV;     // one K or V tile
   static constexpr int OFF_Q = 0;                    // Q_a, Q_b
-  static constexpr int OFF_K = OFF_Q + 2 * T_BYTES;  // 2-deep rings
-  static constexpr int OFF_V = OFF_K + 2 * KV_BYTES;
-  static constexpr int OFF_BAR = OFF_V + 2 * KV_BYTES;
-  static constexpr int SMEM = OFF_BAR + 256 + 1024;
+  static constexpr int OFF_K = OFF_Q + 2 * T_BYTES;  // rings
+  static constexpr int OFF_V = OFF_K + KVS * KV_BYTES;
+  static constexpr int OFF_BAR = OFF_V + KVS * KV_BYTES;
+  static constexpr int BAR_BYTES = 512;
+  static constexpr int SMEM = OFF_BAR + BAR_BYTES + 1024;
   // attn_persist_kernel adds the output staging: per softmax warp two
   // 32-row x 32-column bf16 boxes (64-byte swizzle) for TMA stores
   static constexpr int STAGE_BOX = 32 * 64;
-  static constexpr int OFF_STAGE_P = OFF_V + 2 * KV_BYTES;
+  static constexpr int OFF_STAGE_P = OFF_V + KVS * KV_BYTES;
   static constexpr int OFF_BAR_P = OFF_STAGE_P + 8 * 2 * STAGE_BOX;
-  static constexpr int SMEM_P = OFF_BAR_P + 256 + 1024;
-  // TMEM columns: S_a [0,BKV), S_b [BKV,2BKV) (P_t over the first BKV/2
-  // columns of S_t), O_a [2BKV, 2BKV+D), O_b [2BKV+D, 2BKV+2D)
-  static constexpr uint32_t S_COL = 0, O_COL = 2 * BKV;
-  static constexpr uint32_t TMEM_COLS = 2 * BKV + 2 * D;
+  static constexpr int SMEM_P = OFF_BAR_P + BAR_BYTES + 1024;
+  // TMEM columns: the S regions (P over the first BKV / 2 columns of each), O_a, O_b
+  static constexpr uint32_t O_COL = NB * BKV, TMEM_COLS = O_COL + 2 * D;
+  static_assert(TMEM_COLS * CTAS_PER_SM == 512, "the CTAs of an SM take all of TMEM");
   __host__ __device__ static constexpr uint32_t o_col(int t) { return O_COL + t * D; }
+  // Region of step g of tile t, and the parity of its use.
+  static __device__ __forceinline__ int sb(int t, int g) { return NB == 2 ? t : (2 * g + t) % NB; }
+  static __device__ __forceinline__ uint32_t sp(int t, int g) { return (uint32_t)(NB == 2 ? g : (2 * g + t) / NB) & 1; }
+  static __device__ __forceinline__ int slot(int g) { return g & (KVS - 1); }
+  static __device__ __forceinline__ uint32_t round(int g) { return (uint32_t)(g / KVS); }
+};
+
+// The barriers of a CTA.
+template <class C>
+struct AttnBars {
+  uint64_t *q_full, *q_empty;  // [2] per query tile
+  uint64_t *k_full, *k_empty, *v_full, *v_empty;  // [KVS]
+  uint64_t *s_full, *p_full, *pv_done;  // [NB] per S region
+  uint64_t* drain;  // failure path: the MMAs issued so far have completed
+  uint32_t* tmem_slot;
+  static constexpr int kCount = 4 + 4 * C::KVS + 3 * C::NB + 1;
+  static_assert(kCount * 8 + 4 <= C::BAR_BYTES, "barrier area");
+  __device__ __forceinline__ explicit AttnBars(uint8_t* at) {
+    uint64_t* b = reinterpret_cast<uint64_t*>(at);
+    auto take = [&](int n) { uint64_t* r = b; b += n; return r; };
+    q_full = take(2);
+    q_empty = take(2);
+    k_full = take(C::KVS);
+    k_empty = take(C::KVS);
+    v_full = take(C::KVS);
+    v_empty = take(C::KVS);
+    s_full = take(C::NB);
+    p_full = take(C::NB);
+    pv_done = take(C::NB);
+    drain = take(1);
+    tmem_slot = reinterpret_cast<uint32_t*>(b);
+  }
+  __device__ __forceinline__ void init() const {
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(&q_full[i], 1);
+      mbar_init(&q_empty[i], 1);
+    }
+    for (int i = 0; i < C::KVS; ++i) {
+      mbar_init(&k_full[i], 1);
+      mbar_init(&k_empty[i], 1);
+      mbar_init(&v_full[i], 1);
+      mbar_init(&v_empty[i], 1);
+    }
+    for (int i = 0; i < C::NB; ++i) {
+      mbar_init(&s_full[i], 1);
+      mbar_init(&p_full[i], 128);
+      mbar_init(&pv_done[i], 1);
+    }
+    mbar_init(drain, 1);
+    mbar_fence_init();
+  }
 };
 
 // Softmax of one key tile for this thread's query row (row r of tile t is
 // TMEM lane r): waits for S_t, writes P_t = 2^(s * scale - m) over the S
 // region as bf16 pairs, updates the running reference max m and sum l,
 // rescales O_t when the reference moves, and hands P_t to the MMA warp.
-// phase: this tile's step count in the CTA (barrier parity); first: the
-// item's first key tile; valid: keys of a masked (partial last) tile.
-template <int D, bool MASKED>
-__device__ __forceinline__ bool softmax_tile(uint64_t* s_full, uint64_t* pv_done, uint64_t* p_full, int phase,
-                                             bool first, int valid, uint32_t s_addr, uint32_t o_addr,
-                                             float scale_log2, float& m_run, float& l_run) {
-  using C = AttnCfg<D>;
+// g: this tile's step count in the CTA; first: the item's first key tile;
+// valid: keys of a masked (partial last) tile.
+template <class C, bool MASKED>
+__device__ __forceinline__ bool softmax_tile(const AttnBars<C>& bar, int t, int g, bool first, int valid,
+                                             uint32_t s_base, uint32_t o_addr, float scale_log2, float& m_run,
+                                             float& l_run) {
+  const uint32_t s_addr = s_base + C::sb(t, g) * C::BKV;
   // The lanes of a warp wait on the same phase, so they give up together
   // (after the wait limit) and the warp-collective tcgen05.ld / st below stay
   // convergent; a vote here would rule out a phase that completes exactly at
   // the limit for some lanes only, but costs 2-3% in this loop.
-  if (!mbar_wait(s_full, phase & 1)) return false;
-  // consume pv_done phase - 1 (already complete: s_full(phase) is committed
-  // after PV(phase - 1)) so that no later parity wait is two phases behind;
-  // at an item's first tile the previous item's output pass consumed it
-  if (!first && !mbar_wait(pv_done, (phase - 1) & 1)) return false;
+  if (!mbar_wait(&bar.s_full[C::sb(t, g)], C::sp(t, g))) return false;
   tc_fence_after();
   float s[C::BKV];
 #pragma unroll
@@ -130,23 +190,53 @@ __device__ __forceinline__ bool softmax_tile(uint64_t* s_full, uint64_t* pv_done
     for (int i = 0; i < C::BKV; ++i)
       if (i >= valid) s[i] = -INFINITY;
   }
-  // e = s * scale - m_run in place (packed pairs; the first tile uses 0 as
-  // the reference), with the row max of e alongside in four independent
-  // 3-input max chains on the ALU pipe.  s_full(phase) is committed after
-  // PV(phase - 1), so O_t and the P_t region are free here.  Lazy rescaling:
-  // the reference max moves only on the first tile or when the row max
-  // exceeds it by more than 2^8; then e is shifted in place.
   const uint64_t sc2 = f2_pack(scale_log2, scale_log2);
-  {
-    const float mref = first ? 0.f : m_run;
-    const uint64_t nm2 = f2_pack(-mref, -mref);
+  const float mref = first ? 0.f : m_run;
+  const uint64_t nm2 = f2_pack(-mref, -mref);
+  auto row_max = [](const float* m4) { return fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3])); };
+  auto shift = [&](float me) {
+    const uint64_t sh2 = f2_pack(-me, -me);
+#pragma unroll
+    for (int i = 0; i < C::BKV / 2; ++i) f2_unpack(f2_add(f2_pack(s[2 * i], s[2 * i + 1]), sh2), s[2 * i], s[2 * i + 1]);
+  };
+  // P = 2^e as bf16 pairs over the first BKV/2 columns of S_t, and the row sum
+  // as packed fp32 pairs
+  auto exps = [&]() -> float {
+    uint64_t acc0 = f2_pack(0.f, 0.f), acc1 = acc0;
+#pragma unroll
+    for (int half = 0; half < C::BKV / 64; ++half) {
+      uint32_t pk[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const float p0 = ex2_approx(s[half * 64 + 2 * i]), p1 = ex2_approx(s[half * 64 + 2 * i + 1]);
+        if (i & 1)
+          acc1 = f2_add(acc1, f2_pack(p0, p1));
+        else
+          acc0 = f2_add(acc0, f2_pack(p0, p1));
+        pk[i] = pack_bf16(p0, p1);
+      }
+      tmem_st32(s_addr + half * 32, pk);
+    }
+    float a0, a1, b0, b1;
+    f2_unpack(acc0, a0, a1);
+    f2_unpack(acc1, b0, b1);
+    return (a0 + a1) + (b0 + b1);
+  };
+  // e = s * scale - m_run in place (packed pairs; the first tile uses 0 as the
+  // reference); the row max of e in four independent 3-input max chains on the
+  // ALU pipe.  The P_t region is free here: the MMAs run in order, and S_t(g)
+  // follows the PV that read it.  Lazy rescaling: the reference max moves only
+  // on the first tile or when the row max exceeds it by more than 2^8; then e
+  // is shifted in place.
+  float ls;
+  if constexpr (C::MAX_FIRST) {
     float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
     for (int i = 0; i < C::BKV / 2; ++i) {
       f2_unpack(f2_fma(f2_pack(s[2 * i], s[2 * i + 1]), sc2, nm2), s[2 * i], s[2 * i + 1]);
       m4[i & 3] = fmax3(m4[i & 3], s[2 * i], s[2 * i + 1]);
     }
-    const float me = fmaxf(fmaxf(m4[0], m4[1]), fmaxf(m4[2], m4[3]));
+    const float me = row_max(m4);
     if (first || me > kRescaleLog2) {
       if (!first) {
         resc = true;
@@ -154,36 +244,51 @@ __device__ __forceinline__ bool softmax_tile(uint64_t* s_full, uint64_t* pv_done
         l_run *= f;
       }
       m_run = mref + me;
-      const uint64_t sh2 = f2_pack(-me, -me);
+      shift(me);
+    }
+    ls = exps();
+  } else {
+    // An element above 2^8 makes the row sum larger than 2^8 (or NaN), so the
+    // max is formed on a row's first tile and then only for such a sum.  Where
+    // it moves the reference, the warp writes its P again.  Without the max the
+    // exponentials start as the scores are scaled: 4726 tokens, 30 heads 172.9 ->
+    // 158.9 us (with 96-key tiles).
+    auto max_of_e = [&] {
+      float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
-      for (int i = 0; i < C::BKV / 2; ++i) f2_unpack(f2_add(f2_pack(s[2 * i], s[2 * i + 1]), sh2), s[2 * i], s[2 * i + 1]);
+      for (int i = 0; i < C::BKV / 2; ++i) m4[i & 3] = fmax3(m4[i & 3], s[2 * i], s[2 * i + 1]);
+      return row_max(m4);
+    };
+#pragma unroll
+    for (int i = 0; i < C::BKV / 2; ++i)
+      f2_unpack(f2_fma(f2_pack(s[2 * i], s[2 * i + 1]), sc2, nm2), s[2 * i], s[2 * i + 1]);
+    if (first) {
+      m_run = max_of_e();
+      shift(m_run);
+    }
+    ls = exps();
+    if (!first && !(ls <= kRescale)) {
+      const float me = max_of_e();
+      if (me > kRescaleLog2) {
+        resc = true;
+        f = ex2_approx(-me);
+        l_run *= f;
+        m_run += me;
+        shift(me);
+      }
+    }
+    if (__any_sync(0xffffffffu, resc)) {
+      tmem_wait_st();  // the first P has been written
+      ls = exps();
     }
   }
-  // P = 2^e as bf16 pairs over the first BKV/2 columns of S_t, with the row
-  // sum as packed fp32 pairs
-  uint64_t acc0 = f2_pack(0.f, 0.f), acc1 = acc0;
-#pragma unroll
-  for (int half = 0; half < C::BKV / 64; ++half) {
-    uint32_t pk[32];
-#pragma unroll
-    for (int i = 0; i < 32; ++i) {
-      const float p0 = ex2_approx(s[half * 64 + 2 * i]), p1 = ex2_approx(s[half * 64 + 2 * i + 1]);
-      if (i & 1)
-        acc1 = f2_add(acc1, f2_pack(p0, p1));
-      else
-        acc0 = f2_add(acc0, f2_pack(p0, p1));
-      pk[i] = pack_bf16(p0, p1);
-    }
-    tmem_st32(s_addr + half * 32, pk);
-  }
-  float a0, a1, b0, b1;
-  f2_unpack(acc0, a0, a1);
-  f2_unpack(acc1, b0, b1);
-  const float ls = (a0 + a1) + (b0 + b1);
   l_run += ls;
   if (__any_sync(0xffffffffu, resc)) {
+    // (no later use of that region can have completed: the MMAs of step (t, g) wait for this warp)
+    if (!mbar_wait(&bar.pv_done[C::sb(t, g - 1)], C::sp(t, g - 1))) return false;
+    tc_fence_after();
 #pragma unroll 1
-    for (int c = 0; c < D; c += 32) {
+    for (int c = 0; c < C::D; c += 32) {
       uint32_t o[32];
       tmem_ld32(o_addr + c, o);
       tmem_wait_ld();
@@ -194,19 +299,18 @@ __device__ __forceinline__ bool softmax_tile(uint64_t* s_full, uint64_t* pv_done
   }
   tmem_wait_st();
   tc_fence_before();
-  mbar_arrive(p_full);
+  mbar_arrive(&bar.p_full[C::sb(t, g)]);
   return true;
 }
 
 // S_t = Q_t K^T for one key tile: D/16 MMAs (M128, N = BKV, K16) into TMEM
 // column d; qdesc_t / kdesc_slot: shared-memory descriptors of Q_t and of the
 // K ring slot (an operand at byte offset o is the descriptor plus o >> 4).
-template <int D>
+template <class C>
 __device__ __forceinline__ void issue_s_mma(uint32_t d, uint64_t qdesc_t, uint64_t kdesc_slot) {
-  using C = AttnCfg<D>;
   constexpr uint32_t idesc_s = idesc_bf16_f32(128, C::BKV, false, false);
 #pragma unroll
-  for (int kk = 0; kk < D / 16; ++kk) {
+  for (int kk = 0; kk < C::D / 16; ++kk) {
     const uint64_t off_a = (uint64_t)(((kk >> 2) * C::CHUNK_Q + (kk & 3) * 32) >> 4);
     const uint64_t off_b = (uint64_t)(((kk >> 2) * C::CHUNK_KV + (kk & 3) * 32) >> 4);
     mma_bf16_ss(d, qdesc_t + off_a, kdesc_slot + off_b, idesc_s, kk != 0);
@@ -216,59 +320,75 @@ __device__ __forceinline__ void issue_s_mma(uint32_t d, uint64_t qdesc_t, uint64
 // O_t (+)= P_t V for one key tile: BKV/16 MMAs (M128, N = D, K16), P_t from
 // TMEM at column p (bf16 pairs over the S region), V MN-major from the ring
 // slot; accumulate is false on an item's first key tile.
-template <int D>
+template <class C>
 __device__ __forceinline__ void issue_pv_mma(uint32_t d, uint32_t p, uint64_t vdesc_slot, bool accumulate) {
-  using C = AttnCfg<D>;
-  constexpr uint32_t idesc_o = idesc_bf16_f32(128, D, false, true);
+  constexpr uint32_t idesc_o = idesc_bf16_f32(128, C::D, false, true);
 #pragma unroll
   for (int kk = 0; kk < C::BKV / 16; ++kk)
     mma_bf16_ts(d, p + kk * 8, vdesc_slot + (uint64_t)((kk * 16 * 128) >> 4), idesc_o, accumulate || kk != 0);
 }
 
 // TMA loads of one K or V tile (D / 64 chunks of 64 columns) into a ring slot.
-template <int D>
+template <class C>
 __device__ __forceinline__ void load_kv_tile(uint8_t* dst, const CUtensorMap* map, uint64_t* bar, int col, int row) {
-  using C = AttnCfg<D>;
   mbar_expect_tx(bar, C::KV_BYTES);
   for (int c = 0; c < C::CH; ++c) tma_load_2d(dst + c * C::CHUNK_KV, map, bar, col + c * 64, row);
 }
 
-// Failure path (a wait ran out): the producer waits, bounded, until the loads
-// it has issued have landed (the Q tiles, and the last K and V tiles of each
-// two-slot ring), so that no copy writes into the shared memory of a CTA
-// that has left; the MMA thread waits, bounded, for the MMAs it has issued
-// before tensor memory is freed.  Never called on the normal path.
-__device__ __noinline__ void drain_loads(uint64_t* q_full, uint64_t* k_full, uint64_t* v_full, int nk, int nv) {
-  mbar_wait(q_full, 0);
-  for (int j = nk > 2 ? nk - 2 : 0; j < nk; ++j) mbar_wait(&k_full[j & 1], (j >> 1) & 1);
-  for (int j = nv > 2 ? nv - 2 : 0; j < nv; ++j) mbar_wait(&v_full[j & 1], (j >> 1) & 1);
+// Failure path (a wait ran out): the producer waits, bounded, until the last K
+// and V loads of each ring have landed, so that no copy writes into the shared
+// memory of a CTA that has left; the MMA thread waits, bounded, for the MMAs it
+// has issued before tensor memory is freed.  Never called on the normal path.
+template <class C>
+__device__ __noinline__ void drain_loads(const AttnBars<C>& bar, int nk, int nv) {
+  for (int j = nk > C::KVS ? nk - C::KVS : 0; j < nk; ++j) mbar_wait(&bar.k_full[C::slot(j)], C::round(j) & 1);
+  for (int j = nv > C::KVS ? nv - C::KVS : 0; j < nv; ++j) mbar_wait(&bar.v_full[C::slot(j)], C::round(j) & 1);
 }
 __device__ __noinline__ void drain_mmas(uint64_t* drain) {
   mma_commit(drain);
   mbar_wait(drain, 0);
 }
 
-template <int D>
-__global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
-    attn_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
-                   const __grid_constant__ CUtensorMap tmV, AttnDev a) {
-  using C = AttnCfg<D>;
+// The MMA warp's commits and operands.
+template <class C>
+struct AttnMma {
+  const AttnBars<C>& bar;
+  uint32_t tmem;
+  uint64_t qdesc, kdesc, vdesc;
+  __device__ __forceinline__ AttnMma(const AttnBars<C>& b, uint32_t tm, uint8_t* sQ, uint8_t* sK, uint8_t* sV)
+      : bar(b), tmem(tm) {
+    // Descriptors are built once; an operand at byte offset o from a base is
+    // the base descriptor plus o >> 4 (the 14-bit address field cannot
+    // overflow: shared memory ends below 256 KB).
+    qdesc = smem_desc_sw128(smem_u32(sQ), 16, 1024);
+    kdesc = smem_desc_sw128(smem_u32(sK), 16, 1024);
+    vdesc = smem_desc_sw128(smem_u32(sV), C::CHUNK_KV, 1024);
+  }
+  // S_t = Q_t K^T of step g into its S region of tile t
+  __device__ __forceinline__ void s_step(int t, int g) const {
+    issue_s_mma<C>(tmem + C::sb(t, g) * C::BKV, qdesc + (uint64_t)((t * C::T_BYTES) >> 4), kdesc + (uint64_t)((C::slot(g) * C::KV_BYTES) >> 4));
+    mma_commit(&bar.s_full[C::sb(t, g)]);
+    if (t == 1) mma_commit(&bar.k_empty[C::slot(g)]);
+  }
+  // O_t += P_t V of step g; accumulate is false on an item's first key tile
+  __device__ __forceinline__ void pv_step(int t, int g, bool accumulate) const {
+    issue_pv_mma<C>(tmem + C::o_col(t), tmem + C::sb(t, g) * C::BKV,
+                    vdesc + (uint64_t)((C::slot(g) * C::KV_BYTES) >> 4), accumulate);
+    mma_commit(&bar.pv_done[C::sb(t, g)]);
+    if (t == 1) mma_commit(&bar.v_empty[C::slot(g)]);
+  }
+};
+
+template <class C>
+__global__ void __launch_bounds__(kAttnThreads, C::CTAS_PER_SM)
+    attn_split_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
+                      const __grid_constant__ CUtensorMap tmV, AttnDev a) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = smem + C::OFF_Q;
   uint8_t* sK = smem + C::OFF_K;
   uint8_t* sV = smem + C::OFF_V;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR);
-  uint64_t* q_full = bars + 0;
-  uint64_t* k_full = bars + 1;    // [2]
-  uint64_t* k_empty = bars + 3;   // [2]
-  uint64_t* v_full = bars + 5;    // [2]
-  uint64_t* v_empty = bars + 7;   // [2]
-  uint64_t* s_full = bars + 9;    // [2] per query tile
-  uint64_t* p_full = bars + 11;   // [2] per query tile
-  uint64_t* pv_done = bars + 13;  // [2] per query tile
-  uint64_t* drain = bars + 15;    // failure path: the MMAs issued so far have completed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 16);
+  const AttnBars<C> bar(smem + C::OFF_BAR);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int item = a.item_base + (int)blockIdx.x / a.splits, split = (int)blockIdx.x % a.splits;
@@ -281,114 +401,80 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
     tma_prefetch_desc(&tmQ);
     tma_prefetch_desc(&tmK);
     tma_prefetch_desc(&tmV);
-    mbar_init(q_full, 1);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&k_full[i], 1);
-      mbar_init(&k_empty[i], 1);
-      mbar_init(&v_full[i], 1);
-      mbar_init(&v_empty[i], 1);
-      mbar_init(&s_full[i], 1);
-      mbar_init(&p_full[i], 128);
-      mbar_init(&pv_done[i], 1);
-    }
-    mbar_init(drain, 1);
-    mbar_fence_init();
+    bar.init();
   }
-  if (warp == 1) tmem_alloc(tmem_slot, C::TMEM_COLS);
+  if (warp == 1) tmem_alloc(bar.tmem_slot, C::TMEM_COLS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = *bar.tmem_slot;
   pdl_wait();  // the set-up above overlaps the tail of the kernel before
 
   if (warp == 0) {
     if (lane == 0) {  // ---------------------------------------- TMA producer
-      mbar_expect_tx(q_full, 2 * C::T_BYTES);
+      mbar_expect_tx(&bar.q_full[0], 2 * C::T_BYTES);
       for (int t = 0; t < 2; ++t)
         for (int c = 0; c < C::CH; ++c)
-          tma_load_2d(sQ + t * C::T_BYTES + c * C::CHUNK_Q, &tmQ, q_full, a.q_col + h * D + c * 64,
+          tma_load_2d(sQ + t * C::T_BYTES + c * C::CHUNK_Q, &tmQ, &bar.q_full[0], a.q_col + h * C::D + c * 64,
                       qt * kBQ + t * kTileQ);
       int nk_issued = 0, nv_issued = 0;
       for (int j = 0; j < nkv; ++j) {
-        const int st = j & 1, round = j >> 1;
-        if (round > 0 && !mbar_wait(&k_empty[st], (round - 1) & 1)) break;
-        load_kv_tile<D>(sK + st * C::KV_BYTES, &tmK, &k_full[st], a.k_col + h * D, (jb + j) * C::BKV);
+        const int st = C::slot(j);
+        const uint32_t round = C::round(j);
+        if (round > 0 && !mbar_wait(&bar.k_empty[st], (round - 1) & 1)) break;
+        load_kv_tile<C>(sK + st * C::KV_BYTES, &tmK, &bar.k_full[st], a.k_col + h * C::D, (jb + j) * C::BKV);
         nk_issued = j + 1;
-        if (round > 0 && !mbar_wait(&v_empty[st], (round - 1) & 1)) break;
-        load_kv_tile<D>(sV + st * C::KV_BYTES, &tmV, &v_full[st], a.v_col + h * D, (jb + j) * C::BKV);
+        if (round > 0 && !mbar_wait(&bar.v_empty[st], (round - 1) & 1)) break;
+        load_kv_tile<C>(sV + st * C::KV_BYTES, &tmV, &bar.v_full[st], a.v_col + h * C::D, (jb + j) * C::BKV);
         nv_issued = j + 1;
       }
-      if (nv_issued < nkv) drain_loads(q_full, k_full, v_full, nk_issued, nv_issued);
+      if (nv_issued < nkv) {
+        mbar_wait(&bar.q_full[0], 0);
+        drain_loads<C>(bar, nk_issued, nv_issued);
+      }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer
     // The whole warp walks the loop (descriptors and flags stay in uniform
-    // registers) and one elected lane issues.  Descriptors are built once; an
-    // operand at byte offset o from a base is the base descriptor plus o >> 4
-    // (the 14-bit address field cannot overflow: shared memory ends below
-    // 256 KB).
+    // registers) and one elected lane issues.
     const bool leader = elect_one();
-    const uint64_t qdesc = smem_desc_sw128(smem_u32(sQ), 16, 1024);
-    const uint64_t kdesc = smem_desc_sw128(smem_u32(sK), 16, 1024);
-    const uint64_t vdesc = smem_desc_sw128(smem_u32(sV), C::CHUNK_KV, 1024);
-    // S_t(j) = Q_t K_j^T into the S region of tile t
-    auto issue_s = [&](int t, int j) {
-      issue_s_mma<D>(tmem + C::S_COL + t * C::BKV, qdesc + (uint64_t)((t * C::T_BYTES) >> 4),
-                     kdesc + (uint64_t)(((j & 1) * C::KV_BYTES) >> 4));
-      mma_commit(&s_full[t]);
-    };
-    bool ok = mbar_wait_warp(q_full, 0) && mbar_wait_warp(&k_full[0], 0);
-    if (ok) {
+    const AttnMma<C> mma(bar, tmem, sQ, sK, sV);
+    bool ok = mbar_wait_warp(&bar.q_full[0], 0);
+    auto issue_s = [&](int t, int j) -> bool {
+      if (t == 0 && !mbar_wait_warp(&bar.k_full[C::slot(j)], C::round(j) & 1)) return false;
       tc_fence_after();
-      if (leader) {
-        issue_s(0, 0);
-        issue_s(1, 0);
-        mma_commit(&k_empty[0]);
-      }
+      if (leader) mma.s_step(t, j);
       __syncwarp();
-    }
+      return true;
+    };
+    for (int n = 0; ok && n < 2 * nkv && n < C::NB; ++n) ok = issue_s(n & 1, n >> 1);
     for (int j = 0; ok && j < nkv; ++j) {
-      const int st = j & 1;
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
-        if (!mbar_wait_warp(&p_full[t], j & 1)) { ok = false; break; }
-        if (t == 0 && !mbar_wait_warp(&v_full[st], (j >> 1) & 1)) { ok = false; break; }
+        if (!mbar_wait_warp(&bar.p_full[C::sb(t, j)], C::sp(t, j))) { ok = false; break; }
+        if (t == 0 && !mbar_wait_warp(&bar.v_full[C::slot(j)], C::round(j) & 1)) { ok = false; break; }
         tc_fence_after();
-        if (leader) {
-          // O_t += P_t V_j
-          issue_pv_mma<D>(tmem + C::o_col(t), tmem + C::S_COL + t * C::BKV,
-                          vdesc + (uint64_t)((st * C::KV_BYTES) >> 4), j != 0);
-          mma_commit(&pv_done[t]);
-          if (t == 1) mma_commit(&v_empty[st]);
-        }
+        if (leader) mma.pv_step(t, j, j != 0);
         __syncwarp();
-        if (j + 1 < nkv) {
-          if (t == 0 && !mbar_wait_warp(&k_full[st ^ 1], ((j + 1) >> 1) & 1)) { ok = false; break; }
-          tc_fence_after();
-          if (leader) {
-            issue_s(t, j + 1);
-            if (t == 1) mma_commit(&k_empty[st ^ 1]);
-          }
-          __syncwarp();
-        }
+        const int tn = (t + C::NB) & 1, jn = j + (t + C::NB) / 2;
+        if (jn < nkv && !issue_s(tn, jn)) { ok = false; break; }
       }
     }
-    if (!ok && leader) drain_mmas(drain);
+    if (!ok && leader) drain_mmas(bar.drain);
   } else {  // ---------------------------------------- softmax: warps 2-5 tile a, 6-9 tile b
     const int t = (warp - 2) >> 2;
     const int q = warp & 3;
     const int r = q * 32 + lane;  // row within the query tile == TMEM lane
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const uint32_t s_addr = tmem + lane_base + C::S_COL + t * C::BKV;
+    const uint32_t s_base = tmem + lane_base;
     const uint32_t o_addr = tmem + lane_base + C::o_col(t);
     float m_run = -INFINITY, l_run = 0.f;
     bool ok = true;
     // One key tile; the masked variant (keys past the end of the sequence)
     // is compiled separately and runs only on a partial last tile.
     auto step = [&](int j, auto masked) -> bool {
-      return softmax_tile<D, decltype(masked)::value>(&s_full[t], &pv_done[t], &p_full[t], j, j == 0,
-                                                      (int)(a.nk - (int64_t)(jb + j) * C::BKV), s_addr, o_addr,
-                                                      a.scale_log2, m_run, l_run);
+      return softmax_tile<C, decltype(masked)::value>(bar, t, j, j == 0, (int)(a.nk - (int64_t)(jb + j) * C::BKV),
+                                                      s_base, o_addr, a.scale_log2, m_run, l_run);
     };
     const bool partial_last = (int64_t)(jb + nkv) * C::BKV > a.nk;
     for (int j = 0; j < nkv; ++j) {
@@ -398,35 +484,24 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
         break;
       }
     }
-    // ---------------------------------------------------- epilogue: O_t / l
-    if (ok) ok = mbar_wait(&pv_done[t], (nkv - 1) & 1);
+    // ------------------------------ partial result of this key range: unnormalised O
+    if (ok) ok = mbar_wait(&bar.pv_done[C::sb(t, nkv - 1)], C::sp(t, nkv - 1));
     tc_fence_after();
     const int64_t row = (int64_t)qt * kBQ + t * kTileQ + r;
-    const float inv = 1.0f / l_run;
+    const int64_t slot = (int64_t)blockIdx.x * kBQ + t * kTileQ + r;
 #pragma unroll 1
-    for (int c = 0; c < D; c += 32) {
+    for (int c = 0; c < C::D; c += 32) {
       uint32_t o[32];
       tmem_ld32(o_addr + c, o);
       tmem_wait_ld();
       if (!ok || row >= a.nq) continue;
-      if (a.splits > 1) {  // partial result of this key range: unnormalised O
-        float* pp = a.part_o + ((int64_t)blockIdx.x * kBQ + t * kTileQ + r) * D + c;
+      float* pp = a.part_o + slot * C::D + c;
 #pragma unroll
-        for (int i = 0; i < 32; i += 4)
-          *reinterpret_cast<float4*>(pp + i) = make_float4(__uint_as_float(o[i]), __uint_as_float(o[i + 1]),
-                                                           __uint_as_float(o[i + 2]), __uint_as_float(o[i + 3]));
-        continue;
-      }
-      float v[32];
-#pragma unroll
-      for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(o[i]) * inv;
-      __nv_bfloat16* op = static_cast<__nv_bfloat16*>(a.out) + row * a.ldo + a.o_col + h * D + c;
-#pragma unroll
-      for (int i = 0; i < 32; i += 8) store8(op + i, v + i);
+      for (int i = 0; i < 32; i += 4)
+        *reinterpret_cast<float4*>(pp + i) = make_float4(__uint_as_float(o[i]), __uint_as_float(o[i + 1]),
+                                                         __uint_as_float(o[i + 2]), __uint_as_float(o[i + 3]));
     }
-    if (a.splits > 1 && ok && row < a.nq)
-      *reinterpret_cast<float2*>(a.part_ml + ((int64_t)blockIdx.x * kBQ + t * kTileQ + r) * 2) =
-          make_float2(m_run, l_run);
+    if (ok && row < a.nq) *reinterpret_cast<float2*>(a.part_ml + slot * 2) = make_float2(m_run, l_run);
   }
   tc_fence_before();
   __syncthreads();
@@ -436,7 +511,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
   }
 }
 
-// Persistent variant.  Each CTA walks the items
+// Whole items on persistent CTAs.  Each CTA walks the items
 // item_base + blockIdx.x + k * gridDim.x; one counter g numbers its key-tile
 // steps across items, and every per-step barrier phase and ring slot follows
 // it.  Q_t of the next item is loaded once the current item's last S_t MMA
@@ -444,29 +519,17 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
 // right after the current item's last PV.  The output leaves through two
 // staging boxes per softmax warp and TMA stores, which frees the softmax
 // warps for the next item.
-template <int D>
-__global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
+template <class C>
+__global__ void __launch_bounds__(kAttnThreads, C::CTAS_PER_SM)
     attn_persist_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmO,
                         AttnDev a) {
-  using C = AttnCfg<D>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sQ = smem + C::OFF_Q;
   uint8_t* sK = smem + C::OFF_K;
   uint8_t* sV = smem + C::OFF_V;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + C::OFF_BAR_P);
-  uint64_t* q_full = bars + 0;    // [2] per query tile
-  uint64_t* q_empty = bars + 2;   // [2] per query tile
-  uint64_t* k_full = bars + 4;    // [2]
-  uint64_t* k_empty = bars + 6;   // [2]
-  uint64_t* v_full = bars + 8;    // [2]
-  uint64_t* v_empty = bars + 10;  // [2]
-  uint64_t* s_full = bars + 12;   // [2] per query tile
-  uint64_t* p_full = bars + 14;   // [2] per query tile
-  uint64_t* pv_done = bars + 16;  // [2] per query tile
-  uint64_t* drain = bars + 18;    // failure path: the MMAs issued so far have completed
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 19);
+  const AttnBars<C> bar(smem + C::OFF_BAR_P);
 
   const int warp = warp_index(), lane = threadIdx.x & 31;
   const int item0 = a.item_base + (int)blockIdx.x, item_step = (int)gridDim.x;
@@ -479,25 +542,13 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
     tma_prefetch_desc(&tmK);
     tma_prefetch_desc(&tmV);
     tma_prefetch_desc(&tmO);
-    for (int i = 0; i < 2; ++i) {
-      mbar_init(&q_full[i], 1);
-      mbar_init(&q_empty[i], 1);
-      mbar_init(&k_full[i], 1);
-      mbar_init(&k_empty[i], 1);
-      mbar_init(&v_full[i], 1);
-      mbar_init(&v_empty[i], 1);
-      mbar_init(&s_full[i], 1);
-      mbar_init(&p_full[i], 128);
-      mbar_init(&pv_done[i], 1);
-    }
-    mbar_init(drain, 1);
-    mbar_fence_init();
+    bar.init();
   }
-  if (warp == 1) tmem_alloc(tmem_slot, C::TMEM_COLS);
+  if (warp == 1) tmem_alloc(bar.tmem_slot, C::TMEM_COLS);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = *bar.tmem_slot;
   pdl_wait();  // the set-up above overlaps the tail of the kernel before
 
   if (warp == 0) {
@@ -507,93 +558,77 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
       for (int k = 0, g = 0; ok && k < n_items; ++k) {
         const int item = item0 + k * item_step;
         const int qt = item % a.nqp, h = item / a.nqp;
-        // Q_t of item k replaces Q_t of item k - 1 once that item's last S_t is done
-        for (int t = 0; t < 2 && ok; ++t) {
-          if (k > 0 && !mbar_wait(&q_empty[t], (k - 1) & 1)) { ok = false; break; }
-          mbar_expect_tx(&q_full[t], C::T_BYTES);
+        // Q_t of item k replaces Q_t of item k - 1 once that item's last S_t is
+        // done; the item's first K goes out before Q_b, whose tile finishes later
+        auto load_q = [&](int t) -> bool {
+          if (k > 0 && !mbar_wait(&bar.q_empty[t], (k - 1) & 1)) return false;
+          mbar_expect_tx(&bar.q_full[t], C::T_BYTES);
           for (int c = 0; c < C::CH; ++c)
-            tma_load_2d(sQ + t * C::T_BYTES + c * C::CHUNK_Q, &tmQ, &q_full[t], a.q_col + h * D + c * 64,
+            tma_load_2d(sQ + t * C::T_BYTES + c * C::CHUNK_Q, &tmQ, &bar.q_full[t], a.q_col + h * C::D + c * 64,
                         qt * kBQ + t * kTileQ);
-        }
+          return true;
+        };
+        if (!load_q(0)) { ok = false; break; }
         for (int j = 0; ok && j < nkv; ++j, ++g) {
-          const int st = g & 1, round = g >> 1;
-          if (round > 0 && !mbar_wait(&k_empty[st], (round - 1) & 1)) { ok = false; break; }
-          load_kv_tile<D>(sK + st * C::KV_BYTES, &tmK, &k_full[st], a.k_col + h * D, j * C::BKV);
+          const int st = C::slot(g);
+          const uint32_t round = C::round(g);
+          if (round > 0 && !mbar_wait(&bar.k_empty[st], (round - 1) & 1)) { ok = false; break; }
+          load_kv_tile<C>(sK + st * C::KV_BYTES, &tmK, &bar.k_full[st], a.k_col + h * C::D, j * C::BKV);
           nk_issued = g + 1;
-          if (round > 0 && !mbar_wait(&v_empty[st], (round - 1) & 1)) { ok = false; break; }
-          load_kv_tile<D>(sV + st * C::KV_BYTES, &tmV, &v_full[st], a.v_col + h * D, j * C::BKV);
+          if (j == 0 && !load_q(1)) { ok = false; break; }
+          if (round > 0 && !mbar_wait(&bar.v_empty[st], (round - 1) & 1)) { ok = false; break; }
+          load_kv_tile<C>(sV + st * C::KV_BYTES, &tmV, &bar.v_full[st], a.v_col + h * C::D, j * C::BKV);
           nv_issued = g + 1;
         }
       }
       // after a wait ran out: the last K and V loads of each ring have landed
       // (Q loads of an item are waited on by the MMA thread before any use)
-      if (!ok) {
-        for (int j = nk_issued > 2 ? nk_issued - 2 : 0; j < nk_issued; ++j) mbar_wait(&k_full[j & 1], (j >> 1) & 1);
-        for (int j = nv_issued > 2 ? nv_issued - 2 : 0; j < nv_issued; ++j) mbar_wait(&v_full[j & 1], (j >> 1) & 1);
-      }
+      if (!ok) drain_loads<C>(bar, nk_issued, nv_issued);
     }
   } else if (warp == 1) {
     // ------------------------------------------------------- MMA issuer
-    // (whole warp walks, one elected lane issues, as in attn_tc_kernel)
+    // (whole warp walks, one elected lane issues, as in attn_split_kernel)
     const bool leader = elect_one();
-    const uint64_t qdesc = smem_desc_sw128(smem_u32(sQ), 16, 1024);
-    const uint64_t kdesc = smem_desc_sw128(smem_u32(sK), 16, 1024);
-    const uint64_t vdesc = smem_desc_sw128(smem_u32(sV), C::CHUNK_KV, 1024);
-    // S_t = Q_t K^T of step g into the S region of tile t; after an item's
-    // last key tile (last_tile) the producer may replace Q_t
-    auto issue_s = [&](int t, int g, bool last_tile) {
-      issue_s_mma<D>(tmem + C::S_COL + t * C::BKV, qdesc + (uint64_t)((t * C::T_BYTES) >> 4),
-                     kdesc + (uint64_t)(((g & 1) * C::KV_BYTES) >> 4));
-      mma_commit(&s_full[t]);
-      if (last_tile) mma_commit(&q_empty[t]);
-    };
-    bool ok = total > 0 && mbar_wait_warp(&k_full[0], 0);
-    for (int t = 0; t < 2 && ok; ++t) {
-      if (!mbar_wait_warp(&q_full[t], 0)) { ok = false; break; }
+    const AttnMma<C> mma(bar, tmem, sQ, sK, sV);
+    // S_t of step g, which is key tile j of item k (jn, kn: of the next S to
+    // issue); after an item's last key tile the producer may replace Q_t
+    int jn = 0, kn = 0;
+    auto issue_s = [&](int t, int g) -> bool {
+      if (t == 0 && !mbar_wait_warp(&bar.k_full[C::slot(g)], C::round(g) & 1)) return false;
+      if (jn == 0 && !mbar_wait_warp(&bar.q_full[t], kn & 1)) return false;
       tc_fence_after();
-      if (leader) issue_s(t, 0, nkv == 1);
+      if (leader) {
+        mma.s_step(t, g);
+        if (jn == nkv - 1) mma_commit(&bar.q_empty[t]);
+      }
       __syncwarp();
-    }
-    if (ok && leader) mma_commit(&k_empty[0]);
-    __syncwarp();
-    // step g (key tile j of item k): PV_a(g) S_a(g+1) PV_b(g) S_b(g+1); at an
-    // item boundary S(g+1) reads the next item's Q
-    for (int g = 0, j = 0, k = 0; ok && g < total; ++g) {
-      const int st = g & 1, gn = g + 1;
-      const bool boundary = j + 1 == nkv;  // step gn starts item k + 1
-      const int jn = boundary ? 0 : j + 1;
+      if (t == 1 && ++jn == nkv) {
+        jn = 0;
+        ++kn;
+      }
+      return true;
+    };
+    bool ok = true;
+    for (int n = 0; ok && n < 2 * total && n < C::NB; ++n) ok = issue_s(n & 1, n >> 1);
+    for (int g = 0, j = 0; ok && g < total; ++g) {
 #pragma unroll
       for (int t = 0; t < 2; ++t) {
-        if (!mbar_wait_warp(&p_full[t], g & 1)) { ok = false; break; }
-        if (t == 0 && !mbar_wait_warp(&v_full[st], (g >> 1) & 1)) { ok = false; break; }
+        if (!mbar_wait_warp(&bar.p_full[C::sb(t, g)], C::sp(t, g))) { ok = false; break; }
+        if (t == 0 && !mbar_wait_warp(&bar.v_full[C::slot(g)], C::round(g) & 1)) { ok = false; break; }
         tc_fence_after();
-        if (leader) {
-          issue_pv_mma<D>(tmem + C::o_col(t), tmem + C::S_COL + t * C::BKV,
-                          vdesc + (uint64_t)((st * C::KV_BYTES) >> 4), j != 0);
-          mma_commit(&pv_done[t]);
-          if (t == 1) mma_commit(&v_empty[st]);
-        }
+        if (leader) mma.pv_step(t, g, j != 0);
         __syncwarp();
-        if (gn < total) {
-          if (t == 0 && !mbar_wait_warp(&k_full[st ^ 1], (gn >> 1) & 1)) { ok = false; break; }
-          if (boundary && !mbar_wait_warp(&q_full[t], (k + 1) & 1)) { ok = false; break; }
-          tc_fence_after();
-          if (leader) {
-            issue_s(t, gn, jn == nkv - 1);
-            if (t == 1) mma_commit(&k_empty[st ^ 1]);
-          }
-          __syncwarp();
-        }
+        const int tn = (t + C::NB) & 1, gn = g + (t + C::NB) / 2;
+        if (gn < total && !issue_s(tn, gn)) { ok = false; break; }
       }
-      j = jn;
-      k += boundary;
+      if (++j == nkv) j = 0;
     }
-    if (!ok && leader) drain_mmas(drain);
+    if (!ok && leader) drain_mmas(bar.drain);
   } else {  // ---------------------------------------- softmax: warps 2-5 tile a, 6-9 tile b
     const int t = (warp - 2) >> 2;
     const int q = warp & 3;
     const uint32_t lane_base = (uint32_t)(q * 32) << 16;
-    const uint32_t s_addr = tmem + lane_base + C::S_COL + t * C::BKV;
+    const uint32_t s_base = tmem + lane_base;
     const uint32_t o_addr = tmem + lane_base + C::o_col(t);
     uint8_t* stage = smem + C::OFF_STAGE_P + (warp - 2) * 2 * C::STAGE_BOX;
     const int valid_last = (int)(a.nk - (int64_t)(nkv - 1) * C::BKV);  // keys of the last tile
@@ -603,10 +638,10 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
       float m_run = -INFINITY, l_run = 0.f;
       for (int j = 0; j < nkv; ++j, ++g) {
         const bool ok_j = (j == nkv - 1 && valid_last < C::BKV)
-                              ? softmax_tile<D, true>(&s_full[t], &pv_done[t], &p_full[t], g, j == 0, valid_last,
-                                                      s_addr, o_addr, a.scale_log2, m_run, l_run)
-                              : softmax_tile<D, false>(&s_full[t], &pv_done[t], &p_full[t], g, j == 0, C::BKV,
-                                                       s_addr, o_addr, a.scale_log2, m_run, l_run);
+                              ? softmax_tile<C, true>(bar, t, g, j == 0, valid_last, s_base, o_addr, a.scale_log2,
+                                                      m_run, l_run)
+                              : softmax_tile<C, false>(bar, t, g, j == 0, C::BKV, s_base, o_addr, a.scale_log2, m_run,
+                                                       l_run);
         if (!ok_j) {
           ok = false;
           break;
@@ -615,14 +650,14 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
       // ------------------------------------------------ output: O_t / l
       // (the next PV_t, which overwrites O_t, follows this warpgroup's next
       // p_full arrival, issued after these loads have completed)
-      if (ok) ok = mbar_wait(&pv_done[t], (g - 1) & 1);
+      if (ok) ok = mbar_wait(&bar.pv_done[C::sb(t, g - 1)], C::sp(t, g - 1));
       ok = __all_sync(0xffffffffu, ok);  // the item loop continues for the whole warp or not at all
       tc_fence_after();
       const int qt = item % a.nqp, h = item / a.nqp;
       const int64_t row0 = (int64_t)qt * kBQ + t * kTileQ + q * 32;  // this warp's 32 rows
       const float inv = 1.0f / l_run;
 #pragma unroll 1
-      for (int c = 0; c < D; c += 32) {
+      for (int c = 0; c < C::D; c += 32) {
         uint32_t o[32];
         tmem_ld32(o_addr + c, o);
         tmem_wait_ld();
@@ -647,7 +682,7 @@ __global__ void __launch_bounds__(kAttnThreads, AttnCfg<D>::CTAS_PER_SM)
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) {
-          tma_store_2d(&tmO, box, a.o_col + h * D + c, (int)row0);
+          tma_store_2d(&tmO, box, a.o_col + h * C::D + c, (int)row0);
           bulk_commit_group();
         }
         ++n_st;
@@ -705,16 +740,14 @@ int num_sms_attn() {
   return n;
 }
 
-// Key ranges of at most this many tiles are short: no split of a last wave.
-constexpr int kPersistMaxKeyTiles = 8;
-
-template <int D>
+template <class C>
 acid_status launch_attn_tc(const AttnArgs& x, cudaStream_t s) {
-  using C = AttnCfg<D>;
+  constexpr int D = C::D;
   static bool attr_done = false;
   if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(attn_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    ACID_CUDA(cudaFuncSetAttribute(attn_persist_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_P));
+    ACID_CUDA(cudaFuncSetAttribute(attn_persist_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_P));
+    if constexpr (C::CTAS_PER_SM == 1)
+      ACID_CUDA(cudaFuncSetAttribute(attn_split_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
     attr_done = true;
   }
   CUtensorMap tq, tk, tv;
@@ -739,45 +772,40 @@ acid_status launch_attn_tc(const AttnArgs& x, cudaStream_t s) {
   a.part_ml = nullptr;
   const int items = a.nqp * x.heads;
   const int nkv_all = (int)((x.nk + C::BKV - 1) / C::BKV);
-  // Head dim 128, and short key ranges at head dim 64, run on persistent CTAs
-  // (measured at head dim 128, us, persistent / one item per CTA: 4846 tokens, 24
-  // heads 179 / 188; 7800, 12 heads 248 / 254; 1100, 12 heads 18.5 / 22.2; head
-  // dim 64 at 17776 tokens, 30 heads 2326 / 2154).  Long key ranges: items fill
-  // whole waves of CTAS_PER_SM CTAs per SM; the items of a last, partial wave
-  // are split along the key range so that they fill one wave together, and
-  // their partial results are merged.  Short key ranges: the persistent CTAs
-  // take all items, and the few CTAs that take one item more cost less than a
-  // split wave's start-up and merge (measured: 109 against 121 us for
-  // 32760 x 512 keys).
+  // Items fill whole waves of persistent CTAs, CTAS_PER_SM on an SM (measured at
+  // head dim 128, us, persistent / one item per CTA: 4846 tokens, 24 heads 179 /
+  // 188; 7800, 12 heads 248 / 254; 1100, 12 heads 18.5 / 22.2).  Long key ranges:
+  // the items of a last, partial wave are split along the key range so that
+  // they fill one wave together, and their partial results are merged.  Short
+  // key ranges: the persistent CTAs take all items, and the few CTAs that take
+  // one item more cost less than a split wave's start-up and merge (measured:
+  // 109 against 121 us for 32760 x 512 keys).
   const int slots = num_sms_attn() * C::CTAS_PER_SM;
   const int full = (items / slots) * slots, tail = items - full;
   int splits = tail > 0 ? std::min(std::min(kAttnPartCtas, slots) / tail, nkv_all) : 1;
   const size_t part_need = (size_t)tail * splits * kBQ * (D + 2) * sizeof(float);
-  const bool short_keys = nkv_all <= kPersistMaxKeyTiles;
-  const bool persist = D == 128 || short_keys;
+  const bool short_keys = x.nk <= 8 * D;
   const bool split_tail =
       !short_keys && full > 0 && tail > 0 && splits >= 2 && x.part != nullptr && x.part_bytes >= part_need;
   ProfScope prof(PROF_ATTENTION, 4.0 * (double)x.nq * (double)x.nk * D * x.heads, s);
   const int main_items = split_tail ? full : items;
-  if (persist) {
-    // output: 32-row x 32-column boxes, one per softmax warp and column chunk
-    CUtensorMap to;
-    ACID_TRY(make_tmap_bf16_box(&to, x.out, x.nq, x.ldo, x.ldo, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B));
-    a.item_end = main_items;
-    launch_pdl(attn_persist_kernel<D>, std::min(main_items, slots), kAttnThreads, C::SMEM_P, s, tq, tk, tv, to, a);
-  } else {
-    launch_pdl(attn_tc_kernel<D>, main_items, kAttnThreads, C::SMEM, s, tq, tk, tv, a);
-  }
+  // output: 32-row x 32-column boxes, one per softmax warp and column chunk
+  CUtensorMap to;
+  ACID_TRY(make_tmap_bf16_box(&to, x.out, x.nq, x.ldo, x.ldo, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B));
+  a.item_end = main_items;
+  launch_pdl(attn_persist_kernel<C>, std::min(main_items, slots), kAttnThreads, C::SMEM_P, s, tq, tk, tv, to, a);
   ACID_CHECK_LAUNCH();
   if (!split_tail) return ACID_OK;
   a.item_base = full;
   a.splits = splits;
   a.part_o = static_cast<float*>(x.part);
   a.part_ml = a.part_o + (size_t)tail * splits * kBQ * D;
-  launch_pdl(attn_tc_kernel<D>, tail * splits, kAttnThreads, C::SMEM, s, tq, tk, tv, a);
-  ACID_CHECK_LAUNCH();
-  launch_pdl(attn_merge_kernel<D>, tail * kBQ / 8, 256, 0, s, a, full, tail, splits);
-  ACID_CHECK_LAUNCH();
+  if constexpr (C::CTAS_PER_SM == 1) {
+    launch_pdl(attn_split_kernel<C>, tail * splits, kAttnThreads, C::SMEM, s, tq, tk, tv, a);
+    ACID_CHECK_LAUNCH();
+    launch_pdl(attn_merge_kernel<D>, tail * kBQ / 8, 256, 0, s, a, full, tail, splits);
+    ACID_CHECK_LAUNCH();
+  }
   return ACID_OK;
 }
 
@@ -1056,8 +1084,13 @@ acid_status attention_forward(int dtype, const AttnArgs& x, cudaStream_t s) {
   ACID_REQUIRE(x.q_col % 8 == 0 && x.k_col % 8 == 0 && x.v_col % 8 == 0 && x.o_col % 8 == 0 && x.ldo % 8 == 0,
                ACID_ERR_UNSUPPORTED, "attention bf16: column offsets must be multiples of 8");
   ACID_REQUIRE(aligned(x.out, 16), ACID_ERR_UNSUPPORTED, "attention bf16: output must be 16-byte aligned");
-  if (x.head_dim == 128) return launch_attn_tc<128>(x, s);
-  return launch_attn_tc<64>(x, s);
+  if (x.head_dim == 128) return launch_attn_tc<AttnCfg<128, 128>>(x, s);
+  // Measured at head dim 64 (us, 64-key / 128-key tiles), 17776 x 226 keys, 30
+  // heads: 45.0 / 53.6; 4726 x 400: 21.4 / 24.5; x 450: 23.7 / 24.5; x 512: 23.2 /
+  // 22.6; self-attention of 500 tokens 9.6 / 8.2, of 4726 tokens (64-key tiles,
+  // two CTAs on an SM, as every range took them once) 177 / 147.
+  if (x.nk <= 448) return launch_attn_tc<AttnCfg<64, 64>>(x, s);
+  return launch_attn_tc<AttnCfg<64, 128>>(x, s);
 }
 
 ACID_DEVICE_FLAG_READER(take_device_error_attention)
