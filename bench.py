@@ -42,12 +42,12 @@ MICRO_T = (32760, 67320, 118800)  # drift micro-benchmark rows (x 3072 bf16)
 MICRO_SIGMA = 1e-2
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum, ncu captures of
-# a self-attention call (main launch, split tail launch and merge) and a
+# a self-attention call (whole waves, split last wave and merge) and a
 # cross-attention call (one persistent launch) at this shape, each the mean of
-# two calls) per attention call of the step's 1:1 self/cross mix: 436.9 MB and
-# 159.2 MB.  Valid only for the kernel source it was measured on; any other
+# two calls) per attention call of the step's 1:1 self/cross mix: 431.5 MB and
+# 158.4 MB.  Valid only for the kernel source it was measured on; any other
 # source reports null.
-ATTN_TRAFFIC = {"source_sha256_16": "c918258b40c85349", "bytes_per_launch": (436.88e6 + 159.20e6) / 2}
+ATTN_TRAFFIC = {"source_sha256_16": "1f964e9ed980da0c", "bytes_per_launch": (431.50e6 + 158.42e6) / 2}
 
 
 def _attn_traffic():
