@@ -140,17 +140,34 @@ extern "C" const char* acid_version(void) { return "acid-gb300 0.1 (sm_103a)"; }
 
 namespace acid {
 namespace {
-// One thread waits on an mbarrier that no thread arrives on, through the
-// kernels' bounded wait with a short budget: the wait runs out, raises this
-// unit's device flag and the kernel returns.
+// At which of its steps each warp of wait_selftest_kernel left.
+__device__ int g_selftest_left[4];
+
+// Four warps take three steps together, voting after each (group_all).  In the
+// second, one of them waits on an mbarrier that no thread arrives on, through
+// the kernels' bounded wait with a short budget: the wait runs out and raises
+// this unit's device flag, and all four warps leave at that step, also the one
+// that idles after each vote while the others are a step ahead.
 __global__ void wait_selftest_kernel(long long limit) {
   __shared__ uint64_t bar;
+  const int warp = threadIdx.x >> 5;
   if (threadIdx.x == 0) {
     mbar_init(&bar, 1);
     mbar_fence_init();
   }
   __syncthreads();
-  if (threadIdx.x == 0) (void)mbar_wait_limit(&bar, 0, limit);
+  int step = 0;
+  for (; step < 3; ++step) {
+    const bool waits = step == 1 && warp == 2;
+    const bool go = group_all(1, 128, !waits || mbar_wait_limit(&bar, 0, limit));
+    if (warp == 0) {
+      const long long t0 = clock64(), idle = min(2 * limit, 1LL << 23);
+      while (clock64() - t0 < idle) {
+      }
+    }
+    if (!go) break;
+  }
+  if ((threadIdx.x & 31) == 0) g_selftest_left[warp] = step;
 }
 
 // Evaluates one index check one past the end of an extent of n, with no
@@ -196,9 +213,13 @@ extern "C" acid_status acid_selftest_wait_timeout(int64_t budget_cycles, acid_st
   ACID_REQUIRE(budget_cycles >= 1000 && budget_cycles <= 10000000000LL, ACID_ERR_INVALID_ARG,
                "acid_selftest_wait_timeout: budget must be 1e3..1e10 cycles");
   cudaStream_t s = (cudaStream_t)stream;
-  wait_selftest_kernel<<<1, 32, 0, s>>>((long long)budget_cycles);
+  wait_selftest_kernel<<<1, 128, 0, s>>>((long long)budget_cycles);
   ACID_CHECK_LAUNCH();
   ACID_CUDA(cudaStreamSynchronize(s));
+  int left[4];
+  ACID_CUDA(cudaMemcpyFromSymbol(left, g_selftest_left, sizeof(left)));
+  for (const int step : left)
+    ACID_REQUIRE(step == 1, ACID_ERR_TIMEOUT, "acid_selftest_wait_timeout: a group's warps did not leave together");
   return ACID_OK;
 }
 

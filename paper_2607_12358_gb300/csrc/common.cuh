@@ -341,6 +341,21 @@ __device__ __forceinline__ void cp_async_wait() {
 __device__ __forceinline__ void group_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
+// The same, and whether `vote` is true in all of them: one answer for the whole
+// group, which belongs to this barrier.  (A flag in shared memory read behind
+// the barrier can already hold what a faster warp found in its next round.)
+__device__ __forceinline__ bool group_all(int id, int threads, bool vote) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred v, a;\n\t"
+      "setp.ne.u32 v, %3, 0;\n\t"
+      "bar.red.and.pred a, %1, %2, v;\n\t"
+      "selp.u32 %0, 1, 0, a;\n\t}"
+      : "=r"(r)
+      : "r"(id), "r"(threads), "r"((uint32_t)vote)
+      : "memory");
+  return r != 0;
+}
 
 // ---------------------------------------------------------------------------
 // TMA (cp.async.bulk.tensor), 2D tiles, 128-byte swizzle

@@ -589,8 +589,6 @@ __global__ void __launch_bounds__(32 * (WPR == 1 ? kTemniMaxGroups : kTemniMaxWa
   uint64_t* full = reinterpret_cast<uint64_t*>(ring + (size_t)ngroups * kTemniStages * 2 * d);    // [group][stage]
   __shared__ double rd[2][kTemniMaxWarps];
   __shared__ float4 stats[2][kTemniMaxWarps];  // partial row sums, by row parity
-  __shared__ int gave_up[kTemniMaxWarps];      // by group
-  if (threadIdx.x < kTemniMaxWarps) gave_up[threadIdx.x] = 0;
   const int step = step_dev ? *step_dev : step_host;
   float* wr = ring + (size_t)grp * kTemniStages * 2 * d;
   uint64_t* wf = full + grp * kTemniStages;
@@ -671,9 +669,7 @@ __global__ void __launch_bounds__(32 * (WPR == 1 ? kTemniMaxGroups : kTemniMaxWa
     if constexpr (WPR > 1) {
       // the sums of row k + 2 overwrite these behind the barrier of row k + 1
       if (lane == 0) stats[k & 1][warp] = make_float4(s1c, s2c, s1p, s2p);
-      if (!ok && lane == 0) gave_up[grp] = 1;
-      group_sync(1 + grp, 32 * WPR);
-      if (gave_up[grp]) break;  // a wait of one of its warps ran out: the group leaves together
+      if (!group_all(1 + grp, 32 * WPR, ok)) break;  // a wait of one of its warps ran out: the group leaves together
       if (leader && k + kTemniStages < n_my) issue(k + kTemniStages);  // the whole group holds its values
       s1c = s2c = s1p = s2p = 0.f;
 #pragma unroll

@@ -1,7 +1,8 @@
 """Failure detection on the GPU without a fault: a bounded device wait that
 runs out (an mbarrier nothing arrives on, through the kernels' own wait
 routine with a short budget) must come back as ACID_ERR_TIMEOUT through
-acid_check_device_error, clear itself, and leave the context usable."""
+acid_check_device_error, clear itself, and leave the context usable.  The
+warps of a group whose wait runs out leave at the same step."""
 
 import numpy as np
 import pytest
@@ -40,4 +41,17 @@ def test_bounded_wait_reports_timeout_and_context_survives(acid):
     acid.acid_drift_signal(p, c, out_rel=rel)
     ref = O.rel_l1(S.round_to_bf16(prev).astype(np.float64), S.round_to_bf16(cur).astype(np.float64))
     assert abs(rel.item() - ref) <= 1e-3 * ref
+    acid.check_device_error()
+
+
+@pytest.mark.parametrize("budget", [1_000, 300_000])
+def test_group_of_warps_leaves_together(acid, budget):
+    """One warp's wait runs out in the second step while another warp still
+    idles behind the first step's vote (for longer than the budget)."""
+    from paper_2607_12358_gb300 import _capi as A
+
+    acid.selftest_wait_timeout(budget)  # raises if a warp left at another step
+    with pytest.raises(A.AcidError) as e:
+        acid.check_device_error()
+    assert e.value.status == A.ACID_ERR_TIMEOUT
     acid.check_device_error()
