@@ -16,6 +16,7 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -761,24 +762,52 @@ int num_sms() {
   return n;
 }
 
-// CTA pairs that can be resident at once for the pair kernel (clusters are
-// placed within a GPC, so this can be below half the SM count).
-template <int KIND, bool R32, bool O32>
-int max_pairs() {
-  static int n = -1;
-  if (n < 0) {
-    // the dynamic shared memory limit must be raised before the query
-    if (cudaFuncSetAttribute(gemm_tc2_kernel<KIND, R32, O32>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             Tc2Cfg::SMEM) != cudaSuccess)
-      return 0;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(2 * 76, 1, 1);
-    cfg.blockDim = dim3(kGemmThreads, 1, 1);
-    cfg.dynamicSmemBytes = Tc2Cfg::SMEM;
-    int c = 0;
-    n = (cudaOccupancyMaxActiveClusters(&c, gemm_tc2_kernel<KIND, R32, O32>, &cfg) == cudaSuccess && c > 0) ? c : 0;
+// An instance of the pair kernel and its count of CTA pairs that can be
+// resident at once (clusters are placed within a GPC, so this can be below half
+// the SM count), always positive on success.
+using PairKernel = decltype(&gemm_tc2_kernel<EPI_BIAS, false, false>);
+struct PairInstance {
+  PairKernel kernel;
+  acid_status (*pairs)(int* n);
+};
+
+template <int KIND, bool R32, bool O32, bool SPLIT>
+acid_status max_pairs(int* pairs) {
+  static std::atomic<int> known{0};  // a count once there is one; errors are asked again
+  *pairs = known.load(std::memory_order_relaxed);
+  if (*pairs > 0) return ACID_OK;
+  const PairKernel kernel = gemm_tc2_kernel<KIND, R32, O32, SPLIT>;
+  // the dynamic shared memory limit must be raised before the query (and the launch)
+  ACID_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Tc2Cfg::SMEM));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(2 * 76, 1, 1);
+  cfg.blockDim = dim3(kGemmThreads, 1, 1);
+  cfg.dynamicSmemBytes = Tc2Cfg::SMEM;
+  ACID_CUDA(cudaOccupancyMaxActiveClusters(pairs, kernel, &cfg));
+  ACID_REQUIRE(*pairs > 0, ACID_ERR_CUDA, "linear: no resident CTA pair for the pair GEMM");
+  known.store(*pairs, std::memory_order_relaxed);
+  return ACID_OK;
+}
+
+template <int KIND, bool R32, bool O32, bool SPLIT = false>
+PairInstance pair_instance() {
+  return {gemm_tc2_kernel<KIND, R32, O32, SPLIT>, max_pairs<KIND, R32, O32, SPLIT>};
+}
+
+// The instance that applies an epilogue.
+template <int KIND, bool R32 = false>
+PairInstance pair_instance_out(const Epilogue& e) {
+  return e.out_fp32 ? pair_instance<KIND, R32, true>() : pair_instance<KIND, R32, false>();
+}
+PairInstance pair_instance_for(const Epilogue& e) {
+  switch (e.kind) {
+    case EPI_GELU: return pair_instance_out<EPI_GELU>(e);
+    case EPI_ROPE_QKV: return pair_instance_out<EPI_ROPE_QKV>(e);
+    case EPI_GATED_RES:
+      return e.res_fp32 ? pair_instance_out<EPI_GATED_RES, true>(e) : pair_instance_out<EPI_GATED_RES>(e);
+    case EPI_RES: return e.res_fp32 ? pair_instance_out<EPI_RES, true>(e) : pair_instance_out<EPI_RES>(e);
+    default: return pair_instance_out<EPI_BIAS>(e);
   }
-  return n;
 }
 
 int64_t pair_row_tiles(int64_t M, int64_t text_rows) {
@@ -816,26 +845,21 @@ struct PairMaps {
   CUtensorMap a, b, o, r, bt, ot;
 };
 
-template <int KIND, bool R32, bool O32>
-acid_status launch_tc2_kind1(const PairMaps& t, const GemmDims& g, const Epilogue& epi, int64_t tiles, cudaStream_t s) {
-  const int pairs = max_pairs<KIND, R32, O32>();  // also raises the shared memory limit
-  ACID_REQUIRE(pairs > 0, ACID_ERR_CUDA, "linear: no resident CTA pair for the pair GEMM");
-  const int grid = 2 * (int)std::min<int64_t>(tiles, pairs);
-  launch_pdl(gemm_tc2_kernel<KIND, R32, O32>, grid, kGemmThreads, Tc2Cfg::SMEM, s, t.a, t.b, t.o, t.r, t.bt, t.ot, g, to_dev(epi));
+acid_status launch_pairs(PairKernel kernel, const PairMaps& t, const GemmDims& g, const Epilogue& epi, int64_t units,
+                         int pairs, cudaStream_t s) {
+  const int grid = 2 * (int)std::min<int64_t>(units, pairs);
+  launch_pdl(kernel, grid, kGemmThreads, Tc2Cfg::SMEM, s, t.a, t.b, t.o, t.r, t.bt, t.ot, g, to_dev(epi));
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
 
-template <int KIND, bool R32 = false>
-acid_status launch_tc2_kind(const PairMaps& t, const GemmDims& g, const Epilogue& epi, int64_t tiles, cudaStream_t s) {
-  return g.out_fp32 ? launch_tc2_kind1<KIND, R32, true>(t, g, epi, tiles, s)
-                    : launch_tc2_kind1<KIND, R32, false>(t, g, epi, tiles, s);
-}
-
 acid_status launch_tc2(const void* A, int64_t lda, int64_t M, int K, const void* W, int N, void* out, int64_t ldo,
                        const Epilogue& epi, cudaStream_t s) {
+  const PairInstance inst = pair_instance_for(epi);
+  int pairs = 0;
+  ACID_TRY(inst.pairs(&pairs));
   const int64_t m_tiles = pair_row_tiles(M, epi.text_rows);
-  const int bn = pick_bn(m_tiles, N, K, max_pairs<EPI_BIAS, false, false>());
+  const int bn = pick_bn(m_tiles, N, K, pairs);
   const bool res = epi_reads_res(epi.kind);
   PairMaps t;
   ACID_TRY(make_tmap_bf16(&t.a, A, M, K, lda, BM));
@@ -859,17 +883,7 @@ acid_status launch_tc2(const void* A, int64_t lda, int64_t M, int K, const void*
   }
   const int64_t tiles = m_tiles * ((N + bn - 1) / bn);
   ProfScope prof(PROF_LINEAR, 2.0 * (double)M * N * K, s);
-  switch (epi.kind) {
-    case EPI_GELU: return launch_tc2_kind<EPI_GELU>(t, g, epi, tiles, s);
-    case EPI_ROPE_QKV: return launch_tc2_kind<EPI_ROPE_QKV>(t, g, epi, tiles, s);
-    case EPI_GATED_RES:
-      return epi.res_fp32 ? launch_tc2_kind<EPI_GATED_RES, true>(t, g, epi, tiles, s)
-                          : launch_tc2_kind<EPI_GATED_RES, false>(t, g, epi, tiles, s);
-    case EPI_RES:
-      return epi.res_fp32 ? launch_tc2_kind<EPI_RES, true>(t, g, epi, tiles, s)
-                          : launch_tc2_kind<EPI_RES, false>(t, g, epi, tiles, s);
-    default: return launch_tc2_kind<EPI_BIAS>(t, g, epi, tiles, s);
-  }
+  return launch_pairs(inst.kernel, t, g, epi, tiles, pairs, s);
 }
 
 // ---------------------------------------------------------------------------
@@ -889,7 +903,7 @@ bool splitk_plan(int64_t M, int N, int K, size_t ws_bytes, int pairs, SplitKPlan
   constexpr int64_t bm = 2 * BM;
   const int64_t n_tiles = (N + Tc2Cfg::MAX_BN - 1) / Tc2Cfg::MAX_BN, m_tiles = (M + bm - 1) / bm;
   const int64_t tiles = m_tiles * n_tiles, num_kb = (K + BK - 1) / BK;
-  if (pairs <= 0 || num_kb < 64) return false;  // short mainloops: the last round is cheap
+  if (num_kb < 64) return false;  // short mainloops: the last round is cheap
   const int64_t full = tiles / pairs, last = tiles - full * pairs;
   if (full < 1 || last == 0 || 2 * last >= pairs) return false;
   const int64_t rows_main = (full * pairs / n_tiles) * bm;
@@ -960,18 +974,16 @@ acid_status launch_splitk_fixup_kind(const SplitKPlan& sp, const float* part, in
 // The split-K units of the tail rows [M rows of A], then the fixup into out.
 acid_status launch_tc2_splitk(const void* A, int64_t lda, int64_t M, int K, const void* W, int N, void* out,
                               int64_t ldo, const Epilogue& epi, const SplitKPlan& sp, cudaStream_t s) {
-  using Kern = decltype(&gemm_tc2_kernel<EPI_BIAS, false, true, true>);
-  const Kern kern = gemm_tc2_kernel<EPI_BIAS, false, true, true>;
-  static bool attr_done = false;
-  if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Tc2Cfg::SMEM));
-    attr_done = true;
-  }
+  const PairInstance inst = pair_instance<EPI_BIAS, false, true, true>();
+  int pairs = 0;
+  ACID_TRY(inst.pairs(&pairs));
   float* part = static_cast<float*>(epi.splitk_ws);
-  CUtensorMap ta, tb, to;
-  ACID_TRY(make_tmap_bf16(&ta, A, M, K, lda, BM));
-  ACID_TRY(make_tmap_bf16(&tb, W, N, K, K, Tc2Cfg::MAX_BN / 2));
-  ACID_TRY(make_tmap_out(&to, part, (int64_t)sp.splits * sp.m_pad, N, N, true));
+  PairMaps t;
+  ACID_TRY(make_tmap_bf16(&t.a, A, M, K, lda, BM));
+  ACID_TRY(make_tmap_bf16(&t.b, W, N, K, K, Tc2Cfg::MAX_BN / 2));
+  ACID_TRY(make_tmap_out(&t.o, part, (int64_t)sp.splits * sp.m_pad, N, N, true));
+  t.r = t.ot = t.o;
+  t.bt = t.b;
   GemmDims g{M, N, K, part, N, 1};  // 256 columns per tile
   g.splits = sp.splits;
   g.kb_split = sp.kb_split;
@@ -979,13 +991,9 @@ acid_status launch_tc2_splitk(const void* A, int64_t lda, int64_t M, int K, cons
   Epilogue raw;  // the accumulator as it is: no bias, fp32
   raw.out_fp32 = true;
   const int64_t units = ((M + 2 * BM - 1) / (2 * BM)) * ((N + Tc2Cfg::MAX_BN - 1) / Tc2Cfg::MAX_BN) * sp.splits;
-  const int pairs = max_pairs<EPI_BIAS, false, true>();
-  ACID_REQUIRE(pairs > 0, ACID_ERR_CUDA, "linear: no resident CTA pair for the pair GEMM");
   {
     ProfScope prof(PROF_LINEAR, 2.0 * (double)M * N * K, s);
-    launch_pdl(kern, 2 * (int)std::min<int64_t>(units, pairs), kGemmThreads, Tc2Cfg::SMEM, s, ta, tb, to, to, tb, to, g,
-                                                                                                  to_dev(raw));
-    ACID_CHECK_LAUNCH();
+    ACID_TRY(launch_pairs(inst.kernel, t, g, raw, units, pairs, s));
   }
   switch (epi.kind) {
     case EPI_GELU: return launch_splitk_fixup_kind<EPI_GELU>(sp, part, M, N, out, ldo, epi, s);
@@ -1206,8 +1214,10 @@ acid_status linear_forward(int dtype, const void* A, int64_t lda, int64_t M, int
   ACID_REQUIRE(epi.kind != EPI_ROPE_QKV || (epi.head_dim & (epi.head_dim - 1)) == 0, ACID_ERR_UNSUPPORTED,
                "linear bf16: the RoPE epilogue needs a power-of-two head_dim");
   SplitKPlan sp;
-  if (epi.splitk_ws != nullptr && aligned(epi.splitk_ws, 128) && epi.text_rows == 0 &&
-      splitk_plan(M, N, K, epi.splitk_bytes, max_pairs<EPI_BIAS, false, true>(), &sp)) {
+  int pairs = 0;
+  const bool may_split = epi.splitk_ws != nullptr && aligned(epi.splitk_ws, 128) && epi.text_rows == 0;
+  if (may_split) ACID_TRY(pair_instance_for(epi).pairs(&pairs));
+  if (may_split && splitk_plan(M, N, K, epi.splitk_bytes, pairs, &sp)) {
     ACID_TRY(launch_tc2(A, lda, sp.rows_main, K, W, N, out, ldo, epi, s));
     const size_t osz = epi.out_fp32 ? 4 : 2, rsz = epi.res_fp32 ? 4 : 2;
     Epilogue et = epi;
