@@ -730,26 +730,11 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(AttnDev a, int item0, i
   for (int i = 0; i < D / 32; ++i) op[i * 32 + lane] = __float2bfloat16_rn(acc[i] * inv);
 }
 
-int num_sms_attn() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-  }
-  return n;
-}
-
 template <class C>
 acid_status launch_attn_tc(const AttnArgs& x, cudaStream_t s) {
   constexpr int D = C::D;
-  static bool attr_done = false;
-  if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(attn_persist_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM_P));
-    if constexpr (C::CTAS_PER_SM == 1)
-      ACID_CUDA(cudaFuncSetAttribute(attn_split_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    attr_done = true;
-  }
+  static PerContext allowed, allowed_split;
+  ACID_TRY(allow_smem(allowed, attn_persist_kernel<C>, C::SMEM_P));
   CUtensorMap tq, tk, tv;
   ACID_TRY(make_tmap_bf16(&tq, x.q, x.nq, x.ldq, x.ldq, kTileQ));
   ACID_TRY(make_tmap_bf16(&tk, x.k, x.nk, x.ldk, x.ldk, C::BKV));
@@ -780,7 +765,7 @@ acid_status launch_attn_tc(const AttnArgs& x, cudaStream_t s) {
   // key ranges: the persistent CTAs take all items, and the few CTAs that take
   // one item more cost less than a split wave's start-up and merge (measured:
   // 109 against 121 us for 32760 x 512 keys).
-  const int slots = num_sms_attn() * C::CTAS_PER_SM;
+  const int slots = num_sms() * C::CTAS_PER_SM;
   const int full = (items / slots) * slots, tail = items - full;
   int splits = tail > 0 ? std::min(std::min(kAttnPartCtas, slots) / tail, nkv_all) : 1;
   const size_t part_need = (size_t)tail * splits * kBQ * (D + 2) * sizeof(float);
@@ -793,6 +778,9 @@ acid_status launch_attn_tc(const AttnArgs& x, cudaStream_t s) {
   CUtensorMap to;
   ACID_TRY(make_tmap_bf16_box(&to, x.out, x.nq, x.ldo, x.ldo, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B));
   a.item_end = main_items;
+  if constexpr (C::CTAS_PER_SM == 1) {
+    if (split_tail) ACID_TRY(allow_smem(allowed_split, attn_split_kernel<C>, C::SMEM));
+  }
   launch_pdl(attn_persist_kernel<C>, std::min(main_items, slots), kAttnThreads, C::SMEM_P, s, tq, tk, tv, to, a);
   ACID_CHECK_LAUNCH();
   if (!split_tail) return ACID_OK;
@@ -1046,11 +1034,8 @@ __global__ void __launch_bounds__(128 * kF32Groups) attn_f32_kernel(AttnF32Args 
 template <int D, int BQ>
 acid_status attn_f32_launch(const AttnF32Args& a, int heads, cudaStream_t s) {
   using C = AttnF32Cfg<D, BQ>;
-  static bool attr_done = false;
-  if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(attn_f32_kernel<D, BQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    attr_done = true;
-  }
+  static PerContext allowed;
+  ACID_TRY(allow_smem(allowed, attn_f32_kernel<D, BQ>, C::SMEM));
   const dim3 grid((unsigned)((a.nq + BQ - 1) / BQ), (unsigned)heads);
   launch_pdl(attn_f32_kernel<D, BQ>, grid, 128 * kF32Groups, C::SMEM, s, a);
   ACID_CHECK_LAUNCH();
@@ -1074,7 +1059,7 @@ acid_status launch_attn_f32(const AttnArgs& x, cudaStream_t s) {
   a.vec = aligned(a.q, 16) && aligned(a.k, 16) && aligned(a.v, 16) && x.ldq % 4 == 0 && x.ldk % 4 == 0 && x.ldv % 4 == 0;
   // 32-row tiles reuse each K and V value for twice the rows; 16-row tiles
   // while the 32-row ones would leave SMs without a CTA
-  if ((x.nq + 31) / 32 * x.heads < num_sms_attn()) return attn_f32_launch<D, 16>(a, x.heads, s);
+  if ((x.nq + 31) / 32 * x.heads < num_sms()) return attn_f32_launch<D, 16>(a, x.heads, s);
   return attn_f32_launch<D, 32>(a, x.heads, s);
 }
 

@@ -1,5 +1,6 @@
 // C-ABI entry points for the drift signal and cache apply, plus the
 // library-wide status plumbing.
+#include <cudaTypedefs.h>
 #include <math.h>
 
 #include <atomic>
@@ -37,6 +38,30 @@ std::vector<ProfRec> g_prof;
 void set_error(const std::string& msg) { t_last_error = msg; }
 void clear_error() { t_last_error.clear(); }
 void count_launch() { g_launches.fetch_add(1, std::memory_order_relaxed); }
+
+unsigned long long context_id() {
+  static const auto get_id = [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPointByVersion("cuCtxGetId", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+                    q == cudaDriverEntryPointSuccess;
+    return reinterpret_cast<PFN_cuCtxGetId_v12000>(ok ? p : nullptr);
+  }();
+  unsigned long long id = 0;
+  return get_id != nullptr && get_id(nullptr, &id) == CUDA_SUCCESS ? id : 0;
+}
+
+int num_sms() {
+  static PerContext known;
+  int n = 0;
+  const acid_status st = known.get(&n, [](int* v) {
+    int dev = 0;
+    ACID_CUDA(cudaGetDevice(&dev));
+    ACID_CUDA(cudaDeviceGetAttribute(v, cudaDevAttrMultiProcessorCount, dev));
+    return ACID_OK;
+  });
+  return st == ACID_OK && n > 0 ? n : 148;
+}
 
 ProfScope::ProfScope(int kind, double work, cudaStream_t s) : s_(s) {
   std::lock_guard<std::mutex> lk(g_prof_mu);

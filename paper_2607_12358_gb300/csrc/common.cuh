@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <utility>
 
@@ -37,6 +38,53 @@ void clear_error();
       return ACID_ERR_CUDA;                                                    \
     }                                                                          \
   } while (0)
+
+// Id of the calling thread's CUDA context, never given to another one; 0 if it
+// has none yet (or the driver cannot tell).
+unsigned long long context_id();
+
+// A number in 1 .. 65535 that is asked for once in each CUDA context (so for each
+// device, and again after a device reset): the kernels' shared memory opt-in,
+// which belongs to a device, and what was counted there.  Safe from several
+// threads: two that ask at once both call make, which has to allow that.  A
+// lookup takes 6 ns; cudaFuncSetAttribute at each launch would take 200.
+class PerContext {
+ public:
+  // make(&value) forms the number; a status other than ACID_OK is passed on and nothing is kept.
+  template <typename F>
+  acid_status get(int* value, F make) {
+    unsigned long long id = context_id();
+    const unsigned long long kept = slot_[id % kSlots].load(std::memory_order_acquire);
+    if (id != 0 && kept >> 16 == id) {
+      *value = (int)(kept & 0xffff);
+      return ACID_OK;
+    }
+    const acid_status st = make(value);
+    if (st != ACID_OK) return st;
+    id = context_id();  // make may have been this thread's first use of the device
+    if (id != 0 && *value > 0 && *value < 65536)
+      slot_[id % kSlots].store(id << 16 | (unsigned long long)*value, std::memory_order_release);
+    return ACID_OK;
+  }
+
+ private:
+  static constexpr int kSlots = 16;  // contexts that share a slot ask again
+  std::atomic<unsigned long long> slot_[kSlots] = {};
+};
+
+// Raises a kernel's dynamic shared memory limit where it has not been raised yet.
+template <typename K>
+acid_status allow_smem(PerContext& done, K kernel, size_t bytes) {
+  int yes;
+  return done.get(&yes, [&](int* v) {
+    *v = 1;
+    ACID_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+    return ACID_OK;
+  });
+}
+
+// SMs of the current device.
+int num_sms();
 
 // Counts every kernel launch of the library (acid_launch_count) and checks it.
 void count_launch();

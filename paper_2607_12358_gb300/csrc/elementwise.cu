@@ -15,16 +15,6 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kDriftMaxBlocks = 152 * 4;  // one wave of 4 CTAs per SM on GB300
 
-int num_sms_elem() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-  }
-  return n;
-}
-
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -1172,19 +1162,15 @@ acid_status launch_ln_rows(const LnArgs& a, cudaStream_t s) {
 template <typename Tin, typename Tout, int WPR, int NQ, bool FULL, int MODE>
 acid_status launch_ln_team(const LnArgs& a, cudaStream_t s) {
   constexpr size_t kSmemMax = 216 * 1024 / kLnCtas<WPR>;
-  static bool attr_done = false;
-  if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(ln_mod_team_kernel<Tin, Tout, WPR, NQ, FULL, MODE>,
-                                   cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
-    attr_done = true;
-  }
+  static PerContext allowed;
+  ACID_TRY(allow_smem(allowed, ln_mod_team_kernel<Tin, Tout, WPR, NQ, FULL, MODE>, kSmemMax));
   const size_t row = (size_t)a.d * (MODE == kLnPlain ? sizeof(Tin) : MODE == kLnReuse ? 8 : sizeof(Tin) + 4);
   // Two rows ahead keep HBM busy and its reads in order (bf16, 50000 x 3072: 93 us,
   // 109 with four); rows that largely stay in L2 are latency's, which four cover
   // (16000 x 1920: 19.5 us, 21.4 with two; the line lies between 154 and 200 MB).
   const double bytes = (double)a.rows * a.d * (sizeof(Tin) + sizeof(Tout));
   const int stages = row <= 6144 && bytes < 160e6 ? kLnMaxStages : 2;
-  const unsigned grid = (unsigned)std::min<int64_t>(a.rows, (int64_t)num_sms_elem() * kLnCtas<WPR>);
+  const unsigned grid = (unsigned)std::min<int64_t>(a.rows, (int64_t)num_sms() * kLnCtas<WPR>);
   launch_pdl(ln_mod_team_kernel<Tin, Tout, WPR, NQ, FULL, MODE>, grid, 32 * WPR, stages * row, s, a, stages);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
@@ -1233,12 +1219,8 @@ acid_status launch_temni_drift(const float* h_cur, const float* h_prev, const fl
                                const int* step_dev, int step_host, int64_t rows, int d, float eps, double2* parts,
                                unsigned int* done, double* result, cudaStream_t s, int* grid_out) {
   constexpr int kSmemMax = 225 * 1024;  // dynamic shared memory, below the 227 KB limit less the static part
-  static bool attr_done = false;
-  if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(temni_drift_kernel<NV4, WPR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   kSmemMax));
-    attr_done = true;
-  }
+  static PerContext allowed;
+  ACID_TRY(allow_smem(allowed, temni_drift_kernel<NV4, WPR>, kSmemMax));
   // groups per CTA: as many two-stage rings (8 d bytes per stage) as fit
   // beside the staged modulation vectors (16 d bytes), within the group and
   // warp limits
@@ -1246,7 +1228,7 @@ acid_status launch_temni_drift(const float* h_cur, const float* h_prev, const fl
   const int groups = (int)std::max<size_t>(1, std::min<size_t>(std::min(kTemniMaxGroups, kTemniMaxWarps / WPR),
                                                                (kSmemMax - 16 * (size_t)d) / ring_per_group));
   const size_t smem = 16 * (size_t)d + groups * ring_per_group;
-  const int grid = (int)std::min<int64_t>(std::min<int64_t>(kDriftMaxBlocks, (int64_t)num_sms_elem()),
+  const int grid = (int)std::min<int64_t>(std::min<int64_t>(kDriftMaxBlocks, (int64_t)num_sms()),
                                           std::max<int64_t>(1, (rows + groups - 1) / groups));
   launch_pdl(temni_drift_kernel<NV4, WPR>, grid, 32 * WPR * groups, smem, s, h_cur, h_prev, step_dev, step_host, rows, d,
              mod_cur, mod_cur + d, mod_prev, mod_prev + d, eps, parts, done, result);
@@ -1293,10 +1275,12 @@ acid_status launch_gemv(const GemvMat& m0, const GemvMat& m1, const float* x, in
   const int total = m0.n_out + m1.n_out;
   const size_t smem = sizeof(float) * k;
   // four rows per warp, on as many CTAs as are resident, once every SM gets two
-  auto grid = [&](int rows) { return std::min((total + kThreads / 32 * rows - 1) / (kThreads / 32 * rows), 152 * 3); };
-  if (total >= 152 * 2 * (kThreads / 32) * 4)
+  constexpr int kWarps = kThreads / 32;
+  const int sms = num_sms();
+  auto grid = [&](int rows) { return std::min((total + kWarps * rows - 1) / (kWarps * rows), sms * 3); };
+  if (total >= sms * 2 * kWarps * 4)
     launch_pdl(gemv_kernel<TW, 4>, grid(4), kThreads, smem, s, m0, m1, x, k, silu_input);
-  else if (total >= 152 * 2 * (kThreads / 32) * 2)
+  else if (total >= sms * 2 * kWarps * 2)
     launch_pdl(gemv_kernel<TW, 2>, grid(2), kThreads, smem, s, m0, m1, x, k, silu_input);
   else
     launch_pdl(gemv_kernel<TW, 1>, grid(1), kThreads, smem, s, m0, m1, x, k, silu_input);

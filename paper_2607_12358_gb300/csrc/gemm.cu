@@ -16,7 +16,6 @@
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -752,16 +751,6 @@ acid_status make_tmap_out(CUtensorMap* map, void* out, int64_t M, int N, int64_t
               : make_tmap_2d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, out, M, N, ldo, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
-int num_sms() {
-  static int n = 0;
-  if (n == 0) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-  }
-  return n;
-}
-
 // An instance of the pair kernel and its count of CTA pairs that can be
 // resident at once (clusters are placed within a GPC, so this can be below half
 // the SM count), always positive on success.
@@ -773,20 +762,19 @@ struct PairInstance {
 
 template <int KIND, bool R32, bool O32, bool SPLIT>
 acid_status max_pairs(int* pairs) {
-  static std::atomic<int> known{0};  // a count once there is one; errors are asked again
-  *pairs = known.load(std::memory_order_relaxed);
-  if (*pairs > 0) return ACID_OK;
-  const PairKernel kernel = gemm_tc2_kernel<KIND, R32, O32, SPLIT>;
-  // the dynamic shared memory limit must be raised before the query (and the launch)
-  ACID_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Tc2Cfg::SMEM));
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(2 * 76, 1, 1);
-  cfg.blockDim = dim3(kGemmThreads, 1, 1);
-  cfg.dynamicSmemBytes = Tc2Cfg::SMEM;
-  ACID_CUDA(cudaOccupancyMaxActiveClusters(pairs, kernel, &cfg));
-  ACID_REQUIRE(*pairs > 0, ACID_ERR_CUDA, "linear: no resident CTA pair for the pair GEMM");
-  known.store(*pairs, std::memory_order_relaxed);
-  return ACID_OK;
+  static PerContext known;
+  return known.get(pairs, [](int* n) {
+    const PairKernel kernel = gemm_tc2_kernel<KIND, R32, O32, SPLIT>;
+    // the dynamic shared memory limit must be raised before the query (and the launch)
+    ACID_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, Tc2Cfg::SMEM));
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2 * 76, 1, 1);
+    cfg.blockDim = dim3(kGemmThreads, 1, 1);
+    cfg.dynamicSmemBytes = Tc2Cfg::SMEM;
+    ACID_CUDA(cudaOccupancyMaxActiveClusters(n, kernel, &cfg));
+    ACID_REQUIRE(*n > 0, ACID_ERR_CUDA, "linear: no resident CTA pair for the pair GEMM");
+    return ACID_OK;
+  });
 }
 
 template <int KIND, bool R32, bool O32, bool SPLIT = false>
@@ -1150,11 +1138,8 @@ template <int TM, int TN>
 acid_status launch_f32(const float* A, int64_t lda, int64_t M, int K, const float* W, int N, float* out, int64_t ldo,
                        const Epilogue& epi, cudaStream_t s) {
   using C = F32Cfg<TM, TN>;
-  static bool attr_done = false;
-  if (!attr_done) {
-    ACID_CUDA(cudaFuncSetAttribute(gemm_f32_kernel<TM, TN>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM));
-    attr_done = true;
-  }
+  static PerContext allowed;
+  ACID_TRY(allow_smem(allowed, gemm_f32_kernel<TM, TN>, C::SMEM));
   const bool vec = aligned(A, 16) && aligned(W, 16) && lda % 4 == 0 && K % 4 == 0;
   const dim3 grid((unsigned)((N + TN - 1) / TN), (unsigned)((M + TM - 1) / TM));
   launch_pdl(gemm_f32_kernel<TM, TN>, grid, 64 * kFGroups, C::SMEM, s, A, lda, M, K, W, N, out, ldo, to_dev(epi), vec);

@@ -17,19 +17,39 @@ RUNTIME = r"""
 #include <cudaTypedefs.h>
 #include <cuda_runtime_api.h>
 #include <cstring>
+#include <set>
+#include <utility>
+
+static std::set<std::pair<const void*, int>> opted_in;  // (kernel, device)
+static cudaError_t last_error = cudaSuccess;
 
 extern "C" {
-// what the stand-in answers
-int fk_pairs = 76, fk_occupancy_error = 0;
+// what the stand-in answers; a device's context has the device's number + 1
+int fk_pairs = 76, fk_occupancy_error = 0, fk_device = 0, fk_attribute_error = 0;
 // what it was asked
 int fk_launches = 0, fk_grid = 0;
+
+cudaError_t cudaGetDevice(int* d) { *d = fk_device; return cudaSuccess; }
+cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
+  *a = {};
+  a->type = cudaMemoryTypeDevice;
+  a->devicePointer = const_cast<void*>(p);
+  return cudaSuccess;
+}
+cudaError_t cudaGetLastError() { return std::exchange(last_error, cudaSuccess); }
+cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute, int) {
+  if (fk_attribute_error == 0) opted_in.insert({f, fk_device});
+  return (cudaError_t)fk_attribute_error;
+}
 
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunchConfig_t*) {
   *n = fk_pairs;
   return (cudaError_t)fk_occupancy_error;
 }
-cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { *v = 152; return cudaSuccess; }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**) {
+cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int dev) { *v = dev == 0 ? 152 : 100; return cudaSuccess; }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+  // more than 48 KB of dynamic shared memory has to be asked for on each device
+  if (c->dynamicSmemBytes > 48 * 1024 && !opted_in.count({f, fk_device})) return last_error = cudaErrorInvalidValue;
   ++fk_launches;
   fk_grid = (int)c->gridDim.x;
   return cudaSuccess;
@@ -37,9 +57,12 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void*, void**
 static CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                        const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                        CUtensorMapL2promotion, CUtensorMapFloatOOBfill) { return CUDA_SUCCESS; }
+static CUresult ctx_id(CUcontext, unsigned long long* id) { *id = fk_device + 1; return CUDA_SUCCESS; }
 cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** fn, unsigned int, unsigned long long,
                                              cudaDriverEntryPointQueryResult* q) {
-  *fn = !std::strcmp(name, "cuTensorMapEncodeTiled") ? (void*)encode : nullptr;
+  *fn = !std::strcmp(name, "cuTensorMapEncodeTiled") ? (void*)encode
+        : !std::strcmp(name, "cuCtxGetId")           ? (void*)ctx_id
+                                                      : nullptr;
   *q = *fn ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
   return cudaSuccess;
 }
@@ -67,6 +90,12 @@ def linear(dtype=A.ACID_BF16, M=512, K=1536, N=3072, epi=A.ACID_EPI_BIAS, out_fp
     return lib.acid_linear_forward(dtype, p[0], K, M, K, p[1], None, N, p[2], N, epi,
                                    p[4] if epi == A.ACID_EPI_GATED_RES else None, p[3] if res else None,
                                    N if res else 0, out_fp32, None)
+def attention(dtype, nq, nk, heads, hd, ws=False):
+    w = heads * hd
+    return lib.acid_attention_forward(dtype, p[0], w, p[1], w, p[2], w, p[3], w, nq, nk, heads, hd,
+                                      p[4] if ws else None, 1 << 28 if ws else 0, None)
+def layernorm(tin, tout, rows, d): return lib.acid_layernorm_mod(tin, p[0], tout, p[1], rows, d, p[2], p[3], 1e-6, None)
+def temni(rows, d): return lib.acid_temni_drift(p[0], p[1], p[2], p[3], rows, d, 1e-6, p[4], None, p[5], 1 << 20, None)
 EPIS = (A.ACID_EPI_BIAS, A.ACID_EPI_GELU, A.ACID_EPI_GATED_RES, A.ACID_EPI_RES)
 """
 
@@ -127,4 +156,35 @@ for epi in EPIS:
     assert linear(M=32760, epi=epi) == A.ACID_OK
     assert (fk.launches, fk.grid) == (1, 2 * 76)
     fk.launches = 0
+""", *libs)
+
+
+def test_shared_memory_opt_in_on_every_device(libs):
+    """Every kernel's opt-in is made on each device that it is launched on, and made again after it failed."""
+    run("""
+B, F = A.ACID_BF16, A.ACID_FP32
+calls = [lambda d=d, i=i, o=o: layernorm(i, o, 5000, d) for d in (520, 1536, 1912, 1920, 3064, 3072) for i in (B, F) for o in (B, F)]
+calls += [lambda d=d: temni(5000, d) for d in (512, 1536, 1920, 3072)]
+calls += [lambda e=e, o=o: linear(epi=e, out_fp32=o) for e in EPIS for o in (0, 1)]
+calls += [lambda m=m: linear(F, M=m, K=256, N=256) for m in (16, 1000, 5000)]
+calls += [lambda n=n, h=h: attention(F, n, n, 4, h) for n in (64, 4000) for h in (32, 64, 96, 128)]
+calls += [lambda n=n, k=k, h=h: attention(B, n, k, 12, h, True) for n, k in ((4800, 300), (4800, 4800)) for h in (64, 128)]
+fk.attribute_error = 1
+for i, f in enumerate(calls):
+    assert f() in (A.ACID_OK, A.ACID_ERR_CUDA), i  # below 48 KB nothing has to be asked for
+fk.attribute_error = 0
+for dev in (0, 1, 0):
+    fk.device = dev
+    for i, f in enumerate(calls):
+        assert f() == A.ACID_OK, (dev, i, lib.acid_last_error())
+""", *libs)
+
+
+def test_grids_follow_the_device(libs):
+    """Persistent grids are sized to the SMs of the device that the call runs on."""
+    run("""
+for dev, sms in ((0, 152), (1, 100), (0, 152)):
+    fk.device = dev
+    assert layernorm(A.ACID_BF16, A.ACID_BF16, 100000, 3072) == A.ACID_OK and fk.grid == 4 * sms
+    assert attention(A.ACID_BF16, 30000, 512, 12, 128) == A.ACID_OK and fk.grid == sms
 """, *libs)
