@@ -91,20 +91,33 @@ static void prof_clear() {
   g_prof.clear();
 }
 
-bool is_device_pointer(const void* p) {
+namespace {
+// Where a caller's pointer leads: to memory of a device (or managed), and
+// whether a kernel on the current device may store there: memory of another
+// device is reached by copies alone unless the two are peers.
+struct PointerHome {
+  bool device = false, local = false;
+};
+PointerHome pointer_home(const void* p) {
   cudaPointerAttributes attr;
   if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
     cudaGetLastError();
-    return false;
+    return {};
   }
-  return attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged;
+  int dev = -1;
+  const bool local = attr.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess && dev == attr.device;
+  return {attr.type == cudaMemoryTypeDevice || attr.type == cudaMemoryTypeManaged, local};
 }
+}  // namespace
 
 DriftOutputs::DriftOutputs(double* rel_, double* sums_) : rel(rel_), sums(sums_) {
-  rel_dev = is_device_pointer(rel);
-  sums_dev = sums ? is_device_pointer(sums) : true;
-  if (rel_dev && aligned(rel, sizeof(double))) rel_direct = rel;
-  if (sums && sums_dev && aligned(sums, sizeof(double))) sums_direct = sums;
+  const PointerHome r = pointer_home(rel);
+  rel_dev = r.device;
+  if (r.local && aligned(rel, sizeof(double))) rel_direct = rel;
+  if (sums == nullptr) return;
+  const PointerHome u = pointer_home(sums);
+  sums_dev = u.device;
+  if (u.local && aligned(sums, sizeof(double))) sums_direct = sums;
 }
 
 acid_status DriftOutputs::finish(const double* d_result, cudaStream_t s) const {

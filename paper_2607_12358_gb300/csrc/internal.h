@@ -133,9 +133,9 @@ acid_status drift_launch(int dtype, const void* prev, const void* cur, const voi
                          double* sums_out = nullptr);
 
 // Delivers the results of a drift call, host side: which of the caller's
-// outputs the final kernel can write itself (device memory, aligned for a
-// double), and the copies of the others from d_result afterwards (to host
-// memory, which synchronises the stream).
+// outputs the final kernel can write itself (memory of the current device,
+// aligned for a double), and the copies of the others from d_result afterwards
+// (to host memory, which synchronises the stream).
 struct DriftOutputs {
   double *rel, *sums;                              // as the caller gave them (sums may be null)
   double *rel_direct = nullptr, *sums_direct = nullptr;  // for the kernel

@@ -28,12 +28,20 @@ extern "C" {
 int fk_pairs = 76, fk_occupancy_error = 0, fk_device = 0, fk_attribute_error = 0;
 // what it was asked
 int fk_launches = 0, fk_grid = 0;
+// device of the memory at 0x2......., its type (cudaMemoryType); copies there, and stores by the drift's final kernel
+int fk_home = 0, fk_type = cudaMemoryTypeDevice, fk_copies = 0, fk_stores = 0;
+#define OUTPUT(p) (((size_t)(p) >> 28) == 2)
 
 cudaError_t cudaGetDevice(int* d) { *d = fk_device; return cudaSuccess; }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
   *a = {};
-  a->type = cudaMemoryTypeDevice;
+  a->type = OUTPUT(p) ? (cudaMemoryType)fk_type : cudaMemoryTypeDevice;
+  a->device = OUTPUT(p) ? fk_home : fk_device;
   a->devicePointer = const_cast<void*>(p);
+  return cudaSuccess;
+}
+cudaError_t cudaMemcpyAsync(void* dst, const void*, size_t, cudaMemcpyKind, cudaStream_t) {
+  fk_copies += OUTPUT(dst);
   return cudaSuccess;
 }
 cudaError_t cudaGetLastError() { return std::exchange(last_error, cudaSuccess); }
@@ -47,11 +55,13 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunch
   return (cudaError_t)fk_occupancy_error;
 }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int dev) { *v = dev == 0 ? 152 : 100; return cudaSuccess; }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args) {
   // more than 48 KB of dynamic shared memory has to be asked for on each device
   if (c->dynamicSmemBytes > 48 * 1024 && !opted_in.count({f, fk_device})) return last_error = cudaErrorInvalidValue;
   ++fk_launches;
   fk_grid = (int)c->gridDim.x;
+  if (c->gridDim.x == 1 && c->blockDim.x == 256)  // drift_final_kernel(partials, nparts, result, rel_out, sums_out)
+    fk_stores += OUTPUT(*(void**)args[3]) + OUTPUT(*(void**)args[4]);
   return cudaSuccess;
 }
 static CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
@@ -187,4 +197,22 @@ for dev, sms in ((0, 152), (1, 100), (0, 152)):
     fk.device = dev
     assert layernorm(A.ACID_BF16, A.ACID_BF16, 100000, 3072) == A.ACID_OK and fk.grid == 4 * sms
     assert attention(A.ACID_BF16, 30000, 512, 12, 128) == A.ACID_OK and fk.grid == sms
+""", *libs)
+
+
+def test_drift_results_on_another_device_are_copied(libs):
+    """The final kernel stores to the caller's outputs where they are memory of the device that it runs on; memory of
+    another device, and managed memory, take the copies, which need no peer access."""
+    run("""
+rel, sums, n = 0x20000000, 0x20000100, 4096 * 3072
+calls = [lambda r, s: lib.acid_drift_signal(p[0], p[1], n, A.ACID_BF16, r, s, p[5], 1 << 20, None),
+         lambda r, s: lib.acid_drift_apply(p[0], p[1], p[2], p[3], n, A.ACID_BF16, r, s, p[5], 1 << 20, None),
+         lambda r, s: lib.acid_temni_drift(p[0], p[1], p[2], p[3], 4096, 3072, 1e-6, r, s, p[5], 1 << 20, None)]
+for f in calls:
+    for dev, home, kind, stores in ((0, 0, 2, 2), (0, 1, 2, 0), (1, 0, 2, 0), (1, 1, 2, 2), (0, 0, 3, 0)):
+        fk.device, fk.home, fk.type, fk.copies, fk.stores = dev, home, kind, 0, 0
+        assert f(rel, sums) == A.ACID_OK
+        assert (fk.stores, fk.copies) == (stores, 2 - stores), (dev, home, kind, fk.stores, fk.copies)
+    fk.device, fk.home, fk.type, fk.copies, fk.stores = 0, 0, 2, 0, 0
+    assert f(rel + 4, None) == A.ACID_OK and (fk.stores, fk.copies) == (0, 1)  # not aligned for a double
 """, *libs)
