@@ -4,6 +4,7 @@
 #include <string>
 
 #include "block.h"
+#define ACID_UNIT_WITHOUT_WAITS
 #include "common.cuh"
 #include "internal.h"
 

@@ -141,7 +141,9 @@ inline bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_
 
 // Device flag raised by a bounded wait that ran out (see acid_check_device_error).
 // One copy per translation unit (no relocatable device code); each unit that
-// waits exports a reader through ACID_DEVICE_FLAG_READER.
+// waits exports a reader through ACID_DEVICE_FLAG_READER.  A unit that defines
+// ACID_UNIT_WITHOUT_WAITS has neither the flag nor the functions that raise it.
+#ifndef ACID_UNIT_WITHOUT_WAITS
 static __device__ unsigned int g_device_error = 0;
 
 #define ACID_DEVICE_FLAG_READER(fname)                                              \
@@ -151,6 +153,7 @@ static __device__ unsigned int g_device_error = 0;
     if (v) cudaMemcpyToSymbol(g_device_error, &z, sizeof(z));                      \
     return v;                                                                      \
   }
+#endif
 
 // Debug builds (compiled with ACID_BOUNDS_CHECK, libacid_gb300_debug.so)
 // check the global-memory index of the kernels' hand-computed accesses
@@ -332,6 +335,7 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
 // About 4 s at 2 GHz: far above any legitimate wait in these kernels.
 constexpr long long kWaitLimitCycles = 8000000000LL;
 
+#ifndef ACID_UNIT_WITHOUT_WAITS
 // Returns false (and raises the device flag) if the phase did not complete
 // within `limit` SM clocks.  Callers stop their role's loop on false.
 __device__ __forceinline__ bool mbar_wait_limit(uint64_t* bar, uint32_t parity, long long limit) {
@@ -355,6 +359,7 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity) {
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity) {
   return __all_sync(0xffffffffu, mbar_wait(bar, parity));
 }
+#endif
 // Warp index as a value the compiler knows to be the same in all lanes.
 __device__ __forceinline__ int warp_index() { return __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0); }
 // True in one lane of the (converged) warp.
@@ -586,6 +591,7 @@ __device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t pa
       : "memory");
   return ok != 0;
 }
+#ifndef ACID_UNIT_WITHOUT_WAITS
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity) {
   if (mbar_try_wait_cluster(bar, parity)) return true;
   const long long t0 = clock64();
@@ -599,6 +605,7 @@ __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity
     }
   }
 }
+#endif
 // TMA tile load into this CTA's shared memory whose completion is counted on
 // an mbarrier that may live in either CTA of the pair (cluster address).
 __device__ __forceinline__ void tma_load_2d_pair(void* dst, const CUtensorMap* map, uint32_t bar_cluster, int x,

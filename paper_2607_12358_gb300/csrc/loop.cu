@@ -13,6 +13,7 @@
 #include <utility>
 
 #include "block.h"
+#define ACID_UNIT_WITHOUT_WAITS
 #include "common.cuh"
 #include "internal.h"
 

@@ -13,6 +13,7 @@
 #include <mutex>
 #include <string>
 
+#define ACID_UNIT_WITHOUT_WAITS
 #include "common.cuh"
 #include "internal.h"
 

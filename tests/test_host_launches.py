@@ -17,11 +17,17 @@ RUNTIME = r"""
 #include <cudaTypedefs.h>
 #include <cuda_runtime_api.h>
 #include <cstring>
+#include <map>
 #include <set>
 #include <utility>
 
 static std::set<std::pair<const void*, int>> opted_in;  // (kernel, device)
 static cudaError_t last_error = cudaSuccess;
+// the translation units' device error flags (g_device_error) by their host address, numbered as they are registered
+static std::map<const void*, int>& flags() {
+  static std::map<const void*, int> f;
+  return f;
+}
 
 extern "C" {
 // what the stand-in answers; a device's context has the device's number + 1
@@ -32,6 +38,22 @@ int fk_launches = 0, fk_grid = 0;
 int fk_home = 0, fk_type = cudaMemoryTypeDevice, fk_copies = 0, fk_stores = 0;
 #define OUTPUT(p) (((size_t)(p) >> 28) == 2)
 
+// which of the flags is raised; how many there are
+int fk_raised = -1, fk_flags = 0;
+void __cudaRegisterVar(void**, char* host, char*, const char* name, int, size_t, int, int) {
+  if (std::strstr(name, "g_device_error")) flags()[host] = fk_flags++;
+}
+cudaError_t cudaMemcpyFromSymbol(void* dst, const void* sym, size_t n, size_t, cudaMemcpyKind) {
+  std::memset(dst, 0, n);
+  const auto f = flags().find(sym);
+  if (f != flags().end() && f->second == fk_raised) *(unsigned*)dst = 1;
+  return cudaSuccess;
+}
+cudaError_t cudaMemcpyToSymbol(const void* sym, const void*, size_t, size_t, cudaMemcpyKind) {
+  const auto f = flags().find(sym);
+  if (f != flags().end() && f->second == fk_raised) fk_raised = -1;
+  return cudaSuccess;
+}
 cudaError_t cudaGetDevice(int* d) { *d = fk_device; return cudaSuccess; }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void* p) {
   *a = {};
