@@ -1,7 +1,8 @@
 """Bf16 attention at the edges of its kernels: the last short key range at head
 dim 64 and the first long one, tiles that just fill or overflow, one and two
 tiles per item on CTAs with several items, and rows whose max grows from tile
-to tile, so that the reference moves after P was formed."""
+to tile, so that the reference moves after P was formed, with the items of
+a partial last wave whole and, with a workspace, split along their keys."""
 
 import pytest
 
@@ -36,13 +37,15 @@ def test_attention_regions(acid, nq, nk, heads, hd, grow):
         q.view(nq, heads, hd)[:, :, 0] = (sign * hd ** 0.5)[:, None].to(torch.bfloat16)
         ramp = torch.linspace(0.0, grow, nk, device=DEV, dtype=torch.float32)
         k.view(nk, heads, hd)[:, :, 0] = ramp[:, None].to(torch.bfloat16)
-    got = acid.acid_attention_forward(q, k, v, heads).double()
+    ws = torch.empty(acid.attention_workspace_size(hd), dtype=torch.uint8, device=DEV)
+    outs = [acid.acid_attention_forward(q, k, v, heads, workspace=w).double() for w in (None, ws)]
     acid.check_device_error()
-    for h in (0, heads - 1):
+    for h in (0, heads - 1):  # the last head's items are in the last wave
         c = slice(h * hd, (h + 1) * hd)
         w = torch.softmax(q[:, c].double() @ k[:, c].double().T / hd ** 0.5, dim=1)
         ref = w @ v[:, c].double()
         # weights round to bf16 (2^-9) before P V; fp32 scores of magnitude up to
         # grow + 10 carry 2^-24 of it into the exponent; the output rounds once more
         tol = (2.0 ** -8 + (grow + 10.0) * 2.0 ** -20) * (w @ v[:, c].double().abs()) + 2.0 ** -8 * ref.abs() + 1e-6
-        assert torch.all((got[:, c] - ref).abs() <= tol)
+        for got in outs:
+            assert torch.all((got[:, c] - ref).abs() <= tol)

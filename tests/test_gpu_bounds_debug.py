@@ -6,9 +6,10 @@ an index outside it is recorded (acid_bounds_report) instead of accessed.
 
 The library is loaded in a child process (ACID_LIBRARY=debug), which runs
 every kernel family on small, ragged shapes: partial row and column tiles,
-single-SM and SM-pair GEMMs with each epilogue, head dims 64 and 128 with a
-split tail, odd LayerNorm widths, ragged drift lengths, a bf16 block of each
-joint kind, and loop steps of a bf16 and the fp32 model.  Each result is
+GEMMs with each epilogue and with one residual row for all, a block whose
+FFN2 ends in split-K units, head dims 64 and 128 with a split tail, odd
+LayerNorm widths, ragged drift lengths, a bf16 block of the Wan and of a joint
+kind, and loop steps of a bf16 and the fp32 model.  Each result is
 compared with the oracle, and no index check may have fired.  The self-test
 first shows that a check one past the end is recorded (with no access behind
 it), so a silent report means the checks ran."""
@@ -53,7 +54,7 @@ CHILD = textwrap.dedent(
         assert err <= rel_l2, (what, err)
 
     rng = np.random.default_rng(5)
-    # GEMMs: single-SM tiles (N <= 2048, K <= 2048) and SM pairs, every epilogue
+    # bf16 GEMMs, every epilogue
     for (M, K, N) in [(333, 192, 320), (130, 2176, 2304), (257, 64, 96)]:
         a = S.round_to_bf16(rng.normal(size=(M, K)).astype(np.float32))
         w = S.round_to_bf16((0.05 * rng.normal(size=(N, K))).astype(np.float32))
@@ -71,17 +72,31 @@ CHILD = textwrap.dedent(
                 acc = O.linear(a, w, b)
                 ref = {"bias": acc, "gelu": O.gelu_tanh(acc), "gated_res": r + g * acc, "res": r + acc}[epi]
                 close(out.float().cpu().numpy(), ref, 1e-2, ("linear", M, K, N, epi, fp32))
+    # a residual row that repeats for every output row (row stride 0: plain loads)
+    a = S.round_to_bf16(rng.normal(size=(333, 192)).astype(np.float32))
+    w = S.round_to_bf16((0.05 * rng.normal(size=(320, 192))).astype(np.float32))
+    r = S.round_to_bf16(rng.normal(size=(1, 320)).astype(np.float32))
+    for fp32 in (False, True):
+        res = (f32(r) if fp32 else bf(r)).expand(333, 320)
+        out = acid.acid_linear_forward(bf(a), bf(w), None, epilogue="res", residual=res, out_fp32=fp32)
+        close(out.float().cpu().numpy(), r + O.linear(a, w), 1e-2, ("linear, repeated residual", fp32))
     # fp32 GEMM (FP32 pipes)
     a = rng.normal(size=(77, 96)).astype(np.float32)
     w = (0.1 * rng.normal(size=(130, 96))).astype(np.float32)
     out = acid.acid_linear_forward(f32(a), f32(w), None)
     close(out.cpu().numpy(), O.linear(a, w), 1e-5, "linear fp32")
-    # attention: bf16 head dims 64 and 128 (long key ranges with the split tail
-    # and short ones on persistent CTAs), fp32
-    for (nq, nk, H, D) in [(1300, 1300, 2, 128), (700, 1100, 3, 64), (900, 300, 2, 128)]:
+    def launches(call):
+        before = acid.launch_count()
+        out = call()
+        return out, acid.launch_count() - before
+
+    # attention: bf16 head dims 64 and 128 (long key ranges with three or four items
+    # beyond the 152 of a whole wave, which are split and merged, and short ones), fp32
+    for (nq, nk, H, D) in [(1100, 1100, 31, 128), (700, 600, 52, 64), (900, 300, 2, 128)]:
         q, k, v = (S.round_to_bf16(rng.normal(size=(n, H * D)).astype(np.float32)) for n in (nq, nk, nk))
         ws = torch.empty(acid.attention_workspace_size(D), dtype=torch.uint8, device=dev)
-        out = acid.acid_attention_forward(bf(q), bf(k), bf(v), H, workspace=ws)
+        out, n = launches(lambda: acid.acid_attention_forward(bf(q), bf(k), bf(v), H, workspace=ws))
+        assert n == (3 if H > 2 else 1), ("launches", nq, nk, H, D, n)
         ref = O.attention(q.reshape(nq, H, D), k.reshape(nk, H, D), v.reshape(nk, H, D)).reshape(nq, H * D)
         close(out.float().cpu().numpy(), ref, 1e-2, ("attention", nq, nk, H, D))
     q, k, v = (rng.normal(size=(n, 2 * 64)).astype(np.float32) for n in (50, 70, 70))
@@ -109,7 +124,7 @@ CHILD = textwrap.dedent(
         o, rel, _ = acid.acid_drift_apply(f32(p), f32(c), f32(r))
         assert abs(rel.item() - O.rel_l1(p, c)) <= 1e-3 * O.rel_l1(p, c), ("drift apply", n)
         close(o.cpu().numpy(), c.astype(np.float64) + r, 1e-6, ("drift apply", n))
-    # TEMNI drift, rows in registers (d <= 1536) and re-read from the ring (d > 1536)
+    # TEMNI drift, one warp per row (d <= 1536) and four (d > 1536)
     for (rows, d) in [(301, 1920), (77, 512)]:
         hp = rng.normal(size=(rows, d)).astype(np.float32)
         hc = (hp + 0.05 * rng.normal(size=(rows, d))).astype(np.float32)
@@ -119,6 +134,23 @@ CHILD = textwrap.dedent(
         tp = O.modulate(O.layer_norm(hp), mp[:d], mp[d:])
         tc = O.modulate(O.layer_norm(hc), mc[:d], mc[d:])
         assert abs(rel.item() - O.rel_l1(tp, tc)) <= 1e-3 * O.rel_l1(tp, tc), ("temni", rows, d)
+    # a bf16 block whose FFN2 (K = 4096) runs 12 row tiles as one launch and the other 412 rows as split-K
+    # units with a fixup, and whose attention splits a tail: four launches more than on a short clip
+    cfg = S.get_config("toy", d=1536, heads=12, ffn=4096, latent_f=4, latent_h=26, latent_w=134, dtype="bf16")
+    w = S.block_weights(cfg, 0, seed=9, block_type="wan")
+    blk = acid.DeviceBlock.upload(w, "wan", torch.bfloat16, dev)
+    temb = S.temb_vector(cfg, seed=9)
+    counts = []
+    for c in (cfg, S.get_config("toy", d=1536, heads=12, ffn=4096, latent_f=1, latent_h=26, latent_w=134, dtype="bf16")):
+        x = S.hidden(c, c.n_video, seed=9)
+        tx = bf(x)
+        counts.append(launches(lambda: acid.acid_dit_block_forward(acid.block_desc(c, "wan"), tx, f32(temb), blk))[1])
+        if c is cfg:
+            assert c.n_video == 3484
+            at = np.array([0, 3070, 3071, 3072, 3073, 3483])
+            ref = O.wan_block(x, O.block_modulation(temb, w["mod"]), w, c.grid, c.heads, rows=at)
+            close(tx.float().cpu().numpy()[at], ref, 1e-2, "block, split-K FFN2")
+    assert counts[0] == counts[1] + 4, ("launches of a block", counts)
     # bf16 blocks: Wan (RoPE QKV, cross-attention) and the joint CogVideoX kind
     for kind in ("wan", "cog"):
         over = dict(d=256, heads=4 if kind == "cog" else 2, ffn=512, latent_f=3, latent_h=16, latent_w=22)

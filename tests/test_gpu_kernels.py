@@ -268,7 +268,7 @@ def test_attention_bf16(acid, nq, nk, H, D, qscale):
     assert np.abs(got - ref).max() <= 5e-2
 
 
-@pytest.mark.parametrize("nq,H,D", [(2560, 16, 128), (2048, 19, 64), (32760, 12, 128)])
+@pytest.mark.parametrize("nq,H,D", [(2560, 16, 128), (2048, 19, 64), (2560, 16, 64), (32760, 12, 128)])
 def test_attention_split_last_wave(acid, nq, H, D):
     """With a workspace, the work items of a partial last wave are split along
     the key range and merged; the result matches the oracle and the unsplit

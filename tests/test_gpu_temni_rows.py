@@ -25,7 +25,7 @@ def acid():
 
 
 # 1544 and 1920: the last of four vectors per lane only partly filled; 2048 and
-# 3072: every lane full; 2056 and 3064 on either side.  Three to eight groups a CTA
+# 3072: every lane full; 2056 and 3064 on either side.  Three or four groups a CTA
 # on 152 CTAs: 2500 rows give every group several, 5 rows leave most without one
 @pytest.mark.parametrize("d", [1544, 1920, 2048, 2056, 3064, 3072])
 @pytest.mark.parametrize("rows", [1, 5, 457, 2500])
