@@ -24,7 +24,8 @@
 // output leaves through shared memory and TMA stores.  attn_split_kernel runs
 // the items of a partial last wave, each split along its key range over
 // several CTAs, and attn_merge_kernel puts their parts together.
-// fp32 path: one warp per query row, exact expf, for the fp32 mode.
+// fp32 path: attn_f32_kernel, a tiled flash kernel on the FP32 pipes with exact
+// expf, for the fp32 mode.
 #include <cudaTypedefs.h>
 #include <math.h>
 
@@ -197,7 +198,8 @@ __device__ __forceinline__ bool softmax_tile(const AttnBars<C>& bar, int t, int 
   auto shift = [&](float me) {
     const uint64_t sh2 = f2_pack(-me, -me);
 #pragma unroll
-    for (int i = 0; i < C::BKV / 2; ++i) f2_unpack(f2_add(f2_pack(s[2 * i], s[2 * i + 1]), sh2), s[2 * i], s[2 * i + 1]);
+    for (int i = 0; i < C::BKV / 2; ++i)
+      f2_unpack(f2_add(f2_pack(s[2 * i], s[2 * i + 1]), sh2), s[2 * i], s[2 * i + 1]);
   };
   // P = 2^e as bf16 pairs over the first BKV/2 columns of S_t, and the row sum
   // as packed fp32 pairs
@@ -252,7 +254,11 @@ __device__ __forceinline__ bool softmax_tile(const AttnBars<C>& bar, int t, int 
     // max is formed on a row's first tile and then only for such a sum.  Where
     // it moves the reference, the warp writes its P again.  Without the max the
     // exponentials start as the scores are scaled: 4726 tokens, 30 heads 172.9 ->
-    // 158.9 us (with 96-key tiles).
+    // 158.9 us (with 96-key tiles).  A row that moves at every tile pays its
+    // exponentials twice: with scores that rise by 2^10 from tile to tile 290 us,
+    // where the max first takes 207 to 228 (64-key tiles).  A flag that lets a
+    // tile behind a move form its max first takes 211 there, but ordinary scores
+    // 151 instead of 147 and peaked ones 171 instead of 162, so there is none.
     auto max_of_e = [&] {
       float m4[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
 #pragma unroll
@@ -366,7 +372,8 @@ struct AttnMma {
   }
   // S_t = Q_t K^T of step g into its S region of tile t
   __device__ __forceinline__ void s_step(int t, int g) const {
-    issue_s_mma<C>(tmem + C::sb(t, g) * C::BKV, qdesc + (uint64_t)((t * C::T_BYTES) >> 4), kdesc + (uint64_t)((C::slot(g) * C::KV_BYTES) >> 4));
+    issue_s_mma<C>(tmem + C::sb(t, g) * C::BKV, qdesc + (uint64_t)((t * C::T_BYTES) >> 4),
+                   kdesc + (uint64_t)((C::slot(g) * C::KV_BYTES) >> 4));
     mma_commit(&bar.s_full[C::sb(t, g)]);
     if (t == 1) mma_commit(&bar.k_empty[C::slot(g)]);
   }
@@ -1056,7 +1063,8 @@ acid_status launch_attn_f32(const AttnArgs& x, cudaStream_t s) {
   a.nq = x.nq;
   a.nk = x.nk;
   a.scale = (float)(1.0 / sqrt((double)D));
-  a.vec = aligned(a.q, 16) && aligned(a.k, 16) && aligned(a.v, 16) && x.ldq % 4 == 0 && x.ldk % 4 == 0 && x.ldv % 4 == 0;
+  a.vec = aligned(a.q, 16) && aligned(a.k, 16) && aligned(a.v, 16) && x.ldq % 4 == 0 && x.ldk % 4 == 0 &&
+          x.ldv % 4 == 0;
   // 32-row tiles reuse each K and V value for twice the rows; 16-row tiles
   // while the 32-row ones would leave SMs without a CTA
   if ((x.nq + 31) / 32 * x.heads < num_sms()) return attn_f32_launch<D, 16>(a, x.heads, s);

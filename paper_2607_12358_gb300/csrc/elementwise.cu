@@ -900,7 +900,8 @@ struct PatchTile {
 // then forms the fp32-input patch embedding on tensor cores.  Otherwise fp32
 // tokens.
 template <bool SPLIT>
-__global__ void __launch_bounds__(kThreads) patchify_tile_kernel(const float* __restrict__ lat, void* tok, PatchGeo geo) {
+__global__ void __launch_bounds__(kThreads) patchify_tile_kernel(const float* __restrict__ lat, void* tok,
+                                                                 PatchGeo geo) {
   pdl_wait();
   extern __shared__ float tile[];
   const PatchTile t(geo);
@@ -1090,17 +1091,17 @@ acid_status drift_launch(int dtype, const void* prev, const void* cur, const voi
     using T = __nv_bfloat16;
     if (resid)
       launch_pdl(drift_partials_kernel<T, true>, grid, kThreads, 0, s, (const T*)prev, (const T*)cur, (const T*)resid,
-                                                              (T*)out, n, parts);
+                 (T*)out, n, parts);
     else
-      launch_pdl(drift_partials_kernel<T, false>, grid, kThreads, 0, s, (const T*)prev, (const T*)cur, nullptr, nullptr, n,
-                                                               parts);
+      launch_pdl(drift_partials_kernel<T, false>, grid, kThreads, 0, s, (const T*)prev, (const T*)cur, nullptr, nullptr,
+                 n, parts);
   } else {
     if (resid)
       launch_pdl(drift_partials_kernel<float, true>, grid, kThreads, 0, s, (const float*)prev, (const float*)cur,
-                                                                  (const float*)resid, (float*)out, n, parts);
+                 (const float*)resid, (float*)out, n, parts);
     else
-      launch_pdl(drift_partials_kernel<float, false>, grid, kThreads, 0, s, (const float*)prev, (const float*)cur, nullptr,
-                                                                   nullptr, n, parts);
+      launch_pdl(drift_partials_kernel<float, false>, grid, kThreads, 0, s, (const float*)prev, (const float*)cur,
+                 nullptr, nullptr, n, parts);
   }
   ACID_CHECK_LAUNCH();
   launch_pdl(drift_final_kernel, 1, kThreads, 0, s, parts, grid, d_result, rel_out, sums_out);
@@ -1113,7 +1114,7 @@ acid_status add_same(int dtype, const void* a, const void* b, void* out, int64_t
   const int grid = grid_for(n / V + 1, kThreads, 152 * 8);
   if (dtype == ACID_BF16)
     launch_pdl(add_vec_kernel<__nv_bfloat16>, grid, kThreads, 0, s, (const __nv_bfloat16*)a, (const __nv_bfloat16*)b,
-                                                            (__nv_bfloat16*)out, n);
+               (__nv_bfloat16*)out, n);
   else
     launch_pdl(add_vec_kernel<float>, grid, kThreads, 0, s, (const float*)a, (const float*)b, (float*)out, n);
   ACID_CHECK_LAUNCH();
@@ -1125,12 +1126,11 @@ acid_status add_mixed(int ad, const void* a, int bd, const void* b, int od, void
   using H = __nv_bfloat16;
   const bool vec = aligned(a, 16) && aligned(b, 16) && aligned(out, 16);
   const int grid = vec ? grid_for(n / 8 + 1, kThreads, 152 * 8) : grid_for(n);
-#define ACID_ADD(TA, TB, TO)                                                                                   \
-  (!vec ? launch_pdl(add_mixed_kernel<TA, TB, TO>, grid, kThreads, 0, s, (const TA*)a, (const TB*)b, (TO*)out, n, bs)  \
-   : bs == 0.0f                                                                                                \
-       ? launch_pdl(add_mixed8_kernel<TA, TB, TO, false>, grid, kThreads, 0, s, (const TA*)a, (const TB*)b, (TO*)out, n, \
-                                                                       bs)                                   \
-       : launch_pdl(add_mixed8_kernel<TA, TB, TO, true>, grid, kThreads, 0, s, (const TA*)a, (const TB*)b, (TO*)out, n, bs))
+#define ACID_ADD(TA, TB, TO)                                                                                     \
+  launch_pdl(!vec         ? add_mixed_kernel<TA, TB, TO>                                                         \
+             : bs == 0.0f ? add_mixed8_kernel<TA, TB, TO, false>                                                 \
+                          : add_mixed8_kernel<TA, TB, TO, true>,                                                 \
+             grid, kThreads, 0, s, (const TA*)a, (const TB*)b, (TO*)out, n, bs)
   const int key = ad * 4 + bd * 2 + od;  // ACID_BF16 = 0, ACID_FP32 = 1
   switch (key) {
     case 0: ACID_ADD(H, H, H); break;
@@ -1230,8 +1230,8 @@ acid_status launch_temni_drift(const float* h_cur, const float* h_prev, const fl
   const size_t smem = 16 * (size_t)d + groups * ring_per_group;
   const int grid = (int)std::min<int64_t>(std::min<int64_t>(kDriftMaxBlocks, (int64_t)num_sms()),
                                           std::max<int64_t>(1, (rows + groups - 1) / groups));
-  launch_pdl(temni_drift_kernel<NV4, WPR>, grid, 32 * WPR * groups, smem, s, h_cur, h_prev, step_dev, step_host, rows, d,
-             mod_cur, mod_cur + d, mod_prev, mod_prev + d, eps, parts, done, result);
+  launch_pdl(temni_drift_kernel<NV4, WPR>, grid, 32 * WPR * groups, smem, s, h_cur, h_prev, step_dev, step_host, rows,
+             d, mod_cur, mod_cur + d, mod_prev, mod_prev + d, eps, parts, done, result);
   ACID_CHECK_LAUNCH();
   *grid_out = grid;
   return ACID_OK;
@@ -1249,15 +1249,15 @@ acid_status temni_drift(const float* h_cur, const float* h_prev, const float* mo
   ProfScope prof(PROF_DRIFT, (double)rows * d * 8.0, s);  // read both steps' H_in (fp32)
   int grid = 1;
   auto run = [&](auto nv4, auto wpr) {
-    return launch_temni_drift<decltype(nv4)::value, decltype(wpr)::value>(h_cur, h_prev, mod_cur, mod_prev, step_dev,
-                                                                          step_host, rows, d, eps, parts, done, d_result,
-                                                                          s, &grid);
+    return launch_temni_drift<decltype(nv4)::value, decltype(wpr)::value>(
+        h_cur, h_prev, mod_cur, mod_prev, step_dev, step_host, rows, d, eps, parts, done, d_result, s, &grid);
   };
   using std::integral_constant;
   if (d <= 512)
     ACID_TRY(run(integral_constant<int, 4>{}, integral_constant<int, 1>{}));
   else if (d <= 1536)
-    ACID_TRY(run(integral_constant<int, 12>{}, integral_constant<int, 1>{}));  // 66.5 us at 32760 x 1536; two warps a row: 68.8
+    // 66.5 us at 32760 x 1536; two warps a row: 68.8
+    ACID_TRY(run(integral_constant<int, 12>{}, integral_constant<int, 1>{}));
   else if (d <= 2048)
     ACID_TRY(run(integral_constant<int, 4>{}, integral_constant<int, 4>{}));
   else
@@ -1327,8 +1327,8 @@ acid_status rope_build(RopeTable& t, float2* storage, float theta, cudaStream_t 
   const int64_t total = t.elems();
   if (total == 0) return ACID_OK;
   const dim3 grid((unsigned)((total + kTableThreads - 1) / kTableThreads), 2);
-  launch_pdl(rope_table_kernel, grid, kTableThreads, 0, s, storage, t.grid_f, t.grid_h, t.grid_w, t.pairs_t, t.pairs_h, t.pairs_w,
-                                                   (double)theta);
+  launch_pdl(rope_table_kernel, grid, kTableThreads, 0, s, storage, t.grid_f, t.grid_h, t.grid_w, t.pairs_t, t.pairs_h,
+             t.pairs_w, (double)theta);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1354,7 +1354,8 @@ acid_status patchify(const float* latent, float* tokens, int C, int F, int H, in
   if (patch_tiles(g, &grid, &smem))
     launch_pdl(patchify_tile_kernel<false>, grid, kThreads, smem, s, latent, (void*)tokens, g);
   else
-    launch_pdl(patchify_kernel, grid_for((int64_t)C * F * H * W), kThreads, 0, s, latent, tokens, C, F, H, W, pt, ph, pw);
+    launch_pdl(patchify_kernel, grid_for((int64_t)C * F * H * W), kThreads, 0, s, latent, tokens, C, F, H, W, pt, ph,
+               pw);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -1416,7 +1417,8 @@ acid_status euler_update_sig(float* latent, const float* v, int64_t n, const dou
 
 acid_status timestep_sinusoid_sig(float* out, const double* sig, const int* step, int dim, cudaStream_t s) {
   const int half = dim / 2;
-  launch_pdl(sinusoid_sig_kernel, dim3((half + kTableThreads - 1) / kTableThreads, 2), kTableThreads, 0, s, out, sig, step, half);
+  launch_pdl(sinusoid_sig_kernel, dim3((half + kTableThreads - 1) / kTableThreads, 2), kTableThreads, 0, s, out, sig,
+             step, half);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }

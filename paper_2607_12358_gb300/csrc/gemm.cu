@@ -86,7 +86,7 @@ __device__ __forceinline__ RopePos rope_pos(const RopeTable& t, int pos) {
 
 // Table entry (cos, sin) of the RoPE angle of pair `jj` (within the head) at a
 // decomposed position.
-__device__ __forceinline__ const float2& rope_cs_ptr(const RopeTable& t, const RopePos& p, int jj) {
+__device__ __forceinline__ const float2& rope_cs(const RopeTable& t, const RopePos& p, int jj) {
   if (jj < t.pairs_t) return t.table[p.f * t.pairs_t + jj];
   jj -= t.pairs_t;
   const int off_h = t.grid_f * t.pairs_t;
@@ -95,7 +95,6 @@ __device__ __forceinline__ const float2& rope_cs_ptr(const RopeTable& t, const R
   const int off_w = off_h + t.grid_h * t.pairs_h;
   return t.table[off_w + p.w * t.pairs_w + jj];
 }
-__device__ __forceinline__ float2 rope_cs(const RopeTable& t, const RopePos& p, int jj) { return rope_cs_ptr(t, p, jj); }
 // (debug builds) the table entry's index lies inside the table
 __device__ __forceinline__ bool rope_in_bounds(const RopeTable& t, const float2& e) {
   const int64_t n = (int64_t)t.grid_f * t.pairs_t + (int64_t)t.grid_h * t.pairs_h + (int64_t)t.grid_w * t.pairs_w;
@@ -108,7 +107,8 @@ __device__ __forceinline__ bool rope_in_bounds(const RopeTable& t, const float2&
 __device__ __forceinline__ void rope_cs16(const RopeTable& t, const RopePos& p, int j0, float2* cs) {
   const int end_t = t.pairs_t, end_h = end_t + t.pairs_h;
   const int off_h = t.grid_f * t.pairs_t, off_w = off_h + t.grid_h * t.pairs_h;
-  const int base_t = p.f * t.pairs_t, base_h = off_h + p.h * t.pairs_h - end_t, base_w = off_w + p.w * t.pairs_w - end_h;
+  const int base_t = p.f * t.pairs_t;
+  const int base_h = off_h + p.h * t.pairs_h - end_t, base_w = off_w + p.w * t.pairs_w - end_h;
 #pragma unroll
   for (int k = 0; k < 16; ++k) {
     const int jj = j0 + k;
@@ -163,9 +163,6 @@ constexpr int kGemmThreads = 64 + 32 * kEpiWarps;
 struct GemmDims {
   int64_t M;
   int N, K;
-  void* out;
-  int64_t ldo;
-  int out_fp32;
   // split-K launches only: work unit = (tile, split); split s covers k-blocks
   // [s kb_split, (s + 1) kb_split) and stores its raw fp32 accumulator at
   // rows s m_pad + row of the partial buffer
@@ -228,8 +225,7 @@ __device__ __forceinline__ void load_bias32(const float* src, int col0, float* b
 // Shared-memory traffic is one write and one TMA read of the box.  The caller
 // makes sure the store that last read this stage has finished reading.
 template <int KIND, bool O32>
-__device__ __forceinline__ void epilogue_rows(const GemmDims& g, const EpiDev& e, const CUtensorMap* tmO,
-                                              uint8_t* stage, int64_t row0, int64_t store_row0, int col0,
+__device__ __forceinline__ void epilogue_rows(const CUtensorMap* tmO, uint8_t* stage, int64_t store_row0, int col0,
                                               const uint32_t* r, const float* bias, const float2* cs) {
   const int lane = threadIdx.x & 31;
   uint64_t v[16];
@@ -268,7 +264,8 @@ __device__ __forceinline__ void epilogue_rows(const GemmDims& g, const EpiDev& e
         f2_unpack(v[4 * u + q], a0, a1);
         w[q] = pack_bf16(a0, a1);
       }
-      *reinterpret_cast<uint4*>(stage + lane * 64 + ((u ^ ((lane >> 1) & 3)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+      *reinterpret_cast<uint4*>(stage + lane * 64 + ((u ^ ((lane >> 1) & 3)) << 4)) =
+          make_uint4(w[0], w[1], w[2], w[3]);
     }
   }
   fence_proxy_async_smem();
@@ -300,7 +297,8 @@ __device__ __forceinline__ void tma_kind_chunk(const GemmDims& g, const EpiDev& 
     if (rotate) {
       const int64_t row = row0 + lane, grow = row + e.row_base;
       const bool video = grow >= e.rope_first_video && row < g.M;
-      rope_cs16(e.rope, rope_pos(e.rope, video ? (int)(grow - e.rope_first_video) : 0), (col0 & (e.head_dim - 1)) >> 1, cs);
+      const RopePos pos = rope_pos(e.rope, video ? (int)(grow - e.rope_first_video) : 0);
+      rope_cs16(e.rope, pos, (col0 & (e.head_dim - 1)) >> 1, cs);
       if (!video) {
 #pragma unroll
         for (int k = 0; k < 16; ++k) cs[k] = make_float2(1.f, 0.f);
@@ -317,7 +315,7 @@ __device__ __forceinline__ void tma_kind_chunk(const GemmDims& g, const EpiDev& 
     if (lane == 0) bulk_wait_group_read<1>();
   }
   __syncwarp();
-  epilogue_rows<KIND, O32>(g, e, tmO, st, row0, store_row0, col0, r, bias, rotate ? cs : nullptr);
+  epilogue_rows<KIND, O32>(tmO, st, store_row0, col0, r, bias, rotate ? cs : nullptr);
   ++nstore;
 }
 
@@ -331,9 +329,9 @@ __device__ __forceinline__ void tma_kind_chunk(const GemmDims& g, const EpiDev& 
 // one into the other box, once the store that last used it has read it.
 // Returns false if the wait ran out.
 template <int KIND, bool R32, bool O32, typename Next>
-__device__ __forceinline__ bool res_kind_chunk(const GemmDims& g, const EpiDev& e, const CUtensorMap* tmO, uint8_t* box, uint64_t* box_full,
-                                               uint32_t phase, uint32_t taddr, int64_t row0, int col0,
-                                               const float* bias_src, Next next) {
+__device__ __forceinline__ bool res_kind_chunk(const GemmDims& g, const EpiDev& e, const CUtensorMap* tmO, uint8_t* box,
+                                               uint64_t* box_full, uint32_t phase, uint32_t taddr, int64_t row0,
+                                               int col0, const float* bias_src, Next next) {
   const int lane = threadIdx.x & 31;
   uint32_t r[32];
   float bv[32], gv[32];
@@ -429,8 +427,9 @@ __device__ __forceinline__ bool res_kind_chunk(const GemmDims& g, const EpiDev& 
 //            then arrives on rank 0's acc_empty[b], which counts the epilogue
 //            warps of both CTAs.
 //   What bounds it: long mainloops run into the power cap (FFN1 at 32760 rows,
-// 1536 -> 8960 with GELU: 521 us, 1730 TFLOP/s, at about 1.45 GHz; 571 us before
-// the issue loops below kept to uniform registers).  A k-step's floor is the
+// 1536 -> 8960 with GELU: 529 to 545 us on several GPUs, 1650 to 1705 TFLOP/s, at
+// 1.42 to 1.48 GHz, and 477 us in runs of 20 ms; 579 to 590 us before the issue
+// loops below kept to uniform registers).  A k-step's floor is the
 // issue of its loads and MMAs: 240 SM clocks at bn = 32, where it was 580.
 // ===========================================================================
 struct Tc2Cfg {
@@ -660,14 +659,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kGemmThreads, 1)
           tma_kind_chunk<KIND, O32>(g, e, to, stage, taddr, row0, store_row0, col0, bias, live, nstore);
         } else if (live) {
           const int x = nchunk & 1;
-          ok = res_kind_chunk<KIND, R32, O32>(g, e, to, stage + x * 4096, &rfull[x], (nchunk >> 1) & 1, taddr, row0, col0,
-                                              bias, [&]() {
-                                                // the other box: its chunk's store was issued one chunk ago
-                                                if (lane == 0 && nchunk > 0) {
-                                                  bulk_wait_group_read<0>();
-                                                  if (!g.res_direct) load_next();
-                                                }
-                                              });
+          auto next = [&]() {  // the other box: its chunk's store was issued one chunk ago
+            if (lane == 0 && nchunk > 0) {
+              bulk_wait_group_read<0>();
+              if (!g.res_direct) load_next();
+            }
+          };
+          ok = res_kind_chunk<KIND, R32, O32>(g, e, to, stage + x * 4096, &rfull[x], (nchunk >> 1) & 1, taddr, row0,
+                                              col0, bias, next);
           if (!ok) break;
           ++nchunk;
         }
@@ -747,8 +746,10 @@ namespace {
 // swizzle of the box layout in epilogue_rows (128-byte rows for fp32,
 // 64-byte rows for bf16).
 acid_status make_tmap_out(CUtensorMap* map, void* out, int64_t M, int N, int64_t ldo, bool fp32) {
-  return fp32 ? make_tmap_2d(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, out, M, N, ldo, 32, 32, CU_TENSOR_MAP_SWIZZLE_128B)
-              : make_tmap_2d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, out, M, N, ldo, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
+  return fp32 ? make_tmap_2d(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, out, M, N, ldo, 32, 32,
+                             CU_TENSOR_MAP_SWIZZLE_128B)
+              : make_tmap_2d(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, out, M, N, ldo, 32, 32,
+                             CU_TENSOR_MAP_SWIZZLE_64B);
 }
 
 // An instance of the pair kernel and its count of CTA pairs that can be
@@ -807,11 +808,12 @@ int64_t pair_row_tiles(int64_t M, int64_t text_rows) {
 // on the tensor cores plus about 75, and not below its issue cost; each tile
 // adds about 500 and the last tile's epilogue 700 per pair of 32-column
 // chunks.  Narrower tiles win where a last round of 256-wide ones leaves pairs
-// idle.  Measured (us, CUDA events) at 256 columns and at the width chosen:
-// 7797 x 1920 x 1920 (M x K x N) gated residual 44.8, 40.4 at 160; 7800 x 1536 x
-// 4608 67.1, 63.0 at 192; 512 x 1536 x 3072 16.9, 11.4 at 96; 64 x 8960 x 1536
-// 49.6, 22.6 at 32; the wide layers of a 480p step stay at 256 (1536 -> 8960:
-// 521 us against 542 at 224).
+// idle.  Measured at 256 columns and at the width chosen (us a call, back to back
+// over inputs that change, in runs too short for the power cap; calls below 10 us
+// are bound by the calling program): 7797 x 1920 x 1920 (M x K x N) gated residual
+// 43.6, 39.3 at 160 (41.7 at 128, 42.3 at 192); 7800 x 1536 x 4608 66.7, 65.4 at
+// 192; 512 x 1536 x 3072 13.2, 9.3 at 96; 64 x 8960 x 1536 45.6, 22.9 at 32; the
+// widest layer of a 480p step stays at 256 (1536 -> 8960: 477 against 481 at 224).
 int pick_bn(int64_t m_tiles, int N, int K, int pairs) {
   const int64_t num_kb = (K + BK - 1) / BK;
   int best = Tc2Cfg::MAX_BN;
@@ -859,7 +861,7 @@ acid_status launch_tc2(const void* A, int64_t lda, int64_t M, int K, const void*
     ACID_TRY(make_tmap_out(&t.r, const_cast<void*>(epi.residual), M, N, epi.ldr, epi.res_fp32));
   t.bt = t.b;
   t.ot = t.o;
-  GemmDims g{M, N, K, out, ldo, epi.out_fp32 ? 1 : 0};
+  GemmDims g{M, N, K};
   g.bn = bn;
   g.stages = Tc2Cfg::stages(bn, res);
   g.res_direct = res_direct;
@@ -928,7 +930,8 @@ __global__ void __launch_bounds__(256) splitk_fixup_kernel(const float* __restri
         r0 = rv.x;
         r1 = rv.y;
       } else {
-        const uint32_t rv = *reinterpret_cast<const uint32_t*>(static_cast<const __nv_bfloat16*>(e.res) + row * e.ldr + col);
+        const __nv_bfloat16* res = static_cast<const __nv_bfloat16*>(e.res) + row * e.ldr + col;
+        const uint32_t rv = *reinterpret_cast<const uint32_t*>(res);
         r0 = bf16_lo(rv);
         r1 = bf16_hi(rv);
       }
@@ -947,7 +950,8 @@ acid_status launch_splitk_fixup(const SplitKPlan& sp, const float* part, int64_t
                                 const Epilogue& epi, cudaStream_t s) {
   const int64_t total = M * (N / 2);
   const int grid = (int)std::min<int64_t>((total + 255) / 256, (int64_t)num_sms() * 8);
-  launch_pdl(splitk_fixup_kernel<KIND, R32, O32>, grid, 256, 0, s, part, sp.splits, sp.m_pad, M, N, out, ldo, to_dev(epi));
+  launch_pdl(splitk_fixup_kernel<KIND, R32, O32>, grid, 256, 0, s, part, sp.splits, sp.m_pad, M, N, out, ldo,
+             to_dev(epi));
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -972,7 +976,7 @@ acid_status launch_tc2_splitk(const void* A, int64_t lda, int64_t M, int K, cons
   ACID_TRY(make_tmap_out(&t.o, part, (int64_t)sp.splits * sp.m_pad, N, N, true));
   t.r = t.ot = t.o;
   t.bt = t.b;
-  GemmDims g{M, N, K, part, N, 1};  // 256 columns per tile
+  GemmDims g{M, N, K};  // 256 columns per tile
   g.splits = sp.splits;
   g.kb_split = sp.kb_split;
   g.m_pad = sp.m_pad;

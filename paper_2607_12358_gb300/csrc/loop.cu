@@ -50,8 +50,8 @@ struct LoopWs {
   double* dres;     // [8] device drift results
   uint8_t* drift_ws;
   unsigned int* drift_done;  // TEMNI drift: CTAs finished (zero between launches)
-  // bf16 models with P % 8 == 0: the patch embedding runs on tensor cores
-  // against the patch weights repeated along K, [d, 2P] bf16
+  // bf16 models: the patch embedding runs on tensor cores against the patch
+  // weights repeated along K, [d, 2P] bf16
   bool patch_split;
   uint8_t* patch_w2;
   float2* rope;
@@ -143,7 +143,7 @@ LoopWs loop_layout(const acid_model& m, void* base) {
   w.dres = b.take<double>(8);
   w.drift_ws = b.take<uint8_t>(drift_workspace_bytes(0));
   w.drift_done = b.take<unsigned int>(1);
-  w.patch_split = dt == ACID_BF16 && s.P % 8 == 0;
+  w.patch_split = dt == ACID_BF16;
   w.patch_w2 = b.take<uint8_t>(w.patch_split ? (size_t)s.d * 2 * s.P * 2 : 0);
   RopeTable rt = rope_layout(m.block.grid_f, m.block.grid_h, m.block.grid_w, m.block.d / std::max(1, m.block.heads));
   w.rope = b.take<float2>((size_t)rt.elems());
@@ -341,10 +341,11 @@ int elem_grid(int64_t n) { return (int)std::min<int64_t>(152 * 16, std::max<int6
 
 acid_status dicache_update(int dt, const void* h_out, const float* p_t, const LoopWs& w, int64_t n, cudaStream_t s) {
   if (dt == ACID_BF16)
-    launch_pdl(dicache_update_kernel<__nv_bfloat16>, elem_grid(n), 256, 0, s, static_cast<const __nv_bfloat16*>(h_out), p_t, w.resid, w.dc_d2, w.dc_p1, w.dc_p2, n, w.dc_count);
+    launch_pdl(dicache_update_kernel<__nv_bfloat16>, elem_grid(n), 256, 0, s, static_cast<const __nv_bfloat16*>(h_out),
+               p_t, w.resid, w.dc_d2, w.dc_p1, w.dc_p2, n, w.dc_count);
   else
     launch_pdl(dicache_update_kernel<float>, elem_grid(n), 256, 0, s, static_cast<const float*>(h_out), p_t, w.resid,
-                                                              w.dc_d2, w.dc_p1, w.dc_p2, n, w.dc_count);
+               w.dc_d2, w.dc_p1, w.dc_p2, n, w.dc_count);
   ACID_CHECK_LAUNCH();
   launch_pdl(dicache_count_kernel, 1, 1, 0, s, w.dc_count);
   ACID_CHECK_LAUNCH();
@@ -358,11 +359,11 @@ acid_status dicache_reuse(int dt, void* out, const float* p_t, const LoopWs& w, 
   ACID_TRY(drift_launch(ACID_FP32, w.dc_p2, w.dc_p1, nullptr, nullptr, n, w.dres + 3, w.drift_ws,
                         drift_workspace_bytes(0), s));
   if (dt == ACID_BF16)
-    launch_pdl(dicache_reuse_kernel<__nv_bfloat16>, elem_grid(n), 256, 0, s, static_cast<__nv_bfloat16*>(out), p_t, w.resid,
-                                                                     w.dc_d2, n, w.dres + 1, w.dres + 4);
+    launch_pdl(dicache_reuse_kernel<__nv_bfloat16>, elem_grid(n), 256, 0, s, static_cast<__nv_bfloat16*>(out), p_t,
+               w.resid, w.dc_d2, n, w.dres + 1, w.dres + 4);
   else
     launch_pdl(dicache_reuse_kernel<float>, elem_grid(n), 256, 0, s, static_cast<float*>(out), p_t, w.resid, w.dc_d2, n,
-                                                            w.dres + 1, w.dres + 4);
+               w.dres + 1, w.dres + 4);
   ACID_CHECK_LAUNCH();
   return ACID_OK;
 }
@@ -511,8 +512,8 @@ static acid_status patch_embed(const acid_model& m, const LoopWs& w, const float
     ACID_TRY(patchify_split(latent, w.tokens, m.latent_c, m.latent_f, m.latent_h, m.latent_w, m.pt, m.ph, m.pw, s));
     return linear_forward(ACID_BF16, w.tokens, 2 * sh.P, sh.N, (int)(2 * sh.P), w.patch_w2, sh.d, h_in, sh.d, e, s);
   }
-  ACID_REQUIRE(m.block.dtype == ACID_FP32, ACID_ERR_UNSUPPORTED, "patch embedding: bf16 needs P % 8 == 0");
-  ACID_TRY(patchify(latent, reinterpret_cast<float*>(w.tokens), m.latent_c, m.latent_f, m.latent_h, m.latent_w, m.pt, m.ph, m.pw, s));
+  ACID_TRY(patchify(latent, reinterpret_cast<float*>(w.tokens), m.latent_c, m.latent_f, m.latent_h, m.latent_w, m.pt,
+                    m.ph, m.pw, s));
   return linear_forward_f32(w.tokens, sh.P, sh.N, (int)sh.P, m.patch.w, sh.d, h_in, sh.d, e, s);
 }
 
