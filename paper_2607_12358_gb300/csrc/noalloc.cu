@@ -8,8 +8,6 @@
 // three results) lives in the file-scope array below instead of a
 // caller-provided workspace.  Every GPU that loads this library holds the
 // array until the process exits.
-#include <cudaTypedefs.h>
-
 #include <mutex>
 #include <string>
 
@@ -38,52 +36,28 @@ static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratch
 
 std::mutex g_mu;
 struct ScratchSlot {
-  CUcontext ctx;  // context the address belongs to
+  unsigned long long ctx;  // id of the context that the address belongs to
   void* addr;
 };
 ScratchSlot g_slot[kMaxDevices] = {};
 
-// cuCtxGetCurrent through the runtime's driver entry-point query (the library
-// does not link the driver API).
-PFN_cuCtxGetCurrent_v4000 ctx_get_current() {
-  static PFN_cuCtxGetCurrent_v4000 fn = nullptr;
-  static std::once_flag once;
-  std::call_once(once, [] {
-    void* p = nullptr;
-    cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuCtxGetCurrent", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-        q == cudaDriverEntryPointSuccess)
-      fn = reinterpret_cast<PFN_cuCtxGetCurrent_v4000>(p);
-  });
-  return fn;
-}
-
 // Device address of the scratch array in the current device's context (host
 // code cannot use the symbol itself as a device pointer).  Looked up once per
-// device and looked up again if that device's context has changed since, as
-// after cudaDeviceReset, which reloads the module at a new address.
+// context: after cudaDeviceReset, which unloads the library's device code, the
+// device's context has a new id, though its handle stays the same.
 acid_status scratch_address(void** out) {
   int dev = 0;
   ACID_CUDA(cudaGetDevice(&dev));
   ACID_REQUIRE(dev >= 0 && dev < kMaxDevices, ACID_ERR_UNSUPPORTED, "drift_noalloc: device index too large");
-  auto get_ctx = ctx_get_current();
-  ACID_REQUIRE(get_ctx != nullptr, ACID_ERR_CUDA, "drift_noalloc: cuCtxGetCurrent entry point unavailable");
   std::lock_guard<std::mutex> lk(g_mu);
   ScratchSlot& sl = g_slot[dev];
-  CUcontext ctx = nullptr;
-  if (sl.addr != nullptr && get_ctx(&ctx) == CUDA_SUCCESS && ctx == sl.ctx) {
-    *out = sl.addr;
-    return ACID_OK;
+  const unsigned long long ctx = context_id();
+  if (ctx == 0 || sl.ctx != ctx) {
+    // the lookup also makes the device's context current, so its id is read after it
+    ACID_CUDA(cudaGetSymbolAddress(&sl.addr, g_noalloc_scratch));
+    sl.ctx = context_id();
   }
-  // first call on this device, or its context was replaced: the lookup also
-  // makes the device's primary context current, so the context is read after it
-  void* p = nullptr;
-  ACID_CUDA(cudaGetSymbolAddress(&p, g_noalloc_scratch));
-  ctx = nullptr;
-  ACID_REQUIRE(get_ctx(&ctx) == CUDA_SUCCESS && ctx != nullptr, ACID_ERR_CUDA, "drift_noalloc: no current context");
-  sl.ctx = ctx;
-  sl.addr = p;
-  *out = p;
+  *out = sl.addr;
   return ACID_OK;
 }
 

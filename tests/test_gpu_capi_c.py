@@ -6,7 +6,8 @@ API, links libacid_gb300.so, and checks closed forms.
   elements (a ragged count) gives rel_l1 = 0.25 exactly (every term and
   partial sum is exactly representable), through a host output pointer;
 * cache apply: out = x + r element for element;
-* the zero-denominator reading: rel_l1(0, 0) = 0 and rel_l1(0, c != 0) = inf.
+* the zero-denominator reading: rel_l1(0, 0) = 0 and rel_l1(0, c != 0) = inf;
+* the entry point without a workspace before and after cudaDeviceReset.
 """
 
 import os
@@ -30,7 +31,7 @@ SOURCE = r"""
 #define CHECK(x) do { acid_status st = (x); if (st != ACID_OK) { \
   std::printf("FAIL %s: %d %s\n", #x, (int)st, acid_last_error()); return 1; } } while (0)
 
-static double drift(const std::vector<float>& prev, const std::vector<float>& cur) {
+static double drift(const std::vector<float>& prev, const std::vector<float>& cur, bool noalloc = false) {
   const int64_t n = (int64_t)prev.size();
   float *dp = nullptr, *dc = nullptr;
   void* ws = nullptr;
@@ -40,7 +41,8 @@ static double drift(const std::vector<float>& prev, const std::vector<float>& cu
   cudaMemcpy(dp, prev.data(), n * sizeof(float), cudaMemcpyHostToDevice);
   cudaMemcpy(dc, cur.data(), n * sizeof(float), cudaMemcpyHostToDevice);
   double rel = -3.0;  // host pointer: the call returns with the value written
-  if (acid_drift_signal(dp, dc, n, ACID_FP32, &rel, nullptr, ws, wsb, nullptr) != ACID_OK) rel = -4.0;
+  if (noalloc ? acid_drift_signal_noalloc(dp, dc, n, ACID_FP32, &rel, nullptr, nullptr)
+              : acid_drift_signal(dp, dc, n, ACID_FP32, &rel, nullptr, ws, wsb, nullptr)) rel = -4.0;
   cudaFree(dp);
   cudaFree(dc);
   cudaFree(ws);
@@ -72,6 +74,12 @@ int main() {
   cudaMemcpy(out.data(), dout, n * 4, cudaMemcpyDeviceToHost);
   for (int64_t i = 0; i < n; ++i)
     if (out[i] != cur[i] + r[i]) { std::printf("FAIL cache apply at %lld\n", (long long)i); return 1; }
+  CHECK(acid_check_device_error());
+  const double before = drift(prev, cur, true);
+  if (cudaDeviceReset() != cudaSuccess) { std::printf("FAIL reset\n"); return 1; }
+  const double after = drift(prev, cur, true);
+  std::printf("noalloc %.17g %.17g\n", before, after);
+  if (before != 0.25 || after != 0.25) { std::printf("FAIL noalloc\n"); return 1; }
   CHECK(acid_check_device_error());
   std::printf("launches %lld\n", (long long)acid_launch_count());
   std::printf("OK\n");

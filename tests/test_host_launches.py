@@ -30,10 +30,10 @@ static std::map<const void*, int>& flags() {
 }
 
 extern "C" {
-// what the stand-in answers; a device's context has the device's number + 1
-int fk_pairs = 76, fk_occupancy_error = 0, fk_device = 0, fk_attribute_error = 0;
+// what the stand-in answers; contexts keep their handle over a reset, not their id
+int fk_pairs = 76, fk_occupancy_error = 0, fk_device = 0, fk_attribute_error = 0, fk_resets = 0;
 // what it was asked
-int fk_launches = 0, fk_grid = 0;
+int fk_launches = 0, fk_grid = 0, fk_lookups = 0;
 // device of the memory at 0x2......., its type (cudaMemoryType); copies there, and stores by the drift's final kernel
 int fk_home = 0, fk_type = cudaMemoryTypeDevice, fk_copies = 0, fk_stores = 0;
 #define OUTPUT(p) (((size_t)(p) >> 28) == 2)
@@ -89,11 +89,20 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void
 static CUresult encode(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
                        const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
                        CUtensorMapL2promotion, CUtensorMapFloatOOBfill) { return CUDA_SUCCESS; }
-static CUresult ctx_id(CUcontext, unsigned long long* id) { *id = fk_device + 1; return CUDA_SUCCESS; }
+static CUresult ctx_id(CUcontext, unsigned long long* id) {
+  *id = 2 * fk_resets + fk_device + 1;
+  return CUDA_SUCCESS;
+}
+static CUresult ctx_current(CUcontext* c) { *c = (CUcontext)(size_t)(0x1000 + fk_device); return CUDA_SUCCESS; }
+cudaError_t cudaGetSymbolAddress(void** p, const void*) {
+  *p = (void*)(size_t)(0x30000000 + 0x10000 * ++fk_lookups);
+  return cudaSuccess;
+}
 cudaError_t cudaGetDriverEntryPointByVersion(const char* name, void** fn, unsigned int, unsigned long long,
                                              cudaDriverEntryPointQueryResult* q) {
   *fn = !std::strcmp(name, "cuTensorMapEncodeTiled") ? (void*)encode
         : !std::strcmp(name, "cuCtxGetId")           ? (void*)ctx_id
+        : !std::strcmp(name, "cuCtxGetCurrent")      ? (void*)ctx_current
                                                       : nullptr;
   *q = *fn ? cudaDriverEntryPointSuccess : cudaDriverEntryPointSymbolNotFound;
   return cudaSuccess;
@@ -237,4 +246,16 @@ for f in calls:
         assert (fk.stores, fk.copies) == (stores, 2 - stores), (dev, home, kind, fk.stores, fk.copies)
     fk.device, fk.home, fk.type, fk.copies, fk.stores = 0, 0, 2, 0, 0
     assert f(rel + 4, None) == A.ACID_OK and (fk.stores, fk.copies) == (0, 1)  # not aligned for a double
+""", *libs)
+
+
+def test_scratch_address_after_a_device_reset(libs):
+    """The file-scope scratch array is looked up once in each device's context, and again after a reset."""
+    run("""
+def noalloc(): return lib.acid_drift_signal_noalloc(p[0], p[1], 4096, A.ACID_BF16, 0x20000000, None, None)
+for dev, resets, lookups in ((0, 0, 1), (0, 0, 1), (1, 0, 2), (0, 0, 2), (0, 1, 3), (0, 1, 3), (1, 1, 4), (1, 2, 5)):
+    fk.device = fk.home = dev
+    fk.resets = resets
+    assert noalloc() == A.ACID_OK
+    assert fk.lookups == lookups, (dev, resets, fk.lookups)
 """, *libs)
