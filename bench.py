@@ -44,10 +44,10 @@ MICRO_SIGMA = 1e-2
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum, ncu captures of
 # a self-attention call (whole waves, split last wave and merge) and a
 # cross-attention call (one persistent launch) at this shape, each the mean of
-# two calls) per attention call of the step's 1:1 self/cross mix: 431.5 MB and
-# 158.4 MB.  Valid only for the kernel source it was measured on; any other
+# two calls) per attention call of the step's 1:1 self/cross mix: 432.0 MB and
+# 158.6 MB.  Valid only for the kernel source it was measured on; any other
 # source reports null.
-ATTN_TRAFFIC = {"source_sha256_16": "1f964e9ed980da0c", "bytes_per_launch": (431.50e6 + 158.42e6) / 2}
+ATTN_TRAFFIC = {"source_sha256_16": "a145a415a174bad8", "bytes_per_launch": (432.03e6 + 158.59e6) / 2}
 
 
 def _attn_traffic():
