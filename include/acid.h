@@ -256,7 +256,7 @@ acid_status acid_attention_workspace_size(int32_t head_dim, size_t* bytes);
 
 /* adaLN LayerNorm: y = LN(x) * (1 + scale) + shift per row of x [rows, d]
  * (no affine part, epsilon eps); shift / scale fp32 [d] or both NULL.
- * x and y may have different dtypes (x_dtype, y_dtype). */
+ * x and y may have different dtypes (x_dtype, y_dtype).  All 16-byte aligned. */
 acid_status acid_layernorm_mod(int32_t x_dtype, const void* x, int32_t y_dtype, void* y,
                                int64_t rows, int32_t d, const float* shift, const float* scale,
                                float eps, acid_stream_t stream);

@@ -1196,6 +1196,8 @@ acid_status ln_mod(int in_dtype, const void* x, int out_dtype, void* y, int64_t 
   using H = __nv_bfloat16;
   ACID_REQUIRE(d % 8 == 0 && d <= 3072, ACID_ERR_UNSUPPORTED, "ln_mod: d must be a multiple of 8, <= 3072");
   if (rows == 0) return ACID_OK;
+  ACID_REQUIRE(aligned(shv, 16) && aligned(scv, 16) && aligned(sht, 16) && aligned(sct, 16), ACID_ERR_UNSUPPORTED,
+               "ln_mod: shift and scale must be 16-byte aligned");
   const bool two = scv != nullptr && sht != nullptr && split > 0 && (sht != shv || sct != scv);
   const LnArgs a{x, y, nullptr, nullptr, rows, split, d, scv == nullptr ? 0 : two ? 2 : 1, shv, scv, sht, sct, eps};
   if (in_dtype == ACID_BF16 && out_dtype == ACID_BF16) return ln_mod_types<H, H, kLnPlain>(a, s);
@@ -1292,6 +1294,8 @@ acid_status launch_gemv(const GemvMat& m0, const GemvMat& m1, const float* x, in
 acid_status gemv2(int w_dtype, const void* W, const float* b, float* y, int n_out, const void* W2, const float* b2,
                   float* y2, int n_out2, const float* x, int k, bool silu_input, cudaStream_t s) {
   ACID_REQUIRE(k % 8 == 0 && k <= 16384, ACID_ERR_UNSUPPORTED, "gemv: k must be a multiple of 8, <= 16384");
+  ACID_REQUIRE(aligned(W, 16) && aligned(W2, 16), ACID_ERR_UNSUPPORTED,
+               "gemv: time and modulation weights must be 16-byte aligned");
   const GemvMat m0{W, b, y, n_out}, m1{W2, b2, y2, n_out2};
   return w_dtype == ACID_BF16 ? launch_gemv<__nv_bfloat16>(m0, m1, x, k, silu_input, s)
                               : launch_gemv<float>(m0, m1, x, k, silu_input, s);

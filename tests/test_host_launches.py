@@ -259,3 +259,26 @@ for dev, resets, lookups in ((0, 0, 1), (0, 0, 1), (1, 0, 2), (0, 0, 2), (0, 1, 
     assert noalloc() == A.ACID_OK
     assert fk.lookups == lookups, (dev, resets, fk.lookups)
 """, *libs)
+
+
+def test_vectors_that_wide_loads_cannot_read_are_refused(libs):
+    """The LayerNorm's vectors and the modulation's weights are read 16 bytes at a time: an address that does not allow
+    it is an error before anything is launched."""
+    run("""
+f = lambda sh, sc: lib.acid_layernorm_mod(A.ACID_FP32, p[0], A.ACID_FP32, p[1], 100, 256, sh, sc, 1e-6, None)
+for sh, sc in ((p[2] + 4, p[3]), (p[2], p[3] + 8)):
+    assert f(sh, sc) == A.ACID_ERR_UNSUPPORTED and fk.launches == 0
+assert f(p[2], p[3]) == A.ACID_OK and f(None, None) == A.ACID_OK and fk.launches == 2
+desc = A.acid_block_desc(A.ACID_BLOCK_WAN, A.ACID_FP32, 256, 4, 512, 1, 8, 8, 0, 10000.0, 1e-6)
+n = C.c_size_t()
+assert lib.acid_block_workspace_size(C.byref(desc), C.byref(n)) == A.ACID_OK
+w = A.acid_block_weights()
+for name in ("mod", "qkv", "o", "ff1", "ff2"):
+    setattr(w, name, A.acid_linear(p[5], p[6]))
+cond = A.acid_cond()
+cond.temb = p[7]
+block = lambda: lib.acid_dit_block_forward(C.byref(desc), p[8], C.byref(cond), C.byref(w), p[9], n.value, None)
+assert block() == A.ACID_OK
+w.mod = A.acid_linear(p[5] + 8, p[6])
+assert block() == A.ACID_ERR_UNSUPPORTED
+""", *libs)
